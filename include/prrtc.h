@@ -120,7 +120,8 @@ typedef struct prrtc_robot prrtc_robot;
 
 /* ------------------------------------------------------------ parameters */
 #define PRRTC_MODE_ASYNC 0   /* blocks x warps run Alg. 1 iterations concurrently (Sec. III) */
-#define PRRTC_MODE_SERIAL 1  /* one warp runs the iterations in order: the serial Alg. 1   */
+#define PRRTC_MODE_SERIAL 1  /* the iterations in order: results of the serial Alg. 1 on one
+                                worker (several run side by side where that changes nothing) */
 /* B = params.workers concurrent iterations per round on a fixed schedule (the
  * concurrency of Sec. III made deterministic): in round r, worker b runs
  * iteration r B + b -- sampling, nearest neighbour, pEXTEND and the greedy
@@ -163,9 +164,11 @@ typedef struct prrtc_params {
                              (1 - dd_alpha), not below dd_min_radius, after a collision */
   float dd_min_radius;
   int32_t workers;        /* PRRTC_MODE_LOCKSTEP: concurrent iterations per round, 1..1024
-                             (other modes ignore it); warps_per_block 0 = min(workers, 8)
-                             warps per problem, each running workers / warps iterations
-                             of a round in turn                                       */
+                             (other modes ignore it); warps_per_block 0 = the library
+                             gives each problem as many warps as pay, over several
+                             blocks; else one block of min(workers, warps_per_block)
+                             warps, each running workers / warps iterations of a round
+                             in turn.  The results do not depend on it              */
   int32_t debug_wait_polls;  /* test hook for the bounded device waits; 0 = off.  When > 0, the
                              path extraction of a solved problem first spins, for at most
                              this many polls, on a device flag that nothing sets; the wait

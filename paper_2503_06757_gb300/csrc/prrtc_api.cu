@@ -108,7 +108,8 @@ struct DeviceCtx {
   // CUDA graph of the launch sequence, keyed by everything it bakes in
   struct GraphKey {
     int n, grid, warps, smem, robot_bytes, env_bytes, stage_bytes, max_spheres, max_pairs, max_env, gen, head,
-        lockstep, tile, batch_head, lean;
+        rounds, tile, batch_head, lean;
+    RoundsLaunch rcfg;
     bool operator==(const GraphKey& o) const { return std::memcmp(this, &o, sizeof(GraphKey)) == 0; }
   };
   GraphKey gkey{};
@@ -136,6 +137,7 @@ struct DeviceCtx {
 
 constexpr int kHeadRows = 512;
 constexpr int kBatchHeadRows = 32;
+constexpr size_t kHeldFloats = (size_t)1 << 28;  // held rows of the deterministic schedules: at most 1 GiB
 
 DeviceCtx g_ctx[64];
 std::mutex g_init_mu;
@@ -1037,13 +1039,14 @@ static int plan_batch_impl(const prrtc_problem* problems, int32_t n, const prrtc
     }
     c->gmm_cap = (size_t)n;
   }
-  // lockstep mode: each problem's held rows, [workers][held_rows x dpad].  Every
-  // node lies in the box spanned by the joint limits, the start and the goal
+  // Serial and lockstep mode: rows one iteration can hold back.  Every node
+  // lies in the box spanned by the joint limits, the start and the goal
   // (samples lie in the limits, steps are convex combinations), so a connect
   // takes at most ceil(diagonal / range) steps.
+  const bool ordered = params->mode != PRRTC_MODE_ASYNC;
   std::vector<int> held_rows(n, 0);
-  std::vector<size_t> held_off(n + 1, 0);
-  if (params->mode == PRRTC_MODE_LOCKSTEP) {
+  size_t held_floats = 0;  // per virtual worker, over all problems
+  if (ordered) {
     for (int p = 0; p < n; ++p) {
       const prrtc_problem& pb = problems[p];
       const RobotHeader& H = pb.robot->h->h;
@@ -1053,12 +1056,12 @@ static int plan_batch_impl(const prrtc_problem* problems, int32_t n, const prrtc
         const double hi = std::max({(double)H.lo[j] + (double)H.span[j], (double)pb.q_start[j], (double)pb.q_goal[j]});
         diag2 += (hi - lo) * (hi - lo);
       }
-      held_rows[p] = 3 + (int)std::ceil(std::sqrt(diag2) / (double)params->range * (1.0 + 1e-5));
-      held_off[p + 1] = held_off[p] + (size_t)params->workers * held_rows[p] * H.dpad;
+      const double rows = 3.0 + std::ceil(std::sqrt(diag2) / (double)params->range * (1.0 + 1e-5));
+      held_rows[p] = (int)std::min(rows, 1e9);
+      held_floats += (size_t)held_rows[p] * H.dpad;
     }
-    if (held_off[n] > ((size_t)1 << 28)) return fail(PRRTC_ERR_OOM, "lockstep scratch above 1 GiB");
-    if ((rc = grow_device(&c->d_held, &c->held_cap, held_off[n]))) return rc;
-    if ((rc = grow_device(&c->d_held_meta, &c->held_meta_cap, (size_t)n * params->workers * kHeldMeta))) return rc;
+    if (params->mode == PRRTC_MODE_LOCKSTEP && held_floats * (size_t)params->workers > kHeldFloats)
+      return fail(PRRTC_ERR_OOM, "lockstep scratch above 1 GiB");
   }
   int max_spheres = 1, max_pairs = 0, max_env = 0, max_dof = 1;
   for (int p = 0; p < n; ++p) {
@@ -1088,11 +1091,6 @@ static int plan_batch_impl(const prrtc_problem* problems, int32_t n, const prrtc
     D.key_hi = (uint32_t)(pb.seed >> 32);
     D.pid = pb.problem_id;
     D.gmm = (pb.gmm || (proposals && proposals[p])) ? c->d_gmm + (size_t)p * kGmmStride : nullptr;
-    if (params->mode == PRRTC_MODE_LOCKSTEP) {
-      D.held = c->d_held + held_off[p];
-      D.held_meta = c->d_held_meta + (size_t)p * params->workers * kHeldMeta;
-      D.held_rows = held_rows[p];
-    }
     for (int j = 0; j < H.dof; ++j) {
       D.q_start[j] = pb.q_start[j];
       D.q_goal[j] = pb.q_goal[j];
@@ -1123,9 +1121,29 @@ static int plan_batch_impl(const prrtc_problem* problems, int32_t n, const prrtc
   }
   const PlanLaunch cfg =
       plan_launch_config(n, params->mode, blocks, warps, max_spheres, max_pairs, max_env, c->sms, params->workers);
-  bool lean = params->sampler == PRRTC_SAMPLER_PHILOX && !cfg.lockstep && !(params->dd_radius > 0.f);
+  bool lean = params->sampler == PRRTC_SAMPLER_PHILOX && !(params->dd_radius > 0.f);
   for (int p = 0; p < n && lean; ++p) lean = problem_is_lean(problems[p].robot->h->h, c->h_desc[p]);
   if (cfg.smem > 227 * 1024) return fail(PRRTC_ERR_UNSUPPORTED, "robot + environment exceed shared memory");
+  // The deterministic schedules run in rounds.  A serial batch whose held rows
+  // would take more than a quarter of the lockstep limit (a tiny range over
+  // many problems) keeps to one warp a problem, which holds no rows.
+  const size_t held_limit = params->mode == PRRTC_MODE_LOCKSTEP ? kHeldFloats : kHeldFloats / 4;
+  const bool rounds =
+      params->mode == PRRTC_MODE_LOCKSTEP || (ordered && held_floats * (size_t)kRoundsWarps <= held_limit);
+  RoundsLaunch rcfg{};
+  if (rounds) {
+    rcfg = rounds_launch_config(cfg, n, params->mode, blocks, warps, params->workers, held_floats, held_limit, c->sms);
+    if ((rc = grow_device(&c->d_held, &c->held_cap, held_floats * (size_t)rcfg.workers))) return rc;
+    if ((rc = grow_device(&c->d_held_meta, &c->held_meta_cap, (size_t)n * rcfg.workers * kHeldMeta))) return rc;
+    size_t off = 0;
+    for (int p = 0; p < n; ++p) {
+      ProblemDesc& D = c->h_desc[p];
+      D.held = c->d_held + off;
+      D.held_meta = c->d_held_meta + (size_t)p * rcfg.workers * kHeldMeta;
+      D.held_rows = held_rows[p];
+      off += (size_t)rcfg.workers * held_rows[p] * D.dpad;
+    }
+  }
   const int head_rows = (n == 1) ? std::min(kHeadRows, params->path_capacity) : 0;
   // A batch copies the first rows of every path back with its results; only a
   // longer path needs the gather after the results are read.
@@ -1221,7 +1239,8 @@ static int plan_batch_impl(const prrtc_problem* problems, int32_t n, const prrtc
         launch_setup(c->d_desc, c->d_state, n, max_spheres, max_pairs, max_env, c->stream, nullptr, &c->d_glob->error);
     if (e != cudaSuccess) return cuda_fail("setup launch", e);
     CK(cudaEventRecordWithFlags(c->ev[1], c->stream, ev_flags));
-    e = launch_plan(c->d_glob, c->d_desc, c->d_state, cfg, G.obstacle_tile, lean, c->stream);
+    e = rounds ? launch_rounds(c->d_glob, c->d_desc, c->d_state, rcfg, lean, c->stream)
+               : launch_plan(c->d_glob, c->d_desc, c->d_state, cfg, G.obstacle_tile, lean, c->stream);
     if (e != cudaSuccess) return cuda_fail("plan launch", e);
     CK(cudaEventRecordWithFlags(c->ev[2], c->stream, ev_flags));
     e = launch_record_usage(c->d_desc, c->d_state, n, c->stream);
@@ -1245,7 +1264,7 @@ static int plan_batch_impl(const prrtc_problem* problems, int32_t n, const prrtc
   } else {
     const DeviceCtx::GraphKey key{n, cfg.grid, cfg.warps, cfg.smem, cfg.robot_bytes, cfg.env_bytes, cfg.stage_bytes,
                                   max_spheres, max_pairs, max_env, c->arena_gen, head_rows * c->h_desc[0].dof,
-                                  cfg.lockstep ? 1 : 0, G.obstacle_tile, head_stride, lean ? 1 : 0};
+                                  rounds ? 1 : 0, G.obstacle_tile, head_stride, lean ? 1 : 0, rcfg};
     if (!c->gexec || !(c->gkey == key)) {
       if (c->gexec) cudaGraphExecDestroy(c->gexec);
       c->gexec = nullptr;
@@ -1345,16 +1364,16 @@ static int plan_batch_impl(const prrtc_problem* problems, int32_t n, const prrtc
   for (prrtc_proposal* prop : staged) L.infer_ms += prrtc_internal_proposal_infer_ms(prop);
   L.kernel_ms = plan_ms;
   L.setup_ms = setup_ms;
-  L.grid = cfg.grid;
-  L.block_threads = cfg.warps * 32;
-  L.smem_bytes = cfg.smem;
+  L.grid = rounds ? rcfg.ph[0].grid : cfg.grid;
+  L.block_threads = (rounds ? rcfg.warps : cfg.warps) * 32;
+  L.smem_bytes = rounds ? rcfg.smem : cfg.smem;
   L.problems = n;
   L.h2d_bytes = (int64_t)n * (int64_t)sizeof(ProblemDesc) + (int64_t)sizeof(PlanGlobals) +
                 (gathered ? (int64_t)(n + 1) * (int64_t)sizeof(int) : 0);
   L.d2h_bytes = (int64_t)n * (int64_t)sizeof(ProblemState) + (int64_t)sizeof(PlanGlobals) +
                 ((int64_t)head_rows * c->h_desc[0].dof + (int64_t)n * head_stride + (gathered ? total : 0)) *
                     (int64_t)sizeof(float);
-  L.kernels = 3 + (batch_head ? 1 : 0) + (gathered ? 1 : 0);
+  L.kernels = 2 + (rounds ? rcfg.n_phases : 1) + (batch_head ? 1 : 0) + (gathered ? 1 : 0);
   L.lean_kernel = lean ? 1 : 0;
   const unsigned long long t0 = c->h_glob->t0;
   for (int p = 0; p < n; ++p) {

@@ -31,6 +31,7 @@ struct PlanGlobals {
   unsigned long long t0;             // launch start (min over blocks, %globaltimer ns)
   unsigned long long time_limit_ns;  // 0 = none
   int cursor;            // work-queue ticket counter
+  int queue[3];          // the same, one per launch of the deterministic schedules
   int error;             // device-side error code (PRRTC_ERR_*), 0 = none
   int error_info;
   uint32_t learned_thr;  // learned-vs-uniform draw as a threshold on the top 24 bits of a Philox word
@@ -99,7 +100,7 @@ struct ProblemDesc {
   uint32_t key_lo, key_hi;
   uint32_t pid;
   const float* gmm;      // learned mixture (kGmmStride floats, device) or null
-  // lockstep mode: the rows each worker of a round holds back, [workers][held_rows * dpad],
+  // serial and lockstep mode: the rows each virtual worker holds back, [workers][held_rows * dpad],
   // and per worker kHeldMeta ints (see LockstepHeld in prrtc_plan.cu); null otherwise
   float* held;
   int* held_meta;
@@ -162,25 +163,65 @@ cudaError_t launch_setup(const ProblemDesc* desc, ProblemState* state, int n, in
 struct PlanLaunch {
   int grid;
   int warps;
-  bool lockstep;         // lockstep_kernel (PRRTC_MODE_LOCKSTEP) instead of plan_kernel
   int smem;
   int robot_bytes;
   int env_bytes;
   int stage_bytes;
 };
 
+// Launches of the deterministic schedules (serial and lockstep mode): up to
+// three in a row, with growing clusters of blocks per problem.
+struct RoundsLaunch {
+  int warps;             // per block
+  int smem;
+  int robot_bytes;
+  int env_bytes;
+  int stage_bytes;
+  int workers;           // virtual workers of the largest cluster: slices of a problem's held rows
+  int n_phases;
+  struct Phase {
+    int blocks;          // blocks of a cluster, which runs one problem
+    int grid;
+    int it_limit;        // a problem with this many iterations is left to the next launch
+  } ph[3];
+};
+// Easy problems are solved within a few rounds of 16 workers and rarely let a
+// round of more of them count (one iteration in seven adds a row); the few
+// hard ones, which set the batch's time, add a row in a hundred iterations or
+// more and take all the workers they get.  So each launch gives what the one
+// before left a larger cluster.  Kernel time of four sets of 200 shelf
+// problems (ms; one warp a problem: 121, 270, 33, 160):
+//   16 warps, clusters 1 / 4 / 16, 256 / 1024 iterations   3.3  5.1  3.3  5.5
+//   16 warps, clusters 1 / 16, 256                          3.5  5.6  4.2  5.6
+//   16 warps, clusters 1 / 4 / 8                            4.1  6.7  3.0  8.3
+//   16 warps, clusters 1 / 4 / 16, 64 / 256                 4.1  6.4  4.8  6.3
+//    8 warps, clusters 1 / 4 / 16, 256 / 1024               3.8  6.3  2.8  7.5
+//    8 warps, clusters 1 / 4 / 8, 256 / 1024                5.3  9.7  3.1 12.9
+constexpr int kRoundsWarps = 16;
+constexpr int kRoundsSmem = 226 * 1024;
+constexpr int kRoundsMidCluster = 4, kRoundsMaxCluster = 16;
+constexpr int kRoundsFirstIters = 256, kRoundsMidIters = 1024;
+
+// base: the launch of plan_launch_config for the same arguments.  held_floats:
+// floats of held rows per virtual worker, over all problems; held_limit: the
+// most that may be allocated.
+RoundsLaunch rounds_launch_config(const PlanLaunch& base, int n_problems, int mode, int blocks, int warps, int workers,
+                                  size_t held_floats, size_t held_limit, int sm_count);
+
 // workers: the lockstep round size (PRRTC_MODE_LOCKSTEP), else ignored.
 PlanLaunch plan_launch_config(int n_problems, int mode, int blocks, int warps, int max_spheres, int max_pairs,
                               int max_env_f4, int sm_count, int workers = 1);
 
-// obstacle_tile: 64 launches the 64-obstacle-tile instance of the async/serial
-// kernel, anything else the 32 one (lockstep always uses 32).  lean: the
+// obstacle_tile: 64 launches the 64-obstacle-tile instance of the kernel,
+// anything else the 32 one.  lean: the
 // instance without the learned mixture draw, the Halton sampler, distance
 // fields, oriented boxes and one-stage links; only for batches that use none of
 // them
 // (problem_is_lean).
 cudaError_t launch_plan(const PlanGlobals* g, const ProblemDesc* desc, ProblemState* state, const PlanLaunch& cfg,
                         int obstacle_tile, bool lean, cudaStream_t stream);
+cudaError_t launch_rounds(const PlanGlobals* g, const ProblemDesc* desc, ProblemState* state, const RoundsLaunch& cfg,
+                          bool lean, cudaStream_t stream);
 
 // Whether the lean planner instance serves a problem: no mixture, no distance
 // field, at least one primitive and no oriented box, a bounding sphere on every

@@ -15,8 +15,9 @@
 //     writes the parent, fences, then the coordinates.  Readers scan with L2
 //     loads and skip rows whose distance is NaN, so a row is used only once
 //     all its coordinates are final (each word changes NaN -> value once).
-//   * Serial mode runs one worker per problem; it performs exactly the
-//     iterations of the serial Alg. 1 in order.
+//   * Serial and lockstep mode run rounds of iterations on a fixed schedule,
+//     several rounds side by side where the trees stay as they are (see
+//     "rounds" below); their results are those of the iterations in order.
 #include <algorithm>
 #include <cfloat>
 #include <climits>
@@ -613,13 +614,30 @@ __device__ void worker(const Ctx& c) {
   }
 }
 
-// ------------------------------------------------------------------ lockstep rounds
-// The concurrency of Sec. III on a fixed schedule (PRRTC_MODE_LOCKSTEP): in
-// round r, worker b runs iteration r B + b against the trees as they stood
-// when the round began, holding its new rows back in its slice of D->held;
-// at the end of the round the rows are appended in worker order and the
-// connected worker that checked the fewest edges (ties: lowest b) wins.
-// Virtual worker b runs on warp b % warps of the problem's block.
+// ------------------------------------------------------------------ rounds
+// The deterministic schedules.  Lockstep (PRRTC_MODE_LOCKSTEP): in round r,
+// worker b runs iteration r B + b against the trees as they stood when the
+// round began, holding its new rows back in its slice of D->held; at the end
+// of the round the rows are appended in worker order and the connected worker
+// that checked the fewest edges (ties: lowest b) wins.  Serial mode is the
+// case B = 1.
+//
+// A round that adds no row and changes no radius leaves the trees as they
+// were, so the round after it would have read the same trees.  A batch
+// therefore runs R rounds side by side against one snapshot, iteration
+// it0 + v on virtual worker v; at its end the rounds are taken in order up to
+// and including the first that changed something, and the iterations after it
+// are run again in the next batch.  Results and counters are those of one
+// round at a time: the discarded iterations leave nothing behind.
+//
+// What bounds a round is the latency of one edge check (about 9 us for a warp
+// alone on its SM), and on hard problems hundreds of rounds in a row add
+// nothing (14,160 iterations for 21 rows in one shelf problem).  200 shelf
+// problems: serial 268 -> 5.3 ms a call (one warp a problem before), lockstep
+// with 8 workers 40 -> 4.1 ms (one block a problem, one round at a time).
+//
+// Virtual worker v runs on warp v / C of block v % C of the problem's cluster
+// of C blocks.
 
 // One worker's record for a round (kHeldMeta ints of D->held_meta).
 struct LockstepHeld {
@@ -634,9 +652,15 @@ struct LockstepHeld {
 };
 static_assert(sizeof(LockstepHeld) == kHeldMeta * sizeof(int), "lockstep record layout");
 
+__device__ __forceinline__ LockstepHeld load_held(const LockstepHeld* h) {
+  const int4 a = __ldcg(reinterpret_cast<const int4*>(h)), b = __ldcg(reinterpret_cast<const int4*>(h) + 1);
+  return LockstepHeld{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+}
+
 // Alg. 1 lines 4-15 of iteration `it` against T_s = tree s (its first n_s
 // rows) and T_o (its first n_o rows); new rows go to `rows` (held_rows x
 // dpad), the outcome to *h (written by lane 0).
+template <bool kLean>
 __device__ void lockstep_iteration(const Ctx& c, int it, int s, int n_s, int n_o, LockstepHeld* h, float* rows) {
   const PlanGlobals* g = c.g;
   const ProblemDesc* D = c.D;
@@ -644,12 +668,12 @@ __device__ void lockstep_iteration(const Ctx& c, int it, int s, int n_s, int n_o
   const int o = 1 - s;
   const bool mine = lane < dpad;
   const float range = g->range, res = g->resolution;
-  const bool dd = g->dd_radius > 0.f;
+  const bool dd = !kLean && g->dd_radius > 0.f;  // lean batches have it off
   int n = 0, nn = -1, nno = -1, connected = 0, edges = 0, dd_node = -1, dd_free = 0;
   if (lane == 0) c.cnt->iterations++;
   do {
     bool goal_sample;
-    const float crand = random_config<false>(c, it, o, &goal_sample);
+    const float crand = random_config<kLean>(c, it, o, &goal_sample);
     if (mine) c.v.rnd[lane] = crand;
     __syncwarp();
     // line 5: nearest node of T_s as the round found it
@@ -682,7 +706,7 @@ __device__ void lockstep_iteration(const Ctx& c, int it, int s, int n_s, int n_o
     float ct = 0.f, Dd = 0.f, bval = cnew;
     int n_ext = 0;
     for (int phase = 0;; ++phase) {
-      const bool free_edge = edge_free<32, false>(c, N);  // lockstep: 32-obstacle tiles
+      const bool free_edge = edge_free<32, kLean>(c, N);  // 32-obstacle tiles
       ++edges;
       if (phase == 0 && dd) {
         dd_node = nn;
@@ -727,89 +751,194 @@ __device__ void lockstep_iteration(const Ctx& c, int it, int s, int n_s, int n_o
     }
   } while (false);
   __syncwarp();
-  if (lane == 0) {
-    h->n = n;
-    h->nn = nn;
-    h->nno = nno;
-    h->connected = connected;
-    h->edges = edges;
-    h->dd_node = dd_node;
-    h->dd_free = dd_free;
+  if (lane == 0) {  // read by another SM's block when the problem has a cluster
+    __stcg(reinterpret_cast<int4*>(h), make_int4(n, nn, nno, connected));
+    __stcg(reinterpret_cast<int4*>(h) + 1, make_int4(edges, dd_node, dd_free, 0));
   }
   __syncwarp();
 }
 
-// Rounds of one problem by every warp of the block (block-uniform control
-// flow: every thread meets every barrier).
-__device__ void lockstep_problem(const Ctx& c, int warp, int nwarps) {
-  __shared__ int s_it0, s_s, s_ns, s_no, s_stop, s_nb, s_winner, s_total;
+// A warp's counters into its problem.
+__device__ __forceinline__ void flush_counters(ProblemState* S, const WarpCount& w, int lane) {
+  if (lane >= 14) return;
+  unsigned long long* dst[14] = {&S->sphere_tests, &S->pair_tests,  &S->fk_states,     &S->prim_tests[0],
+                                 &S->prim_tests[1], &S->prim_tests[2], &S->prim_tests[3], &S->edges,
+                                 &S->edge_states,  &S->nn_nodes,    &S->iterations,    &S->insert_fail,
+                                 &S->dd_rejected,  &S->verdict_states};
+  const unsigned long long val = reinterpret_cast<const unsigned long long*>(&w)[lane];
+  if (val) atomicAdd(dst[lane], val);
+}
+
+// What the leading block tells its cluster about the next batch; kept in its
+// shared memory and read by every warp after the cluster barrier.
+struct RoundCtl {
+  int stop;        // 1: leave the problem
+  int it0;         // first iteration of the batch
+  int s, n_s, n_o; // tree extended by every iteration, and the trees' rows
+  int nb;          // iterations of the batch
+  int committed;   // iterations of the batch before that count
+  int prob;        // problem to run, -1: none left
+};
+static_assert(sizeof(RoundCtl) == 8 * sizeof(int), "one int per lane");
+
+// Barrier over the problem's blocks; global and shared writes before it are
+// visible after it.
+__device__ __forceinline__ void cluster_barrier(int blocks) {
+  if (blocks == 1) {
+    __syncthreads();
+    return;
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Word `lane` (lane < 8) of the leading block's control record.
+__device__ __forceinline__ int ctl_word(const RoundCtl* ctl, int lane) {
+  int v = 0;
+  if (lane < 8) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;"
+                 : "=r"(remote)
+                 : "r"(smem_u32(reinterpret_cast<const int*>(ctl) + lane)));
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(remote) : "memory");
+  }
+  return v;
+}
+
+// The next batch of the problem, by lane 0 of the leading warp.
+__device__ __forceinline__ void plan_batch(PlanGlobals* g, const ProblemDesc* D, ProblemState* S, int it_limit,
+                                           int workers, RoundCtl* ctl) {
+  int stop = ld_volatile(&S->done) | ld_volatile(&S->solved) | (slice_over(g) ? 1 : 0);
+  const int it0 = ld_volatile(&S->iter);
+  if (!stop && it0 >= g->max_iters) {
+    atomicExch(&S->done, 1);
+    stop = 1;
+  }
+  if (!stop && g->time_limit_ns && globaltimer_ns() - g->t0 > g->time_limit_ns) {
+    S->timed_out = 1;
+    atomicExch(&S->done, 1);
+    stop = 1;
+  }
+  if (it0 >= it_limit) stop = 1;  // the next launch takes it from here
+  // line 3 at the start of the round: every worker extends the smaller tree
+  const int na = min(ld_volatile(&S->count[0]), D->cap), nb = min(ld_volatile(&S->count[1]), D->cap);
+  ctl->stop = stop;
+  ctl->it0 = it0;
+  ctl->s = (na <= nb) ? 0 : 1;
+  ctl->n_s = min(na, nb);
+  ctl->n_o = max(na, nb);
+  ctl->nb = min(workers, g->max_iters - it0);
+}
+
+// Batches of one problem by every warp of its cluster (uniform control flow:
+// every thread meets every barrier).  `total`: this warp's counters, to which
+// an iteration's counters (c.cnt) are added once it counts.
+template <bool kLean>
+__device__ __forceinline__ void rounds_problem(const Ctx& c, WarpCount* total, RoundCtl* ctl, int rank, int blocks,
+                                               int warp, int nwarps, int it_limit) {
+  __shared__ int s_first, s_winner, s_total;  // the leading block's: round to append, its winner and rows
   PlanGlobals* g = const_cast<PlanGlobals*>(c.g);
   const ProblemDesc* D = c.D;
   ProblemState* S = c.S;
   LockstepHeld* meta = reinterpret_cast<LockstepHeld*>(D->held_meta);
   const int B = g->workers, dpad = D->dpad, cap = D->cap, lane = c.lane;
+  const int slots = blocks * nwarps;             // warps of the cluster
+  const int batch = max(slots / B, 1) * B;       // virtual workers: whole rounds
+  const int me = warp * blocks + rank;
   const size_t held_stride = (size_t)D->held_rows * dpad;
+  unsigned long long* acc = reinterpret_cast<unsigned long long*>(total);
+  unsigned long long* one = reinterpret_cast<unsigned long long*>(c.cnt);
+  if (rank == 0 && threadIdx.x == 0) {
+    plan_batch(g, D, S, it_limit, batch, ctl);
+    ctl->committed = 0;
+  }
+  int ran = 0;  // iterations this warp ran in the batch before
   for (;;) {
-    if (threadIdx.x == 0) {
-      int stop = ld_volatile(&S->done) | ld_volatile(&S->solved) | (slice_over(g) ? 1 : 0);
-      const int it0 = S->iter;
-      if (!stop && it0 >= g->max_iters) {
-        atomicExch(&S->done, 1);
-        stop = 1;
-      }
-      if (!stop && g->time_limit_ns && globaltimer_ns() - g->t0 > g->time_limit_ns) {
-        S->timed_out = 1;
-        atomicExch(&S->done, 1);
-        stop = 1;
-      }
-      // line 3 at the start of the round: every worker extends the smaller tree
-      const int na = min(S->count[0], cap), nb = min(S->count[1], cap);
-      s_s = (na <= nb) ? 0 : 1;
-      s_ns = s_s ? nb : na;
-      s_no = s_s ? na : nb;
-      s_it0 = it0;
-      s_nb = min(B, g->max_iters - it0);
-      s_stop = stop;
+    cluster_barrier(blocks);
+    const int word = ctl_word(ctl, lane);
+    // the iterations of the batch before count, or are forgotten
+    if (ran && me < __shfl_sync(kFull, word, 6)) {
+      if (lane < 14) acc[lane] += one[lane];
     }
-    __syncthreads();
-    if (s_stop) break;
-    const int it0 = s_it0, s = s_s, n_s = s_ns, n_o = s_no, nb = s_nb;
-    for (int b = warp; b < nb; b += nwarps)
-      lockstep_iteration(c, it0 + b, s, n_s, n_o, meta + b, D->held + (size_t)b * held_stride);
-    __syncthreads();
-    // end of the round: radius updates and row offsets in worker order, the winner
-    if (threadIdx.x == 0) {
-      float* rad = D->radius[s];
-      int total = 0, winner = -1;
-      for (int b = 0; b < nb; ++b) {
-        LockstepHeld& h = meta[b];
-        if (h.dd_node >= 0) {
-          const float r = __ldcg(rad + h.dd_node);
-          if (h.dd_free) {
-            if (!isnan(r)) __stcg(rad + h.dd_node, r * (1.f + g->dd_alpha));
-          } else {
-            __stcg(rad + h.dd_node, isnan(r) ? g->dd_radius : fmaxf(r * (1.f - g->dd_alpha), g->dd_min_radius));
+    warp_count_clear(c.cnt, lane);
+    if (__shfl_sync(kFull, word, 0)) break;
+    const int it0 = __shfl_sync(kFull, word, 1), s = __shfl_sync(kFull, word, 2), n_s = __shfl_sync(kFull, word, 3);
+    const int n_o = __shfl_sync(kFull, word, 4), nb = __shfl_sync(kFull, word, 5);
+    ran = me < nb ? 1 : 0;
+    // a warp has several virtual workers only where the batch is one round, all of which count
+    for (int v = me; v < nb; v += slots)
+      lockstep_iteration<kLean>(c, it0 + v, s, n_s, n_o, meta + v, D->held + (size_t)v * held_stride);
+    if (lane == 0) __threadfence();
+    cluster_barrier(blocks);
+    if (rank != 0) continue;
+    // The leading block takes the rounds in order.
+    if (warp == 0) {
+      int first = INT_MAX;  // first worker that changed something
+      for (int v = lane; v < nb; v += 32) {
+        const LockstepHeld h = load_held(meta + v);
+        if (h.n > 0 || h.dd_node >= 0) first = min(first, v);
+      }
+      first = __reduce_min_sync(kFull, first);
+      int committed = nb, winner = -1, sum = 0;
+      if (first != INT_MAX) {
+        first = first / B * B;  // its round
+        committed = min(first + B, nb);
+        float* rad = D->radius[s];
+        if (!kLean && g->dd_radius > 0.f && lane == 0) {  // radius updates in worker order
+          for (int v = first; v < committed; ++v) {
+            const LockstepHeld h = load_held(meta + v);
+            if (h.dd_node < 0) continue;
+            const float r = __ldcg(rad + h.dd_node);
+            if (h.dd_free) {
+              if (!isnan(r)) __stcg(rad + h.dd_node, r * (1.f + g->dd_alpha));
+            } else {
+              __stcg(rad + h.dd_node, isnan(r) ? g->dd_radius : fmaxf(r * (1.f - g->dd_alpha), g->dd_min_radius));
+            }
           }
         }
-        h.offset = total;
-        total += h.n;
-        const bool all_in = n_s + total <= cap;
-        if (h.connected && all_in && (winner < 0 || h.edges < meta[winner].edges)) winner = b;
+        // row offsets in worker order, and the winner among the workers whose rows all fit
+        unsigned long long best = ~0ull;
+        for (int base = first; base < committed; base += 32) {
+          const int v = base + lane;
+          const bool in = v < committed;
+          const LockstepHeld h = in ? load_held(meta + v) : LockstepHeld{};
+          int end = h.n;  // inclusive prefix sum
+#pragma unroll
+          for (int off = 1; off < 32; off <<= 1) {
+            const int up = __shfl_up_sync(kFull, end, off);
+            if (lane >= off) end += up;
+          }
+          end += sum;
+          if (in) __stcg(&meta[v].offset, end - h.n);
+          if (in && h.connected && n_s + end <= cap)
+            best = min(best, ((unsigned long long)(uint32_t)h.edges << 32) | (uint32_t)v);
+          sum = __shfl_sync(kFull, end, 31);
+        }
+#pragma unroll
+        for (int off = 16; off; off >>= 1) best = min(best, __shfl_xor_sync(kFull, best, off));
+        winner = best == ~0ull ? -1 : (int)(uint32_t)best;
       }
-      s_total = total;
-      s_winner = winner;
-      S->iter = it0 + nb;
+      if (lane == 0) {
+        s_first = first;
+        s_winner = winner;
+        s_total = sum;
+        S->iter = it0 + committed;
+        ctl->committed = committed;
+        if (first == INT_MAX || sum == 0) plan_batch(g, D, S, it_limit, batch, ctl);
+      }
     }
     __syncthreads();
-    // append the held rows: row k of worker b at n_s + offset + k, hanging
+    if (s_first == INT_MAX || s_total == 0) continue;
+    // append the held rows: row k of worker v at n_s + offset + k, hanging
     // from the worker's previous row (k > 0) or its snapshot row nn
-    for (int b = warp; b < nb; b += nwarps) {
-      const LockstepHeld h = meta[b];
-      const float* src = D->held + (size_t)b * held_stride;
+    const int committed = ctl->committed;
+    for (int v = s_first + warp; v < committed; v += nwarps) {
+      const LockstepHeld h = load_held(meta + v);
+      const float* src = D->held + (size_t)v * held_stride;
       for (int k = 0; k < h.n; ++k) {
         const int idx = n_s + h.offset + k;
         if (idx >= cap) {
-          if (lane == 0) c.cnt->insert_fail++;
+          if (lane == 0) total->insert_fail++;
           break;
         }
         if (lane == 0) __stcg(D->parent[s] + idx, k == 0 ? h.nn : idx - 1);
@@ -818,12 +947,11 @@ __device__ void lockstep_problem(const Ctx& c, int warp, int nwarps) {
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) S->count[s] = min(n_s + s_total, cap);
-    __syncthreads();
-    const int w = s_winner;
-    if (w >= 0) {
-      if (warp == 0) {
-        const LockstepHeld h = meta[w];
+    if (warp == 0) {
+      const int w = s_winner;
+      if (lane == 0) S->count[s] = min(n_s + s_total, cap);
+      if (w >= 0) {
+        const LockstepHeld h = load_held(meta + w);
         const int join_s = n_s + h.offset + h.n - 1;
         if (lane == 0) {
           S->solved = 1;
@@ -832,15 +960,100 @@ __device__ void lockstep_problem(const Ctx& c, int warp, int nwarps) {
           S->join_s = join_s;
           S->join_o = h.nno;
         }
+        __threadfence();
         __syncwarp();
         extract_path(c, s, join_s, h.nno);
         __threadfence();
         if (lane == 0) atomicExch(&S->done, 1);
       }
-      __syncthreads();
-      break;
+      if (lane == 0) {
+        __threadfence();
+        plan_batch(g, D, S, it_limit, batch, ctl);
+      }
     }
   }
+}
+
+// The launch of the deterministic schedules: clusters of `blocks` blocks take
+// problems from the work queue, stage the problem's robot and environment in
+// each block's shared memory (plain loads: once a problem) and run its
+// batches.  A problem that reaches it_limit iterations is left to the next
+// launch of the call, which gives it a larger cluster.
+template <bool kLean>
+__global__ void __maxnreg__(128) rounds_kernel(PlanGlobals* __restrict__ g, const ProblemDesc* __restrict__ descs,
+                                               ProblemState* __restrict__ states, int robot_bytes, int env_bytes,
+                                               int warp_floats, int blocks, int queue, int it_limit) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ __align__(16) RoundCtl ctl;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int rank = (int)blockIdx.x % blocks;
+  const RobotDev* my_robot = nullptr;
+  const float4* my_env = nullptr;
+  if (threadIdx.x == 0) atomicMin(&g->t0, globaltimer_ns());
+  for (;;) {
+    if (rank == 0 && threadIdx.x == 0) {
+      int p = -1;
+      for (;;) {
+        const int t = atomicAdd(&g->queue[queue], 1);
+        if (t >= g->n_problems) break;
+        p = g->active ? g->active[t] : t;
+        if (!ld_volatile(&states[p].done)) break;
+        p = -1;
+      }
+      ctl.prob = p;
+    }
+    cluster_barrier(blocks);
+    const int p = __shfl_sync(kFull, ctl_word(&ctl, lane), 7);
+    if (p < 0) break;
+    const ProblemDesc* D = descs + p;
+    const int np_pad = (D->n_pairs + 3) & ~3;
+    RobotHeader* R = reinterpret_cast<RobotHeader*>(smem);
+    uint32_t* pair = reinterpret_cast<uint32_t*>(smem + sizeof(RobotHeader));
+    float* thr = reinterpret_cast<float*>(pair + np_pad);
+    float4* senv = reinterpret_cast<float4*>(smem + robot_bytes);
+    auto copy16 = [&](void* dst, const void* src, int bytes) {
+      for (int k = threadIdx.x; k < bytes / 16; k += blockDim.x)
+        reinterpret_cast<float4*>(dst)[k] = __ldg(reinterpret_cast<const float4*>(src) + k);
+    };
+    if (my_robot != D->robot) {
+      copy16(R, &D->robot->h, (int)sizeof(RobotHeader));
+      copy16(pair, D->robot->pair, 4 * np_pad);
+      copy16(thr, D->robot->thr, 4 * np_pad);
+      my_robot = D->robot;
+    }
+    if (my_env != D->env.data) {
+      copy16(senv, D->env.data, 16 * D->env.n_float4());
+      my_env = D->env.data;
+    }
+    __syncthreads();
+    Ctx c;
+    c.g = g;
+    c.D = D;
+    c.S = states + p;
+    c.R = R;
+    c.pair = pair;
+    c.thr = thr;
+    c.env = senv;
+    // per-warp area: counters of the running iterations and of those that
+    // count (128 B each), the three vectors, sphere-centre staging
+    float* warp_area = reinterpret_cast<float*>(smem + robot_bytes + env_bytes) + warp * warp_floats;
+    c.cnt = reinterpret_cast<WarpCount*>(warp_area);
+    WarpCount* total = c.cnt + 1;
+    warp_count_clear(c.cnt, lane);
+    warp_count_clear(total, lane);
+    float* vecs = warp_area + 2 * kCountFloats;
+    c.v.rnd = vecs;
+    c.v.a = vecs + kMaxDof;
+    c.v.b = vecs + 2 * kMaxDof;
+    c.stage = vecs + kWarpVecFloats;
+    c.lane = lane;
+    rounds_problem<kLean>(c, total, &ctl, rank, blocks, warp, nwarps, it_limit);
+    __syncwarp();
+    flush_counters(states + p, *total, lane);
+    // every block has read the last control record before it is written again
+    cluster_barrier(blocks);
+  }
+  cluster_barrier(blocks);  // the leading block's shared memory outlives its readers
 }
 
 __device__ int pick_problem(PlanGlobals* g, const ProblemState* states) {
@@ -857,9 +1070,9 @@ __device__ int pick_problem(PlanGlobals* g, const ProblemState* states) {
 }
 
 // The planner launch: blocks take problems from the work queue, stage each
-// problem's robot and environment in shared memory and run its workers --
-// independent warps (async and serial modes) or the lockstep rounds.
-template <bool kLockstep, int kTile, bool kLean>
+// problem's robot and environment in shared memory and run its workers, one
+// independent warp each.
+template <int kTile, bool kLean>
 __device__ __forceinline__ void plan_body(PlanGlobals* __restrict__ g, const ProblemDesc* __restrict__ descs,
                                           ProblemState* __restrict__ states, int robot_bytes, int env_bytes,
                                           int warp_floats) {
@@ -938,22 +1151,9 @@ __device__ __forceinline__ void plan_body(PlanGlobals* __restrict__ g, const Pro
     c.v.b = vecs + 2 * kMaxDof;
     c.stage = vecs + kWarpVecFloats;
     c.lane = lane;
-    if constexpr (kLockstep)
-      lockstep_problem(c, warp, blockDim.x >> 5);
-    else
-      worker<kTile, kLean>(c);
-    // flush this warp's counters into the problem
+    worker<kTile, kLean>(c);
     __syncwarp();
-    if (lane < 14) {
-      ProblemState* S = states + p;
-      const WarpCount& w = *c.cnt;
-      unsigned long long* dst[14] = {&S->sphere_tests, &S->pair_tests,  &S->fk_states,     &S->prim_tests[0],
-                                     &S->prim_tests[1], &S->prim_tests[2], &S->prim_tests[3], &S->edges,
-                                     &S->edge_states,  &S->nn_nodes,    &S->iterations,    &S->insert_fail,
-                                     &S->dd_rejected,  &S->verdict_states};
-      const unsigned long long val = reinterpret_cast<const unsigned long long*>(&w)[lane];
-      if (val) atomicAdd(dst[lane], val);
-    }
+    flush_counters(states + p, *c.cnt, lane);
     __syncthreads();
   }
 }
@@ -969,18 +1169,12 @@ template <int kTile, bool kLean>
 __global__ void __maxnreg__(128) plan_kernel(PlanGlobals* __restrict__ g, const ProblemDesc* __restrict__ descs,
                                              ProblemState* __restrict__ states, int robot_bytes, int env_bytes,
                                              int warp_floats) {
-  plan_body<false, kTile, kLean>(g, descs, states, robot_bytes, env_bytes, warp_floats);
+  plan_body<kTile, kLean>(g, descs, states, robot_bytes, env_bytes, warp_floats);
 }
 template __global__ void plan_kernel<32, false>(PlanGlobals*, const ProblemDesc*, ProblemState*, int, int, int);
 template __global__ void plan_kernel<64, false>(PlanGlobals*, const ProblemDesc*, ProblemState*, int, int, int);
 template __global__ void plan_kernel<32, true>(PlanGlobals*, const ProblemDesc*, ProblemState*, int, int, int);
 template __global__ void plan_kernel<64, true>(PlanGlobals*, const ProblemDesc*, ProblemState*, int, int, int);
-
-__global__ void __maxnreg__(128) lockstep_kernel(PlanGlobals* __restrict__ g, const ProblemDesc* __restrict__ descs,
-                                                 ProblemState* __restrict__ states, int robot_bytes, int env_bytes,
-                                                 int warp_floats) {
-  plan_body<true, 32, false>(g, descs, states, robot_bytes, env_bytes, warp_floats);
-}
 
 // Reject a start or goal in collision (Alg. 1 lines 1-2): warp 0 checks the
 // start and warp 1 the goal, each with the whole warp; the verdicts meet in
@@ -1146,33 +1340,44 @@ cudaError_t launch_setup(const ProblemDesc* desc, ProblemState* state, int n, in
   return cudaGetLastError();
 }
 
-// Resident planner blocks per SM for a block shape, cached: the occupancy
-// query and the shared-memory attribute cost host time on every call.
-static const void* plan_kernel_fn(bool lockstep, int tile, bool lean) {
-  if (lockstep) return reinterpret_cast<const void*>(lockstep_kernel);
-  if (lean)
-    return tile == 64 ? reinterpret_cast<const void*>(plan_kernel<64, true>)
-                      : reinterpret_cast<const void*>(plan_kernel<32, true>);
-  return tile == 64 ? reinterpret_cast<const void*>(plan_kernel<64, false>)
-                    : reinterpret_cast<const void*>(plan_kernel<32, false>);
+// Kernel instances whose shared-memory attribute and occupancy are cached.
+enum KernelId : int { kPlan32 = 0, kPlan64 = 1, kPlanLean32 = 2, kPlanLean64 = 3, kRounds = 4, kRoundsLean = 5 };
+constexpr int kKernelIds = 6;
+
+static const void* kernel_fn(KernelId id) {
+  switch (id) {
+    case kPlan32: return reinterpret_cast<const void*>(plan_kernel<32, false>);
+    case kPlan64: return reinterpret_cast<const void*>(plan_kernel<64, false>);
+    case kPlanLean32: return reinterpret_cast<const void*>(plan_kernel<32, true>);
+    case kPlanLean64: return reinterpret_cast<const void*>(plan_kernel<64, true>);
+    case kRounds: return reinterpret_cast<const void*>(rounds_kernel<false>);
+    default: return reinterpret_cast<const void*>(rounds_kernel<true>);
+  }
 }
 
-int resident_blocks_per_sm(int warps, int smem, bool lockstep, int tile, bool lean) {
+static KernelId plan_kernel_id(int tile, bool lean) {
+  return (KernelId)((tile == 64 ? 1 : 0) + (lean ? 2 : 0));
+}
+
+// Resident blocks per SM for a block shape, cached: the occupancy query and
+// the shared-memory attribute cost host time on every call.
+static int resident_blocks_per_sm(KernelId id, int warps, int smem) {
   static std::mutex mu;
   static std::map<std::pair<int, int>, int> cache;
   static std::map<int, int> attr_smem;  // per (device, kernel): the attribute value set so far
   int dev = 0;
   cudaGetDevice(&dev);
-  const int kid = 5 * dev + (lockstep ? 4 : (tile == 64 ? 1 : 0) + (lean ? 2 : 0));
+  const int kid = kKernelIds * dev + id;
   const std::pair<int, int> key{warps + 64 * kid, smem};
   std::lock_guard<std::mutex> lk(mu);
   auto it = cache.find(key);
   if (it != cache.end()) return it->second;
-  const void* fn = plan_kernel_fn(lockstep, tile, lean);
+  const void* fn = kernel_fn(id);
   if (smem > attr_smem[kid]) {
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     attr_smem[kid] = smem;
   }
+  if (id >= kRounds) cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, warps * 32, smem);
   if (per_sm < 1) per_sm = 1;
@@ -1180,13 +1385,51 @@ int resident_blocks_per_sm(int warps, int smem, bool lockstep, int tile, bool le
   return per_sm;
 }
 
+// Launch description of a rounds kernel (`at` holds the cluster attribute).
+static cudaLaunchConfig_t rounds_launch(int grid, int blocks, int warps, int smem, cudaStream_t stream,
+                                        cudaLaunchAttribute* at) {
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3(grid);
+  lc.blockDim = dim3(warps * 32);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = stream;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = (unsigned)blocks;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  return lc;
+}
+
+// Largest cluster of the rounds kernels the device can hold at this block
+// shape: 16 blocks are beyond the portable size, so the device is asked.
+static int rounds_max_cluster(int warps, int smem) {
+  static std::mutex mu;
+  static std::map<std::pair<int, int>, int> cache;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lk(mu);
+  const std::pair<int, int> key{warps + 64 * dev, smem};
+  auto it = cache.find(key);
+  if (it != cache.end()) return it->second;
+  int c = kRoundsMaxCluster;
+  for (; c > 1; c /= 2) {
+    int n = 0;
+    cudaLaunchAttribute at{};
+    cudaLaunchConfig_t lc = rounds_launch(c, c, warps, smem, nullptr, &at);
+    if (cudaOccupancyMaxActiveClusters(&n, kernel_fn(kRounds), &lc) == cudaSuccess && n > 0) break;
+    cudaGetLastError();
+  }
+  cache.emplace(key, c);
+  return c;
+}
+
 PlanLaunch plan_launch_config(int n_problems, int mode, int blocks, int warps, int max_spheres, int max_pairs,
                               int max_env_f4, int sm_count, int workers) {
   PlanLaunch c{};
-  c.lockstep = mode == PRRTC_MODE_LOCKSTEP;
   if (mode == PRRTC_MODE_SERIAL)
     c.warps = 1;
-  else if (c.lockstep)  // no more warps than the round has workers
+  else if (mode == PRRTC_MODE_LOCKSTEP)  // no more warps than the round has workers
     c.warps = std::min(warps > 0 ? warps : 8, std::max(workers, 1));
   else
     c.warps = warps > 0 ? warps : 4;
@@ -1196,7 +1439,7 @@ PlanLaunch plan_launch_config(int n_problems, int mode, int blocks, int warps, i
   c.stage_bytes = (int)sizeof(WarpCount) + kWarpVecFloats * (int)sizeof(float) + stage_bytes(max_spheres);  // per warp
   c.smem = c.robot_bytes + c.env_bytes + c.warps * c.stage_bytes;
   // both tile instances take the same registers (capped) and shared memory
-  const int per_sm = resident_blocks_per_sm(c.warps, c.smem, c.lockstep, 32, false);
+  const int per_sm = resident_blocks_per_sm(kPlan32, c.warps, c.smem);
   int resident = per_sm * sm_count;
   if (blocks > 0) {
     c.grid = blocks;
@@ -1213,23 +1456,64 @@ PlanLaunch plan_launch_config(int n_problems, int mode, int blocks, int warps, i
   return c;
 }
 
+RoundsLaunch rounds_launch_config(const PlanLaunch& base, int n_problems, int mode, int blocks, int warps, int workers,
+                                  size_t held_floats, size_t held_limit, int sm_count) {
+  RoundsLaunch c{};
+  c.robot_bytes = base.robot_bytes;
+  c.env_bytes = base.env_bytes;
+  c.stage_bytes = base.stage_bytes + (int)sizeof(WarpCount);  // a second counter block per warp
+  const bool fixed = mode == PRRTC_MODE_LOCKSTEP && warps > 0;  // the caller's warps per block
+  c.warps = fixed ? base.warps : kRoundsWarps;
+  while (c.warps > 1 && c.robot_bytes + c.env_bytes + c.warps * c.stage_bytes > kRoundsSmem) --c.warps;
+  c.smem = c.robot_bytes + c.env_bytes + c.warps * c.stage_bytes;
+  const int resident = resident_blocks_per_sm(kRounds, c.warps, c.smem) * sm_count;
+  const int B = mode == PRRTC_MODE_LOCKSTEP ? workers : 1;
+  // virtual workers of a cluster of C blocks, and whether their held rows fit
+  auto virt = [&](int C) { return std::max(C * c.warps / B, 1) * B; };
+  const int most = (fixed || blocks > 0) ? 1 : rounds_max_cluster(c.warps, c.smem);
+  auto fits = [&](int C) { return C <= most && held_floats * (size_t)virt(C) <= held_limit; };
+  // the first launch: one wave of clusters
+  int first = 1;
+  while (n_problems * first * 2 <= sm_count && fits(2 * first)) first *= 2;
+  int C = first;
+  for (;;) {
+    RoundsLaunch::Phase& ph = c.ph[c.n_phases++];
+    ph.blocks = C;
+    ph.grid = (blocks > 0 ? blocks : std::min(n_problems, std::max(resident / C, 1))) * C;
+    ph.it_limit = INT_MAX;
+    c.workers = virt(C);
+    const int next = std::min(C == 1 ? kRoundsMidCluster : kRoundsMaxCluster, most);
+    if (next <= C || !fits(next) || c.n_phases == 3) break;
+    ph.it_limit = C == 1 ? kRoundsFirstIters : kRoundsMidIters;
+    C = next;
+  }
+  return c;
+}
+
 cudaError_t launch_plan(const PlanGlobals* g, const ProblemDesc* desc, ProblemState* state, const PlanLaunch& cfg,
                         int obstacle_tile, bool lean, cudaStream_t stream) {
   // sets the shared-memory attribute once per size and kernel
-  resident_blocks_per_sm(cfg.warps, cfg.smem, cfg.lockstep, obstacle_tile, lean);
-  cudaError_t e;
-  if (cfg.lockstep)
-    lockstep_kernel<<<cfg.grid, cfg.warps * 32, cfg.smem, stream>>>(const_cast<PlanGlobals*>(g), desc, state,
-                                                                    cfg.robot_bytes, cfg.env_bytes,
-                                                                    cfg.stage_bytes / (int)sizeof(float));
-  else {
-    auto* fn = lean ? (obstacle_tile == 64 ? plan_kernel<64, true> : plan_kernel<32, true>)
-                    : (obstacle_tile == 64 ? plan_kernel<64, false> : plan_kernel<32, false>);
-    fn<<<cfg.grid, cfg.warps * 32, cfg.smem, stream>>>(const_cast<PlanGlobals*>(g), desc, state, cfg.robot_bytes,
-                                                       cfg.env_bytes, cfg.stage_bytes / (int)sizeof(float));
+  resident_blocks_per_sm(plan_kernel_id(obstacle_tile, lean), cfg.warps, cfg.smem);
+  auto* fn = lean ? (obstacle_tile == 64 ? plan_kernel<64, true> : plan_kernel<32, true>)
+                  : (obstacle_tile == 64 ? plan_kernel<64, false> : plan_kernel<32, false>);
+  fn<<<cfg.grid, cfg.warps * 32, cfg.smem, stream>>>(const_cast<PlanGlobals*>(g), desc, state, cfg.robot_bytes,
+                                                     cfg.env_bytes, cfg.stage_bytes / (int)sizeof(float));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rounds(const PlanGlobals* g, const ProblemDesc* desc, ProblemState* state, const RoundsLaunch& cfg,
+                          bool lean, cudaStream_t stream) {
+  resident_blocks_per_sm(lean ? kRoundsLean : kRounds, cfg.warps, cfg.smem);
+  auto* fn = lean ? rounds_kernel<true> : rounds_kernel<false>;
+  for (int k = 0; k < cfg.n_phases; ++k) {
+    const RoundsLaunch::Phase& ph = cfg.ph[k];
+    cudaLaunchAttribute at{};
+    const cudaLaunchConfig_t lc = rounds_launch(ph.grid, ph.blocks, cfg.warps, cfg.smem, stream, &at);
+    const cudaError_t e = cudaLaunchKernelEx(&lc, fn, const_cast<PlanGlobals*>(g), desc, state, cfg.robot_bytes,
+                                             cfg.env_bytes, cfg.stage_bytes / (int)sizeof(float), ph.blocks, k,
+                                             ph.it_limit);
+    if (e != cudaSuccess) return e;
   }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   return cudaSuccess;
 }
 
