@@ -48,7 +48,7 @@ struct prrtc_env {
   // optional distance field
   float* d_esdf = nullptr;
   uint8_t* d_occ = nullptr;
-  int2* d_tmp = nullptr;    // 2 x voxels, scratch of the transform
+  unsigned char* d_tmp = nullptr;  // scratch of the transform
   int dims[3] = {0, 0, 0};
   float origin[3] = {0.f, 0.f, 0.f};
   float voxel = 0.f;
@@ -524,7 +524,7 @@ int prrtc_env_create_esdf(const float origin[3], float voxel, const int32_t dims
   e->voxel = voxel;
   const size_t V = e->voxels();
   if (cudaMalloc(&e->d_esdf, V * sizeof(float)) != cudaSuccess || cudaMalloc(&e->d_occ, V) != cudaSuccess ||
-      cudaMalloc(&e->d_tmp, 2 * V * sizeof(int2)) != cudaSuccess) {
+      cudaMalloc(&e->d_tmp, kEsdfTmpBytes * V) != cudaSuccess) {
     cudaGetLastError();
     prrtc_env_destroy(e);
     return fail(PRRTC_ERR_OOM, "distance field allocation failed");
@@ -548,7 +548,7 @@ int prrtc_env_update_esdf(prrtc_env* env, const uint8_t* occupancy) {
   const size_t V = env->voxels();
   // stream-ordered: planning calls issued before see the old field, later ones the new
   CK(cudaMemcpyAsync(env->d_occ, occupancy, V, cudaMemcpyHostToDevice, c->stream));
-  cudaError_t e = launch_esdf(env->d_occ, env->dims, env->voxel, env->d_tmp, env->d_tmp + V, env->d_esdf, c->stream);
+  cudaError_t e = launch_esdf(env->d_occ, env->dims, env->voxel, env->d_tmp, env->d_esdf, c->stream);
   if (e != cudaSuccess) return cuda_fail("distance transform launch", e);
   CK(cudaStreamSynchronize(c->stream));
   return PRRTC_OK;

@@ -5,18 +5,24 @@
 //
 // The transform is exact: squared distances between voxel centres are
 // integers, and the squared Euclidean distance separates into three 1-D
-// minimisations (along x, then y, then z) of f(j) + (i - j)^2.  Each pass
-// computes, for every voxel, both the distance to the nearest occupied voxel
-// (read by free voxels) and to the nearest free voxel (read by occupied
-// ones).  A thread per voxel scans its line; neighbouring threads scan the
-// same line positions, so the reads are broadcast (x) or coalesced (y, z).
+// minimisations (along x, then y, then z) of f(t) + (i - t)^2.  A free voxel
+// needs the distance to the nearest occupied one and is itself at distance 0
+// from the free ones, an occupied voxel the other way round: one signed number
+// per voxel (positive: free) carries the whole state between the passes.
+//
+// Voxels of the other kind are at distance 0, so along a line only the voxels
+// of the same run of free (or occupied) voxels and the two voxels that bound
+// the run can be nearest.
+#include <algorithm>
+#include <climits>
+
 #include "prrtc.h"
 #include "prrtc_launch.h"
 
 namespace prrtc {
 namespace {
 
-constexpr int kInf = 1 << 29;  // "no site on this line"; + n^2 cannot overflow
+constexpr int kInf = 1 << 29;  // "none on this line"; + n^2 cannot overflow
 
 __global__ void voxelize_kernel(EnvView env, float ox, float oy, float oz, float voxel, int nx, int ny, int nz,
                                 uint8_t* __restrict__ occ) {
@@ -58,54 +64,262 @@ __global__ void voxelize_kernel(EnvView env, float ox, float oy, float oz, float
   }
 }
 
-// Pass along x: squared distance along the row to the nearest occupied
-// (.x) and nearest free (.y) voxel.
-__global__ void edt_x_kernel(const uint8_t* __restrict__ occ, int nx, size_t V, int2* __restrict__ out) {
-  for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(v % nx);
-    const uint8_t* row = occ + (v - i);
-    int bo = kInf, bf = kInf;
-    for (int ii = 0; ii < nx; ++ii) {
-      const int d = (i - ii) * (i - ii);
-      if (row[ii]) bo = min(bo, d);
-      else bf = min(bf, d);
+// Distance to the nearest voxel of the other kind along x, signed; kNoneX: none
+// in the row (256^3: 41 us, a voxel scanning its row 903 us before).  A warp per row: the row as bit words (lane w holds word w, at
+// most 1024 / 32 of them), the nearest set bit of the other kind within the
+// voxel's word or, from two scans over the words, outside it.
+constexpr int kNoneX = 0x7fff;
+
+__global__ void edt_x_kernel(const uint8_t* __restrict__ occ, int nx, size_t rows, int16_t* __restrict__ out) {
+  constexpr int kFar = 1 << 20;
+  const int lane = threadIdx.x & 31, words = (nx + 31) >> 5;
+  const size_t warps = (size_t)gridDim.x * (blockDim.x >> 5);
+  for (size_t r = (size_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < rows; r += warps) {
+    const uint8_t* row = occ + r * nx;
+    uint32_t mine = 0;  // occupied bits of word `lane`
+#pragma unroll 4
+    for (int w = 0; w < words; ++w) {
+      const int i = w * 32 + lane;
+      const uint32_t b = __ballot_sync(kFull, i < nx && row[i]);
+      if (lane == w) mine = b;
     }
-    out[v] = make_int2(bo, bf);
+    const uint32_t in = lane < words ? (lane == words - 1 && (nx & 31) ? (1u << (nx & 31)) - 1u : kFull) : 0u;
+    const uint32_t bits[2] = {~mine & in, mine};  // free, occupied
+    int before[2], after[2];                      // nearest of each kind in the words before / after word `lane`
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      int last = bits[k] ? lane * 32 + 31 - __clz(bits[k]) : -kFar;
+      int first = bits[k] ? lane * 32 + __ffs(bits[k]) - 1 : kFar;
+      for (int off = 1; off < words; off <<= 1) {
+        const int up = __shfl_up_sync(kFull, last, off), down = __shfl_down_sync(kFull, first, off);
+        if (lane >= off) last = max(last, up);
+        if (lane + off < 32) first = min(first, down);
+      }
+      before[k] = __shfl_up_sync(kFull, last, 1);
+      after[k] = __shfl_down_sync(kFull, first, 1);
+      if (lane == 0) before[k] = -kFar;
+      if (lane == 31) after[k] = kFar;
+    }
+#pragma unroll 4
+    for (int w = 0; w < words; ++w) {
+      const int i = w * 32 + lane;
+      const uint32_t f = __shfl_sync(kFull, bits[0], w), o = __shfl_sync(kFull, bits[1], w);
+      const int bf = __shfl_sync(kFull, before[0], w), bo = __shfl_sync(kFull, before[1], w);
+      const int af = __shfl_sync(kFull, after[0], w), ao = __shfl_sync(kFull, after[1], w);
+      const bool is_occ = (o >> lane) & 1u;
+      const uint32_t other = is_occ ? f : o;
+      const uint32_t left = other & ((1u << lane) - 1u), right = other & ~((2u << lane) - 1u);
+      const int lo = left ? w * 32 + 31 - __clz(left) : (is_occ ? bf : bo);
+      const int hi = right ? w * 32 + __ffs(right) - 1 : (is_occ ? af : ao);
+      const int d = min(min(i - lo, hi - i), kNoneX);
+      if (i < nx) out[r * nx + i] = (int16_t)(is_occ ? -d : d);
+    }
   }
 }
+
+// One number of the pass before as a signed squared distance (+-kInf: none).
+__device__ __forceinline__ int load_sq(const int16_t* p) {
+  const int d = __ldg(p), m = abs(d);
+  const int q = m >= kNoneX ? kInf : m * m;
+  return d < 0 ? -q : q;
+}
+__device__ __forceinline__ int load_sq(const int* p) { return __ldg(p); }
+
+// What a pass writes: the signed squared distance, or (last pass) the field,
+// voxel * distance, +- the grid diagonal where no voxel of the other kind exists.
+__device__ __forceinline__ void store_sq(int* p, bool occ, int q, float, float) { *p = occ ? -q : q; }
+__device__ __forceinline__ void store_sq(float* p, bool occ, int q, float voxel, float diag) {
+  const float mag = q >= kInf ? diag : voxel * sqrtf((float)q);
+  *p = occ ? -mag : mag;
+}
+
+// Squared distance that a voxel offers to the voxels of its own kind (v > 0),
+// and 0 to those of the other; "none" stays at or above kInf.
+__device__ __forceinline__ int own_sq(int v, int16_t) { return max(v, 0) * max(v, 0); }
+__device__ __forceinline__ int own_sq(int v, int) { return max(v, 0); }
 
 // Pass along an axis of length n and element stride `stride` (y: nx, z:
-// nx*ny): out(v) = min over positions t of in(t) + (pos(v) - t)^2.
-__global__ void edt_axis_kernel(const int2* __restrict__ in, int n, size_t stride, size_t V, int2* __restrict__ out) {
-  for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (size_t)gridDim.x * blockDim.x) {
-    const int pos = (int)((v / stride) % n);
-    const int2* line = in + (v - (size_t)pos * stride);
-    int bo = kInf, bf = kInf;
-    for (int t = 0; t < n; ++t) {
-      const int2 f = line[(size_t)t * stride];
-      const int d = (pos - t) * (pos - t);
-      if (f.x < kInf) bo = min(bo, f.x + d);
-      if (f.y < kInf) bf = min(bf, f.y + d);
+// nx*ny), small grids: a thread per voxel looks at its whole line, eight
+// voxels in flight; neighbouring threads read neighbouring voxels.
+template <class In, class Out>
+__global__ void edt_scan_kernel(const In* __restrict__ in, int n, size_t stride, size_t V, Out* __restrict__ out,
+                                float voxel, float diag) {
+  const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;  // V < 2^31
+  if (v >= V) return;
+  const int pos = (int)(v / (uint32_t)stride % (uint32_t)n);
+  const In* p = in + (v - (size_t)pos * stride);
+  const bool occ = __ldg(in + v) < 0;
+  const int kind = occ ? -1 : 1;
+  int best = INT_MAX, d = pos, left = n;
+  for (; left >= 8; left -= 8, p += 8 * stride, d -= 8) {
+    int f[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) f[u] = __ldg(p + u * stride);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) best = min(best, own_sq(f[u] * kind, In{}) + (d - u) * (d - u));
+  }
+  for (; left > 0; --left, p += stride, --d) best = min(best, own_sq(__ldg(p) * kind, In{}) + d * d);
+  best = min(best, kInf);
+  store_sq(out + v, occ, best, voxel, diag);
+}
+
+// The same pass for large grids.  For the voxels of one kind, the nearest place t*(i) minimises
+// f(t) + (i - t)^2, with f = 0 at the voxels of the other kind, and the
+// leftmost such t* never decreases with i.  So the place of the middle voxel
+// splits the line: voxels left of it need look no further right than t*, those
+// right of it no further left; log2(n) levels, each n steps a line, all voxels
+// of a level at once.  A block takes 32 lines (lane = line, neighbours in
+// memory) into shared memory; a warp takes one voxel of a level, in all 32
+// lines.  The more frequent kind of the block's voxels goes this way; the
+// others (as a rule the occupied ones: obstacles are thin) look outwards until
+// the offset alone exceeds the best distance, at worst one step a voxel of
+// their run.
+//
+// A candidate is one 32-bit key, (f(t) + (i - t)^2) << 10 | t (t below 1024,
+// values below 2^22 with "none" at kNoneSq), so that a step is one minimum and
+// ties go to the leftmost t.  The lanes of a warp take the union of their
+// ranges, which keeps the loop uniform and finds the same minimum.  The first
+// levels have fewer voxels than the block has warps: the warps share a range.
+constexpr int kAxisWarps = 8;
+constexpr int kNoneSq = 3 << 20;  // above 3 * 1023^2
+
+__host__ __device__ constexpr int axis_smem(int n) { return n * 32 * (int)(sizeof(int) + sizeof(uint16_t)); }
+
+// Smallest key of voxel i over t = lo .. hi of a column of 32-strided values.
+__device__ __forceinline__ uint32_t nearest_key(const int* __restrict__ col, int i, int lo, int hi) {
+  uint32_t k0 = ~0u, k1 = ~0u;
+  int t = lo;
+  for (; t + 7 <= hi; t += 8) {
+    int f[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) f[u] = max(col[(t + u) * 32], 0);
+#pragma unroll
+    for (int u = 0; u < 8; u += 2) {
+      const int d0 = i - t - u, d1 = d0 - 1;
+      k0 = min(k0, (uint32_t)(d0 * d0 + f[u]) << 10 | (uint32_t)(t + u));
+      k1 = min(k1, (uint32_t)(d1 * d1 + f[u + 1]) << 10 | (uint32_t)(t + u + 1));
     }
-    out[v] = make_int2(bo, bf);
+  }
+  for (; t <= hi; ++t) k0 = min(k0, (uint32_t)((i - t) * (i - t) + max(col[t * 32], 0)) << 10 | (uint32_t)t);
+  return min(k0, k1);
+}
+
+template <class In, class Out>
+__global__ void __launch_bounds__(kAxisWarps * 32) edt_axis_kernel(const In* __restrict__ in, int n, size_t stride,
+                                                                   size_t lines, Out* __restrict__ out, float voxel,
+                                                                   float diag) {
+  extern __shared__ int axis_smem_raw[];
+  __shared__ int s_count[kAxisWarps];
+  __shared__ uint32_t s_key[kAxisWarps][32];                    // shared voxels of the first levels
+  int* s = axis_smem_raw;                                       // [n][32], the more frequent kind positive
+  uint16_t* nearest = reinterpret_cast<uint16_t*>(s + n * 32);  // [n][32], t*
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const size_t line = (size_t)blockIdx.x * 32 + lane;
+  const bool live = line < lines;
+  const size_t at = live ? line : lines - 1;
+  const size_t base = (at / stride) * (stride * (size_t)n) + at % stride;
+  in += base;
+  out += base;
+  int count = 0;
+#pragma unroll 8
+  for (int i = warp; i < n; i += kAxisWarps) {
+    const int v = load_sq(in + (size_t)i * stride);
+    s[i * 32 + lane] = max(min(v, kNoneSq), -kNoneSq);
+    count += v < 0 ? -1 : 1;
+  }
+  count = __reduce_add_sync(kFull, count);
+  if (lane == 0) s_count[warp] = count;
+  s_key[warp][lane] = ~0u;
+  __syncthreads();
+  count = 0;
+#pragma unroll
+  for (int w = 0; w < kAxisWarps; ++w) count += s_count[w];
+  const bool flip = count < 0;  // more occupied voxels: they are the positive ones
+  if (flip) {
+    for (int i = warp; i < n; i += kAxisWarps) s[i * 32 + lane] = -s[i * 32 + lane];
+    __syncthreads();
+  }
+  const int* col = s + lane;
+  // voxel i's minimum: its place for the next levels, and the voxel's value
+  auto finish = [&](int i, uint32_t key) {
+    nearest[i * 32 + lane] = (uint16_t)(key & 1023u);
+    const int q = (int)(key >> 10);
+    if (live && col[i * 32] > 0) store_sq(out + (size_t)i * stride, flip, q >= kNoneSq ? kInf : q, voxel, diag);
+  };
+  int half = 1;
+  while (2 * half <= n) half *= 2;
+  for (; half > 0; half >>= 1) {
+    // voxels half - 1, 3 half - 1, ...; those at +-half are done
+    const int nodes = (n - half) / (2 * half) + 1;
+    const int parts = nodes >= kAxisWarps ? 1 : kAxisWarps / nodes;
+    for (int k = parts > 1 ? warp / parts : warp; k < nodes; k += kAxisWarps) {
+      const int i = half - 1 + 2 * half * k;
+      int lo = i - half >= 0 ? nearest[(i - half) * 32 + lane] : 0;
+      int hi = i + half < n ? nearest[(i + half) * 32 + lane] : n - 1;
+      lo = __reduce_min_sync(kFull, lo);
+      hi = __reduce_max_sync(kFull, hi);
+      if (parts == 1) {
+        finish(i, nearest_key(col, i, lo, hi));
+      } else {
+        const int len = (hi - lo + parts) / parts, first = lo + (warp % parts) * len;
+        atomicMin(&s_key[k][lane], nearest_key(col, i, first, min(first + len - 1, hi)));
+      }
+    }
+    __syncthreads();
+    if (parts > 1) {
+      if (warp < nodes) {
+        finish(half - 1 + 2 * half * warp, s_key[warp][lane]);
+        s_key[warp][lane] = ~0u;
+      }
+      __syncthreads();
+    }
+  }
+  // the other kind, outwards, four steps to each side at a time
+  for (int i = warp; i < n; i += kAxisWarps) {
+    int best = live ? -col[i * 32] : -1;
+    const bool mine = best > 0;
+    const int reach = max(i, n - 1 - i);
+    for (int r = 1; r <= reach && r * r < best; r += 4) {
+      int a[4], b[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        a[u] = i - r - u >= 0 ? max(-col[(i - r - u) * 32], 0) : kNoneSq;
+        b[u] = i + r + u < n ? max(-col[(i + r + u) * 32], 0) : kNoneSq;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) best = min(best, min(a[u], b[u]) + (r + u) * (r + u));
+    }
+    if (mine) store_sq(out + (size_t)i * stride, !flip, best >= kNoneSq ? kInf : best, voxel, diag);
   }
 }
 
-// Signed field: free voxels +voxel * sqrt(d2 to occupied), occupied voxels
-// -voxel * sqrt(d2 to free); +/- the grid diagonal when no such voxel exists.
-__global__ void esdf_final_kernel(const uint8_t* __restrict__ occ, const int2* __restrict__ d2, size_t V, float voxel,
-                                  float diag, float* __restrict__ out) {
-  for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (size_t)gridDim.x * blockDim.x) {
-    const int2 d = d2[v];
-    const int q = occ[v] ? d.y : d.x;
-    const float mag = q >= kInf ? diag : voxel * sqrtf((float)q);
-    out[v] = occ[v] ? -mag : mag;
-  }
-}
+// Whether the pass scans whole lines.  It takes about V n / 2.6e6 us, the
+// search by levels about 9 us + V / 1.1e5 us, so the line is V (n - 24) =
+// 2.3e7.  Measured (us, scan / levels): 64^3 9 / 11, 80^3 17 / 14, 100^3
+// 35 / 20, 256^3 1224 / 143; n = 16 of 200 x 16 x 256 8.5 / 20; n = 256 of
+// 16 x 16 x 256 14 / 22.  Before, with both kinds scanned and two numbers per
+// voxel: 64^3 10, 80^3 20, 100^3 42, 256^3 1540 (y) and 2350 (z).
+bool scan_pays(int n, size_t V) { return n <= 24 || V * (size_t)(n - 24) < 23000000; }
 
 int grid_for(size_t V) {
   const size_t blocks = (V + 255) / 256;
   return (int)(blocks < 65535 ? blocks : 65535);
+}
+
+template <class In, class Out>
+cudaError_t launch_axis(const In* in, int n, size_t stride, size_t V, Out* out, float voxel, float diag,
+                        cudaStream_t stream) {
+  if (scan_pays(n, V)) {
+    edt_scan_kernel<<<(int)((V + 255) / 256), 256, 0, stream>>>(in, n, stride, V, out, voxel, diag);
+    return cudaGetLastError();
+  }
+  const cudaError_t e = cudaFuncSetAttribute(edt_axis_kernel<In, Out>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             axis_smem(PRRTC_ESDF_MAX_DIM));
+  if (e != cudaSuccess) return e;
+  const size_t lines = V / n;
+  edt_axis_kernel<<<(int)((lines + 31) / 32), kAxisWarps * 32, axis_smem(n), stream>>>(in, n, stride, lines, out,
+                                                                                       voxel, diag);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -119,17 +333,18 @@ cudaError_t launch_voxelize(const EnvView& env, const float origin[3], float vox
   return cudaGetLastError();
 }
 
-cudaError_t launch_esdf(const uint8_t* occ, const int dims[3], float voxel, int2* tmp_a, int2* tmp_b, float* out,
+cudaError_t launch_esdf(const uint8_t* occ, const int dims[3], float voxel, void* tmp, float* out,
                         cudaStream_t stream) {
-  const size_t V = (size_t)dims[0] * dims[1] * dims[2];
+  const size_t nx = dims[0], ny = dims[1], nz = dims[2], V = nx * ny * nz;
   if (V == 0) return cudaSuccess;
-  const int g = grid_for(V);
-  edt_x_kernel<<<g, 256, 0, stream>>>(occ, dims[0], V, tmp_a);
-  edt_axis_kernel<<<g, 256, 0, stream>>>(tmp_a, dims[1], (size_t)dims[0], V, tmp_b);
-  edt_axis_kernel<<<g, 256, 0, stream>>>(tmp_b, dims[2], (size_t)dims[0] * dims[1], V, tmp_a);
+  int* sq = static_cast<int*>(tmp);
+  int16_t* dx = reinterpret_cast<int16_t*>(sq + V);
+  const size_t rows = ny * nz;
+  edt_x_kernel<<<(int)std::min<size_t>((rows + 7) / 8, 65535), 256, 0, stream>>>(occ, dims[0], rows, dx);
   const float diag = voxel * sqrtf((float)dims[0] * dims[0] + (float)dims[1] * dims[1] + (float)dims[2] * dims[2]);
-  esdf_final_kernel<<<g, 256, 0, stream>>>(occ, tmp_a, V, voxel, diag, out);
-  return cudaGetLastError();
+  cudaError_t e = launch_axis(dx, dims[1], nx, V, sq, voxel, diag, stream);
+  if (e == cudaSuccess) e = launch_axis(sq, dims[2], nx * ny, V, out, voxel, diag, stream);
+  return e;
 }
 
 }  // namespace prrtc

@@ -258,10 +258,11 @@ cudaError_t launch_gather_heads(const ProblemDesc* desc, const ProblemState* sta
 
 // Distance fields (prrtc_esdf.cu): occupancy of voxel centres inside the
 // environment's primitives, and the signed distance transform of an
-// occupancy grid (tmp_a, tmp_b: V int2 each).
+// occupancy grid of V voxels (tmp: kEsdfTmpBytes * V bytes).
+constexpr size_t kEsdfTmpBytes = sizeof(int) + sizeof(int16_t);
 cudaError_t launch_voxelize(const EnvView& env, const float origin[3], float voxel, const int dims[3], uint8_t* occ,
                             cudaStream_t stream);
-cudaError_t launch_esdf(const uint8_t* occ, const int dims[3], float voxel, int2* tmp_a, int2* tmp_b, float* out,
+cudaError_t launch_esdf(const uint8_t* occ, const int dims[3], float voxel, void* tmp, float* out,
                         cudaStream_t stream);
 
 // Tensor-core GEMM (prrtc_gemm.cu): C[M,N] = A[M,K] B[N,K]^T (+bias, ReLU).
