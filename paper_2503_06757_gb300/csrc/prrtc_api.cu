@@ -124,18 +124,27 @@ struct DeviceCtx {
     int blocks, warps, tile, expansions;
   };
   std::map<uint64_t, Tuned> tuned;
-  // check_states scratch
+  // check_states scratch: counters and error word, then the verdicts, in one
+  // buffer, so that they come back in one copy
+  unsigned char* d_check = nullptr;
+  unsigned char* h_check = nullptr;  // pinned image of its first bytes
   float* d_q = nullptr;
-  uint8_t* d_valid = nullptr;
   float* d_spheres = nullptr;
-  size_t q_cap = 0, valid_cap = 0, spheres_cap = 0;
-  unsigned long long* d_counters = nullptr;
-  int* d_error = nullptr;
+  size_t q_cap = 0, check_cap = 0, spheres_cap = 0;
+  int* d_error = nullptr;            // error word of the device-pointer form
   cudaEvent_t ev[4] = {};
   prrtc_launch_stats last{};
 };
 
 constexpr int kHeadRows = 512;
+// A check_states call's counters (7 used) and error word, ahead of its verdicts.
+struct CheckHead {
+  unsigned long long counters[8];
+  int error;
+  int pad[15];
+};
+static_assert(sizeof(CheckHead) == 128, "verdicts start at a 128-byte boundary");
+constexpr size_t kCheckPinned = 64 * 1024;  // verdict bytes that take the pinned way back
 constexpr int kBatchHeadRows = 32;
 constexpr size_t kHeldFloats = (size_t)1 << 28;  // held rows of the deterministic schedules: at most 1 GiB
 
@@ -156,8 +165,8 @@ int current_ctx(DeviceCtx** out) {
     CK(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev));
     CK(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
     for (auto& ev : c->ev) CK(cudaEventCreate(&ev));
-    CK(cudaMalloc(&c->d_counters, 8 * sizeof(unsigned long long)));
     CK(cudaMalloc(&c->d_error, sizeof(int)));
+    CK(cudaMallocHost(&c->h_check, sizeof(CheckHead) + kCheckPinned));
     CK(cudaMallocHost(&c->h_glob, sizeof(PlanGlobals)));
     CK(cudaMalloc(&c->d_glob, sizeof(PlanGlobals)));
     CK(cudaMallocHost(&c->h_path_head, (size_t)kHeadRows * kMaxDof * sizeof(float)));
@@ -882,7 +891,7 @@ int prrtc_check_states_device(const prrtc_robot* robot, const prrtc_env* env, co
   if (robot->device != c->device || env->device != c->device)
     return fail(PRRTC_ERR_INVALID_ARG, "handle belongs to another device");
   cudaError_t e = launch_check_states(robot->d, robot->h->h, env->view(), q_device, n, valid_device, spheres_device,
-                                      c->d_counters, c->d_error, (cudaStream_t)stream);
+                                      nullptr, c->d_error, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail("check_states launch", e);
   return PRRTC_OK;
 }
@@ -953,25 +962,30 @@ int prrtc_check_states(const prrtc_robot* robot, const prrtc_env* env, const flo
   std::lock_guard<std::mutex> lk(c->mu);
   const int dof = robot->h->h.dof, n_raw = robot->h->h.n_raw;
   if ((rc = grow_device(&c->d_q, &c->q_cap, (size_t)n * dof))) return rc;
-  if ((rc = grow_device(&c->d_valid, &c->valid_cap, (size_t)n))) return rc;
+  if ((rc = grow_device(&c->d_check, &c->check_cap, sizeof(CheckHead) + (size_t)n))) return rc;
   if (out_spheres && (rc = grow_device(&c->d_spheres, &c->spheres_cap, (size_t)n * n_raw * 4))) return rc;
+  CheckHead* d_head = reinterpret_cast<CheckHead*>(c->d_check);
+  uint8_t* d_valid = c->d_check + sizeof(CheckHead);
   CK(cudaMemcpyAsync(c->d_q, q, (size_t)n * dof * sizeof(float), cudaMemcpyHostToDevice, c->stream));
-  CK(cudaMemsetAsync(c->d_counters, 0, 8 * sizeof(unsigned long long), c->stream));
-  CK(cudaMemsetAsync(c->d_error, 0, sizeof(int), c->stream));
+  CK(cudaMemsetAsync(d_head, 0, sizeof(CheckHead), c->stream));
   CK(cudaEventRecord(c->ev[0], c->stream));
-  cudaError_t e = launch_check_states(robot->d, robot->h->h, env->view(), c->d_q, n, c->d_valid,
-                                      out_spheres ? c->d_spheres : nullptr, c->d_counters, c->d_error, c->stream);
+  cudaError_t e = launch_check_states(robot->d, robot->h->h, env->view(), c->d_q, n, d_valid,
+                                      out_spheres ? c->d_spheres : nullptr, d_head->counters, &d_head->error,
+                                      c->stream);
   if (e != cudaSuccess) return cuda_fail("check_states launch", e);
   CK(cudaEventRecord(c->ev[1], c->stream));
-  CK(cudaMemcpyAsync(out_valid, c->d_valid, (size_t)n, cudaMemcpyDeviceToHost, c->stream));
+  const bool pinned = (size_t)n <= kCheckPinned;  // one copy for counters and verdicts
+  CK(cudaMemcpyAsync(c->h_check, c->d_check, sizeof(CheckHead) + (pinned ? (size_t)n : 0), cudaMemcpyDeviceToHost,
+                     c->stream));
+  if (!pinned) CK(cudaMemcpyAsync(out_valid, d_valid, (size_t)n, cudaMemcpyDeviceToHost, c->stream));
   if (out_spheres)
     CK(cudaMemcpyAsync(out_spheres, c->d_spheres, (size_t)n * n_raw * 4 * sizeof(float), cudaMemcpyDeviceToHost,
                        c->stream));
-  unsigned long long cnt[7] = {0, 0, 0, 0, 0, 0, 0};
-  int err = 0;
-  CK(cudaMemcpyAsync(cnt, c->d_counters, sizeof(cnt), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaMemcpyAsync(&err, c->d_error, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
+  if (pinned) std::memcpy(out_valid, c->h_check + sizeof(CheckHead), (size_t)n);
+  const CheckHead& head = *reinterpret_cast<const CheckHead*>(c->h_check);
+  const unsigned long long* cnt = head.counters;
+  const int err = head.error;
   float ms = 0.f;
   cudaEventElapsedTime(&ms, c->ev[0], c->ev[1]);
   cudaGetLastError();

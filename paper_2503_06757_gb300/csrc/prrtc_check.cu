@@ -5,6 +5,9 @@
 // against the oracle and as the FP32-roofline microbenchmark (collision-free
 // states: every test must run).
 #include <algorithm>
+#include <map>
+#include <mutex>
+#include <utility>
 
 #include "prrtc.h"
 #include "prrtc_launch.h"
@@ -131,6 +134,38 @@ cudaError_t launch_fma_loop(int sm_count, int iters, float* sink, cudaStream_t s
   return cudaGetLastError();
 }
 
+// Resident blocks of the check kernel on the current device for a shared-memory
+// size, cached: the attribute, the device query and the occupancy query took
+// longer on the host than a small call takes on the device.
+static cudaError_t check_wave(int smem, int* wave) {
+  static std::mutex mu;
+  static std::map<std::pair<int, int>, int> cache;
+  static std::map<int, int> attr_smem;  // per device: the attribute value set so far
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lk(mu);
+  const auto it = cache.find({dev, smem});
+  if (it != cache.end()) {
+    *wave = it->second;
+    return cudaSuccess;
+  }
+  if (smem > attr_smem[dev]) {
+    e = cudaFuncSetAttribute(check_states_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    attr_smem[dev] = smem;
+  }
+  int sms = 0, per_sm = 0;
+  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, check_states_kernel, kCheckWarps * 32, smem);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  *wave = sms * per_sm;
+  cache.emplace(std::make_pair(dev, smem), *wave);
+  return cudaSuccess;
+}
+
 cudaError_t launch_check_states(const RobotDev* robot, const RobotHeader& h, EnvView env, const float* q, int n,
                                 uint8_t* valid, float* spheres, unsigned long long* counters, int* error,
                                 cudaStream_t stream) {
@@ -138,16 +173,11 @@ cudaError_t launch_check_states(const RobotDev* robot, const RobotHeader& h, Env
   const int np_pad = (h.n_pairs + 3) & ~3;
   const int smem = robot_smem_bytes(np_pad) + env.n_float4() * 16 +
                    kCheckWarps * (kQStageFloats * (int)sizeof(float) + stage_bytes(h.n_spheres + h.dof));
-  cudaError_t e = cudaFuncSetAttribute(check_states_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  int wave = 0;
+  const cudaError_t e = check_wave(smem, &wave);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, check_states_kernel, kCheckWarps * 32, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const long long want = ((long long)n + kCheckWarps * 32 - 1) / (kCheckWarps * 32);
-  const int grid = (int)(want < (long long)sms * per_sm ? (want > 0 ? want : 1) : (long long)sms * per_sm);
+  const int grid = (int)std::min<long long>(want, wave);
   check_states_kernel<<<grid, kCheckWarps * 32, smem, stream>>>(robot, env, q, n, valid, spheres, counters, error,
                                                                np_pad);
   return cudaGetLastError();

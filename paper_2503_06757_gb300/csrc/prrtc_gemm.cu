@@ -1054,6 +1054,10 @@ int gemm_take_error() {
   return e;
 }
 
+cudaError_t gemm_read_error(int* out, cudaStream_t stream) {
+  return cudaMemcpyFromSymbolAsync(out, g_gemm_error, sizeof(int), 0, cudaMemcpyDeviceToHost, stream);
+}
+
 }  // namespace prrtc
 
 extern "C" int prrtc_gemm_bf16(const void* a, const void* b, int32_t M, int32_t N, int32_t K, const float* bias,

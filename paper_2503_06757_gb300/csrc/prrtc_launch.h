@@ -273,6 +273,8 @@ int gemm_bf16(const void* a, const void* b, int M, int N, int K, const float* bi
 int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, int K, const float* bias, int relu,
                  float* c32, int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint);
 int gemm_take_error();
+// Copies the kernels' error word to *out on `stream` (does not clear it).
+cudaError_t gemm_read_error(int* out, cudaStream_t stream);
 
 // Fused inference of the learned proposal after the occupancy part of its
 // first layer (prrtc_gemm.cu): first hidden layer from its per-environment

@@ -358,6 +358,10 @@ struct prrtc_proposal {
   size_t envs_cap = 0;
   float** gmm_rows = nullptr;
   size_t gmm_rows_cap = 0;
+  float* d_mix = nullptr;    // prrtc_proposal_mixtures: planner rows, and their host image behind the error word
+  size_t d_mix_cap = 0;
+  unsigned char* h_mix = nullptr;
+  size_t h_mix_cap = 0;
   cudaEvent_t done = nullptr;
   // inference for planning: the per-call inputs staged in one pinned buffer
   // and copied with one transfer; the kernel chain replayed as a CUDA graph
@@ -854,7 +858,8 @@ void prrtc_proposal_destroy(prrtc_proposal* p) {
   }
   cudaFree(p->occ); cudaFree(p->qs); cudaFree(p->qg); cudaFree(p->tgt); cudaFree(p->scene_of); cudaFree(p->rows);
   cudaFree(p->envs); cudaFree(p->gmm_rows);
-  cudaFree(p->d_stage); cudaFree(p->inf_occ);
+  cudaFree(p->d_stage); cudaFree(p->inf_occ); cudaFree(p->d_mix);
+  if (p->h_mix) cudaFreeHost(p->h_mix);
   cudaFree(p->xo16); cudaFree(p->h1o32);
   for (bf16* t : p->atile) cudaFree(t);
   if (p->h_stage) cudaFreeHost(p->h_stage);
@@ -1097,23 +1102,26 @@ int prrtc_proposal_mixtures(prrtc_proposal* p, const prrtc_env* const* envs, con
     if (rc) return rc;
     if (dev != p->device) return mlp_fail(PRRTC_ERR_INVALID_ARG, "environment on another device");
   }
-  float* d = nullptr;
-  MCK(cudaMalloc(&d, (size_t)B * kGmmStride * sizeof(float)));
+  int rc;
+  const size_t floats = (size_t)B * kGmmStride;
+  if ((rc = grow(&p->d_mix, &p->d_mix_cap, floats))) return rc;
+  if ((rc = grow_pinned(&p->h_mix, &p->h_mix_cap, 16 + floats * sizeof(float)))) return rc;
+  int* error = reinterpret_cast<int*>(p->h_mix);
+  const float* padded = reinterpret_cast<const float*>(p->h_mix + 16);
   std::vector<float*> rows(B);
-  for (int b = 0; b < B; ++b) rows[b] = d + (size_t)b * kGmmStride;
-  int rc = prrtc_internal_proposal_mixtures(p, views.data(), q_start, q_goal, B, rows.data(), p->stream);
-  std::vector<float> padded((size_t)B * kGmmStride);
-  cudaError_t e = cudaSuccess;
-  if (!rc) e = cudaMemcpyAsync(padded.data(), d, padded.size() * sizeof(float), cudaMemcpyDeviceToHost, p->stream);
-  if (!rc && e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
-  cudaFree(d);
-  if (rc) return rc;
-  if (e != cudaSuccess) return mlp_fail(PRRTC_ERR_CUDA, cudaGetErrorString(e));
-  if ((rc = check_gemm_error())) return rc;
+  for (int b = 0; b < B; ++b) rows[b] = p->d_mix + (size_t)b * kGmmStride;
+  if ((rc = prrtc_internal_proposal_mixtures(p, views.data(), q_start, q_goal, B, rows.data(), p->stream))) return rc;
+  MCK(cudaMemcpyAsync(p->h_mix + 16, p->d_mix, floats * sizeof(float), cudaMemcpyDeviceToHost, p->stream));
+  MCK(gemm_read_error(error, p->stream));
+  MCK(cudaStreamSynchronize(p->stream));
+  if (*error) {
+    gemm_take_error();
+    return mlp_fail(*error, "a tensor-core kernel wait gave up");
+  }
   // the planner's padded rows -> [logits | means (8 x dof) | log-sigmas (8 x dof)]
   const int stride = kK + 2 * kK * dof;
   for (int b = 0; b < B; ++b) {
-    const float* g = padded.data() + (size_t)b * kGmmStride;
+    const float* g = padded + (size_t)b * kGmmStride;
     float* o = out + (size_t)b * stride;
     for (int k = 0; k < kK; ++k) {
       o[k] = g[k];

@@ -211,6 +211,14 @@ def _fa(a):
     return a, a.ctypes.data_as(_f)
 
 
+def _occ(a):
+    """Occupancy as contiguous bytes, nonzero = occupied; byte and truth arrays go as they are."""
+    a = np.asarray(a)
+    if a.dtype == np.uint8 or a.dtype == np.bool_:
+        return np.ascontiguousarray(a).view(np.uint8)
+    return np.ascontiguousarray(a != 0, dtype=np.uint8)
+
+
 def _ia(a):
     a = np.ascontiguousarray(a, dtype=np.int32)
     return a, a.ctypes.data_as(_i)
@@ -242,7 +250,7 @@ class Env:
     @classmethod
     def from_occupancy(cls, occupancy, origin, voxel: float):
         """Distance-field environment (prrtc_env_create_esdf); occupancy [nz, ny, nx]."""
-        occ = np.ascontiguousarray(np.asarray(occupancy) != 0, dtype=np.uint8)
+        occ = _occ(occupancy)
         nz, ny, nx = occ.shape
         self = cls.__new__(cls)
         self._lib = lib()
@@ -257,20 +265,20 @@ class Env:
         return self
 
     def update_occupancy(self, occupancy):
-        occ = np.ascontiguousarray(np.asarray(occupancy) != 0, dtype=np.uint8)
+        occ = _occ(occupancy)
         _check(self._lib.prrtc_env_update_esdf(self.handle, occ.ctypes.data_as(C.POINTER(C.c_uint8))),
                "prrtc_env_update_esdf")
 
     def esdf(self) -> np.ndarray:
         (nx, ny, nz), _, _ = self.grid
-        out = np.zeros((nz, ny, nx), np.float32)
+        out = np.empty((nz, ny, nx), np.float32)
         _check(self._lib.prrtc_env_esdf_values(self.handle, out.ctypes.data_as(_f)), "prrtc_env_esdf_values")
         return out
 
     def voxelize(self, origin, voxel: float, dims) -> np.ndarray:
         """Occupancy [nz, ny, nx] of this environment's primitives (prrtc_voxelize)."""
         nx, ny, nz = (int(x) for x in dims)
-        out = np.zeros((nz, ny, nx), np.uint8)
+        out = np.empty((nz, ny, nx), np.uint8)
         o = (C.c_float * 3)(*[float(x) for x in origin])
         d = (C.c_int32 * 3)(nx, ny, nz)
         _check(self._lib.prrtc_voxelize(self.handle, o, C.c_float(voxel), d, out.ctypes.data_as(C.POINTER(C.c_uint8))),
@@ -396,8 +404,8 @@ def prrtc_check_states(robot: Robot, env: Env, Q, want_spheres: bool = False):
     """Verdicts (True = collision-free) and, optionally, [n, S, 4] sphere centres+radii."""
     Q, qp = _fa(np.asarray(Q).reshape(-1, robot.dof))
     n = Q.shape[0]
-    valid = np.zeros(n, dtype=np.uint8)
-    sph = np.zeros((n, robot.n_raw, 4), dtype=np.float32) if want_spheres else None
+    valid = np.empty(n, dtype=np.uint8)
+    sph = np.empty((n, robot.n_raw, 4), dtype=np.float32) if want_spheres else None
     _check(lib().prrtc_check_states(robot.handle, env.handle, qp, n, valid.ctypes.data_as(C.POINTER(C.c_uint8)),
                                     sph.ctypes.data_as(_f) if want_spheres else None), "prrtc_check_states")
     return (valid.astype(bool), sph) if want_spheres else valid.astype(bool)
@@ -640,12 +648,12 @@ class Proposal:
         _check(self._lib.prrtc_proposal_save(self.handle, str(path).encode()), "prrtc_proposal_save")
 
     def params(self):
-        out = np.zeros(self.n_params, np.float32)
+        out = np.empty(self.n_params, np.float32)
         _check(self._lib.prrtc_proposal_get_params(self.handle, out.ctypes.data_as(_f), None), "get_params")
         return out
 
     def grads(self):
-        out = np.zeros(self.n_params, np.float32)
+        out = np.empty(self.n_params, np.float32)
         _check(self._lib.prrtc_proposal_get_params(self.handle, None, out.ctypes.data_as(_f)), "get_params")
         return out
 
@@ -654,7 +662,7 @@ class Proposal:
         B = occ.shape[0]
         s, sp = _fa(np.asarray(q_start).reshape(B, self.dof))
         g, gp = _fa(np.asarray(q_goal).reshape(B, self.dof))
-        out = np.zeros((B, self.head), np.float32)
+        out = np.empty((B, self.head), np.float32)
         _check(self._lib.prrtc_proposal_forward(self.handle, occ.ctypes.data_as(C.POINTER(C.c_uint8)), sp, gp, B,
                                                 out.ctypes.data_as(_f)), "prrtc_proposal_forward")
         return out
@@ -709,7 +717,7 @@ class Proposal:
         s, sp = _fa(np.asarray(q_start).reshape(B, self.dof))
         g, gp = _fa(np.asarray(q_goal).reshape(B, self.dof))
         eh = (C.c_void_p * B)(*[e.handle for e in envs])
-        out = np.zeros((B, 8 + 16 * self.dof), np.float32)
+        out = np.empty((B, 8 + 16 * self.dof), np.float32)
         _check(self._lib.prrtc_proposal_mixtures(self.handle, eh, sp, gp, B, out.ctypes.data_as(_f)),
                "prrtc_proposal_mixtures")
         return out
