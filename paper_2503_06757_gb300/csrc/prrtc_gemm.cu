@@ -67,6 +67,7 @@ struct Epilogue {
   int m_tiles, n_tiles, k_tiles;
   int m_pad;             // rows of one split's partial (M rounded up to the tile), so that the
                          // clipped-off rows of an edge tile never reach the next split's rows
+  int ta, tb;            // operand stored transposed: [K x M] / [K x N], M / N contiguous
 };
 
 // Output tensor maps of one launch: workspace (FP32, rows = splits * m_pad),
@@ -89,8 +90,24 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
   return d;
 }
 
-// Instruction descriptor, kind::f16: FP32 accumulator, BF16 A and B, both
-// K-major, N >> 3 at bit 17, M >> 4 at bit 24.
+// The same for an MN-major tile (a transposed operand): 64 rows or columns of
+// the operand are the 128 contiguous bytes, K runs over the tile's lines.
+// Leading byte offset: from one group of 64 to the next (a box of BK lines);
+// stride byte offset: from 8 lines of K to the next 8.
+constexpr int MN_BOX_BYTES = BK * 128;
+__device__ __forceinline__ uint64_t smem_desc_mn(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)(MN_BOX_BYTES >> 4) << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+
+// Instruction descriptor, kind::f16: FP32 accumulator, BF16 A and B, K-major
+// unless the transpose bits (15: A, 16: B) say MN-major, N >> 3 at bit 17,
+// M >> 4 at bit 24.
 __device__ __forceinline__ uint32_t idesc_bf16(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
@@ -309,14 +326,28 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (lane == 0) {
           unsigned char* a = smem + s * STAGE_BYTES;
           mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
-          tma_load_2d(a, &tmA, &full[s], kt * BK, w.m0);
-          tma_load_2d(a + A_BYTES, &tmB, &full[s], kt * BK, w.n0);
+          if (ep.ta) {
+#pragma unroll
+            for (int j = 0; j < BM / 64; ++j)
+              tma_load_2d(a + j * MN_BOX_BYTES, &tmA, &full[s], w.m0 + 64 * j, kt * BK);
+          } else {
+            tma_load_2d(a, &tmA, &full[s], kt * BK, w.m0);
+          }
+          if (ep.tb) {
+#pragma unroll
+            for (int j = 0; j < BN / 64; ++j)
+              tma_load_2d(a + A_BYTES + j * MN_BOX_BYTES, &tmB, &full[s], w.n0 + 64 * j, kt * BK);
+          } else {
+            tma_load_2d(a + A_BYTES, &tmB, &full[s], kt * BK, w.n0);
+          }
         }
         __syncwarp();
       }
     }
   } else if (warp == 1) {
-    const uint32_t idesc = idesc_bf16(BM, BN);
+    const uint32_t idesc = idesc_bf16(BM, BN) | (ep.ta ? 1u << 15 : 0u) | (ep.tb ? 1u << 16 : 0u);
+    // from one K step of 16 to the next: 32 bytes along K, or 16 lines of K
+    const uint32_t step_a = ep.ta ? 2048u : 32u, step_b = ep.tb ? 2048u : 32u;
     int it = 0, i = 0;  // stage counter, local unit counter
     bool ok = true;
     for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x, ++i) {
@@ -349,7 +380,9 @@ __global__ void __launch_bounds__(THREADS, 1)
           const uint32_t b = a + A_BYTES;
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
-            mma_bf16(d, smem_desc(a + 32u * k), smem_desc(b + 32u * k), idesc, (kt > w.kt0 || k > 0) ? 1u : 0u);
+            mma_bf16(d, ep.ta ? smem_desc_mn(a + step_a * k) : smem_desc(a + step_a * k),
+                     ep.tb ? smem_desc_mn(b + step_b * k) : smem_desc(b + step_b * k), idesc,
+                     (kt > w.kt0 || k > 0) ? 1u : 0u);
           mma_commit(&empty[s]);
         }
         __syncwarp();
@@ -827,7 +860,7 @@ PFN_cuTensorMapEncodeTiled_v12000 encoder() {
 }
 
 // Row-major [rows x K] BF16 matrix with row stride ld elements, K
-// contiguous; boxes of 64 x box_rows.
+// contiguous; boxes of 64 x box_rows (for a transposed operand the rows are K).
 bool make_tmap(CUtensorMap* tm, const void* ptr, int rows, int K, int ld, int box_rows) {
   auto enc = encoder();
   if (!enc) return false;
@@ -933,15 +966,18 @@ int g_sms = 0;
 // Host launcher used by the MLP code and the C ABI entry point.  splits_hint:
 // 0 = choose (split K while the tiles fill less than one wave), else forced.
 int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, int K, const float* bias, int relu,
-                 float* c32, int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint) {
+                 float* c32, int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint, int trans) {
+  const int ta = trans & kTransA ? 1 : 0, tb = trans & kTransB ? 1 : 0;
   if (M <= 0 || N <= 0 || K <= 0 || !a || !b || (!c32 && !c16)) return PRRTC_ERR_INVALID_ARG;
   if (K % 8 || N % 8 || (c32 && ldc32 % 4) || (c16 && ldc16 % 8)) return PRRTC_ERR_UNSUPPORTED;
-  if (lda < K || ldb < K || lda % 8 || ldb % 8) return PRRTC_ERR_UNSUPPORTED;
+  if (lda < (ta ? M : K) || ldb < (tb ? N : K) || lda % 8 || ldb % 8) return PRRTC_ERR_UNSUPPORTED;
   if ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) return PRRTC_ERR_INVALID_ARG;
   if ((c32 && (reinterpret_cast<uintptr_t>(c32) & 15)) || (c16 && (reinterpret_cast<uintptr_t>(c16) & 15)))
     return PRRTC_ERR_INVALID_ARG;
-  CUtensorMap ta, tb;
-  if (!cached_map(&ta, a, M, K, lda, 0, BM) || !cached_map(&tb, b, N, K, ldb, 0, BN)) return PRRTC_ERR_CUDA;
+  CUtensorMap ma, mb;
+  if (!(ta ? cached_map(&ma, a, K, M, lda, 0, BK) : cached_map(&ma, a, M, K, lda, 0, BM)) ||
+      !(tb ? cached_map(&mb, b, K, N, ldb, 0, BK) : cached_map(&mb, b, N, K, ldb, 0, BN)))
+    return PRRTC_ERR_CUDA;
   static bool attr = false;
   if (!attr) {
     if (cudaFuncSetAttribute(gemm_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess)
@@ -951,7 +987,7 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
     cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
     attr = true;
   }
-  Epilogue ep{M, N, K, bias, relu, c32 ? 1 : 0, c16 ? 1 : 0, 1, 0, 0, 0, 0};
+  Epilogue ep{M, N, K, bias, relu, c32 ? 1 : 0, c16 ? 1 : 0, 1, 0, 0, 0, 0, ta, tb};
   OutMaps om;
   std::memset(&om, 0, sizeof(om));
   if (c32 && !cached_map(&om.c32, c32, M, N, ldc32, 2)) return PRRTC_ERR_CUDA;
@@ -978,7 +1014,7 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
   }
   const int units = tiles * splits;
   const int grid = std::min(units, sms);
-  gemm_bf16_kernel<<<grid, THREADS, SMEM_BYTES, stream>>>(ta, tb, om, ep);
+  gemm_bf16_kernel<<<grid, THREADS, SMEM_BYTES, stream>>>(ma, mb, om, ep);
   if (cudaGetLastError() != cudaSuccess) return PRRTC_ERR_CUDA;
   if (splits > 1) {
     const size_t work = (size_t)M * (N / 4);
@@ -992,7 +1028,7 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
 
 int gemm_bf16_split(const void* a, const void* b, int M, int N, int K, const float* bias, int relu, float* c32,
                     int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint) {
-  return gemm_bf16_ld(a, K, b, K, M, N, K, bias, relu, c32, ldc32, c16, ldc16, stream, splits_hint);
+  return gemm_bf16_ld(a, K, b, K, M, N, K, bias, relu, c32, ldc32, c16, ldc16, stream, splits_hint, 0);
 }
 
 int gemm_bf16(const void* a, const void* b, int M, int N, int K, const float* bias, int relu, float* c32, int ldc32,

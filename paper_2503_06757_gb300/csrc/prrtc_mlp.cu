@@ -6,9 +6,9 @@
 // everything else is elementwise or per-sample work:
 //   forward   x -> relu(W1 x + b1) -> relu(W2 .) -> relu(W3 .) -> W4 . + b4
 //   loss      mean mixture negative log-likelihood of target configurations
-//   backward  dW = dZ^T H, dH = dZ W (BF16 operands transposed explicitly),
-//             ReLU masks, bias column sums
-//   update    Adam on FP32 master weights, then BF16 copies (and transposes)
+//   backward  dW = dZ^T H, dH = dZ W (operands read as stored), ReLU masks,
+//             bias column sums
+//   update    Adam on FP32 master weights, then BF16 copies
 // The proposal is an addition to pRRTC (the paper samples uniformly).
 #include <cuda_bf16.h>
 
@@ -317,19 +317,14 @@ __global__ void __launch_bounds__(256) colsum_kernel(const ColSums a) {
   if (threadIdx.x < 32) a.out[l][c0 + threadIdx.x] = s;
 }
 
-// out[c, r] = in[r, c] (BF16, 32 x 32 tiles through shared memory).
-__global__ void transpose_kernel(const bf16* __restrict__ in, int rows, int cols, bf16* __restrict__ out) {
+// out[c, r] = in[r, c] (BF16, row strides ldi and ldo, 32 x 32 tiles through
+// shared memory; the grid covers the matrix exactly).
+__global__ void transpose_kernel(const bf16* __restrict__ in, int ldi, bf16* __restrict__ out, int ldo) {
   __shared__ bf16 tile[32][33];
   const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int r = r0 + k, c = c0 + threadIdx.x;
-    if (r < rows && c < cols) tile[k][threadIdx.x] = in[(size_t)r * cols + c];
-  }
+  for (int k = threadIdx.y; k < 32; k += blockDim.y) tile[k][threadIdx.x] = in[(size_t)(r0 + k) * ldi + c0 + threadIdx.x];
   __syncthreads();
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int c = c0 + k, r = r0 + threadIdx.x;
-    if (c < cols && r < rows) out[(size_t)c * rows + r] = tile[threadIdx.x][k];
-  }
+  for (int k = threadIdx.y; k < 32; k += blockDim.y) out[(size_t)(c0 + k) * ldo + r0 + threadIdx.x] = tile[threadIdx.x][k];
 }
 
 __global__ void to_bf16_kernel(const float* __restrict__ in, size_t n, bf16* __restrict__ out) {
@@ -380,7 +375,7 @@ struct prrtc_proposal {
   float* m = nullptr;
   float* v = nullptr;
   bf16* w16[4] = {};
-  bf16* w16t[4] = {};
+  bf16* wq = nullptr;       // start / goal columns of layer 1, transposed: [2 kQPad x kHid0]
   bf16* wtile[3] = {};  // layers 2, 3 and the head, tiled for the fused inference kernel
   int step = 0;
   float lo[kMaxDof], span[kMaxDof];
@@ -388,8 +383,7 @@ struct prrtc_proposal {
   cudaStream_t stream = nullptr;
   // batch scratch
   int cap = 0;
-  bf16 *x16 = nullptr, *xT = nullptr, *h16[3] = {}, *hT[3] = {}, *d16 = nullptr, *dT = nullptr, *z16[3] = {},
-       *zT[3] = {};
+  bf16 *x16 = nullptr, *h16[3] = {}, *d16 = nullptr, *z16[3] = {};
   float *out32 = nullptr, *d32 = nullptr, *dh32 = nullptr, *z32[3] = {}, *loss = nullptr;
   // sample data
   uint8_t* occ = nullptr;
@@ -464,14 +458,14 @@ int grow(T** p, size_t* cap, size_t need) {
 }
 
 void free_scratch(prrtc_proposal* p) {
-  cudaFree(p->x16); cudaFree(p->xT); cudaFree(p->d16); cudaFree(p->dT);
+  cudaFree(p->x16); cudaFree(p->d16);
   cudaFree(p->out32); cudaFree(p->d32); cudaFree(p->dh32); cudaFree(p->loss);
   for (int l = 0; l < 3; ++l) {
-    cudaFree(p->h16[l]); cudaFree(p->hT[l]); cudaFree(p->z16[l]); cudaFree(p->zT[l]); cudaFree(p->z32[l]);
-    p->h16[l] = p->hT[l] = p->z16[l] = p->zT[l] = nullptr;
+    cudaFree(p->h16[l]); cudaFree(p->z16[l]); cudaFree(p->z32[l]);
+    p->h16[l] = p->z16[l] = nullptr;
     p->z32[l] = nullptr;
   }
-  p->x16 = p->xT = p->d16 = p->dT = nullptr;
+  p->x16 = p->d16 = nullptr;
   p->out32 = p->d32 = p->dh32 = p->loss = nullptr;
   p->cap = 0;
 }
@@ -483,18 +477,14 @@ int ensure_scratch(prrtc_proposal* p, int rows) {
   const int P = p->P;
   const int hid[3] = {kHid0, kHid1, kHid2};
   bool ok = cudaMalloc(&p->x16, (size_t)rows * kIn * 2) == cudaSuccess &&
-            cudaMalloc(&p->xT, (size_t)rows * kIn * 2) == cudaSuccess &&
             cudaMalloc(&p->d16, (size_t)rows * P * 2) == cudaSuccess &&
-            cudaMalloc(&p->dT, (size_t)rows * P * 2) == cudaSuccess &&
             cudaMalloc(&p->out32, (size_t)rows * P * 4) == cudaSuccess &&
             cudaMalloc(&p->d32, (size_t)rows * P * 4) == cudaSuccess &&
             cudaMalloc(&p->dh32, (size_t)rows * kHid0 * 4) == cudaSuccess &&
             cudaMalloc(&p->loss, 4) == cudaSuccess;
   for (int l = 0; l < 3 && ok; ++l)
     ok = cudaMalloc(&p->h16[l], (size_t)rows * hid[l] * 2) == cudaSuccess &&
-         cudaMalloc(&p->hT[l], (size_t)rows * hid[l] * 2) == cudaSuccess &&
          cudaMalloc(&p->z16[l], (size_t)rows * hid[l] * 2) == cudaSuccess &&
-         cudaMalloc(&p->zT[l], (size_t)rows * hid[l] * 2) == cudaSuccess &&
          cudaMalloc(&p->z32[l], (size_t)rows * hid[l] * 4) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
@@ -505,22 +495,18 @@ int ensure_scratch(prrtc_proposal* p, int rows) {
   return PRRTC_OK;
 }
 
-int transpose(const bf16* in, int rows, int cols, bf16* out, cudaStream_t s) {
-  dim3 grid((cols + 31) / 32, (rows + 31) / 32), block(32, 8);
-  transpose_kernel<<<grid, block, 0, s>>>(in, rows, cols, out);
-  return cudaGetLastError() == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
-}
-
-// BF16 copies of the weights and their transposes from the FP32 masters.
+// BF16 copies of the weights from the FP32 masters, and what inference reads:
+// the tiled layers and the transposed start / goal columns.
 int refresh_weights(prrtc_proposal* p) {
   for (int l = 0; l < 4; ++l) {
     const size_t n = (size_t)p->out_dim[l] * p->in_dim[l];
     to_bf16_kernel<<<blocks_for(n), 256, 0, p->stream>>>(p->master + p->w_off[l], n, p->w16[l]);
-    int rc = transpose(p->w16[l], p->out_dim[l], p->in_dim[l], p->w16t[l], p->stream);
-    if (rc) return rc;
+    int rc;
     if (l > 0 && (rc = mlp_tile_weights(p->w16[l], p->out_dim[l], p->in_dim[l], p->wtile[l - 1], p->stream)))
       return rc;
   }
+  transpose_kernel<<<dim3(2 * kQPad / 32, kHid0 / 32), dim3(32, 8), 0, p->stream>>>(p->w16[0] + kVox, kIn, p->wq,
+                                                                                    kHid0);
   return cudaGetLastError() == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
 }
 
@@ -544,36 +530,32 @@ int forward_rows(prrtc_proposal* p, int rows, int first_layer = 0) {
   return gemm(in, p->w16[3], rows, p->P, p->in_dim[3], p->master + p->b_off[3], 0, p->out32, nullptr, s);
 }
 
-// Gradients of the mean NLL for `B` samples (rows padded to `rows`) into p->grad.
-int backward_rows(prrtc_proposal* p, int B, int rows) {
+// Gradients of the mean NLL for samples padded to `rows` rows into p->grad.
+int backward_rows(prrtc_proposal* p, int rows) {
   const cudaStream_t s = p->stream;
-  const int P = p->P;
   int rc;
-  // head: dW4 = dout^T h3, db4 = colsum(dout), dh3 = dout W4
-  if ((rc = transpose(p->d16, rows, P, p->dT, s))) return rc;
   const bf16* hprev[4] = {p->x16, p->h16[0], p->h16[1], p->h16[2]};
-  bf16* hprevT[4] = {p->xT, p->hT[0], p->hT[1], p->hT[2]};
   const bf16* dz16 = p->d16;
-  const bf16* dzT = p->dT;
   const float* dz32 = p->d32;
   ColSums cs{};
   cs.rows = rows;
   for (int l = 3; l >= 0; --l) {
     const int in = p->in_dim[l], out = p->out_dim[l];
-    if ((rc = transpose(hprev[l], rows, in, hprevT[l], s))) return rc;
-    // dW_l [out x in] = dZ^T [out x rows] * (H^T [in x rows])^T
-    if ((rc = gemm(dzT, hprevT[l], out, in, rows, nullptr, 0, p->grad + p->w_off[l], nullptr, s))) return rc;
+    // dW_l [out x in] = dZ^T H, both as stored: [rows x out], [rows x in]
+    if ((rc = gemm_bf16_ld(dz16, out, hprev[l], in, out, in, rows, nullptr, 0, p->grad + p->w_off[l], in, nullptr, 0,
+                           s, 0, kTransA | kTransB)))
+      return rc;
     cs.g[l] = dz32;
     cs.out[l] = p->grad + p->b_off[l];
     cs.cols[l] = out;
     if (l == 0) break;
-    // dH_{l-1} [rows x in] = dZ [rows x out] * (W^T [in x out])^T
-    if ((rc = gemm(dz16, p->w16t[l], rows, in, out, nullptr, 0, p->dh32, nullptr, s))) return rc;
+    // dH_{l-1} [rows x in] = dZ [rows x out] W_l [out x in]
+    if ((rc = gemm_bf16_ld(dz16, out, p->w16[l], in, rows, in, out, nullptr, 0, p->dh32, in, nullptr, 0, s, 0,
+                           kTransB)))
+      return rc;
     const size_t n = (size_t)rows * in;
     relu_back_kernel<<<blocks_for(n), 256, 0, s>>>(p->dh32, p->h16[l - 1], n, p->z32[l - 1], p->z16[l - 1]);
-    if ((rc = transpose(p->z16[l - 1], rows, in, p->zT[l - 1], s))) return rc;
     dz16 = p->z16[l - 1];
-    dzT = p->zT[l - 1];
     dz32 = p->z32[l - 1];
   }
   int blocks = 0;
@@ -582,7 +564,6 @@ int backward_rows(prrtc_proposal* p, int B, int rows) {
     blocks += cs.cols[l] / 32;
   }
   colsum_kernel<<<blocks, 256, 0, s>>>(cs);
-  (void)B;
   return cudaGetLastError() == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
 }
 
@@ -632,7 +613,7 @@ int enqueue_inference(prrtc_proposal* p, const EnvView* d_envs, int U, const int
   } else {
     occ_bf16_kernel<<<U, 256, 0, s>>>(p->inf_occ, p->xo16);
     if ((rc = gemm_bf16_ld(p->xo16, kVox, p->w16[0], kIn, U, kHid0, kVox, nullptr, 0, p->h1o32, kHid0, nullptr, 0, s,
-                           0)))
+                           0, 0)))
       return rc;
   }
   MCK(cudaGetLastError());
@@ -651,7 +632,7 @@ int enqueue_inference(prrtc_proposal* p, const EnvView* d_envs, int U, const int
   a.qg = d_qg;
   a.lo = p->d_lims;
   a.span = p->d_lims + kMaxDof;
-  a.wq = p->w16t[0] + (size_t)kVox * kHid0;
+  a.wq = p->wq;
   for (int l = 0; l < 3; ++l) {
     a.w[l] = p->wtile[l];
     a.act[l] = p->atile[l];
@@ -755,7 +736,7 @@ int prrtc_internal_proposal_stage(prrtc_proposal* p, const EnvView* envs, const 
   p->last_infer_B = B;
   q.sig = chain_signature(
       {(uint64_t)B, (uint64_t)rows, (uint64_t)U, (uint64_t)(uintptr_t)p->xo16,
-       (uint64_t)(uintptr_t)p->h1o32, (uint64_t)(uintptr_t)p->w16t[0], (uint64_t)(uintptr_t)p->atile[0],
+       (uint64_t)(uintptr_t)p->h1o32, (uint64_t)(uintptr_t)p->wq, (uint64_t)(uintptr_t)p->atile[0],
        (uint64_t)(uintptr_t)p->atile[1], (uint64_t)(uintptr_t)p->atile[2], (uint64_t)(uintptr_t)p->wtile[0],
        (uint64_t)(uintptr_t)p->wtile[1], (uint64_t)(uintptr_t)p->wtile[2],
        (uint64_t)(uintptr_t)p->d_stage, (uint64_t)(uintptr_t)p->inf_occ,
@@ -874,10 +855,10 @@ int prrtc_proposal_create(int32_t dof, const float* lower, const float* upper, c
             cudaEventCreate(&p->inf_ev[0]) == cudaSuccess && cudaEventCreate(&p->inf_ev[1]) == cudaSuccess &&
             cudaMalloc(&p->master, off * 4) == cudaSuccess && cudaMalloc(&p->grad, off * 4) == cudaSuccess &&
             cudaMalloc(&p->m, off * 4) == cudaSuccess && cudaMalloc(&p->v, off * 4) == cudaSuccess &&
-            cudaMalloc(&p->d_lims, 2 * kMaxDof * 4) == cudaSuccess;
+            cudaMalloc(&p->d_lims, 2 * kMaxDof * 4) == cudaSuccess &&
+            cudaMalloc(&p->wq, (size_t)2 * kQPad * kHid0 * 2) == cudaSuccess;
   for (int l = 0; l < 4 && ok; ++l)
     ok = cudaMalloc(&p->w16[l], (size_t)dims[l + 1] * dims[l] * 2) == cudaSuccess &&
-         cudaMalloc(&p->w16t[l], (size_t)dims[l + 1] * dims[l] * 2) == cudaSuccess &&
          (l == 0 || cudaMalloc(&p->wtile[l - 1], (size_t)dims[l + 1] * dims[l] * 2) == cudaSuccess);
   if (!ok) {
     cudaGetLastError();
@@ -904,9 +885,9 @@ void prrtc_proposal_destroy(prrtc_proposal* p) {
   if (!p) return;
   free_scratch(p);
   cudaFree(p->master); cudaFree(p->grad); cudaFree(p->m); cudaFree(p->v); cudaFree(p->d_lims);
+  cudaFree(p->wq);
   for (int l = 0; l < 4; ++l) {
     cudaFree(p->w16[l]);
-    cudaFree(p->w16t[l]);
     if (l > 0) cudaFree(p->wtile[l - 1]);
   }
   cudaFree(p->occ); cudaFree(p->qs); cudaFree(p->qg); cudaFree(p->tgt); cudaFree(p->scene_of); cudaFree(p->rows);
@@ -1041,7 +1022,7 @@ static int step_on_rows(prrtc_proposal* p, const int* scene_of, const int* rows_
   mixture_loss_kernel<<<(B * 32 + 255) / 256, 256, 0, s>>>(p->out32, p->P, p->tgt, rows_dev, p->d_lims,
                                                             p->d_lims + kMaxDof, B, p->dof, 1.f / (float)B, p->d32,
                                                             p->d16, p->loss);
-  if ((rc = backward_rows(p, B, rows))) return rc;
+  if ((rc = backward_rows(p, rows))) return rc;
   if (lr > 0.f) {
     p->step++;
     const float b1 = 0.9f, b2 = 0.999f;
