@@ -108,31 +108,46 @@ __global__ void occupancy_scatter_kernel(const EnvView* __restrict__ envs, uint8
   }
 }
 
+__device__ __forceinline__ uint2 bf16x4(float4 f) {
+  const __nv_bfloat162 a = __floats2bfloat162_rn(f.x, f.y), b = __floats2bfloat162_rn(f.z, f.w);
+  return make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+}
+
 // One feature row per sample (rows past B are zero): occupancy of the
 // sample's scene, then normalised start and goal, each zero-padded to 32.
+// kVox / 16 threads.
 __global__ void features_kernel(const uint8_t* __restrict__ occ, const int* __restrict__ scene_of,
                                 const int* __restrict__ rows, const float* __restrict__ qs,
                                 const float* __restrict__ qg, const float* __restrict__ lo,
                                 const float* __restrict__ span, int B, int dof, bf16* __restrict__ x) {
   const int b = blockIdx.x;
   bf16* dst = x + (size_t)b * kIn;
-  if (b >= B) {
-    for (int c = threadIdx.x; c < kIn; c += blockDim.x) dst[c] = __float2bfloat16_rn(0.f);
-    return;
-  }
-  const int r = rows ? rows[b] : b;
-  const int s = scene_of ? scene_of[r] : r;
-  const uint8_t* o = occ + (size_t)s * kVox;
-  for (int c = threadIdx.x; c < kIn; c += blockDim.x) {
-    float v;
-    if (c < kVox) {
-      v = o[c] ? 1.f : 0.f;
-    } else {
-      const int j = (c - kVox) % kQPad;
-      const float* q = (c < kVox + kQPad) ? qs : qg;
-      v = (j < dof) ? 2.f * (q[(size_t)r * dof + j] - lo[j]) / span[j] - 1.f : 0.f;
+  const int r = b < B ? (rows ? rows[b] : b) : 0;
+  // 16 voxels a thread: 16 bytes in, 32 bytes out (256 threads, one turn)
+  {
+    const int c = threadIdx.x * 16;
+    uint4 in = make_uint4(0u, 0u, 0u, 0u);
+    if (b < B) {
+      const int s = scene_of ? scene_of[r] : r;
+      in = __ldg(reinterpret_cast<const uint4*>(occ + (size_t)s * kVox + c));
     }
-    dst[c] = __float2bfloat16_rn(v);
+    const uint32_t w[4] = {in.x, in.y, in.z, in.w};
+    uint32_t out[8];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      constexpr uint32_t kOne = 0x3f80u;  // 1.0 in BF16
+      out[2 * k] = ((w[k] & 0xffu) ? kOne : 0u) | ((w[k] & 0xff00u) ? kOne << 16 : 0u);
+      out[2 * k + 1] = ((w[k] & 0xff0000u) ? kOne : 0u) | ((w[k] & 0xff000000u) ? kOne << 16 : 0u);
+    }
+    uint4* o = reinterpret_cast<uint4*>(dst + c);
+    o[0] = make_uint4(out[0], out[1], out[2], out[3]);
+    o[1] = make_uint4(out[4], out[5], out[6], out[7]);
+  }
+  if (threadIdx.x < 2 * kQPad) {
+    const int j = threadIdx.x % kQPad;
+    const float* q = threadIdx.x < kQPad ? qs : qg;
+    const float v = (b < B && j < dof) ? 2.f * (q[(size_t)r * dof + j] - lo[j]) / span[j] - 1.f : 0.f;
+    dst[kVox + threadIdx.x] = __float2bfloat16_rn(v);
   }
 }
 
@@ -327,23 +342,44 @@ __global__ void transpose_kernel(const bf16* __restrict__ in, int ldi, bf16* __r
   for (int k = threadIdx.y; k < 32; k += blockDim.y) out[(size_t)(c0 + k) * ldo + r0 + threadIdx.x] = tile[threadIdx.x][k];
 }
 
-__global__ void to_bf16_kernel(const float* __restrict__ in, size_t n, bf16* __restrict__ out) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    out[i] = __float2bfloat16_rn(in[i]);
+// BF16 copies of all parameters (n a multiple of 4).
+__global__ void to_bf16_kernel(const float4* __restrict__ in, size_t n4, uint2* __restrict__ out) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x)
+    out[i] = bf16x4(in[i]);
 }
 
 // Adam with bias-corrected moments: c1 = 1/(1 - b1^t), c2 = 1/(1 - b2^t).
-__global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, size_t n, float lr, float b1, float b2, float eps, float c1,
-                            float c2) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
-  }
+// The roundings are spelled out: a run of steps carries a different one on
+// into every later step, so they should not follow the compiler's choice.
+__device__ __forceinline__ float adam_one(float p, float g, float& m, float& v, float lr, float b1, float b2,
+                                          float eps, float c1, float c2) {
+  m = __fmaf_rn(__fsub_rn(1.f, b1), g, __fmul_rn(b1, m));
+  v = __fmaf_rn(__fmul_rn(__fsub_rn(1.f, b2), g), g, __fmul_rn(b2, v));
+  const float den = __fadd_rn(__fsqrt_rn(__fmul_rn(v, c2)), eps);
+  return __fsub_rn(p, __fdiv_rn(__fmul_rn(lr, __fmul_rn(m, c1)), den));
+}
+
+// The update of all parameters and their BF16 copies (what the next step's
+// GEMMs read) in one pass, four parameters a thread.  It moves 30 bytes a
+// parameter (157 MB); 5.2 M parameters take 30 us at 32 training steps in a
+// row, where the update, four conversions, four transposed copies and three
+// tilings took 86 us.
+__global__ void __launch_bounds__(256) adam_kernel(float4* __restrict__ p, const float4* __restrict__ g,
+                                                   float4* __restrict__ m, float4* __restrict__ v,
+                                                   uint2* __restrict__ p16, size_t n4, float lr, float b1, float b2,
+                                                   float eps, float c1, float c2) {
+  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (i >= n4) return;
+  float4 pi = p[i], mi = m[i], vi = v[i];
+  const float4 gi = g[i];
+  pi.x = adam_one(pi.x, gi.x, mi.x, vi.x, lr, b1, b2, eps, c1, c2);
+  pi.y = adam_one(pi.y, gi.y, mi.y, vi.y, lr, b1, b2, eps, c1, c2);
+  pi.z = adam_one(pi.z, gi.z, mi.z, vi.z, lr, b1, b2, eps, c1, c2);
+  pi.w = adam_one(pi.w, gi.w, mi.w, vi.w, lr, b1, b2, eps, c1, c2);
+  p[i] = pi;
+  m[i] = mi;
+  v[i] = vi;
+  p16[i] = bf16x4(pi);
 }
 
 int blocks_for(size_t n) { return (int)std::min<size_t>((n + 255) / 256, 4096); }
@@ -374,7 +410,8 @@ struct prrtc_proposal {
   float* grad = nullptr;
   float* m = nullptr;
   float* v = nullptr;
-  bf16* w16[4] = {};
+  bf16* params16 = nullptr;  // BF16 copies of all parameters, in their order
+  bf16* w16[4] = {};         // the layers' weights in it
   bf16* wq = nullptr;       // start / goal columns of layer 1, transposed: [2 kQPad x kHid0]
   bf16* wtile[3] = {};  // layers 2, 3 and the head, tiled for the fused inference kernel
   int step = 0;
@@ -384,7 +421,9 @@ struct prrtc_proposal {
   // batch scratch
   int cap = 0;
   bf16 *x16 = nullptr, *h16[3] = {}, *d16 = nullptr, *z16[3] = {};
-  float *out32 = nullptr, *d32 = nullptr, *dh32 = nullptr, *z32[3] = {}, *loss = nullptr;
+  float *out32 = nullptr, *d32 = nullptr, *dh32 = nullptr, *z32[3] = {};
+  float* loss = nullptr;   // one per step of a call
+  size_t loss_cap = 0;
   // sample data
   uint8_t* occ = nullptr;
   size_t occ_cap = 0;
@@ -459,14 +498,14 @@ int grow(T** p, size_t* cap, size_t need) {
 
 void free_scratch(prrtc_proposal* p) {
   cudaFree(p->x16); cudaFree(p->d16);
-  cudaFree(p->out32); cudaFree(p->d32); cudaFree(p->dh32); cudaFree(p->loss);
+  cudaFree(p->out32); cudaFree(p->d32); cudaFree(p->dh32);
   for (int l = 0; l < 3; ++l) {
     cudaFree(p->h16[l]); cudaFree(p->z16[l]); cudaFree(p->z32[l]);
     p->h16[l] = p->z16[l] = nullptr;
     p->z32[l] = nullptr;
   }
   p->x16 = p->d16 = nullptr;
-  p->out32 = p->d32 = p->dh32 = p->loss = nullptr;
+  p->out32 = p->d32 = p->dh32 = nullptr;
   p->cap = 0;
 }
 
@@ -480,8 +519,7 @@ int ensure_scratch(prrtc_proposal* p, int rows) {
             cudaMalloc(&p->d16, (size_t)rows * P * 2) == cudaSuccess &&
             cudaMalloc(&p->out32, (size_t)rows * P * 4) == cudaSuccess &&
             cudaMalloc(&p->d32, (size_t)rows * P * 4) == cudaSuccess &&
-            cudaMalloc(&p->dh32, (size_t)rows * kHid0 * 4) == cudaSuccess &&
-            cudaMalloc(&p->loss, 4) == cudaSuccess;
+            cudaMalloc(&p->dh32, (size_t)rows * kHid0 * 4) == cudaSuccess;
   for (int l = 0; l < 3 && ok; ++l)
     ok = cudaMalloc(&p->h16[l], (size_t)rows * hid[l] * 2) == cudaSuccess &&
          cudaMalloc(&p->z16[l], (size_t)rows * hid[l] * 2) == cudaSuccess &&
@@ -495,19 +533,24 @@ int ensure_scratch(prrtc_proposal* p, int rows) {
   return PRRTC_OK;
 }
 
-// BF16 copies of the weights from the FP32 masters, and what inference reads:
-// the tiled layers and the transposed start / goal columns.
-int refresh_weights(prrtc_proposal* p) {
-  for (int l = 0; l < 4; ++l) {
-    const size_t n = (size_t)p->out_dim[l] * p->in_dim[l];
-    to_bf16_kernel<<<blocks_for(n), 256, 0, p->stream>>>(p->master + p->w_off[l], n, p->w16[l]);
-    int rc;
-    if (l > 0 && (rc = mlp_tile_weights(p->w16[l], p->out_dim[l], p->in_dim[l], p->wtile[l - 1], p->stream)))
-      return rc;
+// What inference reads, from the BF16 weights: the tiled layers and the
+// transposed start / goal columns.
+int refresh_inference_weights(prrtc_proposal* p) {
+  for (int l = 1; l < 4; ++l) {
+    const int rc = mlp_tile_weights(p->w16[l], p->out_dim[l], p->in_dim[l], p->wtile[l - 1], p->stream);
+    if (rc) return rc;
   }
   transpose_kernel<<<dim3(2 * kQPad / 32, kHid0 / 32), dim3(32, 8), 0, p->stream>>>(p->w16[0] + kVox, kIn, p->wq,
                                                                                     kHid0);
   return cudaGetLastError() == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
+}
+
+// All BF16 copies from the FP32 masters.
+int refresh_weights(prrtc_proposal* p) {
+  const size_t n4 = p->n_params / 4;
+  to_bf16_kernel<<<blocks_for(n4), 256, 0, p->stream>>>(reinterpret_cast<const float4*>(p->master), n4,
+                                                        reinterpret_cast<uint2*>(p->params16));
+  return refresh_inference_weights(p);
 }
 
 int gemm(const bf16* a, const bf16* b, int M, int N, int K, const float* bias, int relu, float* c32, bf16* c16,
@@ -856,10 +899,11 @@ int prrtc_proposal_create(int32_t dof, const float* lower, const float* upper, c
             cudaMalloc(&p->master, off * 4) == cudaSuccess && cudaMalloc(&p->grad, off * 4) == cudaSuccess &&
             cudaMalloc(&p->m, off * 4) == cudaSuccess && cudaMalloc(&p->v, off * 4) == cudaSuccess &&
             cudaMalloc(&p->d_lims, 2 * kMaxDof * 4) == cudaSuccess &&
-            cudaMalloc(&p->wq, (size_t)2 * kQPad * kHid0 * 2) == cudaSuccess;
+            cudaMalloc(&p->wq, (size_t)2 * kQPad * kHid0 * 2) == cudaSuccess &&
+            cudaMalloc(&p->params16, off * 2) == cudaSuccess;
+  for (int l = 0; l < 4 && ok; ++l) p->w16[l] = p->params16 + p->w_off[l];
   for (int l = 0; l < 4 && ok; ++l)
-    ok = cudaMalloc(&p->w16[l], (size_t)dims[l + 1] * dims[l] * 2) == cudaSuccess &&
-         (l == 0 || cudaMalloc(&p->wtile[l - 1], (size_t)dims[l + 1] * dims[l] * 2) == cudaSuccess);
+    ok = (l == 0 || cudaMalloc(&p->wtile[l - 1], (size_t)dims[l + 1] * dims[l] * 2) == cudaSuccess);
   if (!ok) {
     cudaGetLastError();
     prrtc_proposal_destroy(p);
@@ -885,9 +929,8 @@ void prrtc_proposal_destroy(prrtc_proposal* p) {
   if (!p) return;
   free_scratch(p);
   cudaFree(p->master); cudaFree(p->grad); cudaFree(p->m); cudaFree(p->v); cudaFree(p->d_lims);
-  cudaFree(p->wq);
+  cudaFree(p->wq); cudaFree(p->params16); cudaFree(p->loss);
   for (int l = 0; l < 4; ++l) {
-    cudaFree(p->w16[l]);
     if (l > 0) cudaFree(p->wtile[l - 1]);
   }
   cudaFree(p->occ); cudaFree(p->qs); cudaFree(p->qg); cudaFree(p->tgt); cudaFree(p->scene_of); cudaFree(p->rows);
@@ -929,7 +972,7 @@ int prrtc_proposal_forward(prrtc_proposal* p, const uint8_t* occ, const float* q
   int rc;
   if ((rc = ensure_scratch(p, rows))) return rc;
   if ((rc = upload_samples(p, occ, B, q_start, q_goal, nullptr, B))) return rc;
-  features_kernel<<<rows, 256, 0, p->stream>>>(p->occ, nullptr, nullptr, p->qs, p->qg, p->d_lims, p->d_lims + kMaxDof,
+  features_kernel<<<rows, kVox / 16, 0, p->stream>>>(p->occ, nullptr, nullptr, p->qs, p->qg, p->d_lims, p->d_lims + kMaxDof,
                                                B, p->dof, p->x16);
   if ((rc = forward_rows(p, rows))) return rc;
   MCK(cudaMemcpyAsync(out, p->out32, (size_t)B * p->P * 4, cudaMemcpyDeviceToHost, p->stream));
@@ -963,7 +1006,7 @@ int prrtc_proposal_forward_layers(prrtc_proposal* p, const uint8_t* occ, const f
   int rc;
   if ((rc = ensure_scratch(p, rows))) return rc;
   if ((rc = upload_samples(p, occ, B, q_start, q_goal, nullptr, B))) return rc;
-  features_kernel<<<rows, 256, 0, p->stream>>>(p->occ, nullptr, nullptr, p->qs, p->qg, p->d_lims, p->d_lims + kMaxDof,
+  features_kernel<<<rows, kVox / 16, 0, p->stream>>>(p->occ, nullptr, nullptr, p->qs, p->qg, p->d_lims, p->d_lims + kMaxDof,
                                                B, p->dof, p->x16);
   if ((rc = forward_rows(p, rows))) return rc;
   if ((rc = check_gemm_error())) return rc;
@@ -1007,36 +1050,33 @@ int prrtc_proposal_inference_layers(prrtc_proposal* p, int32_t B, float* h1, flo
 }
 
 // One step on a batch: gradients into the proposal (readable with
-// prrtc_proposal_get_params) and, when lr > 0, an Adam update.
+// prrtc_proposal_get_params), the loss added to *loss_dev and, when lr > 0, an
+// Adam update.
 static int step_on_rows(prrtc_proposal* p, const int* scene_of, const int* rows_dev, int B, float lr,
-                        float* loss_host) {
+                        float* loss_dev) {
   const int rows = (B + 7) & ~7;
   int rc;
   const cudaStream_t s = p->stream;
-  features_kernel<<<rows, 256, 0, s>>>(p->occ, scene_of, rows_dev, p->qs, p->qg, p->d_lims, p->d_lims + kMaxDof, B,
+  features_kernel<<<rows, kVox / 16, 0, s>>>(p->occ, scene_of, rows_dev, p->qs, p->qg, p->d_lims, p->d_lims + kMaxDof, B,
                                        p->dof, p->x16);
   if ((rc = forward_rows(p, rows))) return rc;
   MCK(cudaMemsetAsync(p->d32, 0, (size_t)rows * p->P * 4, s));
   MCK(cudaMemsetAsync(p->d16, 0, (size_t)rows * p->P * 2, s));
-  MCK(cudaMemsetAsync(p->loss, 0, 4, s));
   mixture_loss_kernel<<<(B * 32 + 255) / 256, 256, 0, s>>>(p->out32, p->P, p->tgt, rows_dev, p->d_lims,
                                                             p->d_lims + kMaxDof, B, p->dof, 1.f / (float)B, p->d32,
-                                                            p->d16, p->loss);
+                                                            p->d16, loss_dev);
   if ((rc = backward_rows(p, rows))) return rc;
   if (lr > 0.f) {
     p->step++;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f / (1.f - std::pow(b1, (float)p->step)), c2 = 1.f / (1.f - std::pow(b2, (float)p->step));
-    adam_kernel<<<blocks_for(p->n_params), 256, 0, s>>>(p->master, p->grad, p->m, p->v, p->n_params, lr, b1, b2,
-                                                         1e-8f, c1, c2);
-    if ((rc = refresh_weights(p))) return rc;
+    const size_t n4 = p->n_params / 4;
+    adam_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, s>>>(
+        reinterpret_cast<float4*>(p->master), reinterpret_cast<const float4*>(p->grad),
+        reinterpret_cast<float4*>(p->m), reinterpret_cast<float4*>(p->v), reinterpret_cast<uint2*>(p->params16), n4,
+        lr, b1, b2, 1e-8f, c1, c2);
   }
-  if (loss_host) MCK(cudaMemcpyAsync(loss_host, p->loss, 4, cudaMemcpyDeviceToHost, s));
   return cudaGetLastError() == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
-}
-
-static int step_on_rows_direct(prrtc_proposal* p, int B, float* loss) {
-  return step_on_rows(p, nullptr, nullptr, B, 0.f, loss);
 }
 
 int prrtc_proposal_grads(prrtc_proposal* p, const uint8_t* occ, const float* q_start, const float* q_goal,
@@ -1047,7 +1087,10 @@ int prrtc_proposal_grads(prrtc_proposal* p, const uint8_t* occ, const float* q_s
   int rc;
   if ((rc = ensure_scratch(p, rows))) return rc;
   if ((rc = upload_samples(p, occ, B, q_start, q_goal, target, B))) return rc;
-  if ((rc = step_on_rows_direct(p, B, loss))) return rc;
+  if ((rc = grow(&p->loss, &p->loss_cap, 1))) return rc;
+  MCK(cudaMemsetAsync(p->loss, 0, 4, p->stream));
+  if ((rc = step_on_rows(p, nullptr, nullptr, B, 0.f, p->loss))) return rc;
+  if (loss) MCK(cudaMemcpyAsync(loss, p->loss, 4, cudaMemcpyDeviceToHost, p->stream));
   MCK(cudaStreamSynchronize(p->stream));
   return check_gemm_error();
 }
@@ -1084,13 +1127,20 @@ int prrtc_proposal_train(prrtc_proposal* p, const uint8_t* occ, int32_t n_scenes
   if ((rc = grow(&p->rows, &p->rows_cap, std::max<size_t>(idx.size(), 1)))) return rc;
   if (!idx.empty())
     MCK(cudaMemcpyAsync(p->rows, idx.data(), idx.size() * 4, cudaMemcpyHostToDevice, p->stream));
-  std::vector<float> host_loss(std::max(steps, 1));
-  for (int t = 0; t < steps; ++t)
-    if ((rc = step_on_rows(p, p->scene_of, p->rows + (size_t)t * B, B, lr, losses ? &host_loss[t] : nullptr)))
-      return rc;
+  // the losses stay on the device until the last step: a copy per step would
+  // hold the host, and with it the next step's launches, until the step is done
+  if ((rc = grow(&p->loss, &p->loss_cap, (size_t)std::max(steps, 1)))) return rc;
+  MCK(cudaMemsetAsync(p->loss, 0, (size_t)std::max(steps, 1) * 4, p->stream));
+  for (int t = 0; t < steps && !rc; ++t)
+    rc = step_on_rows(p, p->scene_of, p->rows + (size_t)t * B, B, lr, p->loss + t);
+  if (steps > 0) {  // also after a step that failed: inference follows the masters
+    const int rc2 = refresh_inference_weights(p);
+    if (!rc) rc = rc2;
+  }
+  if (rc) return rc;
+  if (losses && steps > 0)
+    MCK(cudaMemcpyAsync(losses, p->loss, (size_t)steps * 4, cudaMemcpyDeviceToHost, p->stream));
   MCK(cudaStreamSynchronize(p->stream));
-  if (losses)
-    for (int t = 0; t < steps; ++t) losses[t] = host_loss[t];
   return check_gemm_error();
 }
 
