@@ -67,7 +67,6 @@ struct Epilogue {
   int m_tiles, n_tiles, k_tiles;
   int m_pad;             // rows of one split's partial (M rounded up to the tile), so that the
                          // clipped-off rows of an edge tile never reach the next split's rows
-  int ta, tb;            // operand stored transposed: [K x M] / [K x N], M / N contiguous
 };
 
 // Output tensor maps of one launch: workspace (FP32, rows = splits * m_pad),
@@ -260,6 +259,8 @@ __device__ __forceinline__ void store_chunk(const Epilogue& ep, const OutMaps& o
   if (ep.has_c16) stage_and_store(&om.c16, tiles, buf, true, col0, row0, lane, f);
 }
 
+// kTA, kTB: operand stored transposed.
+template <bool kTA, bool kTB>
 __global__ void __launch_bounds__(THREADS, 1)
     gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const __grid_constant__ OutMaps om, Epilogue ep) {
@@ -326,14 +327,14 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (lane == 0) {
           unsigned char* a = smem + s * STAGE_BYTES;
           mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
-          if (ep.ta) {
+          if (kTA) {
 #pragma unroll
             for (int j = 0; j < BM / 64; ++j)
               tma_load_2d(a + j * MN_BOX_BYTES, &tmA, &full[s], w.m0 + 64 * j, kt * BK);
           } else {
             tma_load_2d(a, &tmA, &full[s], kt * BK, w.m0);
           }
-          if (ep.tb) {
+          if (kTB) {
 #pragma unroll
             for (int j = 0; j < BN / 64; ++j)
               tma_load_2d(a + A_BYTES + j * MN_BOX_BYTES, &tmB, &full[s], w.n0 + 64 * j, kt * BK);
@@ -345,9 +346,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    const uint32_t idesc = idesc_bf16(BM, BN) | (ep.ta ? 1u << 15 : 0u) | (ep.tb ? 1u << 16 : 0u);
+    const uint32_t idesc = idesc_bf16(BM, BN) | (kTA ? 1u << 15 : 0u) | (kTB ? 1u << 16 : 0u);
     // from one K step of 16 to the next: 32 bytes along K, or 16 lines of K
-    const uint32_t step_a = ep.ta ? 2048u : 32u, step_b = ep.tb ? 2048u : 32u;
+    constexpr uint32_t step_a = kTA ? 2048u : 32u, step_b = kTB ? 2048u : 32u;
     int it = 0, i = 0;  // stage counter, local unit counter
     bool ok = true;
     for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x, ++i) {
@@ -380,8 +381,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           const uint32_t b = a + A_BYTES;
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
-            mma_bf16(d, ep.ta ? smem_desc_mn(a + step_a * k) : smem_desc(a + step_a * k),
-                     ep.tb ? smem_desc_mn(b + step_b * k) : smem_desc(b + step_b * k), idesc,
+            mma_bf16(d, kTA ? smem_desc_mn(a + step_a * k) : smem_desc(a + step_a * k),
+                     kTB ? smem_desc_mn(b + step_b * k) : smem_desc(b + step_b * k), idesc,
                      (kt > w.kt0 || k > 0) ? 1u : 0u);
           mma_commit(&empty[s]);
         }
@@ -479,6 +480,258 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ ws, int splits, i
   }
 }
 
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
+  __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<uint32_t*>(&h);
+}
+
+// ------------------------------------------------------------ GEMMs below one wave
+// The layers' products at training and inference batches fill less than one
+// wave of 128 x 256 tiles even with K split, and are bound by what happens
+// once per launch: the first loads, the tile's way out, the partials' round
+// trip through memory and a second kernel.  Here a cluster of `splits` blocks
+// owns one 128 x kBN output tile (kBN 64 or 128) and each block one range of
+// K, the same ranges as above.  The blocks leave their FP32 partial tiles in
+// shared memory; after a cluster barrier, block r adds up rows
+// [128 r / splits, 128 (r + 1) / splits) over all blocks in split order (the
+// sums of the second kernel, bit for bit) and writes the outputs.
+//
+// Launches in a row, bias, ReLU and BF16 output, in us (128 x 256 tiles and
+// second kernel before): 512 x 512 x 1024 5.6 (9.6), 512 x 512 x 512 5.4 (9.2),
+// 1024 x 4160 x 512 8.1 (15.5), 2048 x 1024 x 4160 19.5 (23.5), 512 x 1024 x
+// 4160 12.7 (12.5: there the eight partial tiles' exchange costs what the
+// second kernel did).  About 1 us goes to the launch, 0.9 to tensor memory and
+// the first loads, 0.3 to each K tile, 1 to the cluster barriers.
+//
+// Roles as above: warp 0 loads, warp 1 issues the MMAs, warps 2-5 read the
+// accumulator; all six add up.  The partial tile takes the ring's place: every
+// load has landed and every MMA has read it by then.  Waits are bounded; a
+// role that gives up records the error, and every thread still meets every
+// barrier.
+template <int kBN>
+struct ClusterTile {
+  static constexpr int kStages = kBN == 64 ? 4 : 3;  // two blocks per SM
+  static constexpr int kBBytes = kBN * BK * 2;
+  static constexpr int kStageBytes = A_BYTES + kBBytes;
+  static constexpr int kSmem = kStages * kStageBytes + 1024 + 256;
+  static_assert(BM * kBN * 4 <= kStages * kStageBytes, "the partial tile fits the ring");
+};
+constexpr int kMaxClusterSplits = 8;  // portable cluster size
+constexpr int kClusterThreads = 256;
+
+struct ClusterEpilogue {
+  int M, N, k_tiles, m_tiles;
+  const float* bias;
+  int relu;
+  const __nv_bfloat16* mask;  // nullable [M x N] of row stride ldm: outputs where mask <= 0 become 0
+  int ldm;
+  float* c32;
+  int ldc32;
+  __nv_bfloat16* c16;
+  int ldc16;
+};
+
+// Byte offset of 16-byte unit u of row i of a partial tile (rows of kBN
+// floats): units of a 128-byte group are exchanged by the row, so that both
+// the row-per-lane writes and the unit-per-thread reads touch every bank once.
+template <int kBN>
+__device__ __forceinline__ uint32_t part_off(int i, int u) {
+  return (uint32_t)i * (kBN * 4) + (uint32_t)((u & ~7) | ((u ^ i) & 7)) * 16u;
+}
+
+template <int kBN, int kSplits, bool kTA, bool kTB>
+__global__ void __launch_bounds__(kClusterThreads, 2)
+    gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                        const ClusterEpilogue ep) {
+  using T = ClusterTile<kBN>;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* smem =
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + T::kStages * T::kStageBytes);
+  uint64_t* empty = full + T::kStages;
+  uint64_t* acc_full = empty + T::kStages;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int split = (int)blockIdx.x % kSplits, tile = (int)blockIdx.x / kSplits;
+  const int m0 = tile % ep.m_tiles * BM, n0 = tile / ep.m_tiles * kBN;
+  const int base = ep.k_tiles / kSplits, rem = ep.k_tiles % kSplits;
+  const int kt0 = split * base + min(split, rem), kts = base + (split < rem ? 1 : 0);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < T::kStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(acc_full, 1);
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"((uint32_t)kBN)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int it = 0;
+      for (; it < kts; ++it) {
+        const int s = it % T::kStages;
+        if (!wait_bar(&empty[s], ((uint32_t)(it / T::kStages) & 1u) ^ 1u)) break;
+        unsigned char* a = smem + s * T::kStageBytes;
+        const int kt = kt0 + it;
+        mbar_arrive_expect_tx(&full[s], T::kStageBytes);
+        if (kTA) {
+#pragma unroll
+          for (int j = 0; j < BM / 64; ++j)
+            tma_load_2d(a + j * MN_BOX_BYTES, &tmA, &full[s], m0 + 64 * j, kt * BK);
+        } else {
+          tma_load_2d(a, &tmA, &full[s], kt * BK, m0);
+        }
+        if (kTB) {
+#pragma unroll
+          for (int j = 0; j < kBN / 64; ++j)
+            tma_load_2d(a + A_BYTES + j * MN_BOX_BYTES, &tmB, &full[s], n0 + 64 * j, kt * BK);
+        } else {
+          tma_load_2d(a + A_BYTES, &tmB, &full[s], kt * BK, n0);
+        }
+      }
+      // the loads have landed before the block can leave, also after a give-up
+      for (int s = 0; s < T::kStages && s < it; ++s) wait_bar(&full[s], (uint32_t)((it - 1 - s) / T::kStages) & 1u);
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    const uint32_t idesc = idesc_bf16(BM, kBN) | (kTA ? 1u << 15 : 0u) | (kTB ? 1u << 16 : 0u);
+    constexpr uint32_t step_a = kTA ? 2048u : 32u, step_b = kTB ? 2048u : 32u;
+    if (lane == 0) {
+      bool ok = true;
+      for (int it = 0; it < kts && ok; ++it) {
+        const int s = it % T::kStages;
+        ok = wait_bar(&full[s], (uint32_t)(it / T::kStages) & 1u);
+        if (!ok) break;
+        fence_after();
+        const uint32_t a = smem_u32(smem + s * T::kStageBytes), b = a + A_BYTES;
+#pragma unroll
+        for (int k = 0; k < BK / 16; ++k)
+          mma_bf16(tmem, kTA ? smem_desc_mn(a + step_a * k) : smem_desc(a + step_a * k),
+                   kTB ? smem_desc_mn(b + step_b * k) : smem_desc(b + step_b * k), idesc,
+                   (it > 0 || k > 0) ? 1u : 0u);
+        mma_commit(&empty[s]);
+      }
+      mma_commit(acc_full);  // completes once every MMA issued so far has
+    }
+    __syncwarp();
+  } else if (warp < 6) {
+    const int q = warp & 3;  // TMEM lane quarter this warp may access
+    int ok = 0;
+    if (lane == 0) ok = wait_bar(acc_full, 0u) ? 1 : 0;
+    ok = __shfl_sync(kFull, ok, 0);
+    if (ok) {
+      fence_after();
+      const int i = 32 * q + lane;
+#pragma unroll
+      for (int c = 0; c < kBN; c += 32) {
+        uint32_t v[32];
+        tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c, v);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          *reinterpret_cast<uint4*>(smem + part_off<kBN>(i, c / 4 + u)) =
+              make_uint4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
+      }
+    }
+    fence_before();
+  }
+  if (kSplits > 1)
+    cluster_sync_all();
+  else
+    __syncthreads();
+  fence_after();
+  if (warp == 1)  // every read of the accumulator is done
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kBN) : "memory");
+
+  // This block's rows, 16 bytes a thread and turn; the loads of kAhead turns
+  // and all blocks are in flight together (one by one this part took as long
+  // as the whole product).
+  constexpr int kUnits = kBN / 4, kRows = BM / kSplits, kTurns = kRows * kUnits / kClusterThreads;
+  constexpr int kAhead = kTurns < 8 / kSplits ? kTurns : (8 / kSplits > 0 ? 8 / kSplits : 1);
+  static_assert(kTurns * kClusterThreads == kRows * kUnits && kTurns % kAhead == 0, "whole turns");
+  const int u = threadIdx.x % kUnits, col = n0 + 4 * u;
+  float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (ep.bias && col < ep.N)  // any alignment
+    bias = make_float4(__ldg(ep.bias + col), __ldg(ep.bias + col + 1), __ldg(ep.bias + col + 2), __ldg(ep.bias + col + 3));
+  for (int turn = 0; turn < kTurns; turn += kAhead) {
+    float4 part[kAhead][kSplits];
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) {
+      const int i = split * kRows + ((turn + j) * kClusterThreads + (int)threadIdx.x) / kUnits;
+      const uint32_t off = smem_u32(smem) + part_off<kBN>(i, u);
+#pragma unroll
+      for (int s = 0; s < kSplits; ++s) {
+        float4& p = part[j][s];
+        if (kSplits == 1) {
+          asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(p.x), "=f"(p.y), "=f"(p.z), "=f"(p.w) : "r"(off));
+        } else {
+          uint32_t remote;
+          asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(off), "r"(s));
+          asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                       : "=f"(p.x), "=f"(p.y), "=f"(p.z), "=f"(p.w)
+                       : "r"(remote));
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) {
+      const int i = split * kRows + ((turn + j) * kClusterThreads + (int)threadIdx.x) / kUnits;
+      const int row = m0 + i;
+      float4 acc = part[j][0];
+#pragma unroll
+      for (int s = 1; s < kSplits; ++s) {
+        acc.x += part[j][s].x;
+        acc.y += part[j][s].y;
+        acc.z += part[j][s].z;
+        acc.w += part[j][s].w;
+      }
+      if (row >= ep.M || col >= ep.N) continue;
+      if (ep.bias) {
+        acc.x += bias.x;
+        acc.y += bias.y;
+        acc.z += bias.z;
+        acc.w += bias.w;
+      }
+      if (ep.relu) {
+        acc.x = fmaxf(acc.x, 0.f);
+        acc.y = fmaxf(acc.y, 0.f);
+        acc.z = fmaxf(acc.z, 0.f);
+        acc.w = fmaxf(acc.w, 0.f);
+      }
+      if (ep.mask) {
+        const uint2 h = *reinterpret_cast<const uint2*>(ep.mask + (size_t)row * ep.ldm + col);
+        const __nv_bfloat162 h0 = *reinterpret_cast<const __nv_bfloat162*>(&h.x);
+        const __nv_bfloat162 h1 = *reinterpret_cast<const __nv_bfloat162*>(&h.y);
+        acc.x = __low2float(h0) > 0.f ? acc.x : 0.f;
+        acc.y = __high2float(h0) > 0.f ? acc.y : 0.f;
+        acc.z = __low2float(h1) > 0.f ? acc.z : 0.f;
+        acc.w = __high2float(h1) > 0.f ? acc.w : 0.f;
+      }
+      if (ep.c32) *reinterpret_cast<float4*>(ep.c32 + (size_t)row * ep.ldc32 + col) = acc;
+      if (ep.c16)
+        *reinterpret_cast<uint2*>(ep.c16 + (size_t)row * ep.ldc16 + col) =
+            make_uint2(pack_bf16x2(acc.x, acc.y), pack_bf16x2(acc.z, acc.w));
+    }
+  }
+  if (kSplits > 1) cluster_sync_all();  // the other blocks have read this one's partial tile
+}
+
 // ------------------------------------------------------------ fused inference
 // The learned proposal's forward pass for planning, after the occupancy part
 // of the first layer, in one launch.  A cluster of kIC CTAs owns 128 problem
@@ -532,11 +785,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // Global writes of this thread -> visible to the cluster's async-proxy reads
 // after the barrier; every thread of the cluster calls it.
 __device__ __forceinline__ void cluster_publish() {
@@ -544,11 +792,6 @@ __device__ __forceinline__ void cluster_publish() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   asm volatile("fence.proxy.async.global;" ::: "memory");
-}
-
-__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
-  __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&h);
 }
 
 // Weight matrix [N x K] (BF16, row-major) -> tiles [kIC slices][K/64 k-blocks]
@@ -959,14 +1202,83 @@ float* workspace(size_t floats, cudaStream_t stream) {
   return w.ptr;
 }
 
-int g_sms = 0;
+}  // namespace
+
+namespace {
+
+// Tile width of the cluster kernel for a product, 0: not its size.  One wave:
+// two blocks per SM.
+int cluster_bn(int m_tiles, int N, int splits, int sms) {
+  for (int bn : {64, 128})
+    if (m_tiles * ((N + bn - 1) / bn) * splits <= 2 * sms) return bn;
+  return 0;
+}
+
+template <int kBN, int kSplits, bool kTA, bool kTB>
+int launch_cluster_as(const CUtensorMap& ma, const CUtensorMap& mb, const ClusterEpilogue& ep, cudaStream_t stream) {
+  using T = ClusterTile<kBN>;
+  auto* fn = gemm_cluster_kernel<kBN, kSplits, kTA, kTB>;
+  static bool attr = false;
+  if (!attr) {
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, T::kSmem) != cudaSuccess)
+      return PRRTC_ERR_CUDA;
+    attr = true;
+  }
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kSplits;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3(ep.m_tiles * ((ep.N + kBN - 1) / kBN) * kSplits);
+  lc.blockDim = dim3(kClusterThreads);
+  lc.dynamicSmemBytes = T::kSmem;
+  lc.stream = stream;
+  lc.attrs = &at;
+  lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, fn, ma, mb, ep) == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
+}
+
+template <int kBN, int kSplits>
+int launch_cluster_split(bool ta, bool tb, const CUtensorMap& ma, const CUtensorMap& mb, const ClusterEpilogue& ep,
+                         cudaStream_t stream) {
+  if (ta) return tb ? launch_cluster_as<kBN, kSplits, true, true>(ma, mb, ep, stream) : PRRTC_ERR_UNSUPPORTED;
+  return tb ? launch_cluster_as<kBN, kSplits, false, true>(ma, mb, ep, stream)
+            : launch_cluster_as<kBN, kSplits, false, false>(ma, mb, ep, stream);
+}
+
+template <int kBN>
+int launch_cluster(int splits, bool ta, bool tb, const CUtensorMap& ma, const CUtensorMap& mb,
+                   const ClusterEpilogue& ep, cudaStream_t stream) {
+  switch (splits) {
+    case 1: return launch_cluster_split<kBN, 1>(ta, tb, ma, mb, ep, stream);
+    case 2: return launch_cluster_split<kBN, 2>(ta, tb, ma, mb, ep, stream);
+    case 4: return launch_cluster_split<kBN, 4>(ta, tb, ma, mb, ep, stream);
+    case 8: return launch_cluster_split<kBN, 8>(ta, tb, ma, mb, ep, stream);
+    default: return PRRTC_ERR_UNSUPPORTED;
+  }
+}
+
+template <bool kTA, bool kTB>
+int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, const OutMaps& om, const Epilogue& ep, int grid,
+                cudaStream_t stream) {
+  auto* fn = gemm_bf16_kernel<kTA, kTB>;
+  static bool attr = false;
+  if (!attr) {
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess)
+      return PRRTC_ERR_CUDA;
+    attr = true;
+  }
+  fn<<<grid, THREADS, SMEM_BYTES, stream>>>(ma, mb, om, ep);
+  return cudaGetLastError() == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
+}
 
 }  // namespace
 
 // Host launcher used by the MLP code and the C ABI entry point.  splits_hint:
 // 0 = choose (split K while the tiles fill less than one wave), else forced.
 int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, int K, const float* bias, int relu,
-                 float* c32, int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint, int trans) {
+                 float* c32, int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint, int trans,
+                 const void* mask, int ldm) {
   const int ta = trans & kTransA ? 1 : 0, tb = trans & kTransB ? 1 : 0;
   if (M <= 0 || N <= 0 || K <= 0 || !a || !b || (!c32 && !c16)) return PRRTC_ERR_INVALID_ARG;
   if (K % 8 || N % 8 || (c32 && ldc32 % 4) || (c16 && ldc16 % 8)) return PRRTC_ERR_UNSUPPORTED;
@@ -975,29 +1287,19 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
   if ((c32 && (reinterpret_cast<uintptr_t>(c32) & 15)) || (c16 && (reinterpret_cast<uintptr_t>(c16) & 15)))
     return PRRTC_ERR_INVALID_ARG;
   CUtensorMap ma, mb;
-  if (!(ta ? cached_map(&ma, a, K, M, lda, 0, BK) : cached_map(&ma, a, M, K, lda, 0, BM)) ||
-      !(tb ? cached_map(&mb, b, K, N, ldb, 0, BK) : cached_map(&mb, b, N, K, ldb, 0, BN)))
-    return PRRTC_ERR_CUDA;
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(gemm_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess)
-      return PRRTC_ERR_CUDA;
-    int dev = 0;
+  if (!(ta ? cached_map(&ma, a, K, M, lda, 0, BK) : cached_map(&ma, a, M, K, lda, 0, BM))) return PRRTC_ERR_CUDA;
+  static const int sms = [] {
+    int dev = 0, n = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
-    attr = true;
-  }
-  Epilogue ep{M, N, K, bias, relu, c32 ? 1 : 0, c16 ? 1 : 0, 1, 0, 0, 0, 0, ta, tb};
-  OutMaps om;
-  std::memset(&om, 0, sizeof(om));
-  if (c32 && !cached_map(&om.c32, c32, M, N, ldc32, 2)) return PRRTC_ERR_CUDA;
-  if (c16 && !cached_map(&om.c16, c16, M, N, ldc16, 3)) return PRRTC_ERR_CUDA;
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n > 0 ? n : 1;
+  }();
+  Epilogue ep{M, N, K, bias, relu, c32 ? 1 : 0, c16 ? 1 : 0, 1, 0, 0, 0, 0};
   ep.m_tiles = (M + BM - 1) / BM;
   ep.n_tiles = (N + BN - 1) / BN;
   ep.k_tiles = (K + BK - 1) / BK;
   ep.m_pad = ep.m_tiles * BM;
   const int tiles = ep.m_tiles * ep.n_tiles;
-  const int sms = g_sms > 0 ? g_sms : 1;
   int splits = splits_hint;
   if (splits <= 0) {
     splits = 1;
@@ -1005,6 +1307,21 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
       splits *= 2;
   }
   splits = std::max(1, std::min(splits, std::min(kMaxSplits, ep.k_tiles)));
+  if (splits <= kMaxClusterSplits && (splits & (splits - 1)) == 0) {
+    const int bn = cluster_bn(ep.m_tiles, N, splits, sms);
+    if (bn) {
+      ClusterEpilogue ce{M, N, ep.k_tiles, ep.m_tiles, bias, relu, static_cast<const __nv_bfloat16*>(mask),
+                         ldm, c32, ldc32, static_cast<__nv_bfloat16*>(c16), ldc16};
+      if (!(tb ? cached_map(&mb, b, K, N, ldb, 0, BK) : cached_map(&mb, b, N, K, ldb, 0, bn))) return PRRTC_ERR_CUDA;
+      return bn == 64 ? launch_cluster<64>(splits, ta, tb, ma, mb, ce, stream) : launch_cluster<128>(splits, ta, tb, ma, mb, ce, stream);
+    }
+  }
+  if (mask) return PRRTC_ERR_UNSUPPORTED;
+  if (!(tb ? cached_map(&mb, b, K, N, ldb, 0, BK) : cached_map(&mb, b, N, K, ldb, 0, BN))) return PRRTC_ERR_CUDA;
+  OutMaps om;
+  std::memset(&om, 0, sizeof(om));
+  if (c32 && !cached_map(&om.c32, c32, M, N, ldc32, 2)) return PRRTC_ERR_CUDA;
+  if (c16 && !cached_map(&om.c16, c16, M, N, ldc16, 3)) return PRRTC_ERR_CUDA;
   ep.splits = splits;
   float* ws = nullptr;
   if (splits > 1) {
@@ -1014,8 +1331,10 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
   }
   const int units = tiles * splits;
   const int grid = std::min(units, sms);
-  gemm_bf16_kernel<<<grid, THREADS, SMEM_BYTES, stream>>>(ma, mb, om, ep);
-  if (cudaGetLastError() != cudaSuccess) return PRRTC_ERR_CUDA;
+  const int rc = ta ? (tb ? launch_gemm<true, true>(ma, mb, om, ep, grid, stream) : PRRTC_ERR_UNSUPPORTED)
+                    : (tb ? launch_gemm<false, true>(ma, mb, om, ep, grid, stream)
+                          : launch_gemm<false, false>(ma, mb, om, ep, grid, stream));
+  if (rc) return rc;
   if (splits > 1) {
     const size_t work = (size_t)M * (N / 4);
     const int blocks = (int)std::min<size_t>((work + 255) / 256, (size_t)sms * 8);
@@ -1028,7 +1347,7 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
 
 int gemm_bf16_split(const void* a, const void* b, int M, int N, int K, const float* bias, int relu, float* c32,
                     int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint) {
-  return gemm_bf16_ld(a, K, b, K, M, N, K, bias, relu, c32, ldc32, c16, ldc16, stream, splits_hint, 0);
+  return gemm_bf16_ld(a, K, b, K, M, N, K, bias, relu, c32, ldc32, c16, ldc16, stream, splits_hint, 0, nullptr, 0);
 }
 
 int gemm_bf16(const void* a, const void* b, int M, int N, int K, const float* bias, int relu, float* c32, int ldc32,

@@ -272,10 +272,13 @@ int gemm_bf16(const void* a, const void* b, int M, int N, int K, const float* bi
 // operands, e.g. a column range of a wider weight matrix; splits_hint 0 = auto.
 // trans: operands stored the other way round, A as [K x M] rows of lda >= M,
 // B as [K x N] rows of ldb >= N (a gradient's operands as the layers wrote
-// them, without a transposed copy).
+// them, without a transposed copy).  mask (nullable, BF16 [M x N], row stride
+// ldm): outputs become 0 where it is not above 0 (a ReLU's gradient);
+// PRRTC_ERR_UNSUPPORTED for products above one wave.
 constexpr int kTransA = 1, kTransB = 2;
 int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, int K, const float* bias, int relu,
-                 float* c32, int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint, int trans);
+                 float* c32, int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint, int trans,
+                 const void* mask, int ldm);
 int gemm_take_error();
 // Copies the kernels' error word to *out on `stream` (does not clear it).
 cudaError_t gemm_read_error(int* out, cudaStream_t stream);

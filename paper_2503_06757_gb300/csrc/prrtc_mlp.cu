@@ -586,18 +586,24 @@ int backward_rows(prrtc_proposal* p, int rows) {
     const int in = p->in_dim[l], out = p->out_dim[l];
     // dW_l [out x in] = dZ^T H, both as stored: [rows x out], [rows x in]
     if ((rc = gemm_bf16_ld(dz16, out, hprev[l], in, out, in, rows, nullptr, 0, p->grad + p->w_off[l], in, nullptr, 0,
-                           s, 0, kTransA | kTransB)))
+                           s, 0, kTransA | kTransB, nullptr, 0)))
       return rc;
     cs.g[l] = dz32;
     cs.out[l] = p->grad + p->b_off[l];
     cs.cols[l] = out;
     if (l == 0) break;
     // dH_{l-1} [rows x in] = dZ [rows x out] W_l [out x in]
-    if ((rc = gemm_bf16_ld(dz16, out, p->w16[l], in, rows, in, out, nullptr, 0, p->dh32, in, nullptr, 0, s, 0,
-                           kTransB)))
-      return rc;
-    const size_t n = (size_t)rows * in;
-    relu_back_kernel<<<blocks_for(n), 256, 0, s>>>(p->dh32, p->h16[l - 1], n, p->z32[l - 1], p->z16[l - 1]);
+    // and dZ_{l-1} = dH_{l-1} where H_{l-1} > 0, in the same launch while the product is below one wave
+    rc = gemm_bf16_ld(dz16, out, p->w16[l], in, rows, in, out, nullptr, 0, p->z32[l - 1], in, p->z16[l - 1], in, s, 0,
+                      kTransB, p->h16[l - 1], in);
+    if (rc == PRRTC_ERR_UNSUPPORTED) {
+      if ((rc = gemm_bf16_ld(dz16, out, p->w16[l], in, rows, in, out, nullptr, 0, p->dh32, in, nullptr, 0, s, 0,
+                             kTransB, nullptr, 0)))
+        return rc;
+      const size_t n = (size_t)rows * in;
+      relu_back_kernel<<<blocks_for(n), 256, 0, s>>>(p->dh32, p->h16[l - 1], n, p->z32[l - 1], p->z16[l - 1]);
+    }
+    if (rc) return rc;
     dz16 = p->z16[l - 1];
     dz32 = p->z32[l - 1];
   }
@@ -656,7 +662,7 @@ int enqueue_inference(prrtc_proposal* p, const EnvView* d_envs, int U, const int
   } else {
     occ_bf16_kernel<<<U, 256, 0, s>>>(p->inf_occ, p->xo16);
     if ((rc = gemm_bf16_ld(p->xo16, kVox, p->w16[0], kIn, U, kHid0, kVox, nullptr, 0, p->h1o32, kHid0, nullptr, 0, s,
-                           0, 0)))
+                           0, 0, nullptr, 0)))
       return rc;
   }
   MCK(cudaGetLastError());
