@@ -765,6 +765,14 @@ int prrtc_robot_create(const prrtc_robot_desc* d, prrtc_robot** out) {
     }
     H.blk_frames[nb] = (uint32_t)fa | ((uint32_t)fb << 16);
     H.blk_range[nb] = (uint32_t)k | ((uint32_t)e << 16);
+    {
+      const int i0 = pairs[k].first, j0 = pairs[k].second;
+      const int ni = pairs[e - 1].first - i0 + 1, nj = pairs[e - 1].second - j0 + 1;
+      bool cross = (size_t)ni * (size_t)nj == e - k;
+      for (size_t t = k; t < e && cross; ++t)
+        cross = pairs[t].first == i0 + (int)(t - k) / nj && pairs[t].second == j0 + (int)(t - k) % nj;
+      H.blk_cross[nb] = cross ? (uint32_t)i0 | (uint32_t)j0 << 8 | (uint32_t)ni << 16 | (uint32_t)nj << 24 : 0u;
+    }
     const float rr = H.grp[fa].w + H.grp[fb].w;
     // one pair, or pairs within one link: no first stage
     H.blk_thr[nb] = (e - k > 1 && fa != fb) ? rr * rr : INFINITY;

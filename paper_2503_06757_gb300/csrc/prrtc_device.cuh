@@ -62,6 +62,9 @@ struct RobotHeader {
   uint32_t blk_frames[kMaxPairBlocks];  // fa | fb << 16
   uint32_t blk_range[kMaxPairBlocks];   // begin | end << 16
   float blk_thr[kMaxPairBlocks];
+  // A block that holds every pair of spheres i0 .. i0 + ni - 1 and
+  // j0 .. j0 + nj - 1: i0 | j0 << 8 | ni << 16 | nj << 24; else 0.
+  uint32_t blk_cross[kMaxPairBlocks];
 };
 
 // Pair table follows the header in device memory: pair[k] = i | (j << 16),
@@ -244,40 +247,6 @@ __device__ __forceinline__ bool sphere_hits_env(float cx, float cy, float cz, fl
   return hit;
 }
 
-// Two-stage test of one frame against the primitives of one type (Sec. III-A,
-// hierarchical check): the frame's bounding sphere (bx, by, bz, br) against
-// every primitive, 32 at a time; the flags of all active lanes are OR-ed, and
-// the frame's fine spheres s0..s1-1 (centres staged in `stage`) are tested
-// against the flagged primitives only.  The flag set is warp-uniform, so the
-// second stage runs without divergence.  Returns this lane's fine verdict and
-// adds the number of flagged primitives to *flagged.
-template <int K>
-__device__ __forceinline__ bool frame_two_stage(const float4* __restrict__ prims, int n, float bx, float by, float bz,
-                                                float br, const float* __restrict__ stage,
-                                                const float4* __restrict__ sph, int s0, int s1, bool active, int lane,
-                                                uint32_t& flagged) {
-  bool hit = false;
-  for (int base = 0; base < n; base += 32) {
-    const int m = min(32, n - base);
-    uint32_t flags = 0;
-#pragma unroll Prim<K>::kUnroll
-    for (int k = 0; k < m; ++k)
-      flags |= (uint32_t)Prim<K>::hit(prims + Prim<K>::kStride * (base + k), bx, by, bz, br) << k;
-    flags = __reduce_or_sync(kFull, active ? flags : 0u);
-    flagged += (uint32_t)__popc(flags);
-    while (flags) {
-      const int k = __ffs(flags) - 1;
-      flags &= flags - 1;
-      const float4* pk = prims + Prim<K>::kStride * (base + k);
-      for (int s = s0; s < s1; ++s) {
-        const float* st = stage + s * 96 + lane;
-        hit |= Prim<K>::hit(pk, st[0], st[32], st[64], sph[s].w);
-      }
-    }
-  }
-  return hit;
-}
-
 // Packs a verdict (bit 63) and four per-type test counts (15 bits each,
 // saturated; AABB lowest).
 __device__ __forceinline__ unsigned long long pack_tests(bool hit, const uint32_t (&t)[4]) {
@@ -285,29 +254,6 @@ __device__ __forceinline__ unsigned long long pack_tests(bool hit, const uint32_
 #pragma unroll
   for (int k = 0; k < 4; ++k) r |= (unsigned long long)min(t[k], 0x7fffu) << (15 * k);
   return r;
-}
-
-// Both stages of one frame against the whole environment, kept out of line so
-// that the register budget of the caller is not set by it.  Returns the
-// lane's verdict and its second-stage tests per primitive type (pack_tests).
-static __device__ __noinline__ unsigned long long env_two_stage(const float4* __restrict__ env, int n_aabb, int n_obb,
-                                                         int n_cyl, int n_sph, float bx, float by, float bz, float br,
-                                                         const float* __restrict__ stage,
-                                                         const float4* __restrict__ sph, int s0, int s1, bool active,
-                                                         int lane) {
-  uint32_t f[4] = {0, 0, 0, 0};
-  bool hit = false;
-  const float4* e = env;
-  hit |= frame_two_stage<kAabb>(e, n_aabb, bx, by, bz, br, stage, sph, s0, s1, active, lane, f[kAabb]);
-  e += 2 * n_aabb;
-  hit |= frame_two_stage<kObb>(e, n_obb, bx, by, bz, br, stage, sph, s0, s1, active, lane, f[kObb]);
-  e += 5 * n_obb;
-  hit |= frame_two_stage<kCyl>(e, n_cyl, bx, by, bz, br, stage, sph, s0, s1, active, lane, f[kCyl]);
-  e += 2 * n_cyl;
-  hit |= frame_two_stage<kSph>(e, n_sph, bx, by, bz, br, stage, sph, s0, s1, active, lane, f[kSph]);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) f[k] *= (uint32_t)(s1 - s0);
-  return pack_tests(hit, f);
 }
 
 // Three-stage test of one frame for a warp whose lanes hold the states of
@@ -434,16 +380,8 @@ __device__ __forceinline__ float4 warp_enclosing_sphere(float x, float y, float 
 }
 
 // ------------------------------------------------------------------ FK + CC
-// Joint-value sources for state_collides: lane-private values staged in
-// shared memory ([joint][lane]) or a point on a warp-uniform edge a -> b
-// (both held in shared memory) at parameter t, exactly b at the endpoint.
-struct LaneQ {
-  const float* q;  // [kMaxDof][32]
-  int lane;
-  __device__ __forceinline__ float operator()(int i) const { return q[i * 32 + lane]; }
-  __device__ __forceinline__ int poll() const { return 0; }
-};
-
+// Joint values of a point on a warp-uniform edge a -> b (both held in shared
+// memory) at parameter t, exactly b at the endpoint.
 struct EdgeQ {
   const float* a;
   const float* b;
@@ -454,30 +392,96 @@ struct EdgeQ {
   __device__ __forceinline__ int poll() const { return *reinterpret_cast<const volatile int*>(solved); }
 };
 
-// Collision test of one configuration per lane.  `stage` is this warp's
-// [n_spheres + dof][3][32] shared-memory buffer of sphere centres (and, with
-// kWarpVote, link group centres).  Without kWarpVote each lane tests its own
-// state link by link, in chain order, and returns its own verdict.  With
-// kWarpVote the lanes are the states of one edge: the joint loop only places
-// and stages every sphere, then the links are tested against the environment
-// from the distal end back (three stages per link) and the whole warp returns
-// true as soon as any active lane collides (the edge verdict).  The joint loop
-// is a runtime loop so that the obstacle loops exist once in the code.
-template <bool kWarpVote, int kTile = 32, bool kLean = false, class QS>
-__device__ __forceinline__ bool state_collides(const RobotHeader* __restrict__ R, const uint32_t* __restrict__ pair,
-                                               const float* __restrict__ thr, const float4* __restrict__ env,
-                                               int n_aabb, int n_obb, int n_cyl, int n_sph, const EsdfGrid& grid,
-                                               float* __restrict__ stage, const QS& qs, bool active, int lane,
-                                               WarpCount* wc) {
+// A joint frame: rotation columns and origin.
+struct Frame {
+  float ax = 1.f, ay = 0.f, az = 0.f;
+  float bx = 0.f, by = 1.f, bz = 0.f;
+  float cx = 0.f, cy = 0.f, cz = 1.f;
+  float px = 0.f, py = 0.f, pz = 0.f;
+  __device__ __forceinline__ float3 at(const float4& o) const {
+    return make_float3(fmaf(ax, o.x, fmaf(bx, o.y, fmaf(cx, o.z, px))), fmaf(ay, o.x, fmaf(by, o.y, fmaf(cy, o.z, py))),
+                       fmaf(az, o.x, fmaf(bz, o.y, fmaf(cz, o.z, pz))));
+  }
+};
+
+__device__ __forceinline__ bool revolute(int type) { return type == kRevZ || type == kRevY || type == kRevX; }
+
+// Sine and cosine of a joint value: the hardware functions (absolute error
+// about 2^-21 on [-pi, pi]: sphere centres within about 1e-6 m of exact FK),
+// the library routine beyond +-3.2 rad.  kNarrow: no value lies there (the
+// host checks).
+template <bool kNarrow>
+__device__ __forceinline__ void joint_sincos(float q, float& s, float& c) {
+  if (kNarrow || fabsf(q) <= 3.2f)
+    __sincosf(q, &s, &c);
+  else
+    sincosf(q, &s, &c);
+}
+
+// Frame of joint i of type ty from its parent's, at joint value qi (revolute
+// joints: its sine s and cosine c).
+__device__ __forceinline__ void fk_apply(const RobotHeader* __restrict__ R, int i, int ty, float qi, float s, float c,
+                                         Frame& T) {
+  if (R->jparent[i] < 0) {
+    T = Frame{};
+    const float4 b = R->jbase[i];
+    T.px = b.x; T.py = b.y; T.pz = b.z;
+  }
+  if (revolute(ty)) {
+    if (ty == kRevZ) {  // R * Rz: col0' = c col0 + s col1, col1' = -s col0 + c col1
+      const float nx = fmaf(c, T.ax, s * T.bx), ny = fmaf(c, T.ay, s * T.by), nz = fmaf(c, T.az, s * T.bz);
+      T.bx = fmaf(c, T.bx, -s * T.ax); T.by = fmaf(c, T.by, -s * T.ay); T.bz = fmaf(c, T.bz, -s * T.az);
+      T.ax = nx; T.ay = ny; T.az = nz;
+    } else if (ty == kRevY) {  // R * Ry: col0' = c col0 - s col2, col2' = s col0 + c col2
+      const float nx = fmaf(c, T.ax, -s * T.cx), ny = fmaf(c, T.ay, -s * T.cy), nz = fmaf(c, T.az, -s * T.cz);
+      T.cx = fmaf(c, T.cx, s * T.ax); T.cy = fmaf(c, T.cy, s * T.ay); T.cz = fmaf(c, T.cz, s * T.az);
+      T.ax = nx; T.ay = ny; T.az = nz;
+    } else {  // R * Rx: col1' = c col1 + s col2, col2' = -s col1 + c col2
+      const float nx = fmaf(c, T.bx, s * T.cx), ny = fmaf(c, T.by, s * T.cy), nz = fmaf(c, T.bz, s * T.cz);
+      T.cx = fmaf(c, T.cx, -s * T.bx); T.cy = fmaf(c, T.cy, -s * T.by); T.cz = fmaf(c, T.cz, -s * T.bz);
+      T.bx = nx; T.by = ny; T.bz = nz;
+    }
+  } else if (ty == kPrismZ) {
+    T.px = fmaf(qi, T.cx, T.px); T.py = fmaf(qi, T.cy, T.py); T.pz = fmaf(qi, T.cz, T.pz);
+  } else if (ty == kPrismX) {
+    T.px = fmaf(qi, T.ax, T.px); T.py = fmaf(qi, T.ay, T.py); T.pz = fmaf(qi, T.az, T.pz);
+  } else {
+    T.px = fmaf(qi, T.bx, T.px); T.py = fmaf(qi, T.by, T.py); T.pz = fmaf(qi, T.bz, T.pz);
+  }
+  const float L = R->jlen[i];
+  T.px = fmaf(L, T.cx, T.px); T.py = fmaf(L, T.cy, T.py); T.pz = fmaf(L, T.cz, T.pz);
+}
+
+template <bool kNarrow>
+__device__ __forceinline__ void fk_joint(const RobotHeader* __restrict__ R, int i, float qi, Frame& T) {
+  const int ty = R->jtype[i];
+  float s = 0.f, c = 1.f;
+  if (revolute(ty)) joint_sincos<kNarrow>(qi, s, c);
+  fk_apply(R, i, ty, qi, s, c, T);
+}
+
+// Collision test of one edge: the lanes are its states.  `stage` is this
+// warp's [n_spheres + dof][3][32] shared-memory buffer of sphere centres and
+// link group centres.  The joint loop only places and stages every sphere;
+// then the links are tested against the environment from the distal end back
+// (three stages per link) and the whole warp returns true as soon as any
+// active lane collides (the edge verdict).  The joint loop is a runtime loop
+// so that the obstacle loops exist once in the code.
+template <int kTile, bool kLean>
+__device__ __forceinline__ bool edge_collides(const RobotHeader* __restrict__ R, const uint32_t* __restrict__ pair,
+                                              const float* __restrict__ thr, const float4* __restrict__ env,
+                                              int n_aabb, int n_obb, int n_cyl, int n_sph, const EsdfGrid& grid,
+                                              float* __restrict__ stage, const EdgeQ& qs, bool active, int lane,
+                                              WarpCount* wc) {
   static_assert(kTile == 32 || kTile == 64, "obstacle tile is 32 or 64 primitives per type");
   // kLean: an instance for batches without distance fields whose links all have
   // bounding spheres (the host checks); the other paths are not compiled in.
   const bool has_grid = !kLean && grid.v != nullptr;
   const bool has_prims = (n_aabb | n_obb | n_cyl | n_sph) != 0;
   const int dof = R->dof;
-  // edge warps read the problem's solved flag now and look at it after
-  // placing the spheres (the load's latency hides behind the FK)
-  const int solved_early = (kWarpVote && lane == 0) ? qs.poll() : 0;
+  // read the problem's solved flag now and look at it after placing the
+  // spheres (the load's latency hides behind the FK)
+  const int solved_early = lane == 0 ? qs.poll() : 0;
   // uniform work of this call, multiplied by the active lanes on the way out
   const unsigned long long na = (unsigned long long)__popc(__ballot_sync(kFull, active));
   uint32_t passes = 0, pairs = 0;
@@ -491,156 +495,86 @@ __device__ __forceinline__ bool state_collides(const RobotHeader* __restrict__ R
       for (int k = 0; k < 4; ++k) wc->prim[k] += na * fine[k];
     }
   };
-  float ax = 1.f, ay = 0.f, az = 0.f;  // rotation column 0 (local x in world)
-  float bx = 0.f, by = 1.f, bz = 0.f;  // column 1
-  float cx = 0.f, cy = 0.f, cz = 1.f;  // column 2
-  float px = 0.f, py = 0.f, pz = 0.f;
+  Frame T;
   bool hit = false;
 #pragma unroll 1
   for (int i = 0; i < dof; ++i) {
-    if (R->jparent[i] < 0) {
-      ax = 1.f; ay = 0.f; az = 0.f;
-      bx = 0.f; by = 1.f; bz = 0.f;
-      cx = 0.f; cy = 0.f; cz = 1.f;
-      const float4 b = R->jbase[i];
-      px = b.x; py = b.y; pz = b.z;
-    }
-    const int ty = R->jtype[i];
-    const float qi = qs(i);
-    if (ty == kRevZ || ty == kRevY || ty == kRevX) {
-      float s, c;
-      // the hardware sine/cosine (absolute error about 2^-21 on [-pi, pi]: sphere
-      // centres within about 1e-6 m of exact FK); the library routine beyond
-      if (kLean || fabsf(qi) <= 3.2f)  // lean batches keep revolute joints within +-3.2
-        __sincosf(qi, &s, &c);
-      else
-        sincosf(qi, &s, &c);
-      if (ty == kRevZ) {  // R * Rz: col0' = c col0 + s col1, col1' = -s col0 + c col1
-        const float nx = fmaf(c, ax, s * bx), ny = fmaf(c, ay, s * by), nz = fmaf(c, az, s * bz);
-        bx = fmaf(c, bx, -s * ax); by = fmaf(c, by, -s * ay); bz = fmaf(c, bz, -s * az);
-        ax = nx; ay = ny; az = nz;
-      } else if (ty == kRevY) {  // R * Ry: col0' = c col0 - s col2, col2' = s col0 + c col2
-        const float nx = fmaf(c, ax, -s * cx), ny = fmaf(c, ay, -s * cy), nz = fmaf(c, az, -s * cz);
-        cx = fmaf(c, cx, s * ax); cy = fmaf(c, cy, s * ay); cz = fmaf(c, cz, s * az);
-        ax = nx; ay = ny; az = nz;
-      } else {  // R * Rx: col1' = c col1 + s col2, col2' = -s col1 + c col2
-        const float nx = fmaf(c, bx, s * cx), ny = fmaf(c, by, s * cy), nz = fmaf(c, bz, s * cz);
-        cx = fmaf(c, cx, -s * bx); cy = fmaf(c, cy, -s * by); cz = fmaf(c, cz, -s * bz);
-        bx = nx; by = ny; bz = nz;
-      }
-    } else if (ty == kPrismZ) {
-      px = fmaf(qi, cx, px); py = fmaf(qi, cy, py); pz = fmaf(qi, cz, pz);
-    } else if (ty == kPrismX) {
-      px = fmaf(qi, ax, px); py = fmaf(qi, ay, py); pz = fmaf(qi, az, pz);
-    } else {
-      px = fmaf(qi, bx, px); py = fmaf(qi, by, py); pz = fmaf(qi, bz, pz);
-    }
-    const float L = R->jlen[i];
-    px = fmaf(L, cx, px); py = fmaf(L, cy, py); pz = fmaf(L, cz, pz);
-
-    const int s0 = R->sph_begin[i], s1 = R->sph_begin[i + 1];
-    const float4 cb = R->coarse[i];
-    const bool two = R->two_stage && cb.w > 0.f && has_prims;  // uniform
+    fk_joint<kLean>(R, i, qs(i), T);
     const float4 gs = R->grp[i];
-    float gx = 0.f, gy = 0.f, gz = 0.f;
-    if (gs.w > 0.f) {  // group sphere of this link (equals cb when the link has a bounding sphere)
-      gx = fmaf(ax, gs.x, fmaf(bx, gs.y, fmaf(cx, gs.z, px)));
-      gy = fmaf(ay, gs.x, fmaf(by, gs.y, fmaf(cy, gs.z, py)));
-      gz = fmaf(az, gs.x, fmaf(bz, gs.y, fmaf(cz, gs.z, pz)));
-      if (kWarpVote) {  // staged for the self-collision first stage (edge warps only)
-        float* gst = stage + (R->n_spheres + i) * 96 + lane;
-        gst[0] = gx;
-        gst[32] = gy;
-        gst[64] = gz;
-      }
+    if (gs.w > 0.f) {  // group sphere of this link: its bounding sphere, or its only one
+      const float3 g = T.at(gs);
+      float* gst = stage + (R->n_spheres + i) * 96 + lane;
+      gst[0] = g.x;
+      gst[32] = g.y;
+      gst[64] = g.z;
     }
+    const int s0 = R->sph_begin[i], s1 = R->sph_begin[i + 1];
     for (int s = s0; s < s1; ++s) {
-      const float4 o = R->sph[s];
-      const float sx = fmaf(ax, o.x, fmaf(bx, o.y, fmaf(cx, o.z, px)));
-      const float sy = fmaf(ay, o.x, fmaf(by, o.y, fmaf(cy, o.z, py)));
-      const float sz = fmaf(az, o.x, fmaf(bz, o.y, fmaf(cz, o.z, pz)));
+      const float3 c = T.at(R->sph[s]);
       float* st = stage + s * 96 + lane;
-      st[0] = sx;
-      st[32] = sy;
-      st[64] = sz;
-      if (kWarpVote) continue;  // edge warps test the environment in a second pass, distal links first
-      if (has_grid) hit |= esdf_read(grid, sx, sy, sz) < o.w;  // the distance field, sphere by sphere
-      if (!two) {
+      st[0] = c.x;
+      st[32] = c.y;
+      st[64] = c.z;
+    }
+  }
+  // Another warp has solved the problem: the verdict no longer matters, and
+  // the warp leaves with "collides" so that it stops at its next check.
+  if (__shfl_sync(kFull, solved_early, 0)) {
+    if (wc && lane == 0) wc->aborted = 1;
+    flush();
+    return true;
+  }
+  // The lanes are the states of one edge, all placed and staged above.  Test
+  // the links against the environment from the last one back: collisions
+  // come mostly at the distal links, and the first hit ends the check.  The
+  // verdict is the OR of the same tests in any order.
+  for (int i = dof - 1; i >= 0; --i) {
+    const int s0 = R->sph_begin[i], s1 = R->sph_begin[i + 1];
+    if (s0 == s1) continue;
+    const float4 cb = R->coarse[i];
+    const bool two = kLean || (R->two_stage && cb.w > 0.f && has_prims);  // uniform
+    if (two) {
+      if (has_grid) {
+        for (int s = s0; s < s1; ++s) {
+          const float* st = stage + s * 96 + lane;
+          hit |= esdf_read(grid, st[0], st[32], st[64]) < R->sph[s].w;
+        }
+      }
+      // the link's bounding sphere, staged as its group centre
+      const float* gst = stage + (R->n_spheres + i) * 96 + lane;
+      const float gx = gst[0], gy = gst[32], gz = gst[64];
+      const float4 u = warp_enclosing_sphere(gx, gy, gz, cb.w, active);
+      const unsigned long long r = env_three_stage<kTile / 32, !kLean>(env, n_aabb, n_obb, n_cyl, n_sph, u.x, u.y, u.z,
+                                                               u.w, gx, gy, gz, cb.w, stage, R->sph, s0, s1,
+                                                               active, lane);
+      hit |= (r >> 63) != 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) fine[k] += (uint32_t)((r >> (15 * k)) & 0x7fffu);
+    } else {
+      for (int s = s0; s < s1; ++s) {
+        const float4 o = R->sph[s];
+        const float* st = stage + s * 96 + lane;
+        const float sx = st[0], sy = st[32], sz = st[64];
+        if (has_grid) hit |= esdf_read(grid, sx, sy, sz) < o.w;
         hit |= sphere_hits_env(sx, sy, sz, o.w, env, n_aabb, n_obb, n_cyl, n_sph);
         passes++;
       }
     }
-    if (two && !kWarpVote) {
-      passes++;
-      const unsigned long long r =
-          env_two_stage(env, n_aabb, n_obb, n_cyl, n_sph, gx, gy, gz, cb.w, stage, R->sph, s0, s1, active, lane);
-      hit |= (r >> 63) != 0;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) fine[k] += (uint32_t)((r >> (15 * k)) & 0x7fffu);
-    }
-  }
-  if (kWarpVote) {
-    // Another warp has solved the problem: the verdict no longer matters, and
-    // the warp leaves with "collides" so that it stops at its next check.
-    if (__shfl_sync(kFull, solved_early, 0)) {
-      if (wc && lane == 0) wc->aborted = 1;
+    if (__any_sync(kFull, hit && active)) {
       flush();
       return true;
     }
-    // The lanes are the states of one edge, all placed and staged above.  Test
-    // the links against the environment from the last one back: collisions
-    // come mostly at the distal links, and the first hit ends the check.  The
-    // verdict is the OR of the same tests in any order.
-    for (int i = dof - 1; i >= 0; --i) {
-      const int s0 = R->sph_begin[i], s1 = R->sph_begin[i + 1];
-      if (s0 == s1) continue;
-      const float4 cb = R->coarse[i];
-      const bool two = kLean || (R->two_stage && cb.w > 0.f && has_prims);  // uniform
-      if (two) {
-        if (has_grid) {
-          for (int s = s0; s < s1; ++s) {
-            const float* st = stage + s * 96 + lane;
-            hit |= esdf_read(grid, st[0], st[32], st[64]) < R->sph[s].w;
-          }
-        }
-        // the link's bounding sphere, staged as its group centre
-        const float* gst = stage + (R->n_spheres + i) * 96 + lane;
-        const float gx = gst[0], gy = gst[32], gz = gst[64];
-        const float4 u = warp_enclosing_sphere(gx, gy, gz, cb.w, active);
-        const unsigned long long r = env_three_stage<kTile / 32, !kLean>(env, n_aabb, n_obb, n_cyl, n_sph, u.x, u.y, u.z,
-                                                                 u.w, gx, gy, gz, cb.w, stage, R->sph, s0, s1,
-                                                                 active, lane);
-        hit |= (r >> 63) != 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) fine[k] += (uint32_t)((r >> (15 * k)) & 0x7fffu);
-      } else {
-        for (int s = s0; s < s1; ++s) {
-          const float4 o = R->sph[s];
-          const float* st = stage + s * 96 + lane;
-          const float sx = st[0], sy = st[32], sz = st[64];
-          if (has_grid) hit |= esdf_read(grid, sx, sy, sz) < o.w;
-          hit |= sphere_hits_env(sx, sy, sz, o.w, env, n_aabb, n_obb, n_cyl, n_sph);
-          passes++;
-        }
-      }
-      if (__any_sync(kFull, hit && active)) {
-        flush();
-        return true;
-      }
-    }
   }
-  // Self-collision by link-pair blocks: when the lanes are the states of one
-  // edge, a block's fine sphere pairs run only if the group spheres of its two
-  // links overlap for some active lane (the group spheres contain the fine
-  // ones, so the verdict is that of testing every pair).  Lanes holding
-  // unrelated states would nearly always find one overlap, so they test every
-  // pair.  Pairs within a block are sorted by their first sphere.
+  // Self-collision by link-pair blocks: a block's fine sphere pairs run only if
+  // the group spheres of its two links overlap for some active lane (the group
+  // spheres contain the fine ones, so the verdict is that of testing every
+  // pair).  Pairs within a block are sorted by their first sphere.
   const int nb = R->n_blocks;
   const int grp_base = R->n_spheres;  // stage slot of frame 0's group centre
   for (int b = 0; b < nb; ++b) {
     const uint32_t fr = R->blk_frames[b], rg = R->blk_range[b];
     const float bt = R->blk_thr[b];
-    if (kWarpVote && bt < INFINITY) {
+    if (bt < INFINITY) {
       const float* ga = stage + (grp_base + (int)(fr & 0xffffu)) * 96 + lane;
       const float* gb = stage + (grp_base + (int)(fr >> 16)) * 96 + lane;
       const float dx = ga[0] - gb[0], dy = ga[32] - gb[32], dz = ga[64] - gb[64];
@@ -664,16 +598,13 @@ __device__ __forceinline__ bool state_collides(const RobotHeader* __restrict__ R
       const float dx = ix - sj[0], dy = iy - sj[32], dz = iz - sj[64];
       hit |= fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < thr[k];
     }
-    if (kWarpVote) {
-      if (__any_sync(kFull, hit && active)) {
-        flush();
-        return true;
-      }
+    if (__any_sync(kFull, hit && active)) {
+      flush();
+      return true;
     }
   }
   flush();
-  if (kWarpVote) return __any_sync(kFull, hit && active);
-  return hit;
+  return __any_sync(kFull, hit && active);
 }
 
 // Byte size of a warp's staging buffer of sphere centres: the robot's
@@ -690,7 +621,7 @@ __host__ __device__ inline int robot_smem_bytes(int n_pairs) {
 // every lane runs the same FK, lane l places spheres l, l + 32, ... , tests
 // them against every primitive (or the distance field) and stages their
 // centres (3 floats each at stage[3 s]); after a warp barrier lane l tests
-// self pairs l, l + 32, ....  Each test is the arithmetic of state_collides's
+// self pairs l, l + 32, ....  Each test is the arithmetic of the edge check's
 // one-stage path, which the bounding-sphere stages reproduce exactly, so the
 // verdict is the same.  Returns the warp-wide verdict.
 static __device__ __noinline__ bool config_collides_warp(const RobotHeader* __restrict__ R, const uint32_t* __restrict__ pair,

@@ -178,7 +178,7 @@ __device__ __forceinline__ bool edge_free(const Ctx& c, int N) {
     const bool active = k <= N;
     const int kk = active ? k : N;
     const EdgeQ qs{c.v.a, c.v.b, __fdiv_rn((float)kk, fN), kk == N, &c.S->solved};
-    if (state_collides<true, kTile, kLean>(c.R, c.pair, c.thr, c.env, c.D->env.n_aabb, c.D->env.n_obb, c.D->env.n_cyl,
+    if (edge_collides<kTile, kLean>(c.R, c.pair, c.thr, c.env, c.D->env.n_aabb, c.D->env.n_obb, c.D->env.n_cyl,
                                     c.D->env.n_sph, c.D->env.esdf, c.stage, qs, active, c.lane, c.cnt)) {
       __syncwarp();  // lane 0 may have just set the flag
       if (c.cnt->aborted) {
