@@ -259,42 +259,44 @@ __device__ __forceinline__ unsigned long long pack_tests(bool hit, const uint32_
 // Three-stage test of one frame for a warp whose lanes hold the states of
 // one edge (the planner).  Stage A: one sphere (ux, uy, uz, ur) around every
 // active lane's bounding sphere against the primitives, one primitive per
-// lane.  Stage B: each lane's bounding sphere (bx, by, bz, br) against the
-// primitives stage A touched.  Stage C: the fine spheres against the
-// primitives some lane's bounding sphere touched.  Each sphere contains the
-// next with a margin, so the verdict equals the one-stage test.  The
-// lane-level tests of the three stages are added to *tests.
+// lane.  Stage B: each lane's bounding sphere (bx, by, bz, br) against a
+// primitive stage A touched.  Stage C: the fine spheres against it when some
+// lane's bounding sphere touched it.  Each sphere contains the next with a
+// margin, so the verdict equals the one-stage test.  A collision of any active
+// lane is the edge's verdict and ends the test: most edges collide, as a rule
+// at their last link, and the primitives after the first hit were two thirds
+// of this function's time.  The lane-level tests of the three stages are added
+// to *tests.
 //
 // Stages B and C of one primitive type for one batch of 32 primitives whose
-// stage-A candidates are `cand`.
+// stage-A candidates are `cand`.  Warp-uniform result.
 template <int K>
 __device__ __forceinline__ bool frame_stages_bc(const float4* __restrict__ prims, int base, uint32_t cand, float bx,
                                                 float by, float bz, float br, const float* __restrict__ stage,
                                                 const float4* __restrict__ sph, int s0, int s1, bool active, int lane,
                                                 uint32_t& tests) {
-  bool hit = false;
-  tests += 1u + (uint32_t)__popc(cand);
-  uint32_t flags = 0;
+  tests += 1u;
   while (cand) {
     const int b = __ffs(cand) - 1;
     cand &= cand - 1;
-    flags |= (uint32_t)Prim<K>::hit(prims + Prim<K>::kStride * (base + b), bx, by, bz, br) << b;
-  }
-  flags = __reduce_or_sync(kFull, active ? flags : 0u);
-  tests += (uint32_t)(s1 - s0) * (uint32_t)__popc(flags);
-  while (flags) {
-    const int b = __ffs(flags) - 1;
-    flags &= flags - 1;
-    const float4* pk = prims + Prim<K>::kStride * (base + b);
+    float4 e[Prim<K>::kStride];
+#pragma unroll
+    for (int k = 0; k < Prim<K>::kStride; ++k) e[k] = prims[Prim<K>::kStride * (base + b) + k];
+    tests += 1u;
+    if (!__any_sync(kFull, active && Prim<K>::hit(e, bx, by, bz, br))) continue;
+    tests += (uint32_t)(s1 - s0);
+    bool hit = false;
     for (int s = s0; s < s1; ++s) {
       const float* st = stage + s * 96 + lane;
-      hit |= Prim<K>::hit(pk, st[0], st[32], st[64], sph[s].w);
+      hit |= Prim<K>::hit(e, st[0], st[32], st[64], sph[s].w);
     }
+    if (__any_sync(kFull, hit && active)) return true;
   }
-  return hit;
+  return false;
 }
 
-// The three stages of one frame (warp = one edge), out of line; same return.
+// The three stages of one frame (warp = one edge), out of line.  Returns the
+// edge's verdict and the tests per primitive type (pack_tests).
 // Stage A of all four primitive types runs first, kHalves x 32 primitives of
 // each type per round (one or two per lane), so that a lane's tests of a round
 // are independent; stages B and C then take the round's candidates in order.
@@ -310,7 +312,6 @@ static __device__ __noinline__ unsigned long long env_three_stage(const float4* 
                                                            bool active, int lane) {
   if (!kObb) n_obb = 0;
   uint32_t t[4] = {0, 0, 0, 0};
-  bool hit = false;
   const float4* ea = env;
   const float4* eo = ea + 2 * n_aabb;
   const float4* ec = eo + 5 * n_obb;
@@ -333,24 +334,28 @@ static __device__ __noinline__ unsigned long long env_three_stage(const float4* 
       const uint32_t cc = __ballot_sync(kFull, nc[h]), cs = __ballot_sync(kFull, ns[h]);
       // a type without stage-A candidates (warp-uniform) needs no stages B and C
       if (b0 < n_aabb) {
-        if (ca) hit |= frame_stages_bc<kAabb>(ea, b0, ca, bx, by, bz, br, stage, sph, s0, s1, active, lane, t[kAabb]);
-        else t[kAabb] += 1u;
+        if (!ca) t[kAabb] += 1u;
+        else if (frame_stages_bc<kAabb>(ea, b0, ca, bx, by, bz, br, stage, sph, s0, s1, active, lane, t[kAabb]))
+          return pack_tests(true, t);
       }
       if (b0 < n_obb) {
-        if (co) hit |= frame_stages_bc<kObb>(eo, b0, co, bx, by, bz, br, stage, sph, s0, s1, active, lane, t[kObb]);
-        else t[kObb] += 1u;
+        if (!co) t[kObb] += 1u;
+        else if (frame_stages_bc<kObb>(eo, b0, co, bx, by, bz, br, stage, sph, s0, s1, active, lane, t[kObb]))
+          return pack_tests(true, t);
       }
       if (b0 < n_cyl) {
-        if (cc) hit |= frame_stages_bc<kCyl>(ec, b0, cc, bx, by, bz, br, stage, sph, s0, s1, active, lane, t[kCyl]);
-        else t[kCyl] += 1u;
+        if (!cc) t[kCyl] += 1u;
+        else if (frame_stages_bc<kCyl>(ec, b0, cc, bx, by, bz, br, stage, sph, s0, s1, active, lane, t[kCyl]))
+          return pack_tests(true, t);
       }
       if (b0 < n_sph) {
-        if (cs) hit |= frame_stages_bc<kSph>(es, b0, cs, bx, by, bz, br, stage, sph, s0, s1, active, lane, t[kSph]);
-        else t[kSph] += 1u;
+        if (!cs) t[kSph] += 1u;
+        else if (frame_stages_bc<kSph>(es, b0, cs, bx, by, bz, br, stage, sph, s0, s1, active, lane, t[kSph]))
+          return pack_tests(true, t);
       }
     }
   }
-  return pack_tests(hit, t);
+  return pack_tests(false, t);
 }
 
 // Order-preserving map of binary32 to uint32 (and back): larger floats give
