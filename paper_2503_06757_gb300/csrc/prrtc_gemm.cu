@@ -581,6 +581,8 @@ __global__ void __launch_bounds__(kClusterThreads, 2)
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
+  let_next_start();
+  wait_before();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1224,18 +1226,10 @@ int launch_cluster_as(const CUtensorMap& ma, const CUtensorMap& mb, const Cluste
       return PRRTC_ERR_CUDA;
     attr = true;
   }
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = kSplits;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cudaLaunchConfig_t lc{};
-  lc.gridDim = dim3(ep.m_tiles * ((ep.N + kBN - 1) / kBN) * kSplits);
-  lc.blockDim = dim3(kClusterThreads);
-  lc.dynamicSmemBytes = T::kSmem;
-  lc.stream = stream;
-  lc.attrs = &at;
-  lc.numAttrs = 1;
-  return cudaLaunchKernelEx(&lc, fn, ma, mb, ep) == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
+  const int grid = ep.m_tiles * ((ep.N + kBN - 1) / kBN) * kSplits;
+  return launch_overlapped(fn, grid, kClusterThreads, T::kSmem, stream, kSplits, ma, mb, ep) == cudaSuccess
+             ? PRRTC_OK
+             : PRRTC_ERR_CUDA;
 }
 
 template <int kBN, int kSplits>

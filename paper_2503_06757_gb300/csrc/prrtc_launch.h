@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <utility>
 
 #include "prrtc.h"
 #include "prrtc_device.cuh"
@@ -264,6 +265,34 @@ cudaError_t launch_voxelize(const EnvView& env, const float origin[3], float vox
                             cudaStream_t stream);
 cudaError_t launch_esdf(const uint8_t* occ, const int dims[3], float voxel, void* tmp, float* out,
                         cudaStream_t stream);
+
+// Launches of a chain of short kernels overlap: a kernel launched with
+// launch_overlapped may start while the kernel before it in the stream still
+// runs; it must call wait_before() ahead of its first access to global memory
+// and may call let_next_start() once its own start-up is over.
+#ifdef __CUDACC__
+__device__ __forceinline__ void wait_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_overlapped(void (*fn)(P...), int grid, int block, size_t smem, cudaStream_t stream, int cluster,
+                              A&&... args) {
+  cudaLaunchAttribute at[2]{};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3((unsigned)grid);
+  lc.blockDim = dim3((unsigned)block);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = stream;
+  lc.attrs = at;
+  lc.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&lc, fn, std::forward<A>(args)...);
+}
+#endif
 
 // Tensor-core GEMM (prrtc_gemm.cu): C[M,N] = A[M,K] B[N,K]^T (+bias, ReLU).
 int gemm_bf16(const void* a, const void* b, int M, int N, int K, const float* bias, int relu, float* c32, int ldc32,

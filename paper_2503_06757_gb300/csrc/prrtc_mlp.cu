@@ -122,6 +122,8 @@ __global__ void features_kernel(const uint8_t* __restrict__ occ, const int* __re
                                 const float* __restrict__ span, int B, int dof, bf16* __restrict__ x) {
   const int b = blockIdx.x;
   bf16* dst = x + (size_t)b * kIn;
+  let_next_start();
+  wait_before();
   const int r = b < B ? (rows ? rows[b] : b) : 0;
   // 16 voxels a thread: 16 bytes in, 32 bytes out (256 threads, one turn)
   {
@@ -212,15 +214,25 @@ __global__ void occ_bf16_kernel(const uint8_t* __restrict__ occ, bf16* __restric
 
 // Mixture negative log-likelihood of each sample's target and its gradient
 // with respect to the head output (scaled by 1/B).  One warp per sample;
-// lane k < 8 owns component k.
+// lane k < 8 owns component k.  Rows B .. n_rows - 1 get zero gradients; the
+// columns behind the head are never written and stay zero.
 __global__ void mixture_loss_kernel(const float* __restrict__ out, int P, const float* __restrict__ target,
                                     const int* __restrict__ rows, const float* __restrict__ lo,
-                                    const float* __restrict__ span, int B, int dof, float invB,
+                                    const float* __restrict__ span, int B, int n_rows, int dof, float invB,
                                     float* __restrict__ dout32, bf16* __restrict__ dout16,
                                     float* __restrict__ loss_sum) {
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (warp >= B) return;
+  let_next_start();
+  wait_before();
+  if (warp >= B) {  // padding rows
+    if (warp < n_rows)
+      for (int c = lane; c < P; c += 32) {
+        dout32[(size_t)warp * P + c] = 0.f;
+        dout16[(size_t)warp * P + c] = __float2bfloat16_rn(0.f);
+      }
+    return;
+  }
   const int r = rows ? rows[warp] : warp;
   const float* o = out + (size_t)warp * P;
   const bool comp = lane < kK;
@@ -299,6 +311,8 @@ __global__ void __launch_bounds__(256) colsum_kernel(const ColSums a) {
   __shared__ __align__(16) float chunk[2][kColChunk][32];
   int l = 0;
   while (l < 3 && (int)blockIdx.x >= a.first_block[l + 1]) ++l;
+  let_next_start();
+  wait_before();
   const int cols = a.cols[l], c0 = ((int)blockIdx.x - a.first_block[l]) * 32;
   const float* g = a.g[l] + c0;
   const int chunks = (a.rows + kColChunk - 1) / kColChunk;
@@ -369,6 +383,8 @@ __global__ void __launch_bounds__(256) adam_kernel(float4* __restrict__ p, const
                                                    uint2* __restrict__ p16, size_t n4, float lr, float b1, float b2,
                                                    float eps, float c1, float c2) {
   const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  let_next_start();
+  wait_before();
   if (i >= n4) return;
   float4 pi = p[i], mi = m[i], vi = v[i];
   const float4 gi = g[i];
@@ -529,6 +545,8 @@ int ensure_scratch(prrtc_proposal* p, int rows) {
     free_scratch(p);
     return mlp_fail(PRRTC_ERR_OOM, "scratch allocation failed");
   }
+  MCK(cudaMemsetAsync(p->d32, 0, (size_t)rows * P * 4, p->stream));
+  MCK(cudaMemsetAsync(p->d16, 0, (size_t)rows * P * 2, p->stream));
   p->cap = rows;
   return PRRTC_OK;
 }
@@ -612,8 +630,7 @@ int backward_rows(prrtc_proposal* p, int rows) {
     cs.first_block[l] = blocks;
     blocks += cs.cols[l] / 32;
   }
-  colsum_kernel<<<blocks, 256, 0, s>>>(cs);
-  return cudaGetLastError() == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
+  return launch_overlapped(colsum_kernel, blocks, 256, 0, s, 1, cs) == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
 }
 
 int upload_samples(prrtc_proposal* p, const uint8_t* occ, int n_occ, const float* qs, const float* qg,
@@ -978,8 +995,8 @@ int prrtc_proposal_forward(prrtc_proposal* p, const uint8_t* occ, const float* q
   int rc;
   if ((rc = ensure_scratch(p, rows))) return rc;
   if ((rc = upload_samples(p, occ, B, q_start, q_goal, nullptr, B))) return rc;
-  features_kernel<<<rows, kVox / 16, 0, p->stream>>>(p->occ, nullptr, nullptr, p->qs, p->qg, p->d_lims, p->d_lims + kMaxDof,
-                                               B, p->dof, p->x16);
+  MCK(launch_overlapped(features_kernel, rows, kVox / 16, 0, p->stream, 1, p->occ, nullptr, nullptr, p->qs, p->qg, p->d_lims,
+                        p->d_lims + kMaxDof, B, p->dof, p->x16));
   if ((rc = forward_rows(p, rows))) return rc;
   MCK(cudaMemcpyAsync(out, p->out32, (size_t)B * p->P * 4, cudaMemcpyDeviceToHost, p->stream));
   MCK(cudaStreamSynchronize(p->stream));
@@ -1012,8 +1029,8 @@ int prrtc_proposal_forward_layers(prrtc_proposal* p, const uint8_t* occ, const f
   int rc;
   if ((rc = ensure_scratch(p, rows))) return rc;
   if ((rc = upload_samples(p, occ, B, q_start, q_goal, nullptr, B))) return rc;
-  features_kernel<<<rows, kVox / 16, 0, p->stream>>>(p->occ, nullptr, nullptr, p->qs, p->qg, p->d_lims, p->d_lims + kMaxDof,
-                                               B, p->dof, p->x16);
+  MCK(launch_overlapped(features_kernel, rows, kVox / 16, 0, p->stream, 1, p->occ, nullptr, nullptr, p->qs, p->qg, p->d_lims,
+                        p->d_lims + kMaxDof, B, p->dof, p->x16));
   if ((rc = forward_rows(p, rows))) return rc;
   if ((rc = check_gemm_error())) return rc;
   if ((rc = bf16_rows_to_host(p->x16, B, kIn, kIn, x, p->stream))) return rc;
@@ -1063,24 +1080,21 @@ static int step_on_rows(prrtc_proposal* p, const int* scene_of, const int* rows_
   const int rows = (B + 7) & ~7;
   int rc;
   const cudaStream_t s = p->stream;
-  features_kernel<<<rows, kVox / 16, 0, s>>>(p->occ, scene_of, rows_dev, p->qs, p->qg, p->d_lims, p->d_lims + kMaxDof, B,
-                                       p->dof, p->x16);
+  MCK(launch_overlapped(features_kernel, rows, kVox / 16, 0, p->stream, 1, p->occ, scene_of, rows_dev, p->qs, p->qg, p->d_lims,
+                        p->d_lims + kMaxDof, B, p->dof, p->x16));
   if ((rc = forward_rows(p, rows))) return rc;
-  MCK(cudaMemsetAsync(p->d32, 0, (size_t)rows * p->P * 4, s));
-  MCK(cudaMemsetAsync(p->d16, 0, (size_t)rows * p->P * 2, s));
-  mixture_loss_kernel<<<(B * 32 + 255) / 256, 256, 0, s>>>(p->out32, p->P, p->tgt, rows_dev, p->d_lims,
-                                                            p->d_lims + kMaxDof, B, p->dof, 1.f / (float)B, p->d32,
-                                                            p->d16, loss_dev);
+  MCK(launch_overlapped(mixture_loss_kernel, (rows * 32 + 255) / 256, 256, 0, s, 1, p->out32, p->P, p->tgt, rows_dev,
+                        p->d_lims, p->d_lims + kMaxDof, B, rows, p->dof, 1.f / (float)B, p->d32, p->d16, loss_dev));
   if ((rc = backward_rows(p, rows))) return rc;
   if (lr > 0.f) {
     p->step++;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f / (1.f - std::pow(b1, (float)p->step)), c2 = 1.f / (1.f - std::pow(b2, (float)p->step));
     const size_t n4 = p->n_params / 4;
-    adam_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, s>>>(
-        reinterpret_cast<float4*>(p->master), reinterpret_cast<const float4*>(p->grad),
-        reinterpret_cast<float4*>(p->m), reinterpret_cast<float4*>(p->v), reinterpret_cast<uint2*>(p->params16), n4,
-        lr, b1, b2, 1e-8f, c1, c2);
+    MCK(launch_overlapped(adam_kernel, (int)((n4 + 255) / 256), 256, 0, s, 1, reinterpret_cast<float4*>(p->master),
+                          reinterpret_cast<const float4*>(p->grad), reinterpret_cast<float4*>(p->m),
+                          reinterpret_cast<float4*>(p->v), reinterpret_cast<uint2*>(p->params16), n4, lr, b1, b2,
+                          1e-8f, c1, c2));
   }
   return cudaGetLastError() == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
 }
