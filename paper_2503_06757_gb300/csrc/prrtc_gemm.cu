@@ -536,6 +536,16 @@ struct ClusterEpilogue {
   int ldc16;
 };
 
+// Up to four products of one launch (a layer's weight gradients, which wait
+// for nothing but their operands): product g has the blocks from first[g] on.
+constexpr int kMaxGroup = 4;
+struct ClusterGroup {
+  CUtensorMap a[kMaxGroup], b[kMaxGroup];
+  ClusterEpilogue ep[kMaxGroup];
+  int first[kMaxGroup];
+  int n;
+};
+
 // Byte offset of 16-byte unit u of row i of a partial tile (rows of kBN
 // floats): units of a 128-byte group are exchanged by the row, so that both
 // the row-per-lane writes and the unit-per-thread reads touch every bank once.
@@ -546,9 +556,14 @@ __device__ __forceinline__ uint32_t part_off(int i, int u) {
 
 template <int kBN, int kSplits, bool kTA, bool kTB>
 __global__ void __launch_bounds__(kClusterThreads, 2)
-    gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                        const ClusterEpilogue ep) {
+    gemm_cluster_kernel(const __grid_constant__ ClusterGroup group) {
   using T = ClusterTile<kBN>;
+  int which = 0;
+  while (which + 1 < group.n && (int)blockIdx.x >= group.first[which + 1]) ++which;
+  const ClusterEpilogue& ep = group.ep[which];
+  const CUtensorMap& tmA = group.a[which];
+  const CUtensorMap& tmB = group.b[which];
+  const int block = (int)blockIdx.x - group.first[which];
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -557,7 +572,7 @@ __global__ void __launch_bounds__(kClusterThreads, 2)
   uint64_t* acc_full = empty + T::kStages;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int split = (int)blockIdx.x % kSplits, tile = (int)blockIdx.x / kSplits;
+  const int split = block % kSplits, tile = block / kSplits;
   const int m0 = tile % ep.m_tiles * BM, n0 = tile / ep.m_tiles * kBN;
   const int base = ep.k_tiles / kSplits, rem = ep.k_tiles % kSplits;
   const int kt0 = split * base + min(split, rem), kts = base + (split < rem ? 1 : 0);
@@ -1208,16 +1223,8 @@ float* workspace(size_t floats, cudaStream_t stream) {
 
 namespace {
 
-// Tile width of the cluster kernel for a product, 0: not its size.  One wave:
-// two blocks per SM.
-int cluster_bn(int m_tiles, int N, int splits, int sms) {
-  for (int bn : {64, 128})
-    if (m_tiles * ((N + bn - 1) / bn) * splits <= 2 * sms) return bn;
-  return 0;
-}
-
 template <int kBN, int kSplits, bool kTA, bool kTB>
-int launch_cluster_as(const CUtensorMap& ma, const CUtensorMap& mb, const ClusterEpilogue& ep, cudaStream_t stream) {
+int launch_cluster_as(const ClusterGroup& group, int grid, cudaStream_t stream) {
   using T = ClusterTile<kBN>;
   auto* fn = gemm_cluster_kernel<kBN, kSplits, kTA, kTB>;
   static bool attr = false;
@@ -1226,30 +1233,82 @@ int launch_cluster_as(const CUtensorMap& ma, const CUtensorMap& mb, const Cluste
       return PRRTC_ERR_CUDA;
     attr = true;
   }
-  const int grid = ep.m_tiles * ((ep.N + kBN - 1) / kBN) * kSplits;
-  return launch_overlapped(fn, grid, kClusterThreads, T::kSmem, stream, kSplits, ma, mb, ep) == cudaSuccess
+  return launch_overlapped(fn, grid, kClusterThreads, T::kSmem, stream, kSplits, group) == cudaSuccess
              ? PRRTC_OK
              : PRRTC_ERR_CUDA;
 }
 
 template <int kBN, int kSplits>
-int launch_cluster_split(bool ta, bool tb, const CUtensorMap& ma, const CUtensorMap& mb, const ClusterEpilogue& ep,
-                         cudaStream_t stream) {
-  if (ta) return tb ? launch_cluster_as<kBN, kSplits, true, true>(ma, mb, ep, stream) : PRRTC_ERR_UNSUPPORTED;
-  return tb ? launch_cluster_as<kBN, kSplits, false, true>(ma, mb, ep, stream)
-            : launch_cluster_as<kBN, kSplits, false, false>(ma, mb, ep, stream);
+int launch_cluster_split(bool ta, bool tb, const ClusterGroup& group, int grid, cudaStream_t stream) {
+  if (ta) return tb ? launch_cluster_as<kBN, kSplits, true, true>(group, grid, stream) : PRRTC_ERR_UNSUPPORTED;
+  return tb ? launch_cluster_as<kBN, kSplits, false, true>(group, grid, stream)
+            : launch_cluster_as<kBN, kSplits, false, false>(group, grid, stream);
 }
 
 template <int kBN>
-int launch_cluster(int splits, bool ta, bool tb, const CUtensorMap& ma, const CUtensorMap& mb,
-                   const ClusterEpilogue& ep, cudaStream_t stream) {
+int launch_cluster_bn(int splits, bool ta, bool tb, const ClusterGroup& group, int grid, cudaStream_t stream) {
   switch (splits) {
-    case 1: return launch_cluster_split<kBN, 1>(ta, tb, ma, mb, ep, stream);
-    case 2: return launch_cluster_split<kBN, 2>(ta, tb, ma, mb, ep, stream);
-    case 4: return launch_cluster_split<kBN, 4>(ta, tb, ma, mb, ep, stream);
-    case 8: return launch_cluster_split<kBN, 8>(ta, tb, ma, mb, ep, stream);
+    case 1: return launch_cluster_split<kBN, 1>(ta, tb, group, grid, stream);
+    case 2: return launch_cluster_split<kBN, 2>(ta, tb, group, grid, stream);
+    case 4: return launch_cluster_split<kBN, 4>(ta, tb, group, grid, stream);
+    case 8: return launch_cluster_split<kBN, 8>(ta, tb, group, grid, stream);
     default: return PRRTC_ERR_UNSUPPORTED;
   }
+}
+
+int launch_cluster(int bn, int splits, bool ta, bool tb, const ClusterGroup& group, int grid, cudaStream_t stream) {
+  return bn == 64 ? launch_cluster_bn<64>(splits, ta, tb, group, grid, stream)
+                  : launch_cluster_bn<128>(splits, ta, tb, group, grid, stream);
+}
+
+int sm_count() {
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n > 0 ? n : 1;
+  }();
+  return sms;
+}
+
+// The library's split of K: doubled while the 128 x 256 tiles fill less than
+// one wave and every range keeps kMinKTilesPerSplit K tiles.
+int auto_splits(int M, int N, int K) {
+  const int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN), k_tiles = (K + BK - 1) / BK;
+  int splits = 1;
+  while (splits < kMaxSplits && tiles * (splits * 2) <= sm_count() && k_tiles / (splits * 2) >= kMinKTilesPerSplit)
+    splits *= 2;
+  return std::min(splits, k_tiles);
+}
+
+int cluster_blocks(int M, int N, int splits, int bn) {
+  return ((M + BM - 1) / BM) * ((N + bn - 1) / bn) * splits;
+}
+
+// Tile width of the cluster kernel for a product, 0: not its size.  One wave:
+// two blocks per SM.
+int cluster_bn(int M, int N, int splits) {
+  if (splits > kMaxClusterSplits || (splits & (splits - 1))) return 0;
+  for (int bn : {64, 128})
+    if (cluster_blocks(M, N, splits, bn) <= 2 * sm_count()) return bn;
+  return 0;
+}
+
+// Adds one product to a group of clusters with tiles of bn columns.
+int group_add(ClusterGroup& g, int& grid, int bn, int splits, const void* a, int lda, bool ta, const void* b, int ldb,
+              bool tb, int M, int N, int K, const float* bias, int relu, const void* mask, int ldm, float* c32,
+              int ldc32, void* c16, int ldc16) {
+  const int k = g.n;
+  if (!(ta ? cached_map(&g.a[k], a, K, M, lda, 0, BK) : cached_map(&g.a[k], a, M, K, lda, 0, BM)) ||
+      !(tb ? cached_map(&g.b[k], b, K, N, ldb, 0, BK) : cached_map(&g.b[k], b, N, K, ldb, 0, bn)))
+    return PRRTC_ERR_CUDA;
+  g.ep[k] = ClusterEpilogue{M, N, (K + BK - 1) / BK, (M + BM - 1) / BM, bias, relu,
+                            static_cast<const __nv_bfloat16*>(mask), ldm, c32, ldc32,
+                            static_cast<__nv_bfloat16*>(c16), ldc16};
+  g.first[k] = grid;
+  g.n = k + 1;
+  grid += cluster_blocks(M, N, splits, bn);
+  return PRRTC_OK;
 }
 
 template <bool kTA, bool kTB>
@@ -1280,37 +1339,26 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
   if ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) return PRRTC_ERR_INVALID_ARG;
   if ((c32 && (reinterpret_cast<uintptr_t>(c32) & 15)) || (c16 && (reinterpret_cast<uintptr_t>(c16) & 15)))
     return PRRTC_ERR_INVALID_ARG;
-  CUtensorMap ma, mb;
-  if (!(ta ? cached_map(&ma, a, K, M, lda, 0, BK) : cached_map(&ma, a, M, K, lda, 0, BM))) return PRRTC_ERR_CUDA;
-  static const int sms = [] {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    return n > 0 ? n : 1;
-  }();
   Epilogue ep{M, N, K, bias, relu, c32 ? 1 : 0, c16 ? 1 : 0, 1, 0, 0, 0, 0};
   ep.m_tiles = (M + BM - 1) / BM;
   ep.n_tiles = (N + BN - 1) / BN;
   ep.k_tiles = (K + BK - 1) / BK;
   ep.m_pad = ep.m_tiles * BM;
   const int tiles = ep.m_tiles * ep.n_tiles;
-  int splits = splits_hint;
-  if (splits <= 0) {
-    splits = 1;
-    while (splits < kMaxSplits && tiles * (splits * 2) <= sms && ep.k_tiles / (splits * 2) >= kMinKTilesPerSplit)
-      splits *= 2;
-  }
+  const int sms = sm_count();
+  int splits = splits_hint > 0 ? splits_hint : auto_splits(M, N, K);
   splits = std::max(1, std::min(splits, std::min(kMaxSplits, ep.k_tiles)));
-  if (splits <= kMaxClusterSplits && (splits & (splits - 1)) == 0) {
-    const int bn = cluster_bn(ep.m_tiles, N, splits, sms);
-    if (bn) {
-      ClusterEpilogue ce{M, N, ep.k_tiles, ep.m_tiles, bias, relu, static_cast<const __nv_bfloat16*>(mask),
-                         ldm, c32, ldc32, static_cast<__nv_bfloat16*>(c16), ldc16};
-      if (!(tb ? cached_map(&mb, b, K, N, ldb, 0, BK) : cached_map(&mb, b, N, K, ldb, 0, bn))) return PRRTC_ERR_CUDA;
-      return bn == 64 ? launch_cluster<64>(splits, ta, tb, ma, mb, ce, stream) : launch_cluster<128>(splits, ta, tb, ma, mb, ce, stream);
-    }
+  if (const int bn = cluster_bn(M, N, splits)) {
+    ClusterGroup g;
+    g.n = 0;
+    int grid = 0;
+    const int rc = group_add(g, grid, bn, splits, a, lda, ta, b, ldb, tb, M, N, K, bias, relu, mask, ldm, c32, ldc32,
+                             c16, ldc16);
+    return rc ? rc : launch_cluster(bn, splits, ta, tb, g, grid, stream);
   }
   if (mask) return PRRTC_ERR_UNSUPPORTED;
+  CUtensorMap ma, mb;
+  if (!(ta ? cached_map(&ma, a, K, M, lda, 0, BK) : cached_map(&ma, a, M, K, lda, 0, BM))) return PRRTC_ERR_CUDA;
   if (!(tb ? cached_map(&mb, b, K, N, ldb, 0, BK) : cached_map(&mb, b, N, K, ldb, 0, BN))) return PRRTC_ERR_CUDA;
   OutMaps om;
   std::memset(&om, 0, sizeof(om));
@@ -1337,6 +1385,38 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
     if (cudaGetLastError() != cudaSuccess) return PRRTC_ERR_CUDA;
   }
   return PRRTC_OK;
+}
+
+int gemm_gradients(const GradientProduct* p, int n, cudaStream_t stream) {
+  // products of one shape of cluster share a launch while it stays one wave
+  ClusterGroup g;
+  g.n = 0;
+  int grid = 0, bn = 0, splits = 0;
+  auto flush = [&]() {
+    const int rc = g.n ? launch_cluster(bn, splits, true, true, g, grid, stream) : PRRTC_OK;
+    g.n = 0;
+    grid = 0;
+    return rc;
+  };
+  int rc = PRRTC_OK;
+  for (int i = 0; i < n && !rc; ++i) {
+    const GradientProduct& q = p[i];
+    const int s = auto_splits(q.out, q.in, q.rows), w = cluster_bn(q.out, q.in, s);
+    if (!w) {
+      rc = gemm_bf16_ld(q.dz, q.out, q.h, q.in, q.out, q.in, q.rows, nullptr, 0, q.dw, q.in, nullptr, 0, stream, 0,
+                        kTransA | kTransB, nullptr, 0);
+      continue;
+    }
+    if (g.n && (g.n == kMaxGroup || w != bn || s != splits ||
+                grid + cluster_blocks(q.out, q.in, s, w) > 2 * sm_count()))
+      rc = flush();
+    bn = w;
+    splits = s;
+    if (!rc)
+      rc = group_add(g, grid, bn, splits, q.dz, q.out, true, q.h, q.in, true, q.out, q.in, q.rows, nullptr, 0, nullptr,
+                     0, q.dw, q.in, nullptr, 0);
+  }
+  return rc ? rc : flush();
 }
 
 int gemm_bf16_split(const void* a, const void* b, int M, int N, int K, const float* bias, int relu, float* c32,

@@ -308,6 +308,16 @@ constexpr int kTransA = 1, kTransB = 2;
 int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, int K, const float* bias, int relu,
                  float* c32, int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint, int trans,
                  const void* mask, int ldm);
+// Weight gradients of n layers, dW [out x in] = dZ [rows x out]^T H [rows x
+// in], in as few launches as their sizes allow (all dimensions multiples of 8,
+// all pointers 16-byte aligned).
+struct GradientProduct {
+  const void* dz;
+  const void* h;
+  float* dw;
+  int out, in, rows;
+};
+int gemm_gradients(const GradientProduct* p, int n, cudaStream_t stream);
 int gemm_take_error();
 // Copies the kernels' error word to *out on `stream` (does not clear it).
 cudaError_t gemm_read_error(int* out, cudaStream_t stream);

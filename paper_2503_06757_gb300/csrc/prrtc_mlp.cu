@@ -600,12 +600,10 @@ int backward_rows(prrtc_proposal* p, int rows) {
   const float* dz32 = p->d32;
   ColSums cs{};
   cs.rows = rows;
+  GradientProduct dw[4];
   for (int l = 3; l >= 0; --l) {
     const int in = p->in_dim[l], out = p->out_dim[l];
-    // dW_l [out x in] = dZ^T H, both as stored: [rows x out], [rows x in]
-    if ((rc = gemm_bf16_ld(dz16, out, hprev[l], in, out, in, rows, nullptr, 0, p->grad + p->w_off[l], in, nullptr, 0,
-                           s, 0, kTransA | kTransB, nullptr, 0)))
-      return rc;
+    dw[3 - l] = GradientProduct{dz16, hprev[l], p->grad + p->w_off[l], out, in, rows};
     cs.g[l] = dz32;
     cs.out[l] = p->grad + p->b_off[l];
     cs.cols[l] = out;
@@ -625,6 +623,8 @@ int backward_rows(prrtc_proposal* p, int rows) {
     dz16 = p->z16[l - 1];
     dz32 = p->z32[l - 1];
   }
+  // dW = dZ^T H of every layer, both as stored: nothing waits for them but the update
+  if ((rc = gemm_gradients(dw, 4, s))) return rc;
   int blocks = 0;
   for (int l = 0; l < 4; ++l) {
     cs.first_block[l] = blocks;
