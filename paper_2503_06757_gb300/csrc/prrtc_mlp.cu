@@ -53,57 +53,66 @@ __device__ __forceinline__ int vox_hi(float x, int axis) {
   return min(kGrid - 1, (int)ceilf((x - grid_origin(axis)) / kCell - 0.5f));
 }
 
-__global__ void occupancy_scatter_kernel(const EnvView* __restrict__ envs, uint8_t* __restrict__ out) {
-  const EnvView env = envs[blockIdx.y];
-  uint8_t* grid = out + (size_t)blockIdx.y * kVox;
+__device__ __forceinline__ void mark_occupied(uint8_t* v) { *v = 1; }
+__device__ __forceinline__ void mark_occupied(bf16* v) { *v = __float2bfloat16_rn(1.f); }
+
+// Voxels whose centre is within kOccRadius of one primitive (at e, box of half
+// extents h around c), by one warp.  n / m for n below 4096 and m up to 16 is
+// exact as a product with 65536 / m + 1.
+template <int K, class Out>
+__device__ __forceinline__ void scatter_primitive(const float4* __restrict__ e, float4 c, float3 h, int lane,
+                                                  Out* __restrict__ grid) {
+  const float m = kOccRadius;
+  const int i0 = vox_lo(c.x - (h.x + m), 0), i1 = vox_hi(c.x + (h.x + m), 0);
+  const int j0 = vox_lo(c.y - (h.y + m), 1), j1 = vox_hi(c.y + (h.y + m), 1);
+  const int k0 = vox_lo(c.z - (h.z + m), 2), k1 = vox_hi(c.z + (h.z + m), 2);
+  if (i1 < i0 || j1 < j0 || k1 < k0) return;
+  const uint32_t ni = i1 - i0 + 1, nj = j1 - j0 + 1, nk = k1 - k0 + 1;
+  const uint32_t by_i = 65536u / ni + 1u, by_j = 65536u / nj + 1u;
+  for (uint32_t t = lane; t < ni * nj * nk; t += 32) {
+    const uint32_t t_i = t * by_i >> 16, t_j = t_i * by_j >> 16;
+    const int i = i0 + (int)(t - t_i * ni), j = j0 + (int)(t_i - t_j * nj), k = k0 + (int)t_j;
+    const float px = grid_origin(0) + (i + 0.5f) * kCell;
+    const float py = grid_origin(1) + (j + 0.5f) * kCell;
+    const float pz = grid_origin(2) + (k + 0.5f) * kCell;
+    if (Prim<K>::hit(e, px, py, pz, kOccRadius)) mark_occupied(grid + i + kGrid * j + kGrid * kGrid * k);
+  }
+}
+
+template <class Out>
+__global__ void occupancy_scatter_kernel(const EnvView* __restrict__ envs, Out* __restrict__ out) {
+  wait_before();
+  const EnvView& env = envs[blockIdx.y];
+  const int n_aabb = env.n_aabb, n_obb = env.n_obb, n_cyl = env.n_cyl, n_sph = env.n_sph;
+  const float4* data = env.data;
+  Out* grid = out + (size_t)blockIdx.y * kVox;
   const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
-  const int n_obs = env.n_aabb + env.n_obb + env.n_cyl + env.n_sph;
+  const int n_obs = n_aabb + n_obb + n_cyl + n_sph;
   for (int o = (int)(blockIdx.x * warps + (threadIdx.x >> 5)); o < n_obs; o += gridDim.x * warps) {
-    // locate obstacle o in the blob and bound it
-    EnvView one{};
-    float3 c, e;
-    const float m = kOccRadius;
-    if (o < env.n_aabb) {
-      one.data = env.data + 2 * o;
-      one.n_aabb = 1;
-      const float4 a = one.data[0], h = one.data[1];
-      c = make_float3(a.x, a.y, a.z);
-      e = make_float3(h.x + m, h.y + m, h.z + m);
-    } else if (o < env.n_aabb + env.n_obb) {
-      one.data = env.data + 2 * env.n_aabb + 5 * (o - env.n_aabb);
-      one.n_obb = 1;
-      const float4 a = one.data[0], h = one.data[1], r0 = one.data[2], r1 = one.data[3], r2 = one.data[4];
-      c = make_float3(a.x, a.y, a.z);
+    const float4* e = data;
+    int k = o;
+    if (k < n_aabb) {
+      e += 2 * k;
+      const float4 h = e[1];
+      scatter_primitive<kAabb>(e, e[0], make_float3(h.x, h.y, h.z), lane, grid);
+    } else if ((k -= n_aabb) < n_obb) {
+      e += 2 * n_aabb + 5 * k;
+      const float4 h = e[1], r0 = e[2], r1 = e[3], r2 = e[4];
       // world half extents of the rotated box: sum_j |R[k][j]| h_j (r_j = column j of R)
-      e = make_float3(fabsf(r0.x) * h.x + fabsf(r1.x) * h.y + fabsf(r2.x) * h.z + m,
-                      fabsf(r0.y) * h.x + fabsf(r1.y) * h.y + fabsf(r2.y) * h.z + m,
-                      fabsf(r0.z) * h.x + fabsf(r1.z) * h.y + fabsf(r2.z) * h.z + m);
-    } else if (o < env.n_aabb + env.n_obb + env.n_cyl) {
-      one.data = env.data + 2 * env.n_aabb + 5 * env.n_obb + 2 * (o - env.n_aabb - env.n_obb);
-      one.n_cyl = 1;
-      const float4 a = one.data[0], ax = one.data[1];
-      c = make_float3(a.x, a.y, a.z);
-      const float rb = sqrtf(a.w * a.w + ax.w * ax.w) + m;
-      e = make_float3(rb, rb, rb);
+      scatter_primitive<kObb>(e, e[0],
+                              make_float3(fabsf(r0.x) * h.x + fabsf(r1.x) * h.y + fabsf(r2.x) * h.z,
+                                          fabsf(r0.y) * h.x + fabsf(r1.y) * h.y + fabsf(r2.y) * h.z,
+                                          fabsf(r0.z) * h.x + fabsf(r1.z) * h.y + fabsf(r2.z) * h.z),
+                              lane, grid);
+    } else if ((k -= n_obb) < n_cyl) {
+      e += 2 * n_aabb + 5 * n_obb + 2 * k;
+      const float4 c = e[0], ax = e[1];
+      const float rb = sqrtf(c.w * c.w + ax.w * ax.w);
+      scatter_primitive<kCyl>(e, c, make_float3(rb, rb, rb), lane, grid);
     } else {
-      one.data = env.data + 2 * env.n_aabb + 5 * env.n_obb + 2 * env.n_cyl + (o - env.n_aabb - env.n_obb - env.n_cyl);
-      one.n_sph = 1;
-      const float4 a = one.data[0];
-      c = make_float3(a.x, a.y, a.z);
-      e = make_float3(a.w + m, a.w + m, a.w + m);
-    }
-    const int i0 = vox_lo(c.x - e.x, 0), i1 = vox_hi(c.x + e.x, 0);
-    const int j0 = vox_lo(c.y - e.y, 1), j1 = vox_hi(c.y + e.y, 1);
-    const int k0 = vox_lo(c.z - e.z, 2), k1 = vox_hi(c.z + e.z, 2);
-    if (i1 < i0 || j1 < j0 || k1 < k0) continue;
-    const int ni = i1 - i0 + 1, nj = j1 - j0 + 1, nk = k1 - k0 + 1;
-    for (int t = lane; t < ni * nj * nk; t += 32) {
-      const int i = i0 + t % ni, j = j0 + (t / ni) % nj, k = k0 + t / (ni * nj);
-      const float px = grid_origin(0) + (i + 0.5f) * kCell;
-      const float py = grid_origin(1) + (j + 0.5f) * kCell;
-      const float pz = grid_origin(2) + (k + 0.5f) * kCell;
-      if (sphere_hits_env(px, py, pz, kOccRadius, one.data, one.n_aabb, one.n_obb, one.n_cyl, one.n_sph))
-        grid[i + kGrid * j + kGrid * kGrid * k] = 1;
+      e += 2 * n_aabb + 5 * n_obb + 2 * n_cyl + (k - n_cyl);
+      const float4 c = e[0];
+      scatter_primitive<kSph>(e, c, make_float3(c.w, c.w, c.w), lane, grid);
     }
   }
 }
@@ -205,11 +214,82 @@ __global__ void __launch_bounds__(256) l1_occ_gemv_kernel(const uint8_t* __restr
   }
 }
 
-// Occupancy rows (one per distinct environment) as BF16 inputs of the
-// occupancy part of the first layer, for batches with many environments.
-__global__ void occ_bf16_kernel(const uint8_t* __restrict__ occ, bf16* __restrict__ x) {
-  const size_t base = (size_t)blockIdx.x * kVox;
-  for (int c = threadIdx.x; c < kVox; c += blockDim.x) x[base + c] = __float2bfloat16_rn(occ[base + c] ? 1.f : 0.f);
+// First hidden layer of the inference rows: the occupancy part of the row's
+// environment plus the start / goal columns, ReLU(W1 x + b1) in BF16 (rows past
+// B: zeros).  A block takes 16 rows and 128 columns, a thread eight columns of
+// a row.
+constexpr int kH1Rows = 16, kH1Cols = 128;
+__global__ void __launch_bounds__(256) hidden1_kernel(const float* __restrict__ h1o, const int* __restrict__ row_env,
+                                                       const float* __restrict__ qs, const float* __restrict__ qg,
+                                                       const float* __restrict__ lo, const float* __restrict__ span,
+                                                       const bf16* __restrict__ wq, const float* __restrict__ bias,
+                                                       int B, int n_rows, int dof, bf16* __restrict__ h1) {
+  __shared__ float s_w[2 * kMaxDof][kH1Cols];
+  __shared__ float s_x[kH1Rows][2 * kMaxDof];
+  let_next_start();
+  wait_before();
+  constexpr int kSlices = kHid0 / kH1Cols;
+  const int c0 = (int)blockIdx.x % kSlices * kH1Cols, r0 = (int)blockIdx.x / kSlices * kH1Rows;
+  const int nq = 2 * dof;
+  for (int i = threadIdx.x; i < nq * kH1Cols; i += 256) {
+    const int c = i / kH1Cols, j = i % kH1Cols;
+    s_w[c][j] = __bfloat162float(wq[(size_t)(c < dof ? c : kQPad + c - dof) * kHid0 + c0 + j]);
+  }
+  for (int i = threadIdx.x; i < kH1Rows * nq; i += 256) {
+    const int rr = i / nq, c = i % nq, row = r0 + rr;
+    float v = 0.f;
+    if (row < B) {
+      const int j = c < dof ? c : c - dof;
+      const float* q = c < dof ? qs : qg;
+      v = __bfloat162float(__float2bfloat16_rn(2.f * (q[(size_t)row * dof + j] - lo[j]) / span[j] - 1.f));
+    }
+    s_x[rr][c] = v;
+  }
+  __syncthreads();
+  const int rr = threadIdx.x / (kH1Cols / 8), j8 = threadIdx.x % (kH1Cols / 8) * 8, row = r0 + rr;
+  if (row >= n_rows) return;
+  uint4 pk = make_uint4(0u, 0u, 0u, 0u);
+  if (row < B) {
+    const float4* src = reinterpret_cast<const float4*>(h1o + (size_t)row_env[row] * kHid0 + c0 + j8);
+    const float4 a = src[0], b = src[1];
+    float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] += bias[c0 + j8 + e];
+    for (int c = 0; c < nq; ++c) {
+      const float x = s_x[rr][c];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = fmaf(s_w[c][j8 + e], x, v[e]);
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = fmaxf(v[e], 0.f);
+    const uint2 l = bf16x4(make_float4(v[0], v[1], v[2], v[3])), h = bf16x4(make_float4(v[4], v[5], v[6], v[7]));
+    pk = make_uint4(l.x, l.y, h.x, h.y);
+  }
+  *reinterpret_cast<uint4*>(h1 + (size_t)row * kHid0 + c0 + j8) = pk;
+}
+
+// Head rows into the planner's mixture rows: logits[8] | means[8][kMaxDof] |
+// log-sigmas[8][kMaxDof], clamped.  Entries of joints from dof on are not
+// written; the planner skips them.
+__global__ void mixture_rows_kernel(const float* __restrict__ out, int P, int B, int dof,
+                                    float* const* __restrict__ gmm_rows) {
+  let_next_start();
+  wait_before();
+  const int head = kK * (1 + 2 * dof);
+  const int at = blockIdx.x * blockDim.x + threadIdx.x;
+  if (at >= B * head) return;
+  const int b = at / head, t = at % head;
+  const float val = out[(size_t)b * P + t];
+  float* g = gmm_rows[b];
+  if (t < kK) {
+    g[t] = val;
+  } else if (t < kK + kK * dof) {
+    const int k = (t - kK) / dof, j = (t - kK) % dof;
+    g[kK + k * kMaxDof + j] = val;
+  } else {
+    const int k = (t - kK - kK * dof) / dof, j = (t - kK - kK * dof) % dof;
+    g[kK + kK * kMaxDof + k * kMaxDof + j] = fminf(fmaxf(val, kLogSigMin), kLogSigMax);
+  }
 }
 
 // Mixture negative log-likelihood of each sample's target and its gradient
@@ -429,7 +509,6 @@ struct prrtc_proposal {
   bf16* params16 = nullptr;  // BF16 copies of all parameters, in their order
   bf16* w16[4] = {};         // the layers' weights in it
   bf16* wq = nullptr;       // start / goal columns of layer 1, transposed: [2 kQPad x kHid0]
-  bf16* wtile[3] = {};  // layers 2, 3 and the head, tiled for the fused inference kernel
   int step = 0;
   float lo[kMaxDof], span[kMaxDof];
   float* d_lims = nullptr;  // lo[16] | span[16]
@@ -468,9 +547,9 @@ struct prrtc_proposal {
   size_t xo16_cap = 0;
   float* h1o32 = nullptr;  // [envs x kHid0]
   size_t h1o32_cap = 0;
-  bf16* atile[3] = {};     // tiled hidden activations, 128-row tiles
+  bf16* ih16[3] = {};      // hidden activations of the last inference batch
   int last_infer_B = 0;    // problems of the last staged inference batch
-  size_t atile_cap[3] = {};
+  size_t ih16_cap[3] = {};
   Pending pend;            // the staged, not yet submitted, inference batch
   bool pend_ok = false;
   cudaEvent_t inf_ev[2] = {};  // timing of the last submitted chain
@@ -551,13 +630,8 @@ int ensure_scratch(prrtc_proposal* p, int rows) {
   return PRRTC_OK;
 }
 
-// What inference reads, from the BF16 weights: the tiled layers and the
-// transposed start / goal columns.
+// The start / goal columns of layer 1 transposed, which inference reads.
 int refresh_inference_weights(prrtc_proposal* p) {
-  for (int l = 1; l < 4; ++l) {
-    const int rc = mlp_tile_weights(p->w16[l], p->out_dim[l], p->in_dim[l], p->wtile[l - 1], p->stream);
-    if (rc) return rc;
-  }
   transpose_kernel<<<dim3(2 * kQPad / 32, kHid0 / 32), dim3(32, 8), 0, p->stream>>>(p->w16[0] + kVox, kIn, p->wq,
                                                                                     kHid0);
   return cudaGetLastError() == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
@@ -671,45 +745,33 @@ uint64_t chain_signature(std::initializer_list<uint64_t> vals) {
 int enqueue_inference(prrtc_proposal* p, const EnvView* d_envs, int U, const int* d_row_env, float* const* d_rows,
                       const float* d_qs, const float* d_qg, int B, int rows) {
   const cudaStream_t s = p->stream;
-  MCK(cudaMemsetAsync(p->inf_occ, 0, (size_t)U * kVox, s));
-  occupancy_scatter_kernel<<<dim3(4, U), 256, 0, s>>>(d_envs, p->inf_occ);
   int rc;
+  const dim3 scatter(8, U);
   if (U <= kGemvMaxEnvs) {
+    MCK(cudaMemsetAsync(p->inf_occ, 0, (size_t)U * kVox, s));
+    occupancy_scatter_kernel<<<scatter, 256, 0, s>>>(d_envs, p->inf_occ);
     l1_occ_gemv_kernel<<<kHid0 / 8, 256, 0, s>>>(p->inf_occ, U, p->w16[0], p->h1o32);
   } else {
-    occ_bf16_kernel<<<U, 256, 0, s>>>(p->inf_occ, p->xo16);
+    MCK(cudaMemsetAsync(p->xo16, 0, (size_t)U * kVox * sizeof(bf16), s));
+    occupancy_scatter_kernel<<<scatter, 256, 0, s>>>(d_envs, p->xo16);
     if ((rc = gemm_bf16_ld(p->xo16, kVox, p->w16[0], kIn, U, kHid0, kVox, nullptr, 0, p->h1o32, kHid0, nullptr, 0, s,
                            0, 0, nullptr, 0)))
       return rc;
   }
   MCK(cudaGetLastError());
-  MlpInferArgs a{};
-  a.rows = rows;
-  a.B = B;
-  a.dof = p->dof;
-  a.h0 = kHid0;
-  a.h1 = kHid1;
-  a.h2 = kHid2;
-  a.head = p->P;
-  a.qpad = kQPad;
-  a.h1o = p->h1o32;
-  a.row_env = d_row_env;
-  a.qs = d_qs;
-  a.qg = d_qg;
-  a.lo = p->d_lims;
-  a.span = p->d_lims + kMaxDof;
-  a.wq = p->wq;
-  for (int l = 0; l < 3; ++l) {
-    a.w[l] = p->wtile[l];
-    a.act[l] = p->atile[l];
+  MCK(launch_overlapped(hidden1_kernel, kHid0 / kH1Cols * ((rows + kH1Rows - 1) / kH1Rows), 256, 0, s, 1, p->h1o32,
+                        d_row_env, d_qs, d_qg, p->d_lims, p->d_lims + kMaxDof, p->wq, p->master + p->b_off[0], B, rows,
+                        p->dof, p->ih16[0]));
+  // one chain of accumulation per output: K is not split, whatever the batch
+  for (int l = 1; l < 4; ++l) {
+    const int in = p->in_dim[l], out = p->out_dim[l];
+    if ((rc = gemm_bf16_ld(p->ih16[l - 1], in, p->w16[l], in, rows, out, in, p->master + p->b_off[l], l < 3,
+                           l < 3 ? nullptr : p->out32, out, l < 3 ? p->ih16[l] : nullptr, out, s, 1, 0, nullptr, 0)))
+      return rc;
   }
-  for (int l = 0; l < 4; ++l) a.bias[l] = p->master + p->b_off[l];
-  a.gmm_rows = d_rows;
-  a.mix_k = kK;
-  a.gmm_dof = kMaxDof;
-  a.logsig_lo = kLogSigMin;
-  a.logsig_hi = kLogSigMax;
-  return mlp_infer(a, s);
+  const int head = kK * (1 + 2 * p->dof);
+  MCK(launch_overlapped(mixture_rows_kernel, (B * head + 255) / 256, 256, 0, s, 1, p->out32, p->P, B, p->dof, d_rows));
+  return PRRTC_OK;
 }
 
 }  // namespace
@@ -773,10 +835,9 @@ int prrtc_internal_proposal_stage(prrtc_proposal* p, const EnvView* envs, const 
   if (U > kGemvMaxEnvs && (rc = grow(&p->xo16, &p->xo16_cap, (size_t)U * kVox))) return rc;
   if ((rc = grow(&p->h1o32, &p->h1o32_cap, (size_t)U * kHid0))) return rc;
   {
-    const size_t m_pad = (size_t)((rows + 127) / 128) * 128;
     const int width[3] = {kHid0, kHid1, kHid2};
     for (int l = 0; l < 3; ++l)
-      if ((rc = grow(&p->atile[l], &p->atile_cap[l], m_pad * width[l]))) return rc;
+      if ((rc = grow(&p->ih16[l], &p->ih16_cap[l], (size_t)rows * width[l]))) return rc;
   }
   // one staging block: env views | row -> env | planner row pointers | starts | goals
   auto up16 = [](size_t x) { return (x + 15) & ~size_t(15); };
@@ -802,9 +863,8 @@ int prrtc_internal_proposal_stage(prrtc_proposal* p, const EnvView* envs, const 
   p->last_infer_B = B;
   q.sig = chain_signature(
       {(uint64_t)B, (uint64_t)rows, (uint64_t)U, (uint64_t)(uintptr_t)p->xo16,
-       (uint64_t)(uintptr_t)p->h1o32, (uint64_t)(uintptr_t)p->wq, (uint64_t)(uintptr_t)p->atile[0],
-       (uint64_t)(uintptr_t)p->atile[1], (uint64_t)(uintptr_t)p->atile[2], (uint64_t)(uintptr_t)p->wtile[0],
-       (uint64_t)(uintptr_t)p->wtile[1], (uint64_t)(uintptr_t)p->wtile[2],
+       (uint64_t)(uintptr_t)p->h1o32, (uint64_t)(uintptr_t)p->wq, (uint64_t)(uintptr_t)p->ih16[0],
+       (uint64_t)(uintptr_t)p->ih16[1], (uint64_t)(uintptr_t)p->ih16[2],
        (uint64_t)(uintptr_t)p->d_stage, (uint64_t)(uintptr_t)p->inf_occ,
        (uint64_t)(uintptr_t)p->x16, (uint64_t)(uintptr_t)p->h16[0], (uint64_t)(uintptr_t)p->h16[1],
        (uint64_t)(uintptr_t)p->h16[2], (uint64_t)(uintptr_t)p->out32, (uint64_t)(uintptr_t)p->w16[0],
@@ -896,7 +956,6 @@ int prrtc_proposal_create(int32_t dof, const float* lower, const float* upper, c
     return mlp_fail(PRRTC_ERR_NO_DEVICE, "no CUDA device");
   for (int j = 0; j < dof; ++j)
     if (!(upper[j] > lower[j])) return mlp_fail(PRRTC_ERR_INVALID_ARG, "joint limits must have upper > lower");
-  if (mlp_check_shapes(kHid0, kHid1, kHid2, head_pad(dof))) return mlp_fail(PRRTC_ERR_UNSUPPORTED, "layer widths");
   prrtc_proposal* p = new prrtc_proposal();
   p->device = dev;
   p->dof = dof;
@@ -925,8 +984,6 @@ int prrtc_proposal_create(int32_t dof, const float* lower, const float* upper, c
             cudaMalloc(&p->wq, (size_t)2 * kQPad * kHid0 * 2) == cudaSuccess &&
             cudaMalloc(&p->params16, off * 2) == cudaSuccess;
   for (int l = 0; l < 4 && ok; ++l) p->w16[l] = p->params16 + p->w_off[l];
-  for (int l = 0; l < 4 && ok; ++l)
-    ok = (l == 0 || cudaMalloc(&p->wtile[l - 1], (size_t)dims[l + 1] * dims[l] * 2) == cudaSuccess);
   if (!ok) {
     cudaGetLastError();
     prrtc_proposal_destroy(p);
@@ -953,15 +1010,12 @@ void prrtc_proposal_destroy(prrtc_proposal* p) {
   free_scratch(p);
   cudaFree(p->master); cudaFree(p->grad); cudaFree(p->m); cudaFree(p->v); cudaFree(p->d_lims);
   cudaFree(p->wq); cudaFree(p->params16); cudaFree(p->loss);
-  for (int l = 0; l < 4; ++l) {
-    if (l > 0) cudaFree(p->wtile[l - 1]);
-  }
   cudaFree(p->occ); cudaFree(p->qs); cudaFree(p->qg); cudaFree(p->tgt); cudaFree(p->scene_of); cudaFree(p->rows);
   cudaFree(p->envs); cudaFree(p->gmm_rows);
   cudaFree(p->d_stage); cudaFree(p->inf_occ); cudaFree(p->d_mix);
   if (p->h_mix) cudaFreeHost(p->h_mix);
   cudaFree(p->xo16); cudaFree(p->h1o32);
-  for (bf16* t : p->atile) cudaFree(t);
+  for (bf16* t : p->ih16) cudaFree(t);
   if (p->h_stage) cudaFreeHost(p->h_stage);
   if (p->infer_exec) cudaGraphExecDestroy(p->infer_exec);
   if (p->done) cudaEventDestroy(p->done);
@@ -1049,25 +1103,9 @@ int prrtc_proposal_inference_layers(prrtc_proposal* p, int32_t B, float* h1, flo
   MCK(cudaStreamSynchronize(p->stream));
   const int width[3] = {kHid0, kHid1, kHid2};
   float* outs[3] = {h1, h2, h3};
-  const int tiles = (B + 127) / 128;
   for (int l = 0; l < 3; ++l) {
-    if (!outs[l]) continue;
-    // [row tile][64-column k-block] blocks of 128 rows x 128 bytes, 16-byte
-    // unit u of row i stored at unit u ^ (i % 8)
-    const size_t elems = (size_t)tiles * 128 * width[l];
-    std::vector<uint16_t> raw(elems);
-    MCK(cudaMemcpy(raw.data(), p->atile[l], elems * 2, cudaMemcpyDeviceToHost));
-    const int kbs = width[l] / 64;
-    for (int r = 0; r < B; ++r) {
-      const int mt = r / 128, i = r % 128;
-      for (int c = 0; c < width[l]; ++c) {
-        const int kb = c / 64, cc = c % 64;
-        const size_t byte = ((size_t)mt * kbs + kb) * (128 * 128) + (size_t)i * 128 +
-                            ((size_t)((cc >> 3) ^ (i & 7)) << 4) + ((size_t)(cc & 7) << 1);
-        const uint32_t bits = (uint32_t)raw[byte / 2] << 16;
-        std::memcpy(outs[l] + (size_t)r * width[l] + c, &bits, 4);
-      }
-    }
+    const int rc = bf16_rows_to_host(p->ih16[l], B, width[l], width[l], outs[l], p->stream);
+    if (rc) return rc;
   }
   return PRRTC_OK;
 }
