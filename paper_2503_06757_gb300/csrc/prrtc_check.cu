@@ -486,7 +486,8 @@ constexpr int kStateFloats = 3 * (kMaxDistinctSpheres + kMaxDof);
 
 __global__ void __launch_bounds__(kStateWarps * 32) check_state_warps_kernel(
     const RobotDev* __restrict__ robot, EnvView env, const float* __restrict__ q, int n, uint8_t* __restrict__ valid,
-    float* __restrict__ spheres, unsigned long long* __restrict__ counters, int* __restrict__ error, int np_pad) {
+    float* __restrict__ spheres, unsigned long long* __restrict__ counters, uint4* __restrict__ slots,
+    int* __restrict__ error, int np_pad, int dof) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(8) uint64_t bar;
   __shared__ int s_ok;
@@ -496,11 +497,14 @@ __global__ void __launch_bounds__(kStateWarps * 32) check_state_warps_kernel(
   float* thr = reinterpret_cast<float*>(pair + np_pad);
   const int env_f4 = env.n_float4();
   float4* senv = reinterpret_cast<float4*>(thr + np_pad);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int idx = blockIdx.x * kStateWarps + warp;
+  // on its way while the tables are staged (it may come from host memory)
+  const float ql = idx < n && lane < dof ? q[(size_t)idx * dof + lane] : 0.f;
   if (threadIdx.x == 0) s_ok = stage_tables(robot, env, R, pair, thr, senv, np_pad, &bar, error);
   __syncthreads();
-  if (!s_ok) return;  // block-uniform
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int dof = R->dof, n_raw = R->n_raw, n_pairs = R->n_pairs;
+  if (!s_ok || idx >= n) return;  // nothing below waits for another warp
+  const int n_raw = R->n_raw, n_pairs = R->n_pairs;
   float* stage = s_stage[warp];                    // sphere centres, then the links' bounding spheres
   float* bounds = stage + 3 * kMaxDistinctSpheres;
   const bool has_grid = env.esdf.v != nullptr;
@@ -508,73 +512,72 @@ __global__ void __launch_bounds__(kStateWarps * 32) check_state_warps_kernel(
   const float4* e_obb = senv + 2 * env.n_aabb;
   const float4* e_cyl = e_obb + 5 * env.n_obb;
   const float4* e_sph = e_cyl + 2 * env.n_cyl;
-  uint32_t states = 0, passes = 0, pairs = 0, fine[4] = {0, 0, 0, 0};
-  for (int idx = blockIdx.x * kStateWarps + warp; idx < n; idx += gridDim.x * kStateWarps) {
-    const float ql = lane < dof ? q[(size_t)idx * dof + lane] : 0.f;
-    float sl = 0.f, cl = 1.f;
-    if (lane < dof && revolute(R->jtype[lane])) joint_sincos<false>(ql, sl, cl);
-    __syncwarp();
-    Frame T;
-    for (int i = 0; i < dof; ++i) {
-      fk_apply(R, i, R->jtype[i], __shfl_sync(kFull, ql, i), __shfl_sync(kFull, sl, i), __shfl_sync(kFull, cl, i), T);
-      const int s0 = R->sph_begin[i], cnt = R->sph_begin[i + 1] - s0;
-      for (int k = lane; k <= cnt; k += 32) {  // one more: the link's bounding sphere, or its only one
-        const float3 c = T.at(k < cnt ? R->sph[s0 + k] : R->grp[i]);
-        float* st = k < cnt ? stage + 3 * (s0 + k) : bounds + 3 * i;
-        st[0] = c.x;
-        st[1] = c.y;
-        st[2] = c.z;
-      }
+  uint32_t passes = 0, pairs = 0, fine[4] = {0, 0, 0, 0};
+  float sl = 0.f, cl = 1.f;
+  if (lane < dof && revolute(R->jtype[lane])) joint_sincos<false>(ql, sl, cl);
+  Frame T;
+  for (int i = 0; i < dof; ++i) {
+    fk_apply(R, i, R->jtype[i], __shfl_sync(kFull, ql, i), __shfl_sync(kFull, sl, i), __shfl_sync(kFull, cl, i), T);
+    const int s0 = R->sph_begin[i], cnt = R->sph_begin[i + 1] - s0;
+    for (int k = lane; k <= cnt; k += 32) {  // one more: the link's bounding sphere, or its only one
+      const float3 c = T.at(k < cnt ? R->sph[s0 + k] : R->grp[i]);
+      float* st = k < cnt ? stage + 3 * (s0 + k) : bounds + 3 * i;
+      st[0] = c.x;
+      st[1] = c.y;
+      st[2] = c.z;
     }
-    __syncwarp();
-    states++;
-    bool hit = false;
-    for (int i = dof - 1; i >= 0 && env_f4; --i) {
-      const int s0 = R->sph_begin[i], cnt = R->sph_begin[i + 1] - s0;
-      if (!cnt) continue;
-      const float3 b = make_float3(bounds[3 * i], bounds[3 * i + 1], bounds[3 * i + 2]);
-      const float br = R->grp[i].w;
-      const float* st = stage + 3 * s0;
-      passes += filter ? 1u : (uint32_t)cnt;
-      hit |= warp_link_stage<kAabb>(senv, env.n_aabb, b, br, filter, st, R->sph + s0, cnt, lane, fine[kAabb]);
-      hit |= warp_link_stage<kObb>(e_obb, env.n_obb, b, br, filter, st, R->sph + s0, cnt, lane, fine[kObb]);
-      hit |= warp_link_stage<kCyl>(e_cyl, env.n_cyl, b, br, filter, st, R->sph + s0, cnt, lane, fine[kCyl]);
-      hit |= warp_link_stage<kSph>(e_sph, env.n_sph, b, br, filter, st, R->sph + s0, cnt, lane, fine[kSph]);
-      if (__any_sync(kFull, hit)) break;
-    }
-    if (has_grid) {
-      for (int s = lane; s < R->n_spheres; s += 32)
-        hit |= esdf_read(env.esdf, stage[3 * s], stage[3 * s + 1], stage[3 * s + 2]) < R->sph[s].w;
-      passes += (uint32_t)R->n_spheres;
-    }
-    if (!__any_sync(kFull, hit)) {
-      for (int k = lane; k < n_pairs; k += 32) {
-        const uint32_t pr = pair[k];
-        const float* si = stage + 3 * (pr & 0xffffu);
-        const float* sj = stage + 3 * (pr >> 16);
-        const float dx = si[0] - sj[0], dy = si[1] - sj[1], dz = si[2] - sj[2];
-        hit |= fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < thr[k];
-      }
-      pairs += (uint32_t)n_pairs;
-    }
-    hit = __any_sync(kFull, hit);
-    if (lane == 0) valid[idx] = hit ? 0 : 1;
-    if (spheres) {
-      float4* out = reinterpret_cast<float4*>(spheres) + (size_t)idx * n_raw;
-      for (int r = lane; r < n_raw; r += 32) {
-        const int ds = robot->raw_to_distinct[r];
-        out[r] = make_float4(stage[3 * ds], stage[3 * ds + 1], stage[3 * ds + 2], R->sph[ds].w);
-      }
-    }
-    __syncwarp();
   }
-  if (lane == 0 && counters && states) {
+  __syncwarp();
+  bool hit = false;
+  for (int i = dof - 1; i >= 0 && env_f4; --i) {
+    const int s0 = R->sph_begin[i], cnt = R->sph_begin[i + 1] - s0;
+    if (!cnt) continue;
+    const float3 b = make_float3(bounds[3 * i], bounds[3 * i + 1], bounds[3 * i + 2]);
+    const float br = R->grp[i].w;
+    const float* st = stage + 3 * s0;
+    passes += filter ? 1u : (uint32_t)cnt;
+    hit |= warp_link_stage<kAabb>(senv, env.n_aabb, b, br, filter, st, R->sph + s0, cnt, lane, fine[kAabb]);
+    hit |= warp_link_stage<kObb>(e_obb, env.n_obb, b, br, filter, st, R->sph + s0, cnt, lane, fine[kObb]);
+    hit |= warp_link_stage<kCyl>(e_cyl, env.n_cyl, b, br, filter, st, R->sph + s0, cnt, lane, fine[kCyl]);
+    hit |= warp_link_stage<kSph>(e_sph, env.n_sph, b, br, filter, st, R->sph + s0, cnt, lane, fine[kSph]);
+    if (__any_sync(kFull, hit)) break;
+  }
+  if (has_grid) {
+    for (int s = lane; s < R->n_spheres; s += 32)
+      hit |= esdf_read(env.esdf, stage[3 * s], stage[3 * s + 1], stage[3 * s + 2]) < R->sph[s].w;
+    passes += (uint32_t)R->n_spheres;
+  }
+  if (!__any_sync(kFull, hit)) {
+    for (int k = lane; k < n_pairs; k += 32) {
+      const uint32_t pr = pair[k];
+      const float* si = stage + 3 * (pr & 0xffffu);
+      const float* sj = stage + 3 * (pr >> 16);
+      const float dx = si[0] - sj[0], dy = si[1] - sj[1], dz = si[2] - sj[2];
+      hit |= fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < thr[k];
+    }
+    pairs += (uint32_t)n_pairs;
+  }
+  hit = __any_sync(kFull, hit);
+  if (lane == 0) valid[idx] = hit ? 0 : 1;
+  if (spheres) {
+    float4* out = reinterpret_cast<float4*>(spheres) + (size_t)idx * n_raw;
+    for (int r = lane; r < n_raw; r += 32) {
+      const int ds = robot->raw_to_distinct[r];
+      out[r] = make_float4(stage[3 * ds], stage[3 * ds + 1], stage[3 * ds + 2], R->sph[ds].w);
+    }
+  }
+  if (lane != 0) return;
+  if (slots) {
+    slots[2 * idx] = make_uint4(passes, pairs, fine[0], fine[1]);
+    slots[2 * idx + 1] = make_uint4(fine[2], fine[3], 0u, 0u);
+  } else if (counters) {
     atomicAdd(counters + 0, (unsigned long long)passes);
     atomicAdd(counters + 1, (unsigned long long)pairs);
-    atomicAdd(counters + 2, (unsigned long long)states);
+    atomicAdd(counters + 2, 1ull);
     for (int k = 0; k < 4; ++k) atomicAdd(counters + 3 + k, (unsigned long long)fine[k]);
   }
 }
+
 
 // Shared memory of a block of `warps` warps.
 struct CheckShape {
@@ -699,15 +702,15 @@ static cudaError_t state_warps_attribute() {
 }
 
 cudaError_t launch_check_states(const RobotDev* robot, const RobotHeader& h, EnvView env, const float* q, int n,
-                                uint8_t* valid, float* spheres, unsigned long long* counters, int* error,
+                                uint8_t* valid, float* spheres, unsigned long long* counters, uint4* slots, int* error,
                                 cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
   const CheckShape shape = check_shape(h, env);
-  if (n <= kWarpPerState) {
+  if (n <= kWarpPerState || slots) {
     const cudaError_t e = state_warps_attribute();
     if (e != cudaSuccess) return e;
     check_state_warps_kernel<<<(n - 1) / kStateWarps + 1, kStateWarps * 32, shape.table_bytes, stream>>>(
-        robot, env, q, n, valid, spheres, counters, error, shape.np_pad);
+        robot, env, q, n, valid, spheres, counters, slots, error, shape.np_pad, h.dof);
     return cudaGetLastError();
   }
   CheckWave wave{};

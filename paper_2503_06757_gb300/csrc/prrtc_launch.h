@@ -143,9 +143,13 @@ inline int reported_iterations(const ProblemState& S, const prrtc_params& p) {
 }
 
 // Launchers (return cudaError_t of the launch).
+// slots (nullable): a warp per state whatever n, and its counters (sphere
+// passes, pair tests, the four second-stage counts, as 32-bit words) at
+// slots[2 * state] instead of summed into counters[7].  All pointers may be
+// pinned host memory.
 cudaError_t launch_check_states(const RobotDev* robot, const RobotHeader& host_header, EnvView env, const float* q,
-                                int n, uint8_t* valid, float* spheres, unsigned long long* counters, int* error,
-                                cudaStream_t stream);
+                                int n, uint8_t* valid, float* spheres, unsigned long long* counters, uint4* slots,
+                                int* error, cudaStream_t stream);
 
 // Philox4x32-10 of n counters (device arrays of 4n words each).
 cudaError_t launch_philox(const uint32_t* ctr, int n, uint64_t key, uint32_t* out, cudaStream_t stream);

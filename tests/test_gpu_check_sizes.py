@@ -77,7 +77,10 @@ def test_few_and_many_states_agree(name):
     assert 0 < valid.sum() or "600" in name
     plain = P.prrtc_check_states(rb, ev, Q)  # without centres
     np.testing.assert_array_equal(plain, valid)
-    for lo, hi in ((0, 1), (1, 34), (34, 1500), (1500, n - 1000), (n - 1000, n)):
+    # up to 1024 states go through pinned host memory, unless their centres are too many
+    for lo, hi in ((0, 1), (1, 34), (34, 1058), (1058, 2083), (2083, n)):
+        np.testing.assert_array_equal(P.prrtc_check_states(rb, ev, Q[lo:hi]), valid[lo:hi])
+        assert P.prrtc_last_launch_stats()["fk_states"] == hi - lo
         v, s = P.prrtc_check_states(rb, ev, Q[lo:hi], want_spheres=True)
         np.testing.assert_array_equal(v, valid[lo:hi])
         np.testing.assert_array_equal(s, spheres[lo:hi])
