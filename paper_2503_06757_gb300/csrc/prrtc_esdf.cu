@@ -177,31 +177,62 @@ __global__ void edt_scan_kernel(const In* __restrict__ in, int n, size_t stride,
 //
 // A candidate is one 32-bit key, (f(t) + (i - t)^2) << 10 | t (t below 1024,
 // values below 2^22 with "none" at kNoneSq), so that a step is one minimum and
-// ties go to the leftmost t.  The lanes of a warp take the union of their
-// ranges, which keeps the loop uniform and finds the same minimum.  The first
-// levels have fewer voxels than the block has warps: the warps share a range.
+// ties go to the leftmost t.  The first levels have fewer voxels than the block
+// has warps: the warps share a range.  What bounds the pass is instruction
+// issue (75% of the slots), so the last two levels, three quarters of the
+// voxels, go together: three voxels share the loads, the loop and the range,
+// and store no place (256^3: 142 us a pass with every level by itself, 111 so;
+// 80^3 14.5 and 9.5).
 constexpr int kAxisWarps = 8;
-constexpr int kNoneSq = 3 << 20;  // above 3 * 1023^2
+constexpr int kNoneSq = 3140000;  // above 3 * 1023^2; with 1026^2 (padded positions) still below 2^22
 
-__host__ __device__ constexpr int axis_smem(int n) { return n * 32 * (int)(sizeof(int) + sizeof(uint16_t)); }
+constexpr int kAxisPad = 3;       // rows past the line that a step of four may touch
 
-// Smallest key of voxel i over t = lo .. hi of a column of 32-strided values.
-__device__ __forceinline__ uint32_t nearest_key(const int* __restrict__ col, int i, int lo, int hi) {
+__host__ __device__ constexpr int axis_smem(int n) {
+  return 32 * ((n + kAxisPad) * (int)sizeof(int) + n * (int)sizeof(uint16_t));
+}
+
+// Smallest key of voxel i over at least t = lo .. hi of the lane's column of
+// 32-strided values (n of them, then kAxisPad rows of "none").  The lanes take
+// as many steps as the longest range needs, four at a time, each from its own
+// lo or, near the line's end, from farther left: positions outside the range
+// lose against its leftmost minimum.
+__device__ __forceinline__ uint32_t nearest_key(const int* __restrict__ col, int i, int lo, int hi, int n) {
+  const int steps = (__reduce_max_sync(kFull, hi - lo) + 4) & ~3;
+  int t = max(min(lo, n + kAxisPad - steps), 0);
   uint32_t k0 = ~0u, k1 = ~0u;
-  int t = lo;
-  for (; t + 7 <= hi; t += 8) {
-    int f[8];
+  const int* p = col + t * 32;
+  for (int left = steps; left > 0; left -= 4, p += 128, t += 4) {
+    int f[4];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) f[u] = max(col[(t + u) * 32], 0);
+    for (int u = 0; u < 4; ++u) f[u] = max(p[u * 32], 0);
+    const int d = i - t;
+    k0 = min(k0, (uint32_t)(d * d + f[0]) << 10 | (uint32_t)t);
+    k1 = min(k1, (uint32_t)((d - 1) * (d - 1) + f[1]) << 10 | (uint32_t)(t + 1));
+    k0 = min(k0, (uint32_t)((d - 2) * (d - 2) + f[2]) << 10 | (uint32_t)(t + 2));
+    k1 = min(k1, (uint32_t)((d - 3) * (d - 3) + f[3]) << 10 | (uint32_t)(t + 3));
+  }
+  return min(k0, k1);
+}
+
+// The same for voxels i, i + 1 and i + 2 over one range.
+__device__ __forceinline__ void nearest_keys(const int* __restrict__ col, int i, int lo, int hi, int n,
+                                             uint32_t (&key)[3]) {
+  const int steps = (__reduce_max_sync(kFull, hi - lo) + 4) & ~3;
+  int t = max(min(lo, n + kAxisPad - steps), 0);
+  const int* p = col + t * 32;
+  key[0] = key[1] = key[2] = ~0u;
+  for (int left = steps; left > 0; left -= 4, p += 128) {
+    int f[4];
 #pragma unroll
-    for (int u = 0; u < 8; u += 2) {
-      const int d0 = i - t - u, d1 = d0 - 1;
-      k0 = min(k0, (uint32_t)(d0 * d0 + f[u]) << 10 | (uint32_t)(t + u));
-      k1 = min(k1, (uint32_t)(d1 * d1 + f[u + 1]) << 10 | (uint32_t)(t + u + 1));
+    for (int u = 0; u < 4; ++u) f[u] = max(p[u * 32], 0);
+#pragma unroll
+    for (int u = 0; u < 4; ++u, ++t) {
+      const int d = i - t;
+#pragma unroll
+      for (int v = 0; v < 3; ++v) key[v] = min(key[v], (uint32_t)((d + v) * (d + v) + f[u]) << 10 | (uint32_t)t);
     }
   }
-  for (; t <= hi; ++t) k0 = min(k0, (uint32_t)((i - t) * (i - t) + max(col[t * 32], 0)) << 10 | (uint32_t)t);
-  return min(k0, k1);
 }
 
 template <class In, class Out>
@@ -211,8 +242,8 @@ __global__ void __launch_bounds__(kAxisWarps * 32) edt_axis_kernel(const In* __r
   extern __shared__ int axis_smem_raw[];
   __shared__ int s_count[kAxisWarps];
   __shared__ uint32_t s_key[kAxisWarps][32];                    // shared voxels of the first levels
-  int* s = axis_smem_raw;                                       // [n][32], the more frequent kind positive
-  uint16_t* nearest = reinterpret_cast<uint16_t*>(s + n * 32);  // [n][32], t*
+  int* s = axis_smem_raw;  // [n + kAxisPad][32], the more frequent kind positive
+  uint16_t* nearest = reinterpret_cast<uint16_t*>(s + (n + kAxisPad) * 32);  // [n][32], t*
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const size_t line = (size_t)blockIdx.x * 32 + lane;
   const bool live = line < lines;
@@ -230,6 +261,7 @@ __global__ void __launch_bounds__(kAxisWarps * 32) edt_axis_kernel(const In* __r
   count = __reduce_add_sync(kFull, count);
   if (lane == 0) s_count[warp] = count;
   s_key[warp][lane] = ~0u;
+  if (warp < kAxisPad) s[(n + warp) * 32 + lane] = kNoneSq;
   __syncthreads();
   count = 0;
 #pragma unroll
@@ -241,28 +273,29 @@ __global__ void __launch_bounds__(kAxisWarps * 32) edt_axis_kernel(const In* __r
   }
   const int* col = s + lane;
   // voxel i's minimum: its place for the next levels, and the voxel's value
-  auto finish = [&](int i, uint32_t key) {
-    nearest[i * 32 + lane] = (uint16_t)(key & 1023u);
+  auto write = [&](int i, uint32_t key) {
     const int q = (int)(key >> 10);
     if (live && col[i * 32] > 0) store_sq(out + (size_t)i * stride, flip, q >= kNoneSq ? kInf : q, voxel, diag);
   };
+  auto finish = [&](int i, uint32_t key) {
+    nearest[i * 32 + lane] = (uint16_t)(key & 1023u);
+    write(i, key);
+  };
   int half = 1;
   while (2 * half <= n) half *= 2;
-  for (; half > 0; half >>= 1) {
+  for (; half > 2; half >>= 1) {
     // voxels half - 1, 3 half - 1, ...; those at +-half are done
     const int nodes = (n - half) / (2 * half) + 1;
     const int parts = nodes >= kAxisWarps ? 1 : kAxisWarps / nodes;
     for (int k = parts > 1 ? warp / parts : warp; k < nodes; k += kAxisWarps) {
       const int i = half - 1 + 2 * half * k;
-      int lo = i - half >= 0 ? nearest[(i - half) * 32 + lane] : 0;
-      int hi = i + half < n ? nearest[(i + half) * 32 + lane] : n - 1;
-      lo = __reduce_min_sync(kFull, lo);
-      hi = __reduce_max_sync(kFull, hi);
+      const int lo = i - half >= 0 ? nearest[(i - half) * 32 + lane] : 0;
+      const int hi = i + half < n ? nearest[(i + half) * 32 + lane] : n - 1;
       if (parts == 1) {
-        finish(i, nearest_key(col, i, lo, hi));
+        finish(i, nearest_key(col, i, lo, hi, n));
       } else {
-        const int len = (hi - lo + parts) / parts, first = lo + (warp % parts) * len;
-        atomicMin(&s_key[k][lane], nearest_key(col, i, first, min(first + len - 1, hi)));
+        const int len = (hi - lo + parts) / parts, first = min(lo + (warp % parts) * len, hi);
+        atomicMin(&s_key[k][lane], nearest_key(col, i, first, min(first + len - 1, hi), n));
       }
     }
     __syncthreads();
@@ -274,6 +307,19 @@ __global__ void __launch_bounds__(kAxisWarps * 32) edt_axis_kernel(const In* __r
       __syncthreads();
     }
   }
+  // The last two levels at once: voxels 4 k, 4 k + 1 and 4 k + 2 between the
+  // places of 4 k - 1 and 4 k + 3.  Three quarters of the voxels share a range
+  // by three and need no place of their own.
+  for (int i = 4 * warp; i < n; i += 4 * kAxisWarps) {
+    const int lo = i > 0 ? nearest[(i - 1) * 32 + lane] : 0;
+    const int hi = i + 3 < n ? nearest[(i + 3) * 32 + lane] : n - 1;
+    uint32_t key[3];
+    nearest_keys(col, i, lo, hi, n, key);
+#pragma unroll
+    for (int v = 0; v < 3; ++v)
+      if (i + v < n) write(i + v, key[v]);
+  }
+  if (abs(count) == n * 32) return;  // no voxel of the other kind
   // the other kind, outwards, four steps to each side at a time
   for (int i = warp; i < n; i += kAxisWarps) {
     int best = live ? -col[i * 32] : -1;
@@ -293,13 +339,14 @@ __global__ void __launch_bounds__(kAxisWarps * 32) edt_axis_kernel(const In* __r
   }
 }
 
-// Whether the pass scans whole lines.  It takes about V n / 2.6e6 us, the
-// search by levels about 9 us + V / 1.1e5 us, so the line is V (n - 24) =
-// 2.3e7.  Measured (us, scan / levels): 64^3 9 / 11, 80^3 17 / 14, 100^3
-// 35 / 20, 256^3 1224 / 143; n = 16 of 200 x 16 x 256 8.5 / 20; n = 256 of
-// 16 x 16 x 256 14 / 22.  Before, with both kinds scanned and two numbers per
-// voxel: 64^3 10, 80^3 20, 100^3 42, 256^3 1540 (y) and 2350 (z).
-bool scan_pays(int n, size_t V) { return n <= 24 || V * (size_t)(n - 24) < 23000000; }
+// Whether the pass scans whole lines.  It takes about V n / 2.4e6 us, the
+// search by levels about 7 us + V / 1.5e5 us, so the line is V (n - 24) =
+// 1.4e7.  Measured (us, scan / levels): 48^3 5 / 9, 64^3 8.7 / 9, 80^3 17 / 11,
+// 100^3 33 / 16, 256^3 1225 / 111; n = 16 of 200 x 16 x 256 9 / 15; n = 256 of
+// 16 x 16 x 256 14 / 14; n = 128 of 16 x 128 x 128 14 / 9.5.  Before, with both
+// kinds scanned and two numbers per voxel: 64^3 10, 80^3 20, 100^3 42, 256^3
+// 1540 (y) and 2350 (z).
+bool scan_pays(int n, size_t V) { return n <= 24 || V * (size_t)(n - 24) < 14000000; }
 
 int grid_for(size_t V) {
   const size_t blocks = (V + 255) / 256;

@@ -43,6 +43,7 @@ def runs(rng, shape, mean, start):
 
 @pytest.mark.parametrize("dims", [
     (31, 33, 40), (64, 64, 64), (65, 66, 67),             # cubes around the rule's line
+    (67, 68, 69), (40, 101, 90), (36, 103, 100),          # ... and every remainder of the levels' last step
     (1024, 5, 7), (3, 1024, 24), (37, 3, 1024),           # the longest line along each axis: scanned
     (2, 1024, 40), (40, 2, 1024),                         # ... and searched by levels
     (130, 131, 25), (129, 24, 120), (33, 250, 96), (2, 2, 2),
