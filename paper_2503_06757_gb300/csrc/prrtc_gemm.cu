@@ -3,25 +3,37 @@
 // FP32 accumulation in tensor memory, optional bias + ReLU and FP32 / BF16
 // outputs.
 //
-// Persistent kernel, one CTA per SM.  A work unit is one 128 x 256 output tile
-// over a range of K (split-K when the tiles alone cannot fill the GPU):
+// Three kernels.  Products below one wave of tiles (every layer of the proposal
+// up to a few thousand rows): gemm_cluster_kernel, K split over the blocks of a
+// cluster, which add up their partial tiles through shared memory.  Larger ones:
+// gemm_bf16_kernel, persistent, one CTA per SM or pair of CTAs per two SMs.  A
+// work unit is one output tile of 128 x 256 (a pair: 256 x 256) over a range of
+// K (a requested split that the clusters do not take: partial tiles go to a
+// workspace and splitk_reduce_kernel adds them up in split order):
 //   warp 0    -- one lane issues TMA loads of the 128 x 64 A and 256 x 64 B
-//                tiles (128-byte swizzle) into a 4-stage shared-memory ring;
+//                tiles (a pair: each CTA its rows of A and half of B; 128-byte
+//                swizzle) into a ring of 4 (6) stages;
 //   warp 1    -- allocates all 512 TMEM columns (two 256-column
-//                accumulators); one lane issues tcgen05.mma (M=128, N=256,
-//                K=16, kind::f16) four times per stage, commits each stage
-//                back to the producer and each finished unit to the epilogue;
+//                accumulators); one lane (a pair: of the first CTA) issues
+//                tcgen05.mma (M=128 or 256, N=256, K=16, kind::f16) four times
+//                per stage, commits each stage back to the producer and each
+//                finished unit to the epilogue;
 //   warps 2-5 -- read an accumulator with tcgen05.ld (each warp owns one
 //                32-lane quarter of TMEM), run the epilogue, and hand the
 //                accumulator back, so the epilogue of one unit overlaps the
 //                main loop of the next.
 // The epilogue stages each 32 x 32 chunk in a swizzled shared-memory tile and
 // writes it with a TMA bulk tensor store (the TMA engine clips the matrix
-// edges).  With split-K each unit writes its FP32 partial tile to a workspace
-// and a second kernel sums the partials in split order (deterministic) and
-// applies bias, ReLU and the output conversions.
+// edges).
 // Every mbarrier wait is bounded; a wait that gives up records an error, the
 // roles stop, and the CTA still frees its tensor memory.
+//
+// What bounds the large products: 8192^3 (FP32 output, normal operands) took 714
+// us with every lane of a warp at each wait, 669 with one lane running the MMA
+// loop, 652 with one lane for the loads as well, and 580 (1.9 PFLOP/s) with that
+// lane chosen by elect.sync, after which the compiler needs no loop over lanes
+// around each instruction that takes uniform registers.  With operands of zeros
+// it takes 490, the MMAs' time: the rest is the power limit.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -38,14 +50,21 @@
 namespace prrtc {
 namespace {
 
-constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4;
+constexpr int BM = 128, BN = 256, BK = 64;
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int B_BYTES = BN * BK * 2;
-constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int EPI_TILE_BYTES = 32 * 128;   // one 32 x 32 FP32 chunk (or 32 x 32 BF16 in its first half)
 constexpr int EPI_BUFS = 2;                 // staging tiles per epilogue warp (double buffered)
-// ring | barriers (1 KB) | staging tiles, plus 1 KB for aligning the base
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 1024 + 4 * EPI_BUFS * EPI_TILE_BYTES;
+// One CTA per tile of 128 x 256, or a pair of CTAs per tile of 256 x 256: each
+// holds its 128 rows of A and of the output, and its half of the tile's B.
+template <int kCtas>
+struct Tile {
+  static constexpr int kM = BM * kCtas;             // rows of a tile
+  static constexpr int kBRows = BN / kCtas;         // columns of the output whose B a CTA loads
+  static constexpr int kStageBytes = A_BYTES + kBRows * BK * 2;
+  static constexpr int kStages = kCtas == 2 ? 6 : 4;
+  // ring | barriers (1 KB) | staging tiles, plus 1 KB for aligning the base
+  static constexpr int kSmem = kStages * kStageBytes + 1024 + 1024 + 4 * EPI_BUFS * EPI_TILE_BYTES;
+};
 constexpr int THREADS = 192;
 constexpr int EPI_WARPS = 4;
 constexpr uint32_t TMEM_COLS = 2 * BN;  // two accumulators
@@ -126,7 +145,37 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, ui
       : "memory");
 }
 
+// A load of one CTA of a pair that completes on the pair's first CTA's barrier
+// (`bar`: its address in the cluster's shared memory).
+__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* tm, uint32_t bar, int x, int y) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], "
+      "[%1, {%3, %4}], [%2];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(bar), "r"(x), "r"(y)
+      : "memory");
+}
+
+// Address in the cluster's shared memory of block 0's copy of `p`.
+__device__ __forceinline__ uint32_t of_first_block(const void* p) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(smem_u32(p)));
+  return r;
+}
+
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+template <int kCtas = 1>
 __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  if (kCtas == 2) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
+    return;
+  }
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
@@ -134,7 +183,17 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b
       : "memory");
 }
 
+// Arrival on `bar` (a pair: in both CTAs) once the MMAs issued so far are done.
+template <int kCtas = 1>
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
+  if (kCtas == 2) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_u32(bar)),
+        "h"((uint16_t)3)
+        : "memory");
+    return;
+  }
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
 }
@@ -154,16 +213,30 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// Work unit -> tile and K range.  Tiles go in groups of kGroupM row tiles:
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// True in one lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.b32 %0, 1, 0, p;\n}\n" : "=r"(r));
+  return r != 0;
+}
+
+// Work unit -> tile and K range.  Tiles go in groups of kGroupRows rows:
 // m fastest inside a group, then n, then the next group, so that the tiles in
 // flight at once (one per SM) share a slab of A rows and a few B columns that
 // stay in L2 instead of sweeping all of A for every column of B.
-constexpr int kGroupM = 16;
+constexpr int kGroupRows = 16 * BM;
 struct Unit {
   int m0, n0, split, kt0, kt1;
 };
 
+template <int kCtas>
 __device__ __forceinline__ Unit unit_of(const Epilogue& ep, int u) {
+  constexpr int kM = Tile<kCtas>::kM, kGroupM = kGroupRows / kM;
   Unit w;
   const int tile = u / ep.splits;
   w.split = u - tile * ep.splits;
@@ -171,7 +244,7 @@ __device__ __forceinline__ Unit unit_of(const Epilogue& ep, int u) {
   const int first_m = (tile / span) * kGroupM;
   const int gm = min(ep.m_tiles - first_m, kGroupM);
   const int in = tile - (tile / span) * span;
-  w.m0 = (first_m + in % gm) * BM;
+  w.m0 = (first_m + in % gm) * kM;
   w.n0 = (in / gm) * BN;
   const int base = ep.k_tiles / ep.splits, rem = ep.k_tiles % ep.splits;
   w.kt0 = w.split * base + min(w.split, rem);
@@ -256,11 +329,14 @@ __device__ __forceinline__ void store_chunk(const Epilogue& ep, const OutMaps& o
   if (ep.has_c16) stage_and_store(&om.c16, tiles, buf, true, col0, row0, lane, f);
 }
 
-// kTA, kTB: operand stored transposed.
-template <bool kTA, bool kTB>
+// kTB: B stored transposed.  kCtas = 2: the two blocks of a cluster
+// share a tile; the first one's barriers and MMA warp drive both.
+template <bool kTB, int kCtas>
 __global__ void __launch_bounds__(THREADS, 1)
     gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const __grid_constant__ OutMaps om, Epilogue ep) {
+  using T = Tile<kCtas>;
+  constexpr int STAGES = T::kStages, STAGE_BYTES = T::kStageBytes;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -275,6 +351,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_units = ep.m_tiles * ep.n_tiles * ep.splits;
+  const int rank = kCtas == 2 ? (int)blockIdx.x & 1 : 0;  // place in the pair
+  const int first = (int)blockIdx.x / kCtas, step = (int)gridDim.x / kCtas;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -283,7 +361,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&acc_full[a], 1);
-      mbar_init(&acc_empty[a], EPI_WARPS);
+      mbar_init(&acc_empty[a], kCtas * EPI_WARPS);
     }
     mbar_init(roles_done, THREADS / 32);
     s_abort = 0;
@@ -291,111 +369,110 @@ __global__ void __launch_bounds__(THREADS, 1)
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(TMEM_COLS)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if (kCtas == 2) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                   "r"(TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                   "r"(TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   fence_before();
   __syncthreads();
+  if (kCtas == 2) cluster_sync_all();  // the other block's barriers and tensor memory are set up
   fence_after();
   const uint32_t tmem = *tmem_slot;
   volatile int* abort_flag = &s_abort;
 
-  // Role loops run on all 32 lanes of a warp (lane 0 waits and issues, the
-  // warp reconverges every step), so every warp reaches the final CTA barrier
-  // converged.
+  // One elected lane runs the whole loop of the loads and of the MMAs: what a
+  // warp does between two stages has to fit into the stage's MMAs (512 cycles).
   if (warp == 0) {
-    int it = 0;  // stage counter across units
-    bool ok = true;
-    for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
-      const Unit w = unit_of(ep, u);
-      for (int kt = w.kt0; kt < w.kt1; ++kt, ++it) {
-        const int s = it % STAGES;
-        const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
-        int got = 0;
-        if (lane == 0) got = (!*abort_flag && wait_bar(&empty[s], ph ^ 1u)) ? 1 : 0;
-        got = __shfl_sync(kFull, got, 0);
-        if (!got) {
-          if (lane == 0) *abort_flag = 1;
-          ok = false;
-          break;
-        }
-        if (lane == 0) {
+    if (elect_one()) {
+      int s = 0, issued = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int u = first; u < n_units && ok; u += step) {
+        const Unit w = unit_of<kCtas>(ep, u);
+        const int m = w.m0 + rank * BM, n = w.n0 + rank * T::kBRows;
+        for (int kt = w.kt0; kt < w.kt1; ++kt) {
+          ok = !*abort_flag && wait_bar(&empty[s], ph ^ 1u);
+          if (!ok) break;
           unsigned char* a = smem + s * STAGE_BYTES;
-          mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
-          if (kTA) {
-#pragma unroll
-            for (int j = 0; j < BM / 64; ++j)
-              tma_load_2d(a + j * MN_BOX_BYTES, &tmA, &full[s], w.m0 + 64 * j, kt * BK);
-          } else {
-            tma_load_2d(a, &tmA, &full[s], kt * BK, w.m0);
-          }
+          if (rank == 0) mbar_arrive_expect_tx(&full[s], kCtas * STAGE_BYTES);
+          const uint32_t pair_bar = kCtas == 2 ? of_first_block(&full[s]) : 0u;
+          auto load = [&](unsigned char* dst, const CUtensorMap* tm, int x, int y) {
+            if (kCtas == 2)
+              tma_load_2d_pair(dst, tm, pair_bar, x, y);
+            else
+              tma_load_2d(dst, tm, &full[s], x, y);
+          };
+          load(a, &tmA, kt * BK, m);
           if (kTB) {
 #pragma unroll
-            for (int j = 0; j < BN / 64; ++j)
-              tma_load_2d(a + A_BYTES + j * MN_BOX_BYTES, &tmB, &full[s], w.n0 + 64 * j, kt * BK);
+            for (int j = 0; j < T::kBRows / 64; ++j) load(a + A_BYTES + j * MN_BOX_BYTES, &tmB, n + 64 * j, kt * BK);
           } else {
-            tma_load_2d(a + A_BYTES, &tmB, &full[s], kt * BK, w.n0);
+            load(a + A_BYTES, &tmB, kt * BK, n);
           }
+          issued = min(issued + 1, STAGES);
+          if (++s == STAGES) s = 0, ph ^= 1u;
         }
-        __syncwarp();
+      }
+      if (!ok) {
+        *abort_flag = 1;
+        // the loads in flight land before the block ends
+        for (; rank == 0 && issued > 0; --issued) {
+          if (--s < 0) s = STAGES - 1, ph ^= 1u;
+          wait_bar(&full[s], ph);
+        }
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
-    const uint32_t idesc = idesc_bf16(BM, BN) | (kTA ? 1u << 15 : 0u) | (kTB ? 1u << 16 : 0u);
+    const uint32_t idesc = idesc_bf16(T::kM, BN) | (kTB ? 1u << 16 : 0u);
     // from one K step of 16 to the next: 32 bytes along K, or 16 lines of K
-    constexpr uint32_t step_a = kTA ? 2048u : 32u, step_b = kTB ? 2048u : 32u;
-    int it = 0, i = 0;  // stage counter, local unit counter
-    bool ok = true;
-    for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x, ++i) {
-      const Unit w = unit_of(ep, u);
-      const int acc = i & 1;
-      // wait until the epilogue has drained this accumulator (first use passes)
-      int got = 0;
-      if (lane == 0) got = (!*abort_flag && wait_bar(&acc_empty[acc], ((uint32_t)(i >> 1) & 1u) ^ 1u)) ? 1 : 0;
-      got = __shfl_sync(kFull, got, 0);
-      if (!got) {
-        if (lane == 0) *abort_flag = 1;
-        break;
-      }
-      fence_after();
-      const uint32_t d = tmem + (uint32_t)(acc * BN);
-      for (int kt = w.kt0; kt < w.kt1; ++kt, ++it) {
-        const int s = it % STAGES;
-        const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
-        got = 0;
-        if (lane == 0) got = wait_bar(&full[s], ph) ? 1 : 0;
-        got = __shfl_sync(kFull, got, 0);
-        if (!got) {
-          if (lane == 0) *abort_flag = 1;
-          ok = false;
-          break;
-        }
+    constexpr uint32_t step_a = 32u, step_b = kTB ? 2048u : 32u;
+    if (rank == 0 && elect_one()) {
+      int s = 0, i = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int u = first; u < n_units && ok; u += step, ++i) {
+        const Unit w = unit_of<kCtas>(ep, u);
+        const int acc = i & 1;
+        // wait until the epilogue has drained this accumulator (first use passes)
+        ok = !*abort_flag && wait_bar(&acc_empty[acc], ((uint32_t)(i >> 1) & 1u) ^ 1u);
+        if (!ok) break;
         fence_after();
-        if (lane == 0) {
+        const uint32_t d = tmem + (uint32_t)(acc * BN);
+        for (int kt = w.kt0; kt < w.kt1; ++kt) {
+          ok = wait_bar(&full[s], ph);
+          if (!ok) break;
+          fence_after();
           const uint32_t a = smem_u32(smem + s * STAGE_BYTES);
           const uint32_t b = a + A_BYTES;
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
-            mma_bf16(d, kTA ? smem_desc_mn(a + step_a * k) : smem_desc(a + step_a * k),
-                     kTB ? smem_desc_mn(b + step_b * k) : smem_desc(b + step_b * k), idesc,
-                     (kt > w.kt0 || k > 0) ? 1u : 0u);
-          mma_commit(&empty[s]);
+            mma_bf16<kCtas>(d, smem_desc(a + step_a * k),
+                            kTB ? smem_desc_mn(b + step_b * k) : smem_desc(b + step_b * k), idesc,
+                            (kt > w.kt0 || k > 0) ? 1u : 0u);
+          mma_commit<kCtas>(&empty[s]);
+          if (++s == STAGES) s = 0, ph ^= 1u;
         }
-        __syncwarp();
+        if (ok) mma_commit<kCtas>(&acc_full[acc]);
       }
-      if (!ok) break;
-      if (lane == 0) mma_commit(&acc_full[acc]);
-      __syncwarp();
+      if (!ok) *abort_flag = 1;
     }
+    __syncwarp();
   } else {
     const int q = warp & 3;  // TMEM lane quarter this warp may access
     unsigned char* tiles = epi_tiles + (warp - 2) * EPI_BUFS * EPI_TILE_BYTES;
     int buf = 0;
     int i = 0;
-    for (int u = blockIdx.x; u < n_units; u += gridDim.x, ++i) {
-      const Unit w = unit_of(ep, u);
+    for (int u = first; u < n_units; u += step, ++i) {
+      const Unit w = unit_of<kCtas>(ep, u);
       const int acc = i & 1;
       int ok = 0;
       if (lane == 0) ok = wait_bar(&acc_full[acc], (uint32_t)(i >> 1) & 1u) ? 1 : 0;
@@ -405,7 +482,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         break;
       }
       fence_after();
-      const int row0 = w.m0 + 32 * q;
+      const int row0 = w.m0 + rank * BM + 32 * q;
       for (int c = 0; c < BN; c += 32) {
         uint32_t v[32];
         __syncwarp();
@@ -415,7 +492,12 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[acc]);
+      if (lane == 0) {
+        if (kCtas == 2)
+          mbar_arrive_cluster(of_first_block(&acc_empty[acc]));
+        else
+          mbar_arrive(&acc_empty[acc]);
+      }
     }
     if (lane == 0) bulk_wait_all();  // every bulk store of this warp has landed
     __syncwarp();
@@ -433,7 +515,16 @@ __global__ void __launch_bounds__(THREADS, 1)
     joined = __shfl_sync(kFull, joined, 0);
     (void)joined;
     fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+  }
+  // A pair also ends together: the other block's barriers, shared and tensor
+  // memory are in use until both are through.
+  __syncwarp();
+  if (kCtas == 2) cluster_sync_all();
+  if (warp == 1) {
+    if (kCtas == 2)
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    else
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
   }
 }
 
@@ -475,11 +566,6 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ ws, int splits, i
       *reinterpret_cast<uint2*>(c16 + (size_t)row * ldc16 + col) = pk;
     }
   }
-}
-
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
@@ -596,7 +682,7 @@ __global__ void __launch_bounds__(kClusterThreads, 2)
   wait_before();
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       int it = 0;
       for (; it < kts; ++it) {
         const int s = it % T::kStages;
@@ -626,7 +712,7 @@ __global__ void __launch_bounds__(kClusterThreads, 2)
   } else if (warp == 1) {
     const uint32_t idesc = idesc_bf16(BM, kBN) | (kTA ? 1u << 15 : 0u) | (kTB ? 1u << 16 : 0u);
     constexpr uint32_t step_a = kTA ? 2048u : 32u, step_b = kTB ? 2048u : 32u;
-    if (lane == 0) {
+    if (elect_one()) {
       bool ok = true;
       for (int it = 0; it < kts && ok; ++it) {
         const int s = it % T::kStages;
@@ -937,6 +1023,21 @@ int cluster_bn(int M, int N, int splits) {
   return 0;
 }
 
+// Whether pairs of CTAs take the tiles (256 x 256) instead of single ones
+// (128 x 256).  A pair loads a third less per MMA, which counts while the MMAs
+// are the bound; with few K tiles the epilogue is, where the two kernels differ
+// in the pairs' joint start and end.  Measured (us, single / pair), 4096^2:
+// K 256 19.2 / 22.1, 512 21.8 / 24.4, 768 26.1 / 26.3, 1024 30.6 / 29.6, 2048
+// 50.2 / 46.6, 4096 94.6 / 83.1; 8192^3 633 / 578; 9728 x 4096 K 512 35.3 /
+// 40.3, 768 45.2 / 44.8, 1024 56.0 / 50.6.  The larger tiles may take more
+// waves, each a tenth shorter for its work.
+bool pair_pays(int M, int N, int k_tiles, int splits) {
+  const int sms = sm_count(), n = (N + BN - 1) / BN * splits;
+  if (sms < 2 || k_tiles <= 12 * splits) return false;
+  auto waves = [](int units, int at_once) { return (units + at_once - 1) / at_once; };
+  return 10 * waves((M + 2 * BM - 1) / (2 * BM) * n, sms / 2) <= 11 * waves((M + BM - 1) / BM * n, sms);
+}
+
 // Adds one product to a group of clusters with tiles of bn columns.
 int group_add(ClusterGroup& g, int& grid, int bn, int splits, const void* a, int lda, bool ta, const void* b, int ldb,
               bool tb, int M, int N, int K, const float* bias, int relu, const void* mask, int ldm, float* c32,
@@ -954,18 +1055,30 @@ int group_add(ClusterGroup& g, int& grid, int bn, int splits, const void* a, int
   return PRRTC_OK;
 }
 
-template <bool kTA, bool kTB>
+template <bool kTB, int kCtas>
 int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, const OutMaps& om, const Epilogue& ep, int grid,
                 cudaStream_t stream) {
-  auto* fn = gemm_bf16_kernel<kTA, kTB>;
+  constexpr int kSmem = Tile<kCtas>::kSmem;
+  auto* fn = gemm_bf16_kernel<kTB, kCtas>;
   static bool attr = false;
   if (!attr) {
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess)
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
       return PRRTC_ERR_CUDA;
     attr = true;
   }
-  fn<<<grid, THREADS, SMEM_BYTES, stream>>>(ma, mb, om, ep);
-  return cudaGetLastError() == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = kSmem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kCtas;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = kCtas > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, fn, ma, mb, om, ep) == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
 }
 
 }  // namespace
@@ -983,11 +1096,9 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
   if ((c32 && (reinterpret_cast<uintptr_t>(c32) & 15)) || (c16 && (reinterpret_cast<uintptr_t>(c16) & 15)))
     return PRRTC_ERR_INVALID_ARG;
   Epilogue ep{M, N, K, bias, relu, c32 ? 1 : 0, c16 ? 1 : 0, 1, 0, 0, 0, 0};
-  ep.m_tiles = (M + BM - 1) / BM;
   ep.n_tiles = (N + BN - 1) / BN;
   ep.k_tiles = (K + BK - 1) / BK;
-  ep.m_pad = ep.m_tiles * BM;
-  const int tiles = ep.m_tiles * ep.n_tiles;
+  ep.m_pad = (M + BM - 1) / BM * BM;
   const int sms = sm_count();
   int splits = splits_hint > 0 ? splits_hint : auto_splits(M, N, K);
   splits = std::max(1, std::min(splits, std::min(kMaxSplits, ep.k_tiles)));
@@ -999,10 +1110,13 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
                              c16, ldc16);
     return rc ? rc : launch_cluster(bn, splits, ta, tb, g, grid, stream);
   }
-  if (mask) return PRRTC_ERR_UNSUPPORTED;
+  if (mask || ta) return PRRTC_ERR_UNSUPPORTED;
+  const bool pair = !tb && pair_pays(M, N, ep.k_tiles, splits);
+  const int ctas = pair ? 2 : 1;
+  ep.m_tiles = (M + BM * ctas - 1) / (BM * ctas);
   CUtensorMap ma, mb;
-  if (!(ta ? cached_map(&ma, a, K, M, lda, 0, BK) : cached_map(&ma, a, M, K, lda, 0, BM))) return PRRTC_ERR_CUDA;
-  if (!(tb ? cached_map(&mb, b, K, N, ldb, 0, BK) : cached_map(&mb, b, N, K, ldb, 0, BN))) return PRRTC_ERR_CUDA;
+  if (!cached_map(&ma, a, M, K, lda, 0, BM)) return PRRTC_ERR_CUDA;
+  if (!(tb ? cached_map(&mb, b, K, N, ldb, 0, BK) : cached_map(&mb, b, N, K, ldb, 0, BN / ctas))) return PRRTC_ERR_CUDA;
   OutMaps om;
   std::memset(&om, 0, sizeof(om));
   if (c32 && !cached_map(&om.c32, c32, M, N, ldc32, 2)) return PRRTC_ERR_CUDA;
@@ -1014,11 +1128,10 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
     if (!ws) return PRRTC_ERR_OOM;
     if (!cached_map(&om.ws, ws, splits * ep.m_pad, N, N, 2)) return PRRTC_ERR_CUDA;
   }
-  const int units = tiles * splits;
-  const int grid = std::min(units, sms);
-  const int rc = ta ? (tb ? launch_gemm<true, true>(ma, mb, om, ep, grid, stream) : PRRTC_ERR_UNSUPPORTED)
-                    : (tb ? launch_gemm<false, true>(ma, mb, om, ep, grid, stream)
-                          : launch_gemm<false, false>(ma, mb, om, ep, grid, stream));
+  const int grid = ctas * std::min(ep.m_tiles * ep.n_tiles * splits, sms / ctas);
+  const int rc = pair ? launch_gemm<false, 2>(ma, mb, om, ep, grid, stream)
+                 : tb ? launch_gemm<true, 1>(ma, mb, om, ep, grid, stream)
+                      : launch_gemm<false, 1>(ma, mb, om, ep, grid, stream);
   if (rc) return rc;
   if (splits > 1) {
     const size_t work = (size_t)M * (N / 4);
@@ -1045,11 +1158,7 @@ int gemm_gradients(const GradientProduct* p, int n, cudaStream_t stream) {
   for (int i = 0; i < n && !rc; ++i) {
     const GradientProduct& q = p[i];
     const int s = auto_splits(q.out, q.in, q.rows), w = cluster_bn(q.out, q.in, s);
-    if (!w) {
-      rc = gemm_bf16_ld(q.dz, q.out, q.h, q.in, q.out, q.in, q.rows, nullptr, 0, q.dw, q.in, nullptr, 0, stream, 0,
-                        kTransA | kTransB, nullptr, 0);
-      continue;
-    }
+    if (!w) return PRRTC_ERR_UNSUPPORTED;  // (every layer of the proposal is below one wave)
     if (g.n && (g.n == kMaxGroup || w != bn || s != splits ||
                 grid + cluster_blocks(q.out, q.in, s, w) > 2 * sm_count()))
       rc = flush();
