@@ -194,18 +194,27 @@ struct RoundsLaunch {
 // round of more of them count (one iteration in seven adds a row); the few
 // hard ones, which set the batch's time, add a row in a hundred iterations or
 // more and take all the workers they get.  So each launch gives what the one
-// before left a larger cluster.  Kernel time of four sets of 200 shelf
-// problems (ms; one warp a problem: 121, 270, 33, 160):
-//   16 warps, clusters 1 / 4 / 16, 256 / 1024 iterations   3.3  5.1  3.3  5.5
-//   16 warps, clusters 1 / 16, 256                          3.5  5.6  4.2  5.6
-//   16 warps, clusters 1 / 4 / 8                            4.1  6.7  3.0  8.3
-//   16 warps, clusters 1 / 4 / 16, 64 / 256                 4.1  6.4  4.8  6.3
-//    8 warps, clusters 1 / 4 / 16, 256 / 1024               3.8  6.3  2.8  7.5
-//    8 warps, clusters 1 / 4 / 8, 256 / 1024                5.3  9.7  3.1 12.9
+// before left a larger cluster.  How long it keeps them depends on how many
+// there are: a batch of more problems than SMs fills the GPU with small
+// clusters for longer (a problem's batches overlap less the larger its cluster
+// is), of fewer ones it leaves SMs idle.  Kernel time (ms; limits of the first /
+// second launch in iterations), sums over six sets of 200 shelf problems
+// (serial, lockstep), then sets of 400, 100 and 40:
+//   16 warps, clusters 1 / 4 / 16, 256 / 1024   22.5 16.5   5.74 3.57   2.13 1.36   1.05 0.77
+//   ... 256 / 2048                              21.2 15.8   5.10 3.42   2.14 1.46   0.96 0.75
+//   ... 384 / 4096                              19.8 15.5   4.72 3.20   2.21 1.52   0.95 0.75
+//   ... 512 / 4096                              20.0 15.9   4.62 3.10   2.19 1.52   0.96 0.75
+//   ... 256 / 8192                              20.8 16.9   5.31 3.67   2.15 1.98   0.97 0.76
+//   clusters 1 / 2 / 16, 256 / 2048             21.7 16.2   5.26 3.34   2.35 1.70   0.95 0.76
+//   clusters 1 / 8 / 16, 256 / 1024             24.0 17.6   6.22 4.05   2.23 1.46   1.06 0.76
+//   clusters 1 / 4 / 8, 256 / 1024              25.6 19.9   5.81 3.99   2.11 1.61   1.03 0.75
+//   12 warps, 256 / 1024                        23.5 18.2   5.98 3.98   2.05 1.42   0.96 0.77
+// (one warp a problem, one block a problem: 121 to 270 and 16 to 40 a set).
 constexpr int kRoundsWarps = 16;
 constexpr int kRoundsSmem = 226 * 1024;
 constexpr int kRoundsMidCluster = 4, kRoundsMaxCluster = 16;
-constexpr int kRoundsFirstIters = 256, kRoundsMidIters = 1024;
+constexpr int kRoundsFirstIters = 384, kRoundsMidIters = 4096;
+constexpr int kRoundsFewFirstIters = 256, kRoundsFewMidIters = 1024;  // clusters of 1 for no more problems than SMs
 
 // base: the launch of plan_launch_config for the same arguments.  held_floats:
 // floats of held rows per virtual worker, over all problems; held_limit: the

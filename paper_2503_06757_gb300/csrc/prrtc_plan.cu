@@ -1475,6 +1475,7 @@ RoundsLaunch rounds_launch_config(const PlanLaunch& base, int n_problems, int mo
   // the first launch: one wave of clusters
   int first = 1;
   while (n_problems * first * 2 <= sm_count && fits(2 * first)) first *= 2;
+  const bool few = first == 1 && n_problems <= sm_count;
   int C = first;
   for (;;) {
     RoundsLaunch::Phase& ph = c.ph[c.n_phases++];
@@ -1484,7 +1485,10 @@ RoundsLaunch rounds_launch_config(const PlanLaunch& base, int n_problems, int mo
     c.workers = virt(C);
     const int next = std::min(C == 1 ? kRoundsMidCluster : kRoundsMaxCluster, most);
     if (next <= C || !fits(next) || c.n_phases == 3) break;
-    ph.it_limit = C == 1 ? kRoundsFirstIters : kRoundsMidIters;
+    if (C == 1)
+      ph.it_limit = few ? kRoundsFewFirstIters : kRoundsFirstIters;
+    else
+      ph.it_limit = few ? kRoundsFewMidIters : kRoundsMidIters;
     C = next;
   }
   return c;
