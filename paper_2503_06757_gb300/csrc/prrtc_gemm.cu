@@ -329,9 +329,9 @@ __device__ __forceinline__ void store_chunk(const Epilogue& ep, const OutMaps& o
   if (ep.has_c16) stage_and_store(&om.c16, tiles, buf, true, col0, row0, lane, f);
 }
 
-// kTB: B stored transposed.  kCtas = 2: the two blocks of a cluster
+// kTA, kTB: operand stored transposed.  kCtas = 2: the two blocks of a cluster
 // share a tile; the first one's barriers and MMA warp drive both.
-template <bool kTB, int kCtas>
+template <bool kTA, bool kTB, int kCtas>
 __global__ void __launch_bounds__(THREADS, 1)
     gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const __grid_constant__ OutMaps om, Epilogue ep) {
@@ -410,7 +410,12 @@ __global__ void __launch_bounds__(THREADS, 1)
             else
               tma_load_2d(dst, tm, &full[s], x, y);
           };
-          load(a, &tmA, kt * BK, m);
+          if (kTA) {
+#pragma unroll
+            for (int j = 0; j < BM / 64; ++j) load(a + j * MN_BOX_BYTES, &tmA, m + 64 * j, kt * BK);
+          } else {
+            load(a, &tmA, kt * BK, m);
+          }
           if (kTB) {
 #pragma unroll
             for (int j = 0; j < T::kBRows / 64; ++j) load(a + A_BYTES + j * MN_BOX_BYTES, &tmB, n + 64 * j, kt * BK);
@@ -432,9 +437,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    const uint32_t idesc = idesc_bf16(T::kM, BN) | (kTB ? 1u << 16 : 0u);
+    const uint32_t idesc = idesc_bf16(T::kM, BN) | (kTA ? 1u << 15 : 0u) | (kTB ? 1u << 16 : 0u);
     // from one K step of 16 to the next: 32 bytes along K, or 16 lines of K
-    constexpr uint32_t step_a = 32u, step_b = kTB ? 2048u : 32u;
+    constexpr uint32_t step_a = kTA ? 2048u : 32u, step_b = kTB ? 2048u : 32u;
     if (rank == 0 && elect_one()) {
       int s = 0, i = 0;
       uint32_t ph = 0;
@@ -455,7 +460,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           const uint32_t b = a + A_BYTES;
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
-            mma_bf16<kCtas>(d, smem_desc(a + step_a * k),
+            mma_bf16<kCtas>(d, kTA ? smem_desc_mn(a + step_a * k) : smem_desc(a + step_a * k),
                             kTB ? smem_desc_mn(b + step_b * k) : smem_desc(b + step_b * k), idesc,
                             (kt > w.kt0 || k > 0) ? 1u : 0u);
           mma_commit<kCtas>(&empty[s]);
@@ -1055,11 +1060,11 @@ int group_add(ClusterGroup& g, int& grid, int bn, int splits, const void* a, int
   return PRRTC_OK;
 }
 
-template <bool kTB, int kCtas>
+template <bool kTA, bool kTB, int kCtas>
 int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, const OutMaps& om, const Epilogue& ep, int grid,
                 cudaStream_t stream) {
   constexpr int kSmem = Tile<kCtas>::kSmem;
-  auto* fn = gemm_bf16_kernel<kTB, kCtas>;
+  auto* fn = gemm_bf16_kernel<kTA, kTB, kCtas>;
   static bool attr = false;
   if (!attr) {
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
@@ -1110,12 +1115,12 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
                              c16, ldc16);
     return rc ? rc : launch_cluster(bn, splits, ta, tb, g, grid, stream);
   }
-  if (mask || ta) return PRRTC_ERR_UNSUPPORTED;
-  const bool pair = !tb && pair_pays(M, N, ep.k_tiles, splits);
+  if (mask || (ta && !tb)) return PRRTC_ERR_UNSUPPORTED;
+  const bool pair = !ta && !tb && pair_pays(M, N, ep.k_tiles, splits);
   const int ctas = pair ? 2 : 1;
   ep.m_tiles = (M + BM * ctas - 1) / (BM * ctas);
   CUtensorMap ma, mb;
-  if (!cached_map(&ma, a, M, K, lda, 0, BM)) return PRRTC_ERR_CUDA;
+  if (!(ta ? cached_map(&ma, a, K, M, lda, 0, BK) : cached_map(&ma, a, M, K, lda, 0, BM))) return PRRTC_ERR_CUDA;
   if (!(tb ? cached_map(&mb, b, K, N, ldb, 0, BK) : cached_map(&mb, b, N, K, ldb, 0, BN / ctas))) return PRRTC_ERR_CUDA;
   OutMaps om;
   std::memset(&om, 0, sizeof(om));
@@ -1129,9 +1134,10 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
     if (!cached_map(&om.ws, ws, splits * ep.m_pad, N, N, 2)) return PRRTC_ERR_CUDA;
   }
   const int grid = ctas * std::min(ep.m_tiles * ep.n_tiles * splits, sms / ctas);
-  const int rc = pair ? launch_gemm<false, 2>(ma, mb, om, ep, grid, stream)
-                 : tb ? launch_gemm<true, 1>(ma, mb, om, ep, grid, stream)
-                      : launch_gemm<false, 1>(ma, mb, om, ep, grid, stream);
+  const int rc = pair       ? launch_gemm<false, false, 2>(ma, mb, om, ep, grid, stream)
+                 : ta && tb ? launch_gemm<true, true, 1>(ma, mb, om, ep, grid, stream)
+                 : tb       ? launch_gemm<false, true, 1>(ma, mb, om, ep, grid, stream)
+                            : launch_gemm<false, false, 1>(ma, mb, om, ep, grid, stream);
   if (rc) return rc;
   if (splits > 1) {
     const size_t work = (size_t)M * (N / 4);
@@ -1158,7 +1164,11 @@ int gemm_gradients(const GradientProduct* p, int n, cudaStream_t stream) {
   for (int i = 0; i < n && !rc; ++i) {
     const GradientProduct& q = p[i];
     const int s = auto_splits(q.out, q.in, q.rows), w = cluster_bn(q.out, q.in, s);
-    if (!w) return PRRTC_ERR_UNSUPPORTED;  // (every layer of the proposal is below one wave)
+    if (!w) {  // from 4096 rows on: more splits than a cluster takes
+      rc = gemm_bf16_ld(q.dz, q.out, q.h, q.in, q.out, q.in, q.rows, nullptr, 0, q.dw, q.in, nullptr, 0, stream, 0,
+                        kTransA | kTransB, nullptr, 0);
+      continue;
+    }
     if (g.n && (g.n == kMaxGroup || w != bn || s != splits ||
                 grid + cluster_blocks(q.out, q.in, s, w) > 2 * sm_count()))
       rc = flush();
