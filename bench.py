@@ -363,8 +363,8 @@ def learned_section(args, P):
     ev_25 = L.evaluate(rb, args.learned_eval_scenes, 1, 9000, prop, ratio=0.25)["learned"]
     return dict(workload="cubby shelf, 7-DoF arm; held-out scenes 9000.. (one problem each), Philox keys 1..3",
                 ratio=0.5, train=train, eval=ev, learned_ratio_0_25=ev_25,
-                note="TTFS includes the on-device inference (occupancy grids, layer 1 per distinct scene, one "
-                     "fused kernel for the rest) that precedes planning"), prop
+                note="TTFS includes the on-device inference (occupancy grids, layer 1 per distinct scene, the "
+                     "rest of the network) that precedes planning"), prop
 
 
 def learned_full_section(P, dofs=(7, 14), paths=50000, steps=20000, eval_scenes=500):

@@ -440,10 +440,11 @@ int prrtc_gemm_bf16(const void* a, const void* b, int32_t M, int32_t N, int32_t 
                     int32_t relu, float* c32, void* c16, void* stream);
 /* As prrtc_gemm_bf16 with the K dimension split into `splits` ranges (0 = the
  * library's choice, which splits while the 128 x 256 output tiles fill less
- * than one wave of SMs).  Each range writes an FP32 partial tile to a
- * library-owned workspace (per device and stream, grown on demand); a second
- * kernel sums the partials in range order, so results do not depend on
- * timing, then applies bias, ReLU and the output conversions. */
+ * than one wave of SMs).  The ranges' FP32 partial tiles are summed in range
+ * order, so results do not depend on timing, then bias, ReLU and the output
+ * conversions are applied.  Up to 8 ranges (a power of two) of a product below
+ * one wave are one launch; others write their partial tiles to a library-owned
+ * workspace (per device and stream, grown on demand) for a second kernel. */
 int prrtc_gemm_bf16_splitk(const void* a, const void* b, int32_t M, int32_t N, int32_t K, const float* bias,
                            int32_t relu, float* c32, void* c16, int32_t splits, void* stream);
 int prrtc_gemm_error(void);
@@ -488,7 +489,7 @@ int prrtc_proposal_forward_layers(prrtc_proposal* proposal, const uint8_t* occ, 
 /* The hidden activations (BF16 widened to FP32, host [B * 1024], [B * 512],
  * [B * 512]; any may be null) of the first B problems of the last inference
  * batch of this proposal (prrtc_proposal_mixtures or prrtc_plan_batch_learned),
- * for element-wise tests of the fused inference kernel.  B larger than that
+ * for element-wise tests of the inference kernels.  B larger than that
  * batch: PRRTC_ERR_INVALID_ARG. */
 int prrtc_proposal_inference_layers(prrtc_proposal* proposal, int32_t B, float* h1, float* h2, float* h3);
 /* Mean mixture negative log-likelihood of target [B * dof] and its gradient

@@ -630,11 +630,13 @@ __device__ void worker(const Ctx& c) {
 // are run again in the next batch.  Results and counters are those of one
 // round at a time: the discarded iterations leave nothing behind.
 //
-// What bounds a round is the latency of one edge check (about 9 us for a warp
-// alone on its SM), and on hard problems hundreds of rounds in a row add
-// nothing (14,160 iterations for 21 rows in one shelf problem).  200 shelf
-// problems: serial 268 -> 5.3 ms a call (one warp a problem before), lockstep
-// with 8 workers 40 -> 4.1 ms (one block a problem, one round at a time).
+// What bounds a round is the latency of an edge check (13k cycles on average
+// with 16 warps on the SM: FK 5.7k, environment 6.3k, self pairs 1k), a batch
+// the slowest of its iterations (23k cycles on average, 47k the batch), and on
+// hard problems hundreds of rounds in a row add nothing (14,160 iterations for
+// 21 rows in one shelf problem).  200 shelf problems: serial 289 -> 4.4 ms a
+// call (one warp a problem before), lockstep with 8 workers 52 -> 3.5 ms (one
+// block a problem, one round at a time).
 //
 // Virtual worker v runs on warp v / C of block v % C of the problem's cluster
 // of C blocks.
