@@ -282,7 +282,10 @@ cudaError_t launch_esdf(const uint8_t* occ, const int dims[3], float voxel, void
 // Launches of a chain of short kernels overlap: a kernel launched with
 // launch_overlapped may start while the kernel before it in the stream still
 // runs; it must call wait_before() ahead of its first access to global memory
-// and may call let_next_start() once its own start-up is over.
+// and may call let_next_start() once its own start-up is over.  A kernel that
+// needs nothing of the one before it (and whose operands that one waited for
+// ahead of its let_next_start()) may call wait_before() at its end instead: the
+// two run side by side, and launches still end in order.
 #ifdef __CUDACC__
 __device__ __forceinline__ void wait_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -391,8 +391,8 @@ __global__ void __launch_bounds__(256) colsum_kernel(const ColSums a) {
   __shared__ __align__(16) float chunk[2][kColChunk][32];
   int l = 0;
   while (l < 3 && (int)blockIdx.x >= a.first_block[l + 1]) ++l;
-  let_next_start();
   wait_before();
+  let_next_start();  // the weight gradients: they read what this launch waited for, and run beside it
   const int cols = a.cols[l], c0 = ((int)blockIdx.x - a.first_block[l]) * 32;
   const float* g = a.g[l] + c0;
   const int chunks = (a.rows + kColChunk - 1) / kColChunk;
@@ -697,14 +697,15 @@ int backward_rows(prrtc_proposal* p, int rows) {
     dz16 = p->z16[l - 1];
     dz32 = p->z32[l - 1];
   }
-  // dW = dZ^T H of every layer, both as stored: nothing waits for them but the update
-  if ((rc = gemm_gradients(dw, 4, s))) return rc;
   int blocks = 0;
   for (int l = 0; l < 4; ++l) {
     cs.first_block[l] = blocks;
     blocks += cs.cols[l] / 32;
   }
-  return launch_overlapped(colsum_kernel, blocks, 256, 0, s, 1, cs) == cudaSuccess ? PRRTC_OK : PRRTC_ERR_CUDA;
+  MCK(launch_overlapped(colsum_kernel, blocks, 256, 0, s, 1, cs));
+  // dW = dZ^T H of every layer, both as stored, beside the bias gradients and
+  // one another: nothing waits for them but the update
+  return gemm_gradients(dw, 4, s);
 }
 
 int upload_samples(prrtc_proposal* p, const uint8_t* occ, int n_occ, const float* qs, const float* qg,
