@@ -124,15 +124,16 @@ __device__ __forceinline__ uint2 bf16x4(float4 f) {
 
 // One feature row per sample (rows past B are zero): occupancy of the
 // sample's scene, then normalised start and goal, each zero-padded to 32.
-// kVox / 16 threads.
+// kVox / 16 threads.  late: runs beside the end of the update of the step
+// before, which waited for the last reader of x (a training step 106 -> 102 us).
 __global__ void features_kernel(const uint8_t* __restrict__ occ, const int* __restrict__ scene_of,
                                 const int* __restrict__ rows, const float* __restrict__ qs,
                                 const float* __restrict__ qg, const float* __restrict__ lo,
-                                const float* __restrict__ span, int B, int dof, bf16* __restrict__ x) {
+                                const float* __restrict__ span, int B, int dof, bf16* __restrict__ x, int late) {
   const int b = blockIdx.x;
   bf16* dst = x + (size_t)b * kIn;
   let_next_start();
-  wait_before();
+  if (!late) wait_before();
   const int r = b < B ? (rows ? rows[b] : b) : 0;
   // 16 voxels a thread: 16 bytes in, 32 bytes out (256 threads, one turn)
   {
@@ -160,6 +161,7 @@ __global__ void features_kernel(const uint8_t* __restrict__ occ, const int* __re
     const float v = (b < B && j < dof) ? 2.f * (q[(size_t)r * dof + j] - lo[j]) / span[j] - 1.f : 0.f;
     dst[kVox + threadIdx.x] = __float2bfloat16_rn(v);
   }
+  if (late) wait_before();
 }
 
 // Occupancy part of the first layer for a few environments, W[:, :4096] x_occ,
@@ -455,16 +457,17 @@ __device__ __forceinline__ float adam_one(float p, float g, float& m, float& v, 
 
 // The update of all parameters and their BF16 copies (what the next step's
 // GEMMs read) in one pass, four parameters a thread.  It moves 30 bytes a
-// parameter (157 MB); 5.2 M parameters take 30 us at 32 training steps in a
-// row, where the update, four conversions, four transposed copies and three
-// tilings took 86 us.
+// parameter (157 MB); 5.2 M parameters take 22 us, where the update, four
+// conversions, four transposed copies and three tilings took 86 us.  One turn a
+// thread: with 608 to 1216 blocks of several turns a training step was 2 - 7%
+// slower.
 __global__ void __launch_bounds__(256) adam_kernel(float4* __restrict__ p, const float4* __restrict__ g,
                                                    float4* __restrict__ m, float4* __restrict__ v,
                                                    uint2* __restrict__ p16, size_t n4, float lr, float b1, float b2,
                                                    float eps, float c1, float c2) {
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  let_next_start();
   wait_before();
+  let_next_start();  // the next step's features, into the SMs that this launch's last blocks leave
+  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (i >= n4) return;
   float4 pi = p[i], mi = m[i], vi = v[i];
   const float4 gi = g[i];
@@ -1051,7 +1054,7 @@ int prrtc_proposal_forward(prrtc_proposal* p, const uint8_t* occ, const float* q
   if ((rc = ensure_scratch(p, rows))) return rc;
   if ((rc = upload_samples(p, occ, B, q_start, q_goal, nullptr, B))) return rc;
   MCK(launch_overlapped(features_kernel, rows, kVox / 16, 0, p->stream, 1, p->occ, nullptr, nullptr, p->qs, p->qg, p->d_lims,
-                        p->d_lims + kMaxDof, B, p->dof, p->x16));
+                        p->d_lims + kMaxDof, B, p->dof, p->x16, 0));
   if ((rc = forward_rows(p, rows))) return rc;
   MCK(cudaMemcpyAsync(out, p->out32, (size_t)B * p->P * 4, cudaMemcpyDeviceToHost, p->stream));
   MCK(cudaStreamSynchronize(p->stream));
@@ -1085,7 +1088,7 @@ int prrtc_proposal_forward_layers(prrtc_proposal* p, const uint8_t* occ, const f
   if ((rc = ensure_scratch(p, rows))) return rc;
   if ((rc = upload_samples(p, occ, B, q_start, q_goal, nullptr, B))) return rc;
   MCK(launch_overlapped(features_kernel, rows, kVox / 16, 0, p->stream, 1, p->occ, nullptr, nullptr, p->qs, p->qg, p->d_lims,
-                        p->d_lims + kMaxDof, B, p->dof, p->x16));
+                        p->d_lims + kMaxDof, B, p->dof, p->x16, 0));
   if ((rc = forward_rows(p, rows))) return rc;
   if ((rc = check_gemm_error())) return rc;
   if ((rc = bf16_rows_to_host(p->x16, B, kIn, kIn, x, p->stream))) return rc;
@@ -1115,12 +1118,12 @@ int prrtc_proposal_inference_layers(prrtc_proposal* p, int32_t B, float* h1, flo
 // prrtc_proposal_get_params), the loss added to *loss_dev and, when lr > 0, an
 // Adam update.
 static int step_on_rows(prrtc_proposal* p, const int* scene_of, const int* rows_dev, int B, float lr,
-                        float* loss_dev) {
+                        float* loss_dev, bool after_update) {
   const int rows = (B + 7) & ~7;
   int rc;
   const cudaStream_t s = p->stream;
   MCK(launch_overlapped(features_kernel, rows, kVox / 16, 0, p->stream, 1, p->occ, scene_of, rows_dev, p->qs, p->qg, p->d_lims,
-                        p->d_lims + kMaxDof, B, p->dof, p->x16));
+                        p->d_lims + kMaxDof, B, p->dof, p->x16, after_update ? 1 : 0));
   if ((rc = forward_rows(p, rows))) return rc;
   MCK(launch_overlapped(mixture_loss_kernel, (rows * 32 + 255) / 256, 256, 0, s, 1, p->out32, p->P, p->tgt, rows_dev,
                         p->d_lims, p->d_lims + kMaxDof, B, rows, p->dof, 1.f / (float)B, p->d32, p->d16, loss_dev));
@@ -1148,7 +1151,7 @@ int prrtc_proposal_grads(prrtc_proposal* p, const uint8_t* occ, const float* q_s
   if ((rc = upload_samples(p, occ, B, q_start, q_goal, target, B))) return rc;
   if ((rc = grow(&p->loss, &p->loss_cap, 1))) return rc;
   MCK(cudaMemsetAsync(p->loss, 0, 4, p->stream));
-  if ((rc = step_on_rows(p, nullptr, nullptr, B, 0.f, p->loss))) return rc;
+  if ((rc = step_on_rows(p, nullptr, nullptr, B, 0.f, p->loss, false))) return rc;
   if (loss) MCK(cudaMemcpyAsync(loss, p->loss, 4, cudaMemcpyDeviceToHost, p->stream));
   MCK(cudaStreamSynchronize(p->stream));
   return check_gemm_error();
@@ -1191,7 +1194,7 @@ int prrtc_proposal_train(prrtc_proposal* p, const uint8_t* occ, int32_t n_scenes
   if ((rc = grow(&p->loss, &p->loss_cap, (size_t)std::max(steps, 1)))) return rc;
   MCK(cudaMemsetAsync(p->loss, 0, (size_t)std::max(steps, 1) * 4, p->stream));
   for (int t = 0; t < steps && !rc; ++t)
-    rc = step_on_rows(p, p->scene_of, p->rows + (size_t)t * B, B, lr, p->loss + t);
+    rc = step_on_rows(p, p->scene_of, p->rows + (size_t)t * B, B, lr, p->loss + t, t > 0);
   if (steps > 0) {  // also after a step that failed: inference follows the masters
     const int rc2 = refresh_inference_weights(p);
     if (!rc) rc = rc2;
