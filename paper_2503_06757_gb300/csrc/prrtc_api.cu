@@ -195,7 +195,11 @@ int grow_device(T** p, size_t* cap, size_t need) {
   *p = nullptr;
   *cap = 0;
   size_t n = std::max<size_t>(need, 1);
-  if (cudaMalloc(p, n * sizeof(T)) != cudaSuccess) return fail(PRRTC_ERR_OOM, "device allocation failed");
+  if (cudaMalloc(p, n * sizeof(T)) != cudaSuccess) {
+    *p = nullptr;
+    cudaGetLastError();  // the caller may go on with less
+    return fail(PRRTC_ERR_OOM, "device allocation failed");
+  }
   *cap = n;
   return PRRTC_OK;
 }
@@ -1189,15 +1193,22 @@ static int plan_batch_impl(const prrtc_problem* problems, int32_t n, const prrtc
   if (cfg.smem > 227 * 1024) return fail(PRRTC_ERR_UNSUPPORTED, "robot + environment exceed shared memory");
   // The deterministic schedules run in rounds.  A serial batch whose held rows
   // would take more than a quarter of the lockstep limit (a tiny range over
-  // many problems) keeps to one warp a problem, which holds no rows.
-  const size_t held_limit = params->mode == PRRTC_MODE_LOCKSTEP ? kHeldFloats : kHeldFloats / 4;
-  const bool rounds =
-      params->mode == PRRTC_MODE_LOCKSTEP || (ordered && held_floats * (size_t)kRoundsWarps <= held_limit);
+  // many problems) keeps to one warp a problem, which holds no rows.  Where the
+  // device has no room for the rows, fewer workers run side by side, down to
+  // one round (lockstep) or none (serial).
+  const bool lockstep = params->mode == PRRTC_MODE_LOCKSTEP;
+  bool rounds = false;
   RoundsLaunch rcfg{};
-  if (rounds) {
+  for (size_t held_limit = lockstep ? kHeldFloats : kHeldFloats / 4;; held_limit /= 2) {
+    rounds = lockstep || (ordered && held_floats * (size_t)kRoundsWarps <= held_limit);
+    if (!rounds) break;
     rcfg = rounds_launch_config(cfg, n, params->mode, blocks, warps, params->workers, held_floats, held_limit, c->sms);
-    if ((rc = grow_device(&c->d_held, &c->held_cap, held_floats * (size_t)rcfg.workers))) return rc;
-    if ((rc = grow_device(&c->d_held_meta, &c->held_meta_cap, (size_t)n * rcfg.workers * kHeldMeta))) return rc;
+    rc = grow_device(&c->d_held, &c->held_cap, held_floats * (size_t)rcfg.workers);
+    if (!rc) rc = grow_device(&c->d_held_meta, &c->held_meta_cap, (size_t)n * rcfg.workers * kHeldMeta);
+    if (!rc) break;
+    if (rc != PRRTC_ERR_OOM || (lockstep && rcfg.workers <= params->workers)) return rc;
+  }
+  if (rounds) {
     size_t off = 0;
     for (int p = 0; p < n; ++p) {
       ProblemDesc& D = c->h_desc[p];

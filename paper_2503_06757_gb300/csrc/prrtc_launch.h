@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <utility>
 
@@ -221,6 +222,53 @@ constexpr int kRoundsFewFirstIters = 256, kRoundsFewMidIters = 1024;  // cluster
 // most that may be allocated.
 RoundsLaunch rounds_launch_config(const PlanLaunch& base, int n_problems, int mode, int blocks, int warps, int workers,
                                   size_t held_floats, size_t held_limit, int sm_count);
+
+// The rule behind rounds_launch_config.  per_sm(warps, smem): resident blocks
+// of that shape; max_cluster(warps, smem): its largest cluster.  The held rows
+// of every launch stay within held_limit: fewer warps where those of a single
+// block would exceed it, down to one round of `workers`, which the caller has
+// checked.
+template <class PerSm, class MaxCluster>
+inline RoundsLaunch rounds_shape(const PlanLaunch& base, int n_problems, int mode, int blocks, int warps, int workers,
+                                 size_t held_floats, size_t held_limit, int sm_count, PerSm per_sm,
+                                 MaxCluster max_cluster) {
+  RoundsLaunch c{};
+  c.robot_bytes = base.robot_bytes;
+  c.env_bytes = base.env_bytes;
+  c.stage_bytes = base.stage_bytes + (int)sizeof(WarpCount);  // a second counter block per warp
+  const bool fixed = mode == PRRTC_MODE_LOCKSTEP && warps > 0;  // the caller's warps per block
+  const int B = mode == PRRTC_MODE_LOCKSTEP ? workers : 1;
+  // virtual workers of a cluster of C blocks, and whether their held rows fit
+  auto virt = [&](int C) { return std::max(C * c.warps / B, 1) * B; };
+  auto held = [&](int C) { return held_floats * (size_t)virt(C); };
+  c.warps = fixed ? base.warps : kRoundsWarps;
+  while (c.warps > 1 && c.robot_bytes + c.env_bytes + c.warps * c.stage_bytes > kRoundsSmem) --c.warps;
+  while (c.warps > B && held(1) > held_limit) --c.warps;
+  c.smem = c.robot_bytes + c.env_bytes + c.warps * c.stage_bytes;
+  const int resident = per_sm(c.warps, c.smem) * sm_count;
+  const int most = (fixed || blocks > 0) ? 1 : max_cluster(c.warps, c.smem);
+  auto fits = [&](int C) { return C <= most && held(C) <= held_limit; };
+  // the first launch: one wave of clusters
+  int first = 1;
+  while (n_problems * first * 2 <= sm_count && fits(2 * first)) first *= 2;
+  const bool few = first == 1 && n_problems <= sm_count;
+  int C = first;
+  for (;;) {
+    RoundsLaunch::Phase& ph = c.ph[c.n_phases++];
+    ph.blocks = C;
+    ph.grid = (blocks > 0 ? blocks : std::min(n_problems, std::max(resident / C, 1))) * C;
+    ph.it_limit = INT_MAX;
+    c.workers = virt(C);
+    const int next = std::min(C == 1 ? kRoundsMidCluster : kRoundsMaxCluster, most);
+    if (next <= C || !fits(next) || c.n_phases == 3) break;
+    if (C == 1)
+      ph.it_limit = few ? kRoundsFewFirstIters : kRoundsFirstIters;
+    else
+      ph.it_limit = few ? kRoundsFewMidIters : kRoundsMidIters;
+    C = next;
+  }
+  return c;
+}
 
 // workers: the lockstep round size (PRRTC_MODE_LOCKSTEP), else ignored.
 PlanLaunch plan_launch_config(int n_problems, int mode, int blocks, int warps, int max_spheres, int max_pairs,

@@ -1460,40 +1460,9 @@ PlanLaunch plan_launch_config(int n_problems, int mode, int blocks, int warps, i
 
 RoundsLaunch rounds_launch_config(const PlanLaunch& base, int n_problems, int mode, int blocks, int warps, int workers,
                                   size_t held_floats, size_t held_limit, int sm_count) {
-  RoundsLaunch c{};
-  c.robot_bytes = base.robot_bytes;
-  c.env_bytes = base.env_bytes;
-  c.stage_bytes = base.stage_bytes + (int)sizeof(WarpCount);  // a second counter block per warp
-  const bool fixed = mode == PRRTC_MODE_LOCKSTEP && warps > 0;  // the caller's warps per block
-  c.warps = fixed ? base.warps : kRoundsWarps;
-  while (c.warps > 1 && c.robot_bytes + c.env_bytes + c.warps * c.stage_bytes > kRoundsSmem) --c.warps;
-  c.smem = c.robot_bytes + c.env_bytes + c.warps * c.stage_bytes;
-  const int resident = resident_blocks_per_sm(kRounds, c.warps, c.smem) * sm_count;
-  const int B = mode == PRRTC_MODE_LOCKSTEP ? workers : 1;
-  // virtual workers of a cluster of C blocks, and whether their held rows fit
-  auto virt = [&](int C) { return std::max(C * c.warps / B, 1) * B; };
-  const int most = (fixed || blocks > 0) ? 1 : rounds_max_cluster(c.warps, c.smem);
-  auto fits = [&](int C) { return C <= most && held_floats * (size_t)virt(C) <= held_limit; };
-  // the first launch: one wave of clusters
-  int first = 1;
-  while (n_problems * first * 2 <= sm_count && fits(2 * first)) first *= 2;
-  const bool few = first == 1 && n_problems <= sm_count;
-  int C = first;
-  for (;;) {
-    RoundsLaunch::Phase& ph = c.ph[c.n_phases++];
-    ph.blocks = C;
-    ph.grid = (blocks > 0 ? blocks : std::min(n_problems, std::max(resident / C, 1))) * C;
-    ph.it_limit = INT_MAX;
-    c.workers = virt(C);
-    const int next = std::min(C == 1 ? kRoundsMidCluster : kRoundsMaxCluster, most);
-    if (next <= C || !fits(next) || c.n_phases == 3) break;
-    if (C == 1)
-      ph.it_limit = few ? kRoundsFewFirstIters : kRoundsFirstIters;
-    else
-      ph.it_limit = few ? kRoundsFewMidIters : kRoundsMidIters;
-    C = next;
-  }
-  return c;
+  return rounds_shape(
+      base, n_problems, mode, blocks, warps, workers, held_floats, held_limit, sm_count,
+      [](int w, int smem) { return resident_blocks_per_sm(kRounds, w, smem); }, rounds_max_cluster);
 }
 
 cudaError_t launch_plan(const PlanGlobals* g, const ProblemDesc* desc, ProblemState* state, const PlanLaunch& cfg,
