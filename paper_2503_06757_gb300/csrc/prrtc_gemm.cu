@@ -963,16 +963,22 @@ float* workspace(size_t floats, cudaStream_t stream) {
 
 namespace {
 
+// Dynamic shared memory of a kernel on the current device, set once (`done`).
+template <class Fn>
+cudaError_t smem_attribute(std::atomic<uint64_t>& done, Fn* fn, int bytes) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return once_per_device(
+      done, dev, [&] { return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
+}
+
 template <int kBN, int kSplits, bool kTA, bool kTB>
 int launch_cluster_as(const ClusterGroup& group, int grid, cudaStream_t stream) {
   using T = ClusterTile<kBN>;
   auto* fn = gemm_cluster_kernel<kBN, kSplits, kTA, kTB>;
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, T::kSmem) != cudaSuccess)
-      return PRRTC_ERR_CUDA;
-    attr = true;
-  }
+  static std::atomic<uint64_t> attr{0};
+  if (smem_attribute(attr, fn, T::kSmem) != cudaSuccess) return PRRTC_ERR_CUDA;
   return launch_overlapped(fn, grid, kClusterThreads, T::kSmem, stream, kSplits, group) == cudaSuccess
              ? PRRTC_OK
              : PRRTC_ERR_CUDA;
@@ -1001,14 +1007,16 @@ int launch_cluster(int bn, int splits, bool ta, bool tb, const ClusterGroup& gro
                   : launch_cluster_bn<128>(splits, ta, tb, group, grid, stream);
 }
 
+// SMs of the current device.
 int sm_count() {
-  static const int sms = [] {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    return n > 0 ? n : 1;
-  }();
-  return sms;
+  static std::atomic<int> known[64];
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  const bool keep = dev >= 0 && dev < 64;
+  if (keep && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) return 1;
+  if (keep) known[dev].store(n, std::memory_order_relaxed);
+  return n;
 }
 
 // The library's split of K: doubled while the 128 x 256 tiles fill less than
@@ -1071,12 +1079,8 @@ int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, const OutMaps& om,
                 cudaStream_t stream) {
   constexpr int kSmem = Tile<kCtas>::kSmem;
   auto* fn = gemm_bf16_kernel<kTA, kTB, kCtas>;
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
-      return PRRTC_ERR_CUDA;
-    attr = true;
-  }
+  static std::atomic<uint64_t> attr{0};
+  if (smem_attribute(attr, fn, kSmem) != cudaSuccess) return PRRTC_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(THREADS);

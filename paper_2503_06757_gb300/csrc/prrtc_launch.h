@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <cmath>
 #include <utility>
@@ -326,6 +327,19 @@ cudaError_t launch_voxelize(const EnvView& env, const float origin[3], float vox
                             cudaStream_t stream);
 cudaError_t launch_esdf(const uint8_t* occ, const int dims[3], float voxel, void* tmp, float* out,
                         cudaStream_t stream);
+
+// Runs set(), a kernel attribute of the current device `dev`, unless it has
+// succeeded there before (`done`: one bit per device, one word per kernel).  An
+// attribute belongs to a device: a process may use several, from several
+// threads.
+template <class F>
+inline cudaError_t once_per_device(std::atomic<uint64_t>& done, int dev, F set) {
+  const bool known = dev >= 0 && dev < 64;
+  if (known && (done.load(std::memory_order_acquire) >> dev & 1u)) return cudaSuccess;
+  const cudaError_t e = set();
+  if (e == cudaSuccess && known) done.fetch_or((uint64_t)1 << dev, std::memory_order_release);
+  return e;
+}
 
 // Launches of a chain of short kernels overlap: a kernel launched with
 // launch_overlapped may start while the kernel before it in the stream still
