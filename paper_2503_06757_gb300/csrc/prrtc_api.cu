@@ -1,6 +1,8 @@
 // prrtc_api.cu -- host runtime of libprrtc: handles, device arenas, launch
 // sequencing and the extern "C" entry points declared in include/prrtc.h.
 #include <algorithm>
+#include <array>
+#include <cfloat>
 #include <climits>
 #include <cmath>
 #include <cstdio>
@@ -41,7 +43,8 @@ struct prrtc_env {
   std::mutex mu;            // guards h_data against concurrent updates and snapshots
   int device = -1;
   float4* d_data = nullptr;
-  std::vector<float4> h_data;
+  std::vector<float4> h_data;  // primitives, then the corners of the box around them (kEnvBox)
+  std::vector<std::array<float, 6>> bounds;  // per obstacle id: lower and upper corner
   int n_aabb = 0, n_obb = 0, n_cyl = 0, n_sph = 0;
   std::vector<int> kind;    // per obstacle id: 0 aabb, 1 obb, 2 cylinder, 3 sphere
   std::vector<int> offset;  // per obstacle id: first float4 in the blob
@@ -410,6 +413,22 @@ static int pack_obstacle(const prrtc_obstacle& o, int* kind, float4* out) {
   return -1;
 }
 
+// The corners of the box around all obstacles, in the last words of the host
+// blob; true when they changed.
+static bool refresh_env_box(prrtc_env* e) {
+  float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
+  for (const auto& b : e->bounds)
+    for (int a = 0; a < 3; ++a) {
+      lo[a] = std::min(lo[a], b[a]);
+      hi[a] = std::max(hi[a], b[3 + a]);
+    }
+  const float4 box[kEnvBox] = {make_float4(lo[0], lo[1], lo[2], 0.f), make_float4(hi[0], hi[1], hi[2], 0.f)};
+  float4* at = e->h_data.data() + e->h_data.size() - kEnvBox;
+  if (!std::memcmp(at, box, sizeof(box))) return false;
+  std::memcpy(at, box, sizeof(box));
+  return true;
+}
+
 int prrtc_env_create(const prrtc_obstacle* obstacles, int32_t n, prrtc_env** out) {
   if (!out) return fail(PRRTC_ERR_INVALID_ARG, "out is null");
   *out = nullptr;
@@ -441,9 +460,10 @@ int prrtc_env_create(const prrtc_obstacle* obstacles, int32_t n, prrtc_env** out
   base[0] = 0;
   for (int k = 1; k < 4; ++k) base[k] = base[k - 1] + cnt[k - 1] * width[k - 1];
   const int total = base[3] + cnt[3] * width[3];
-  e->h_data.assign(std::max(total, 1), make_float4(0.f, 0.f, 0.f, 0.f));
+  e->h_data.assign(total + kEnvBox, make_float4(0.f, 0.f, 0.f, 0.f));
   e->kind.resize(n);
   e->offset.resize(n);
+  e->bounds.resize(n);
   int fill[4] = {0, 0, 0, 0};
   for (int i = 0; i < n; ++i) {
     const int k = kinds[i];
@@ -452,7 +472,9 @@ int prrtc_env_create(const prrtc_obstacle* obstacles, int32_t n, prrtc_env** out
     e->kind[i] = k;
     e->offset[i] = off;
     std::copy(packed[i].begin(), packed[i].end(), e->h_data.begin() + off);
+    obstacle_bounds(k, packed[i].data(), e->bounds[i].data(), e->bounds[i].data() + 3);
   }
+  refresh_env_box(e);
   if (cudaMalloc(&e->d_data, e->h_data.size() * sizeof(float4)) != cudaSuccess) {
     cudaGetLastError();
     delete e;
@@ -476,19 +498,27 @@ int prrtc_env_update(prrtc_env* env, const int32_t* ids, const prrtc_obstacle* o
   if (c->device != env->device) return fail(PRRTC_ERR_INVALID_ARG, "env belongs to another device");
   std::lock_guard<std::mutex> lk(c->mu);
   std::lock_guard<std::mutex> lk_env(env->mu);
-  int lo = INT_MAX, hi = -1;
+  // all of them are looked at before the first is taken: the host blob and its
+  // box go on describing what the device holds
+  std::vector<std::array<float4, 5>> packed(n);
   for (int k = 0; k < n; ++k) {
     const int id = ids[k];
     if (id < 0 || id >= (int)env->kind.size()) return fail(PRRTC_ERR_INVALID_ARG, "obstacle id out of range");
-    float4 tmp[5];
     int kind = 0;
-    const int m = pack_obstacle(obstacles[k], &kind, tmp);
-    if (m < 0 || kind != env->kind[id]) return fail(PRRTC_ERR_INVALID_ARG, "update changes an obstacle's kind");
-    std::copy(tmp, tmp + m, env->h_data.begin() + env->offset[id]);
+    if (pack_obstacle(obstacles[k], &kind, packed[k].data()) < 0 || kind != env->kind[id])
+      return fail(PRRTC_ERR_INVALID_ARG, "update changes an obstacle's kind");
+  }
+  static const int width[4] = {2, 5, 2, 1};  // words of a kind
+  int lo = INT_MAX, hi = -1;
+  for (int k = 0; k < n; ++k) {
+    const int id = ids[k], kind = env->kind[id];
+    std::copy_n(packed[k].begin(), width[kind], env->h_data.begin() + env->offset[id]);
+    obstacle_bounds(kind, packed[k].data(), env->bounds[id].data(), env->bounds[id].data() + 3);
     lo = std::min(lo, env->offset[id]);
-    hi = std::max(hi, env->offset[id] + m);
+    hi = std::max(hi, env->offset[id] + width[kind]);
   }
   if (hi < 0) return PRRTC_OK;
+  if (refresh_env_box(env)) hi = (int)env->h_data.size();  // in the same copy
   // Stream-ordered upload: lands between the planning launches around it.
   CK(cudaMemcpyAsync(env->d_data + lo, env->h_data.data() + lo, (size_t)(hi - lo) * sizeof(float4),
                      cudaMemcpyHostToDevice, c->stream));

@@ -21,11 +21,11 @@ constexpr int kMaxCheckWarps = 16;
 // Lanes that make a link pair's tests pay at once instead of through the queue.
 constexpr int kDirect = 24;
 
-// Robot header, pair tables and environment into shared memory by bulk copies
-// (one thread); 0 when they did not complete within the bounded wait.
+// Robot header, pair tables and the first env_f4 words of the environment into
+// shared memory by bulk copies (one thread); 0 when they did not complete within
+// the bounded wait.
 __device__ int stage_tables(const RobotDev* robot, const EnvView& env, RobotHeader* R, uint32_t* pair, float* thr,
-                            float4* senv, int np_pad, uint64_t* bar, int* error) {
-  const int env_f4 = env.n_float4();
+                            float4* senv, int env_f4, int np_pad, uint64_t* bar, int* error) {
   mbar_init(bar, 1);
   mbar_arrive_expect_tx(bar, (uint32_t)sizeof(RobotHeader) + 8u * (uint32_t)np_pad + 16u * (uint32_t)env_f4);
   bulk_g2s(R, &robot->h, sizeof(RobotHeader), bar);
@@ -179,50 +179,6 @@ __device__ __forceinline__ bool block_hits(const RobotHeader* __restrict__ R, co
   return hit;
 }
 
-// Lower and upper corner of a box around every primitive, enlarged by 1e-4 m
-// and 1e-5 of the coordinates; by all threads of the block.  keys: 6 words.
-__device__ void env_box(const float4* __restrict__ env, const EnvView& v, uint32_t* keys, float3& lo, float3& hi) {
-  if (threadIdx.x < 6) keys[threadIdx.x] = threadIdx.x < 3 ? 0xffffffffu : 0u;
-  __syncthreads();
-  const int total = v.n_aabb + v.n_obb + v.n_cyl + v.n_sph;
-  for (int o = threadIdx.x; o < total; o += blockDim.x) {
-    const float4* e = env;
-    float4 c;
-    float3 h;
-    int k = o;
-    if (k < v.n_aabb) {
-      c = e[2 * k];
-      h = make_float3(e[2 * k + 1].x, e[2 * k + 1].y, e[2 * k + 1].z);
-    } else if ((k -= v.n_aabb) < v.n_obb) {
-      e += 2 * v.n_aabb + 5 * k;
-      c = e[0];
-      const float4 s = e[1];  // world half extents: sum over the box's axes (rows of R^T)
-      h = make_float3(fabsf(e[2].x) * s.x + fabsf(e[3].x) * s.y + fabsf(e[4].x) * s.z,
-                      fabsf(e[2].y) * s.x + fabsf(e[3].y) * s.y + fabsf(e[4].y) * s.z,
-                      fabsf(e[2].z) * s.x + fabsf(e[3].z) * s.y + fabsf(e[4].z) * s.z);
-    } else if ((k -= v.n_obb) < v.n_cyl) {
-      e += 2 * v.n_aabb + 5 * v.n_obb + 2 * k;
-      c = e[0];
-      const float r = c.w + e[1].w * 1.01f;  // axes are unit length within 1e-3
-      h = make_float3(r, r, r);
-    } else {
-      k -= v.n_cyl;
-      c = e[2 * v.n_aabb + 5 * v.n_obb + 2 * v.n_cyl + k];
-      h = make_float3(c.w, c.w, c.w);
-    }
-    const float cs[3] = {c.x, c.y, c.z}, hs[3] = {h.x, h.y, h.z};
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const float m = hs[a] + 1e-4f + 1e-5f * (fabsf(cs[a]) + hs[a]);
-      atomicMin(&keys[a], f2key(cs[a] - m));
-      atomicMax(&keys[3 + a], f2key(cs[a] + m));
-    }
-  }
-  __syncthreads();
-  lo = make_float3(key2f(keys[0]), key2f(keys[1]), key2f(keys[2]));
-  hi = make_float3(key2f(keys[3]), key2f(keys[4]), key2f(keys[5]));
-}
-
 // Verdicts of given configurations.  A lane places the spheres of one state
 // and stages them.  Then the links that come near the box around the obstacles
 // queue up, distal ones first; every 32 of them meet the primitives with their
@@ -249,7 +205,6 @@ __global__ void __launch_bounds__(kMaxCheckWarps * 32) check_states_kernel(
   __shared__ int s_ok;
   __shared__ WarpCount s_count[kMaxCheckWarps];
   __shared__ int16_t s_raw[PRRTC_MAX_SPHERES];
-  __shared__ uint32_t s_box[6];
   __shared__ uint32_t s_hit[kMaxCheckWarps];  // states of the warp known to collide
   __shared__ int16_t s_bslot[kMaxDof];        // stage slot of the link's bounding sphere (its only sphere's own)
   RobotHeader* R = reinterpret_cast<RobotHeader*>(smem);
@@ -257,9 +212,10 @@ __global__ void __launch_bounds__(kMaxCheckWarps * 32) check_states_kernel(
   float* thr = reinterpret_cast<float*>(pair + np_pad);
   const int env_f4 = env.n_float4();
   float4* senv = reinterpret_cast<float4*>(thr + np_pad);
-  float* warp_all = reinterpret_cast<float*>(senv + env_f4);
+  const int box_f4 = env_f4 ? kEnvBox : 0;  // corners of the box around the obstacles
+  float* warp_all = reinterpret_cast<float*>(senv + env_f4 + kEnvBox);
 
-  if (threadIdx.x == 0) s_ok = stage_tables(robot, env, R, pair, thr, senv, np_pad, &bar, error);
+  if (threadIdx.x == 0) s_ok = stage_tables(robot, env, R, pair, thr, senv, env_f4 + box_f4, np_pad, &bar, error);
   if (spheres)
     for (int r = threadIdx.x; r < PRRTC_MAX_SPHERES; r += blockDim.x) s_raw[r] = robot->raw_to_distinct[r];
   __syncthreads();
@@ -270,11 +226,12 @@ __global__ void __launch_bounds__(kMaxCheckWarps * 32) check_states_kernel(
   const uint32_t below = (1u << lane) - 1u;
   float* qst = warp_all + warp * warp_floats;  // [joint][lane], then the queues
   float* stage = qst + q_floats;               // [sphere, then link][x, y, z][lane]
-  float3 box_lo, box_hi;
-  env_box(senv, env, s_box, box_lo, box_hi);
-  if (threadIdx.x == 0) {
-    int slot = R->n_spheres;
-    for (int i = 0; i < dof; ++i) s_bslot[i] = (int16_t)(R->coarse[i].w > 0.f ? slot++ : R->sph_begin[i]);
+  float4 box_lo, box_hi;
+  if (env_f4) box_lo = senv[env_f4], box_hi = senv[env_f4 + 1];
+  if (warp == 0) {
+    const uint32_t bounds = __ballot_sync(kFull, lane < dof && R->coarse[lane].w > 0.f);
+    if (lane < dof)
+      s_bslot[lane] = (int16_t)((bounds >> lane & 1u) ? R->n_spheres + __popc(bounds & below) : R->sph_begin[lane]);
   }
   __syncthreads();
   const int gw = blockIdx.x * warps + warp;
@@ -332,7 +289,7 @@ __global__ void __launch_bounds__(kMaxCheckWarps * 32) check_states_kernel(
       for (int i = dof - 1; i >= 0; --i) {
         if (R->sph_begin[i] != R->sph_begin[i + 1]) {
           const float* st = stage + s_bslot[i] * 96 + lane;
-          const float r = R->grp[i].w;
+          const float r = R->grp[i].w * kReachSlack;
           const float dx = fmaxf(fmaxf(box_lo.x - st[0], st[0] - box_hi.x), 0.f);
           const float dy = fmaxf(fmaxf(box_lo.y - st[32], st[32] - box_hi.y), 0.f);
           const float dz = fmaxf(fmaxf(box_lo.z - st[64], st[64] - box_hi.z), 0.f);
@@ -501,7 +458,7 @@ __global__ void __launch_bounds__(kStateWarps * 32) check_state_warps_kernel(
   const int idx = blockIdx.x * kStateWarps + warp;
   // on its way while the tables are staged (it may come from host memory)
   const float ql = idx < n && lane < dof ? q[(size_t)idx * dof + lane] : 0.f;
-  if (threadIdx.x == 0) s_ok = stage_tables(robot, env, R, pair, thr, senv, np_pad, &bar, error);
+  if (threadIdx.x == 0) s_ok = stage_tables(robot, env, R, pair, thr, senv, env_f4, np_pad, &bar, error);
   __syncthreads();
   if (!s_ok || idx >= n) return;  // nothing below waits for another warp
   const int n_raw = R->n_raw, n_pairs = R->n_pairs;
@@ -593,7 +550,7 @@ CheckShape check_shape(const RobotHeader& h, const EnvView& env) {
   s.np_pad = (h.n_pairs + 3) & ~3;
   int bounds = 0;
   for (int f = 0; f < h.dof; ++f) bounds += h.coarse[f].w > 0.f ? 1 : 0;
-  s.table_bytes = (int)sizeof(RobotHeader) + 8 * s.np_pad + env.n_float4() * 16;
+  s.table_bytes = (int)sizeof(RobotHeader) + 8 * s.np_pad + (env.n_float4() + kEnvBox) * 16;
   s.q_floats = std::max(h.dof * 32, (int)sizeof(CheckQueues) / 4);
   s.warp_floats = s.q_floats + (h.n_spheres + bounds) * 96;
   return s;

@@ -88,7 +88,10 @@ struct EsdfGrid {
 // Environment: one float4 array laid out as
 //   [AABB x2: centre|0, half|0][OBB x5: centre, half, R^T rows][CYL x2:
 //   centre|radius, axis|half_len][SPH x1: centre|radius],
-// plus an optional distance field (read from global memory / L2).
+// plus an optional distance field (read from global memory / L2).  Behind the
+// primitives an environment handle's own blob holds kEnvBox words more: the
+// corners of a box around them all, for the check kernel.
+constexpr int kEnvBox = 2;
 struct EnvView {
   const float4* data;
   int n_aabb, n_obb, n_cyl, n_sph;

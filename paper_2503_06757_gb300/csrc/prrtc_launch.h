@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cfloat>
 #include <climits>
 #include <cmath>
 #include <utility>
@@ -144,11 +145,75 @@ inline int reported_iterations(const ProblemState& S, const prrtc_params& p) {
   return (int)(n < p.max_iters ? n : p.max_iters);
 }
 
+// The check kernel lets a link skip the obstacles when its bounding sphere, its
+// radius times kReachSlack, stays clear of a box around all of them.
+constexpr float kReachSlack = 1.0012f;
+
+// Box (lo, hi) that every sphere touching the obstacle (packed as in EnvView,
+// kind 0..3) reaches with its radius times kReachSlack.  The kernels test a box
+// in the coordinates A v of its rows as they were given: the box reaches as far
+// as the rows of A^-1 say, and a sphere's radius grows by at most |A^-1|.  Rows
+// that are not close to orthonormal (|A^-1| above 1.001, or a row longer than
+// 1.1) get an unbounded box.  Cylinder axes may be off unit length by 1e-3.  The
+// margin covers the kernels' own roundings.
+inline void obstacle_bounds(int kind, const float4* e, float lo[3], float hi[3]) {
+  const double c[3] = {e[0].x, e[0].y, e[0].z};
+  double ext[3];
+  if (kind == 0) {
+    ext[0] = e[1].x; ext[1] = e[1].y; ext[2] = e[1].z;
+  } else if (kind == 1) {
+    double A[3][3], cross[3][3], longest = 0.0;
+    for (int j = 0; j < 3; ++j) {
+      A[j][0] = e[2 + j].x; A[j][1] = e[2 + j].y; A[j][2] = e[2 + j].z;
+      longest = std::max(longest, std::sqrt(A[j][0] * A[j][0] + A[j][1] * A[j][1] + A[j][2] * A[j][2]));
+    }
+    for (int j = 0; j < 3; ++j) {  // column j of A^-1 times the determinant
+      const double* u = A[(j + 1) % 3];
+      const double* w = A[(j + 2) % 3];
+      for (int a = 0; a < 3; ++a) cross[j][a] = u[(a + 1) % 3] * w[(a + 2) % 3] - u[(a + 2) % 3] * w[(a + 1) % 3];
+    }
+    const double det = A[0][0] * cross[0][0] + A[0][1] * cross[0][1] + A[0][2] * cross[0][2];
+    const double h[3] = {e[1].x, e[1].y, e[1].z};
+    double inv[3][3];
+    for (int a = 0; a < 3; ++a) {
+      ext[a] = 0.0;
+      for (int j = 0; j < 3; ++j) {
+        inv[a][j] = cross[j][a] / det;
+        ext[a] += std::fabs(inv[a][j]) * h[j];
+      }
+    }
+    bool bounded = longest < 1.1;
+    for (int a = 0; a < 3; ++a) {  // |A^-1|^2 is at most the largest row sum of A^-1 A^-T
+      double sum = 0.0;
+      for (int b = 0; b < 3; ++b)
+        sum += std::fabs(inv[a][0] * inv[b][0] + inv[a][1] * inv[b][1] + inv[a][2] * inv[b][2]);
+      bounded = bounded && sum < 1.002;
+    }
+    if (!bounded) ext[0] = ext[1] = ext[2] = INFINITY;
+  } else if (kind == 2) {
+    const double ax[3] = {e[1].x, e[1].y, e[1].z};
+    const double len = std::sqrt(ax[0] * ax[0] + ax[1] * ax[1] + ax[2] * ax[2]);
+    for (int a = 0; a < 3; ++a) {
+      const double u = std::fabs(ax[a]) / len;
+      ext[a] = (double)e[0].w * std::sqrt(std::max(0.0, 1.0 - u * u)) + (double)e[1].w / len * u;
+    }
+  } else {
+    ext[0] = ext[1] = ext[2] = e[0].w;
+  }
+  for (int a = 0; a < 3; ++a) {
+    const double m = ext[a] + 1e-4 + 1e-5 * (std::fabs(c[a]) + ext[a]);
+    lo[a] = (float)std::max(c[a] - m, -(double)FLT_MAX);
+    hi[a] = (float)std::min(c[a] + m, (double)FLT_MAX);
+  }
+}
+
 // Launchers (return cudaError_t of the launch).
 // slots (nullable): a warp per state whatever n, and its counters (sphere
 // passes, pair tests, the four second-stage counts, as 32-bit words) at
 // slots[2 * state] instead of summed into counters[7].  All pointers may be
 // pinned host memory.
+// env.data holds two float4 more than its primitives: the lower and the upper
+// corner of the box around all of them (obstacle_bounds).
 cudaError_t launch_check_states(const RobotDev* robot, const RobotHeader& host_header, EnvView env, const float* q,
                                 int n, uint8_t* valid, float* spheres, unsigned long long* counters, uint4* slots,
                                 int* error, cudaStream_t stream);
