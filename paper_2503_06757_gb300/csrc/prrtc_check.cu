@@ -263,7 +263,8 @@ __global__ void __maxnreg__(128) check_states_kernel(
     Frame T;
 #pragma unroll 1
     for (int i = 0; i < dof; ++i) {
-      fk_joint<false>(R, i, qst[i * 32 + lane], T);
+      const float qi = qst[i * 32 + lane];
+      fk_joint(R, i, qi, [qi](float& sn, float& cs) { joint_sincos<false>(qi, sn, cs); }, T);
       const int s0 = R->sph_begin[i], s1 = R->sph_begin[i + 1];
       if (R->coarse[i].w > 0.f) {
         const float3 c = T.at(R->coarse[i]);
@@ -475,7 +476,8 @@ __global__ void __launch_bounds__(kStateWarps * 32) check_state_warps_kernel(
   if (lane < dof && revolute(R->jtype[lane])) joint_sincos<false>(ql, sl, cl);
   Frame T;
   for (int i = 0; i < dof; ++i) {
-    fk_apply(R, i, R->jtype[i], __shfl_sync(kFull, ql, i), __shfl_sync(kFull, sl, i), __shfl_sync(kFull, cl, i), T);
+    const float qi = __shfl_sync(kFull, ql, i), si = __shfl_sync(kFull, sl, i), ci = __shfl_sync(kFull, cl, i);
+    fk_joint(R, i, qi, [si, ci](float& sn, float& cs) { sn = si, cs = ci; }, T);
     const int s0 = R->sph_begin[i], cnt = R->sph_begin[i + 1] - s0;
     for (int k = lane; k <= cnt; k += 32) {  // one more: the link's bounding sphere, or its only one
       const float3 c = T.at(k < cnt ? R->sph[s0 + k] : R->grp[i]);
