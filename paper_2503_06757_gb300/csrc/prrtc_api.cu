@@ -1232,7 +1232,8 @@ static int plan_batch_impl(const prrtc_problem* problems, int32_t n, const prrtc
   for (size_t held_limit = lockstep ? kHeldFloats : kHeldFloats / 4;; held_limit /= 2) {
     rounds = lockstep || (ordered && held_floats * (size_t)kRoundsWarps <= held_limit);
     if (!rounds) break;
-    rcfg = rounds_launch_config(cfg, n, params->mode, blocks, warps, params->workers, held_floats, held_limit, c->sms);
+    rcfg = rounds_launch_config(cfg, n, params->mode, blocks, warps, params->workers, held_floats, held_limit,
+                                params->dd_radius > 0.f, c->sms);
     rc = grow_device(&c->d_held, &c->held_cap, held_floats * (size_t)rcfg.workers);
     if (!rc) rc = grow_device(&c->d_held_meta, &c->held_meta_cap, (size_t)n * rcfg.workers * kHeldMeta);
     if (!rc) break;
@@ -1469,8 +1470,8 @@ static int plan_batch_impl(const prrtc_problem* problems, int32_t n, const prrtc
   L.kernel_ms = plan_ms;
   L.setup_ms = setup_ms;
   L.grid = rounds ? rcfg.ph[0].grid : cfg.grid;
-  L.block_threads = (rounds ? rcfg.warps : cfg.warps) * 32;
-  L.smem_bytes = rounds ? rcfg.smem : cfg.smem;
+  L.block_threads = (rounds ? rcfg.ph[0].warps : cfg.warps) * 32;
+  L.smem_bytes = rounds ? rcfg.ph[0].smem : cfg.smem;
   L.problems = n;
   L.h2d_bytes = (int64_t)n * (int64_t)sizeof(ProblemDesc) + (int64_t)sizeof(PlanGlobals) +
                 (gathered ? (int64_t)(n + 1) * (int64_t)sizeof(int) : 0);

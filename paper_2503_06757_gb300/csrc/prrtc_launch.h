@@ -36,6 +36,8 @@ struct PlanGlobals {
   unsigned long long time_limit_ns;  // 0 = none
   int cursor;            // work-queue ticket counter
   int queue[3];          // the same, one per launch of the deterministic schedules
+  int left[2];           // problems that the first and the second of those left to the next
+  int closed;            // problems that have ended
   int error;             // device-side error code (PRRTC_ERR_*), 0 = none
   int error_info;
   uint32_t learned_thr;  // learned-vs-uniform draw as a threshold on the top 24 bits of a Philox word
@@ -132,6 +134,9 @@ struct ProblemState {
   unsigned long long dd_rejected;
   unsigned long long prim_tests[4];
   unsigned long long verdict_states;
+  // deterministic schedules: entry k of the lists of problems left to the second and third launch
+  int left[2];
+  int ahead;             // and how many rounds ran between two that changed a tree lately, x 16
   // arena bookkeeping, preserved across launches
   int used_rows[2];
   int used_dpad;
@@ -244,50 +249,54 @@ struct PlanLaunch {
 // Launches of the deterministic schedules (serial and lockstep mode): up to
 // three in a row, with growing clusters of blocks per problem.
 struct RoundsLaunch {
-  int warps;             // per block
-  int smem;
   int robot_bytes;
   int env_bytes;
   int stage_bytes;
   int workers;           // virtual workers of the largest cluster: slices of a problem's held rows
   int n_phases;
   struct Phase {
+    int warps;           // per block
+    int smem;
     int blocks;          // blocks of a cluster, which runs one problem
     int grid;
-    int it_limit;        // a problem with this many iterations is left to the next launch
+    int it_limit;        // from this many iterations on a problem is left to the next launch ...
+    int open;            // ... once this many problems or fewer are open
   } ph[3];
 };
 // Easy problems are solved within a few rounds of 16 workers and rarely let a
 // round of more of them count (one iteration in seven adds a row); the few
 // hard ones, which set the batch's time, add a row in a hundred iterations or
 // more and take all the workers they get.  So each launch gives what the one
-// before left a larger cluster.  How long it keeps them depends on how many
-// there are: a batch of more problems than SMs fills the GPU with small
-// clusters for longer (a problem's batches overlap less the larger its cluster
-// is), of fewer ones it leaves SMs idle.  Kernel time (ms; limits of the first /
-// second launch in iterations), sums over six sets of 200 shelf problems
+// before left a larger cluster: from a number of iterations on, once no more
+// problems are open than the next launch has clusters at once (Phase::open).
+// Where many stay open they keep their clusters: 35 of 90 problems in clusters
+// of 16, nine at a time, took twice as long as side by side in small ones, and
+// a part of them sent on ran after the rest.  Kernel time (ms; limits of the
+// first / second launch in iterations), sums over six sets of 200 shelf problems
 // (serial, lockstep), then sets of 400, 100 and 40:
-//   16 warps, clusters 1 / 4 / 16, 256 / 1024   22.5 16.5   5.74 3.57   2.13 1.36   1.05 0.77
-//   ... 256 / 2048                              21.2 15.8   5.10 3.42   2.14 1.46   0.96 0.75
-//   ... 384 / 4096                              19.8 15.5   4.72 3.20   2.21 1.52   0.95 0.75
-//   ... 512 / 4096                              20.0 15.9   4.62 3.10   2.19 1.52   0.96 0.75
-//   ... 256 / 8192                              20.8 16.9   5.31 3.67   2.15 1.98   0.97 0.76
-//   clusters 1 / 2 / 16, 256 / 2048             21.7 16.2   5.26 3.34   2.35 1.70   0.95 0.76
-//   clusters 1 / 8 / 16, 256 / 1024             24.0 17.6   6.22 4.05   2.23 1.46   1.06 0.76
-//   clusters 1 / 4 / 8, 256 / 1024              25.6 19.9   5.81 3.99   2.11 1.61   1.03 0.75
-//   12 warps, 256 / 1024                        23.5 18.2   5.98 3.98   2.05 1.42   0.96 0.77
-// (one warp a problem, one block a problem: 121 to 270 and 16 to 40 a set).
-constexpr int kRoundsWarps = 16;
+//   16 warps, clusters 1 / 4 / 16, 256 / 1024   16.7 13.8   3.64 2.69   1.62 1.24   0.89 0.70
+//   ... no smaller blocks at first              16.3 13.3   3.81 2.66   1.62 1.24   0.88 0.70
+//   ... 64 / 512                                16.2 13.9   3.63 2.74   1.59 1.21   0.97 0.77
+//   ... 384 / 4096                              18.1 15.0   3.77 2.75   2.07 1.42   0.94 0.73
+//   ... 768 / 8192                              20.2 17.6   4.20 3.30   2.11 1.86   0.94 0.73
+//   clusters 1 / 2 / 16                         18.5 14.7   4.09 2.96   1.84 1.29   0.89 0.69
+//   clusters 1 / 8 / 16                         18.0 16.0   3.81 2.98   1.44 1.09   0.88 0.70
+//   clusters 1 / 4 / 8                          21.3 18.2   4.23 3.31   1.79 1.37   0.92 0.70
+//   12 warps (6 at first)                       19.0 15.8   4.11 3.22   1.67 1.29   0.97 0.76
+// (one warp a problem, one block a problem: 121 to 270 and 16 to 40 a set).  The
+// smaller blocks of the first launch, two on an SM, are for batches of more
+// problems than SMs that are over soon: 200 problems of eight iterations 156 ->
+// 128 us with 8 workers a round, 50 of them waited for an SM before.
+constexpr int kRoundsWarps = 16, kRoundsManyWarps = 8;
 constexpr int kRoundsSmem = 226 * 1024;
 constexpr int kRoundsMidCluster = 4, kRoundsMaxCluster = 16;
-constexpr int kRoundsFirstIters = 384, kRoundsMidIters = 4096;
-constexpr int kRoundsFewFirstIters = 256, kRoundsFewMidIters = 1024;  // clusters of 1 for no more problems than SMs
+constexpr int kRoundsFirstIters = 256, kRoundsMidIters = 1024;
 
 // base: the launch of plan_launch_config for the same arguments.  held_floats:
 // floats of held rows per virtual worker, over all problems; held_limit: the
-// most that may be allocated.
+// most that may be allocated.  radii: dynamic domain is on.
 RoundsLaunch rounds_launch_config(const PlanLaunch& base, int n_problems, int mode, int blocks, int warps, int workers,
-                                  size_t held_floats, size_t held_limit, int sm_count);
+                                  size_t held_floats, size_t held_limit, bool radii, int sm_count);
 
 // The rule behind rounds_launch_config.  per_sm(warps, smem): resident blocks
 // of that shape; max_cluster(warps, smem): its largest cluster.  The held rows
@@ -296,7 +305,7 @@ RoundsLaunch rounds_launch_config(const PlanLaunch& base, int n_problems, int mo
 // checked.
 template <class PerSm, class MaxCluster>
 inline RoundsLaunch rounds_shape(const PlanLaunch& base, int n_problems, int mode, int blocks, int warps, int workers,
-                                 size_t held_floats, size_t held_limit, int sm_count, PerSm per_sm,
+                                 size_t held_floats, size_t held_limit, bool radii, int sm_count, PerSm per_sm,
                                  MaxCluster max_cluster) {
   RoundsLaunch c{};
   c.robot_bytes = base.robot_bytes;
@@ -304,33 +313,40 @@ inline RoundsLaunch rounds_shape(const PlanLaunch& base, int n_problems, int mod
   c.stage_bytes = base.stage_bytes + (int)sizeof(WarpCount);  // a second counter block per warp
   const bool fixed = mode == PRRTC_MODE_LOCKSTEP && warps > 0;  // the caller's warps per block
   const int B = mode == PRRTC_MODE_LOCKSTEP ? workers : 1;
-  // virtual workers of a cluster of C blocks, and whether their held rows fit
-  auto virt = [&](int C) { return std::max(C * c.warps / B, 1) * B; };
-  auto held = [&](int C) { return held_floats * (size_t)virt(C); };
-  c.warps = fixed ? base.warps : kRoundsWarps;
-  while (c.warps > 1 && c.robot_bytes + c.env_bytes + c.warps * c.stage_bytes > kRoundsSmem) --c.warps;
-  while (c.warps > B && held(1) > held_limit) --c.warps;
-  c.smem = c.robot_bytes + c.env_bytes + c.warps * c.stage_bytes;
-  const int resident = per_sm(c.warps, c.smem) * sm_count;
-  const int most = (fixed || blocks > 0) ? 1 : max_cluster(c.warps, c.smem);
-  auto fits = [&](int C) { return C <= most && held(C) <= held_limit; };
+  auto smem = [&](int w) { return c.robot_bytes + c.env_bytes + w * c.stage_bytes; };
+  // virtual workers of a cluster of C blocks of w warps
+  auto virt = [&](int C, int w) { return std::max(C * w / B, 1) * B; };
+  auto held = [&](int C, int w) { return held_floats * (size_t)virt(C, w); };
+  int w = fixed ? base.warps : kRoundsWarps;
+  while (w > 1 && smem(w) > kRoundsSmem) --w;
+  while (w > B && held(1, w) > held_limit) --w;
+  int most = (fixed || blocks > 0) ? 1 : max_cluster(w, smem(w));
+  if (radii)  // one round at a time, as a rule: no larger cluster than it has work for
+    for (int C = 1; C < most; C *= 2)
+      if (C * w >= B) most = C;
+  auto fits = [&](int C) { return C <= most && held(C, w) <= held_limit; };
   // the first launch: one wave of clusters
-  int first = 1;
-  while (n_problems * first * 2 <= sm_count && fits(2 * first)) first *= 2;
-  const bool few = first == 1 && n_problems <= sm_count;
-  int C = first;
+  int C = 1;
+  while (n_problems * C * 2 <= sm_count && fits(2 * C)) C *= 2;
   for (;;) {
-    RoundsLaunch::Phase& ph = c.ph[c.n_phases++];
+    RoundsLaunch::Phase& ph = c.ph[c.n_phases];
+    // more problems than SMs: two smaller blocks on each at first
+    const bool many = n_problems > sm_count && !fixed && c.n_phases == 0 && B <= kRoundsManyWarps;
+    ph.warps = many ? std::min(w, kRoundsManyWarps) : w;
+    ph.smem = smem(ph.warps);
     ph.blocks = C;
-    ph.grid = (blocks > 0 ? blocks : std::min(n_problems, std::max(resident / C, 1))) * C;
+    ph.grid = (blocks > 0 ? blocks : std::min(n_problems, std::max(per_sm(ph.warps, ph.smem) * sm_count / C, 1))) * C;
     ph.it_limit = INT_MAX;
-    c.workers = virt(C);
-    const int next = std::min(C == 1 ? kRoundsMidCluster : kRoundsMaxCluster, most);
+    ph.open = 0;
+    if (c.n_phases++) {
+      RoundsLaunch::Phase& prev = c.ph[c.n_phases - 2];
+      // each problem at once, or as many times as a round of many workers gets shorter
+      prev.open = ph.grid / C * std::max(1, std::min(C / prev.blocks, B / (prev.blocks * prev.warps)));
+    }
+    c.workers = std::max(c.workers, virt(C, ph.warps));
+    const int next = std::min(C < kRoundsMidCluster ? kRoundsMidCluster : kRoundsMaxCluster, most);
     if (next <= C || !fits(next) || c.n_phases == 3) break;
-    if (C == 1)
-      ph.it_limit = few ? kRoundsFewFirstIters : kRoundsFirstIters;
-    else
-      ph.it_limit = few ? kRoundsFewMidIters : kRoundsMidIters;
+    ph.it_limit = C == 1 ? kRoundsFirstIters : kRoundsMidIters;
     C = next;
   }
   return c;

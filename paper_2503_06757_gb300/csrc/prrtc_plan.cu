@@ -632,10 +632,10 @@ __device__ void worker(const Ctx& c) {
 //
 // What bounds a round is the latency of an edge check (13k cycles on average
 // with 16 warps on the SM: FK 5.7k, environment 6.3k, self pairs 1k), a batch
-// the slowest of its iterations (23k cycles on average, 47k the batch), and on
-// hard problems hundreds of rounds in a row add nothing (14,160 iterations for
-// 21 rows in one shelf problem).  200 shelf problems: serial 289 -> 4.4 ms a
-// call (one warp a problem before), lockstep with 8 workers 52 -> 3.5 ms (one
+// the slowest of its iterations (23k cycles on average, 47k the batch of 16),
+// and on hard problems hundreds of rounds in a row add nothing (14,160 iterations
+// for 21 rows in one shelf problem).  200 shelf problems, kernel: serial 76 ->
+// 2.2 ms (one warp a problem before), lockstep with 8 workers 15.5 -> 1.7 ms (one
 // block a problem, one round at a time).
 //
 // Virtual worker v runs on warp v / C of block v % C of the problem's cluster
@@ -807,38 +807,87 @@ __device__ __forceinline__ int ctl_word(const RoundCtl* ctl, int lane) {
   return v;
 }
 
-// The next batch of the problem, by lane 0 of the leading warp.
-__device__ __forceinline__ void plan_batch(PlanGlobals* g, const ProblemDesc* D, ProblemState* S, int it_limit,
-                                           int workers, RoundCtl* ctl) {
-  int stop = ld_volatile(&S->done) | ld_volatile(&S->solved) | (slice_over(g) ? 1 : 0);
-  const int it0 = ld_volatile(&S->iter);
+// How many rounds the next batch runs side by side: twice as many as ran of late
+// between two that changed a tree, less one; twice the rounds since the
+// last change if that is more.  What follows the first change is run again, and
+// every iteration makes its batch slower -- the slowest counts, and the warps
+// share the SM -- so where most rounds change something (open scenes; dynamic
+// domain: every edge moves a radius) few pay, and where hundreds add nothing all
+// do.  Only the schedule depends on it, not the results.  Serial plans, kernel,
+// with every warp of the cluster always at work / so / one warp a problem: one
+// problem among eight boxes 325 / 199 / 185 us, 60 with ten obstacles 26 / 20 /
+// 22 ms, 40 with a dynamic domain among eight boxes 53 / 23 / 22 ms; 200 shelf
+// problems 2.5 / 2.2 / 76 ms.
+struct RoundsAhead {
+  int len;      // rounds between two changes, x 16, smoothed
+  int run;      // rounds since the last change
+  int batches;
+};
+constexpr int kAheadStart = 2;  // iterations of a problem's first batch
+
+// When a launch leaves its problems to the next one, which has larger clusters:
+// from `iters` iterations on, once no more than `open` are left, so that each
+// gets a larger cluster at once.  All of them go or none: those that stayed
+// would run before the others, not beside them.
+struct RoundsLimit {
+  int iters, open;
+};
+
+__device__ __forceinline__ void rounds_done(RoundsAhead& a, int rounds, bool changed) {
+  a.run += rounds;
+  ++a.batches;
+  if (changed) {
+    a.len += (16 * min(a.run, 1 << 16) - a.len) / 4;
+    a.run = 0;
+  }
+}
+
+// The next batch of the problem, by lane 0 of the leading warp: iteration it0 on
+// trees of na and nb rows.  most: virtual workers of the cluster; phase: the
+// launch's place among the call's.  Nobody else changes the problem, so its
+// state is handed on instead of read back.
+__device__ __forceinline__ void plan_batch(PlanGlobals* g, ProblemState* S, ProblemState* states, int phase,
+                                           const RoundsLimit& lim, int most, const RoundsAhead& a, RoundCtl* ctl,
+                                           int it0, int na, int nb, bool ended) {
+  const int B = g->workers;
+  const int usual = a.len / 8 - 1;  // rounds
+  int stop = (ended || slice_over(g)) ? 1 : 0;
   if (!stop && it0 >= g->max_iters) {
     atomicExch(&S->done, 1);
-    stop = 1;
+    ended = true;
   }
-  if (!stop && g->time_limit_ns && globaltimer_ns() - g->t0 > g->time_limit_ns) {
+  if (!stop && !ended && g->time_limit_ns && globaltimer_ns() - g->t0 > g->time_limit_ns) {
     S->timed_out = 1;
     atomicExch(&S->done, 1);
+    ended = true;
+  }
+  if (ended) {
+    atomicAdd(&g->closed, 1);
     stop = 1;
   }
-  if (it0 >= it_limit) stop = 1;  // the next launch takes it from here
+  if (!stop && it0 >= lim.iters && (a.batches & 3) == 0 && g->n_problems - ld_volatile(&g->closed) <= lim.open) {
+    states[atomicAdd(&g->left[phase], 1)].left[phase] = (int)(S - states);
+    stop = 1;
+  }
+  if (stop) S->ahead = a.len;
   // line 3 at the start of the round: every worker extends the smaller tree
-  const int na = min(ld_volatile(&S->count[0]), D->cap), nb = min(ld_volatile(&S->count[1]), D->cap);
   ctl->stop = stop;
   ctl->it0 = it0;
   ctl->s = (na <= nb) ? 0 : 1;
   ctl->n_s = min(na, nb);
   ctl->n_o = max(na, nb);
-  ctl->nb = min(workers, g->max_iters - it0);
+  ctl->nb = min(min(max(max(usual, 2 * a.run), 1), most / B) * B, g->max_iters - it0);
 }
 
 // Batches of one problem by every warp of its cluster (uniform control flow:
 // every thread meets every barrier).  `total`: this warp's counters, to which
 // an iteration's counters (c.cnt) are added once it counts.
 template <bool kLean>
-__device__ __forceinline__ void rounds_problem(const Ctx& c, WarpCount* total, RoundCtl* ctl, int rank, int blocks,
-                                               int warp, int nwarps, int it_limit) {
+__device__ __forceinline__ void rounds_problem(const Ctx& c, ProblemState* states, WarpCount* total, RoundCtl* ctl,
+                                               int rank, int blocks, int warp, int nwarps, int phase,
+                                               const RoundsLimit& lim) {
   __shared__ int s_first, s_winner, s_total;  // the leading block's: round to append, its winner and rows
+  __shared__ RoundsAhead s_ahead;
   PlanGlobals* g = const_cast<PlanGlobals*>(c.g);
   const ProblemDesc* D = c.D;
   ProblemState* S = c.S;
@@ -851,7 +900,11 @@ __device__ __forceinline__ void rounds_problem(const Ctx& c, WarpCount* total, R
   unsigned long long* acc = reinterpret_cast<unsigned long long*>(total);
   unsigned long long* one = reinterpret_cast<unsigned long long*>(c.cnt);
   if (rank == 0 && threadIdx.x == 0) {
-    plan_batch(g, D, S, it_limit, batch, ctl);
+    s_ahead.len = S->ahead ? S->ahead : max(16 * kAheadStart / (2 * B), 8);
+    s_ahead.run = s_ahead.batches = 0;
+    plan_batch(g, S, states, phase, lim, batch, s_ahead, ctl, ld_volatile(&S->iter),
+               min(ld_volatile(&S->count[0]), cap), min(ld_volatile(&S->count[1]), cap),
+               (ld_volatile(&S->done) | ld_volatile(&S->solved)) != 0);
     ctl->committed = 0;
   }
   int ran = 0;  // iterations this warp ran in the batch before
@@ -870,7 +923,6 @@ __device__ __forceinline__ void rounds_problem(const Ctx& c, WarpCount* total, R
     // a warp has several virtual workers only where the batch is one round, all of which count
     for (int v = me; v < nb; v += slots)
       lockstep_iteration<kLean>(c, it0 + v, s, n_s, n_o, meta + v, D->held + (size_t)v * held_stride);
-    if (lane == 0) __threadfence();
     cluster_barrier(blocks);
     if (rank != 0) continue;
     // The leading block takes the rounds in order.
@@ -926,7 +978,10 @@ __device__ __forceinline__ void rounds_problem(const Ctx& c, WarpCount* total, R
         s_total = sum;
         S->iter = it0 + committed;
         ctl->committed = committed;
-        if (first == INT_MAX || sum == 0) plan_batch(g, D, S, it_limit, batch, ctl);
+        rounds_done(s_ahead, (committed + B - 1) / B, first != INT_MAX);
+        if (first == INT_MAX || sum == 0)
+          plan_batch(g, S, states, phase, lim, batch, s_ahead, ctl, it0 + committed, s ? n_o : n_s, s ? n_s : n_o,
+                     false);
       }
     }
     __syncthreads();
@@ -947,11 +1002,10 @@ __device__ __forceinline__ void rounds_problem(const Ctx& c, WarpCount* total, R
         if (lane < dpad) __stcg(D->nodes[s] + (size_t)idx * dpad + lane, __ldcg(src + (size_t)k * dpad + lane));
       }
     }
-    __threadfence();
     __syncthreads();
     if (warp == 0) {
-      const int w = s_winner;
-      if (lane == 0) S->count[s] = min(n_s + s_total, cap);
+      const int w = s_winner, rows = min(n_s + s_total, cap);
+      if (lane == 0) S->count[s] = rows;
       if (w >= 0) {
         const LockstepHeld h = load_held(meta + w);
         const int join_s = n_s + h.offset + h.n - 1;
@@ -968,10 +1022,9 @@ __device__ __forceinline__ void rounds_problem(const Ctx& c, WarpCount* total, R
         __threadfence();
         if (lane == 0) atomicExch(&S->done, 1);
       }
-      if (lane == 0) {
-        __threadfence();
-        plan_batch(g, D, S, it_limit, batch, ctl);
-      }
+      if (lane == 0)
+        plan_batch(g, S, states, phase, lim, batch, s_ahead, ctl, it0 + committed, s ? n_o : rows, s ? rows : n_o,
+                   w >= 0);
     }
   }
 }
@@ -984,7 +1037,7 @@ __device__ __forceinline__ void rounds_problem(const Ctx& c, WarpCount* total, R
 template <bool kLean>
 __global__ void __maxnreg__(128) rounds_kernel(PlanGlobals* __restrict__ g, const ProblemDesc* __restrict__ descs,
                                                ProblemState* __restrict__ states, int robot_bytes, int env_bytes,
-                                               int warp_floats, int blocks, int queue, int it_limit) {
+                                               int warp_floats, int blocks, int phase, RoundsLimit lim) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(16) RoundCtl ctl;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -996,10 +1049,15 @@ __global__ void __maxnreg__(128) rounds_kernel(PlanGlobals* __restrict__ g, cons
     if (rank == 0 && threadIdx.x == 0) {
       int p = -1;
       for (;;) {
-        const int t = atomicAdd(&g->queue[queue], 1);
+        const int t = atomicAdd(&g->queue[phase], 1);
+        if (phase) {  // what the launch before left
+          if (t < g->left[phase - 1]) p = states[t].left[phase - 1];
+          break;
+        }
         if (t >= g->n_problems) break;
         p = g->active ? g->active[t] : t;
         if (!ld_volatile(&states[p].done)) break;
+        atomicAdd(&g->closed, 1);
         p = -1;
       }
       ctl.prob = p;
@@ -1049,7 +1107,7 @@ __global__ void __maxnreg__(128) rounds_kernel(PlanGlobals* __restrict__ g, cons
     c.v.b = vecs + 2 * kMaxDof;
     c.stage = vecs + kWarpVecFloats;
     c.lane = lane;
-    rounds_problem<kLean>(c, total, &ctl, rank, blocks, warp, nwarps, it_limit);
+    rounds_problem<kLean>(c, states, total, &ctl, rank, blocks, warp, nwarps, phase, lim);
     __syncwarp();
     flush_counters(states + p, *total, lane);
     // every block has read the last control record before it is written again
@@ -1251,6 +1309,7 @@ __global__ void setup_kernel(const ProblemDesc* __restrict__ descs, ProblemState
       S->solved = 0;
       S->done = 0;
       S->timed_out = 0;
+      S->ahead = 0;
       S->pre_status = 0;
       S->s_tree = -1;
       S->join_s = S->join_o = -1;
@@ -1406,6 +1465,7 @@ static cudaLaunchConfig_t rounds_launch(int grid, int blocks, int warps, int sme
 // Largest cluster of the rounds kernels the device can hold at this block
 // shape: 16 blocks are beyond the portable size, so the device is asked.
 static int rounds_max_cluster(int warps, int smem) {
+  resident_blocks_per_sm(kRounds, warps, smem);  // sets the attributes that the device is asked with
   static std::mutex mu;
   static std::map<std::pair<int, int>, int> cache;
   int dev = 0;
@@ -1459,9 +1519,9 @@ PlanLaunch plan_launch_config(int n_problems, int mode, int blocks, int warps, i
 }
 
 RoundsLaunch rounds_launch_config(const PlanLaunch& base, int n_problems, int mode, int blocks, int warps, int workers,
-                                  size_t held_floats, size_t held_limit, int sm_count) {
+                                  size_t held_floats, size_t held_limit, bool radii, int sm_count) {
   return rounds_shape(
-      base, n_problems, mode, blocks, warps, workers, held_floats, held_limit, sm_count,
+      base, n_problems, mode, blocks, warps, workers, held_floats, held_limit, radii, sm_count,
       [](int w, int smem) { return resident_blocks_per_sm(kRounds, w, smem); }, rounds_max_cluster);
 }
 
@@ -1478,15 +1538,15 @@ cudaError_t launch_plan(const PlanGlobals* g, const ProblemDesc* desc, ProblemSt
 
 cudaError_t launch_rounds(const PlanGlobals* g, const ProblemDesc* desc, ProblemState* state, const RoundsLaunch& cfg,
                           bool lean, cudaStream_t stream) {
-  resident_blocks_per_sm(lean ? kRoundsLean : kRounds, cfg.warps, cfg.smem);
   auto* fn = lean ? rounds_kernel<true> : rounds_kernel<false>;
   for (int k = 0; k < cfg.n_phases; ++k) {
     const RoundsLaunch::Phase& ph = cfg.ph[k];
+    resident_blocks_per_sm(lean ? kRoundsLean : kRounds, ph.warps, ph.smem);  // sets the attributes
     cudaLaunchAttribute at{};
-    const cudaLaunchConfig_t lc = rounds_launch(ph.grid, ph.blocks, cfg.warps, cfg.smem, stream, &at);
+    const cudaLaunchConfig_t lc = rounds_launch(ph.grid, ph.blocks, ph.warps, ph.smem, stream, &at);
     const cudaError_t e = cudaLaunchKernelEx(&lc, fn, const_cast<PlanGlobals*>(g), desc, state, cfg.robot_bytes,
                                              cfg.env_bytes, cfg.stage_bytes / (int)sizeof(float), ph.blocks, k,
-                                             ph.it_limit);
+                                             RoundsLimit{ph.it_limit, ph.open});
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

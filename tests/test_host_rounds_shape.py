@@ -29,9 +29,9 @@ int main() {
             base.robot_bytes = 9000;
             base.env_bytes = 1600;
             base.stage_bytes = 11000;
-            const RoundsLaunch c = rounds_shape(base, n, mode, 0, given, workers, held, limit, 152,
+            const RoundsLaunch c = rounds_shape(base, n, mode, 0, given, workers, held, limit, false, 152,
                                                 [](int, int) { return 1; }, [](int, int) { return 16; });
-            printf("%d %d %d %d %d %zu %d %d %d %d\n", mode, workers, n, given, (int)part, held, c.warps, c.workers,
+            printf("%d %d %d %d %d %zu %d %d %d %d\n", mode, workers, n, given, (int)part, held, c.ph[c.n_phases - 1].warps, c.workers,
                    c.n_phases, c.ph[c.n_phases - 1].blocks);
           }
   return 0;
