@@ -182,7 +182,9 @@ typedef struct prrtc_params {
                              the budget runs out, ids claimed but not yet started are dropped */
   int32_t obstacle_tile;  /* primitives of each type tested per round of the warp-wide first
                              stage of the collision check (one or two per lane): 32 or 64;
-                             0 = 32.  The verdicts do not depend on it */
+                             0 = 32.  Async mode and the server; serial and lockstep mode
+                             take 32 (64 where a batch has no room for rounds side by side).
+                             The verdicts do not depend on it */
   int32_t reserved[2];
 } prrtc_params;
 

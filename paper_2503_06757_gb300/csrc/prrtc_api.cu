@@ -1634,8 +1634,9 @@ int prrtc_autotune(const prrtc_problem* problems, int32_t n, const prrtc_params*
   }
   for (size_t i = 0; i < cands.size(); ++i)
     if (cands[i].first == q.blocks && cands[i].second == q.warps_per_block) best_t = times[i];
-  // 2. obstacle tile: primitives per first-stage round (one or two per lane)
-  if (params->obstacle_tile == 0) {
+  // 2. obstacle tile: primitives per first-stage round (one or two per lane; the
+  //    rounds of serial mode always take one)
+  if (params->obstacle_tile == 0 && params->mode == PRRTC_MODE_ASYNC) {
     prrtc_params r = q;
     r.obstacle_tile = 64;
     double t = 0.0;

@@ -357,7 +357,7 @@ PlanLaunch plan_launch_config(int n_problems, int mode, int blocks, int warps, i
                               int max_env_f4, int sm_count, int workers = 1);
 
 // obstacle_tile: 64 launches the 64-obstacle-tile instance of the kernel,
-// anything else the 32 one.  lean: the
+// anything else the 32 one (launch_rounds always uses 32).  lean: the
 // instance without the learned mixture draw, the Halton sampler, distance
 // fields, oriented boxes and one-stage links; only for batches that use none of
 // them

@@ -63,3 +63,10 @@ def test_lockstep(name, workers):
     got = P.prrtc_plan_batch(items, P.params(**kw))
     for k in range(len(items)):
         same(got[k], want[k], (name, workers, k))
+
+
+def test_tuner_leaves_the_tile_of_serial_plans_alone():
+    """Serial rounds have one obstacle tile: the tuner does not choose between two."""
+    items = problems(W.arm7(), shelf(W.arm7(), 2), 4)
+    prm = P.params(mode=P.MODE_SERIAL, max_iters=50, tree_capacity=4096)
+    assert all(P.prrtc_autotune(items, prm, trials=1)[0].obstacle_tile == 32 for _ in range(12))
