@@ -1021,10 +1021,10 @@ int sm_count() {
 
 // The library's split of K: doubled while the 128 x 256 tiles fill less than
 // one wave and every range keeps kMinKTilesPerSplit K tiles.
-int auto_splits(int M, int N, int K) {
+int auto_splits(int M, int N, int K, int sms) {
   const int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN), k_tiles = (K + BK - 1) / BK;
   int splits = 1;
-  while (splits < kMaxSplits && tiles * (splits * 2) <= sm_count() && k_tiles / (splits * 2) >= kMinKTilesPerSplit)
+  while (splits < kMaxSplits && tiles * (splits * 2) <= sms && k_tiles / (splits * 2) >= kMinKTilesPerSplit)
     splits *= 2;
   return std::min(splits, k_tiles);
 }
@@ -1035,10 +1035,10 @@ int cluster_blocks(int M, int N, int splits, int bn) {
 
 // Tile width of the cluster kernel for a product, 0: not its size.  One wave:
 // two blocks per SM.
-int cluster_bn(int M, int N, int splits) {
+int cluster_bn(int M, int N, int splits, int sms) {
   if (splits > kMaxClusterSplits || (splits & (splits - 1))) return 0;
   for (int bn : {64, 128})
-    if (cluster_blocks(M, N, splits, bn) <= 2 * sm_count()) return bn;
+    if (cluster_blocks(M, N, splits, bn) <= 2 * sms) return bn;
   return 0;
 }
 
@@ -1050,8 +1050,8 @@ int cluster_bn(int M, int N, int splits) {
 // 50.2 / 46.6, 4096 94.6 / 83.1; 8192^3 633 / 578; 9728 x 4096 K 512 35.3 /
 // 40.3, 768 45.2 / 44.8, 1024 56.0 / 50.6.  The larger tiles may take more
 // waves, each a tenth shorter for its work.
-bool pair_pays(int M, int N, int k_tiles, int splits) {
-  const int sms = sm_count(), n = (N + BN - 1) / BN * splits;
+bool pair_pays(int M, int N, int k_tiles, int splits, int sms) {
+  const int n = (N + BN - 1) / BN * splits;
   if (sms < 2 || k_tiles <= 12 * splits) return false;
   auto waves = [](int units, int at_once) { return (units + at_once - 1) / at_once; };
   return 10 * waves((M + 2 * BM - 1) / (2 * BM) * n, sms / 2) <= 11 * waves((M + BM - 1) / BM * n, sms);
@@ -1115,9 +1115,9 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
   ep.k_tiles = (K + BK - 1) / BK;
   ep.m_pad = (M + BM - 1) / BM * BM;
   const int sms = sm_count();
-  int splits = splits_hint > 0 ? splits_hint : auto_splits(M, N, K);
+  int splits = splits_hint > 0 ? splits_hint : auto_splits(M, N, K, sms);
   splits = std::max(1, std::min(splits, std::min(kMaxSplits, ep.k_tiles)));
-  if (const int bn = cluster_bn(M, N, splits)) {
+  if (const int bn = cluster_bn(M, N, splits, sms)) {
     ClusterGroup g;
     g.n = 0;
     g.late = 0;
@@ -1127,7 +1127,7 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
     return rc ? rc : launch_cluster(bn, splits, ta, tb, g, grid, stream);
   }
   if (mask || (ta && !tb)) return PRRTC_ERR_UNSUPPORTED;
-  const bool pair = !ta && !tb && pair_pays(M, N, ep.k_tiles, splits);
+  const bool pair = !ta && !tb && pair_pays(M, N, ep.k_tiles, splits, sms);
   const int ctas = pair ? 2 : 1;
   ep.m_tiles = (M + BM * ctas - 1) / (BM * ctas);
   CUtensorMap ma, mb;
@@ -1166,6 +1166,7 @@ int gemm_gradients(const GradientProduct* p, int n, cudaStream_t stream) {
   g.n = 0;
   g.late = 1;
   int grid = 0, bn = 0, splits = 0;
+  const int sms = sm_count();
   auto flush = [&]() {
     const int rc = g.n ? launch_cluster(bn, splits, true, true, g, grid, stream) : PRRTC_OK;
     g.n = 0;
@@ -1175,14 +1176,14 @@ int gemm_gradients(const GradientProduct* p, int n, cudaStream_t stream) {
   int rc = PRRTC_OK;
   for (int i = 0; i < n && !rc; ++i) {
     const GradientProduct& q = p[i];
-    const int s = auto_splits(q.out, q.in, q.rows), w = cluster_bn(q.out, q.in, s);
+    const int s = auto_splits(q.out, q.in, q.rows, sms), w = cluster_bn(q.out, q.in, s, sms);
     if (!w) {  // from 4096 rows on: more splits than a cluster takes
       rc = gemm_bf16_ld(q.dz, q.out, q.h, q.in, q.out, q.in, q.rows, nullptr, 0, q.dw, q.in, nullptr, 0, stream, 0,
                         kTransA | kTransB, nullptr, 0);
       continue;
     }
     if (g.n && (g.n == kMaxGroup || w != bn || s != splits ||
-                grid + cluster_blocks(q.out, q.in, s, w) > 2 * sm_count()))
+                grid + cluster_blocks(q.out, q.in, s, w) > 2 * sms))
       rc = flush();
     bn = w;
     splits = s;
