@@ -589,12 +589,14 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 // [128 r / splits, 128 (r + 1) / splits) over all blocks in split order (the
 // sums of the second kernel, bit for bit) and writes the outputs.
 //
-// Launches in a row, bias, ReLU and BF16 output, in us (128 x 256 tiles and
-// second kernel before): 512 x 512 x 1024 5.6 (9.6), 512 x 512 x 512 5.4 (9.2),
-// 1024 x 4160 x 512 8.1 (15.5), 2048 x 1024 x 4160 19.5 (23.5), 512 x 1024 x
-// 4160 12.7 (12.5: there the eight partial tiles' exchange costs what the
-// second kernel did).  About 1 us goes to the launch, 0.9 to tensor memory and
-// the first loads, 0.3 to each K tile, 1 to the cluster barriers.
+// Launches in a row, bias, ReLU and BF16 output, in us: where the next one may
+// start early (the proposal's) / where not (a caller's) (128 x 256 tiles and
+// second kernel before): 512 x 512 x 1024 4.5 / 5.3 (9.6), 512 x 512 x 512 4.1 /
+// 4.9 (9.2), 1024 x 4160 x 512 8.3 / 8.6 (15.5), 2048 x 1024 x 4160 17.6 / 18.7
+// (23.5), 512 x 1024 x 4160 11.2 / 12.6 (12.5: there the eight partial tiles'
+// exchange costs what the second kernel did).  About 1 us goes to the launch, 0.9
+// to tensor memory and the first loads, 0.3 to each K tile, 1 to the cluster
+// barriers.
 //
 // Roles as above: warp 0 loads, warp 1 issues the MMAs, warps 2-5 read the
 // accumulator; all six add up.  The partial tile takes the ring's place: every
@@ -637,6 +639,9 @@ struct ClusterGroup {
   // gradients run beside the bias gradients and each other so (a training step
   // 109 -> 106 us).
   int late;
+  // The launch after this one may start before the outputs are written: only
+  // where that one is known to wait for this (kNextMayStart).
+  int early;
 };
 
 // Byte offset of 16-byte unit u of row i of a partial tile (rows of kBN
@@ -760,7 +765,7 @@ __global__ void __launch_bounds__(kClusterThreads, 2)
     }
     fence_before();
   }
-  let_next_start();
+  if (group.early) let_next_start();
   if (kSplits > 1)
     cluster_sync_all();
   else
@@ -1101,9 +1106,9 @@ int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, const OutMaps& om,
 // Host launcher used by the MLP code and the C ABI entry point.  splits_hint:
 // 0 = choose (split K while the tiles fill less than one wave), else forced.
 int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, int K, const float* bias, int relu,
-                 float* c32, int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint, int trans,
+                 float* c32, int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint, int flags,
                  const void* mask, int ldm) {
-  const int ta = trans & kTransA ? 1 : 0, tb = trans & kTransB ? 1 : 0;
+  const int ta = flags & kTransA ? 1 : 0, tb = flags & kTransB ? 1 : 0;
   if (M <= 0 || N <= 0 || K <= 0 || !a || !b || (!c32 && !c16)) return PRRTC_ERR_INVALID_ARG;
   if (K % 8 || N % 8 || (c32 && ldc32 % 4) || (c16 && ldc16 % 8)) return PRRTC_ERR_UNSUPPORTED;
   if (lda < (ta ? M : K) || ldb < (tb ? N : K) || lda % 8 || ldb % 8) return PRRTC_ERR_UNSUPPORTED;
@@ -1121,6 +1126,7 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
     ClusterGroup g;
     g.n = 0;
     g.late = 0;
+    g.early = flags & kNextMayStart ? 1 : 0;
     int grid = 0;
     const int rc = group_add(g, grid, bn, splits, a, lda, ta, b, ldb, tb, M, N, K, bias, relu, mask, ldm, c32, ldc32,
                              c16, ldc16);
@@ -1165,6 +1171,7 @@ int gemm_gradients(const GradientProduct* p, int n, cudaStream_t stream) {
   ClusterGroup g;
   g.n = 0;
   g.late = 1;
+  g.early = 1;
   int grid = 0, bn = 0, splits = 0;
   const int sms = sm_count();
   auto flush = [&]() {
@@ -1194,14 +1201,9 @@ int gemm_gradients(const GradientProduct* p, int n, cudaStream_t stream) {
   return rc ? rc : flush();
 }
 
-int gemm_bf16_split(const void* a, const void* b, int M, int N, int K, const float* bias, int relu, float* c32,
-                    int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint) {
-  return gemm_bf16_ld(a, K, b, K, M, N, K, bias, relu, c32, ldc32, c16, ldc16, stream, splits_hint, 0, nullptr, 0);
-}
-
 int gemm_bf16(const void* a, const void* b, int M, int N, int K, const float* bias, int relu, float* c32, int ldc32,
               void* c16, int ldc16, cudaStream_t stream) {
-  return gemm_bf16_split(a, b, M, N, K, bias, relu, c32, ldc32, c16, ldc16, stream, 0);
+  return gemm_bf16_ld(a, K, b, K, M, N, K, bias, relu, c32, ldc32, c16, ldc16, stream, 0, kNextMayStart, nullptr, 0);
 }
 
 // Changes whenever a split-K workspace is allocated or moved: work captured
@@ -1222,16 +1224,19 @@ cudaError_t gemm_read_error(int* out, cudaStream_t stream) {
 
 }  // namespace prrtc
 
-extern "C" int prrtc_gemm_bf16(const void* a, const void* b, int32_t M, int32_t N, int32_t K, const float* bias,
-                               int32_t relu, float* c32, void* c16, void* stream) {
-  return prrtc::gemm_bf16(a, b, M, N, K, bias, relu, c32, N, c16, N, static_cast<cudaStream_t>(stream));
-}
-
+// On the caller's stream nothing starts before the outputs are written, whatever
+// launch attributes it has: the next launch there is not the library's own.
 extern "C" int prrtc_gemm_bf16_splitk(const void* a, const void* b, int32_t M, int32_t N, int32_t K,
                                       const float* bias, int32_t relu, float* c32, void* c16, int32_t splits,
                                       void* stream) {
   if (splits < 0) return PRRTC_ERR_INVALID_ARG;
-  return prrtc::gemm_bf16_split(a, b, M, N, K, bias, relu, c32, N, c16, N, static_cast<cudaStream_t>(stream), splits);
+  return prrtc::gemm_bf16_ld(a, K, b, K, M, N, K, bias, relu, c32, N, c16, N, static_cast<cudaStream_t>(stream),
+                             splits, 0, nullptr, 0);
+}
+
+extern "C" int prrtc_gemm_bf16(const void* a, const void* b, int32_t M, int32_t N, int32_t K, const float* bias,
+                               int32_t relu, float* c32, void* c16, void* stream) {
+  return prrtc_gemm_bf16_splitk(a, b, M, N, K, bias, relu, c32, c16, 0, stream);
 }
 
 extern "C" int prrtc_gemm_error(void) { return prrtc::gemm_take_error(); }

@@ -458,14 +458,16 @@ int gemm_bf16(const void* a, const void* b, int M, int N, int K, const float* bi
               void* c16, int ldc16, cudaStream_t stream);
 // The same with row strides lda / ldb (elements, multiples of 8, >= K) of the
 // operands, e.g. a column range of a wider weight matrix; splits_hint 0 = auto.
-// trans: operands stored the other way round, A as [K x M] rows of lda >= M,
+// flags: operands stored the other way round, A as [K x M] rows of lda >= M,
 // B as [K x N] rows of ldb >= N (a gradient's operands as the layers wrote
 // them, without a transposed copy).  mask (nullable, BF16 [M x N], row stride
 // ldm): outputs become 0 where it is not above 0 (a ReLU's gradient);
-// PRRTC_ERR_UNSUPPORTED for products above one wave.
-constexpr int kTransA = 1, kTransB = 2;
+// PRRTC_ERR_UNSUPPORTED for products above one wave.  kNextMayStart: the next
+// launch on the stream calls wait_before() ahead of its first access to memory
+// (or is an ordinary one), so it may start up while this one still runs.
+constexpr int kTransA = 1, kTransB = 2, kNextMayStart = 4;
 int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, int K, const float* bias, int relu,
-                 float* c32, int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint, int trans,
+                 float* c32, int ldc32, void* c16, int ldc16, cudaStream_t stream, int splits_hint, int flags,
                  const void* mask, int ldm);
 // Weight gradients of n layers, dW [out x in] = dZ [rows x out]^T H [rows x
 // in], in as few launches as their sizes allow (all dimensions multiples of 8,

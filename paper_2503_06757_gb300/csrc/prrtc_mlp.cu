@@ -688,7 +688,7 @@ int backward_rows(prrtc_proposal* p, int rows) {
     // dH_{l-1} [rows x in] = dZ [rows x out] W_l [out x in]
     // and dZ_{l-1} = dH_{l-1} where H_{l-1} > 0, in the same launch while the product is below one wave
     rc = gemm_bf16_ld(dz16, out, p->w16[l], in, rows, in, out, nullptr, 0, p->z32[l - 1], in, p->z16[l - 1], in, s, 0,
-                      kTransB, p->h16[l - 1], in);
+                      kTransB | kNextMayStart, p->h16[l - 1], in);
     if (rc == PRRTC_ERR_UNSUPPORTED) {
       if ((rc = gemm_bf16_ld(dz16, out, p->w16[l], in, rows, in, out, nullptr, 0, p->dh32, in, nullptr, 0, s, 0,
                              kTransB, nullptr, 0)))
@@ -759,7 +759,7 @@ int enqueue_inference(prrtc_proposal* p, const EnvView* d_envs, int U, const int
     MCK(cudaMemsetAsync(p->xo16, 0, (size_t)U * kVox * sizeof(bf16), s));
     occupancy_scatter_kernel<<<scatter, 256, 0, s>>>(d_envs, p->xo16);
     if ((rc = gemm_bf16_ld(p->xo16, kVox, p->w16[0], kIn, U, kHid0, kVox, nullptr, 0, p->h1o32, kHid0, nullptr, 0, s,
-                           0, 0, nullptr, 0)))
+                           0, kNextMayStart, nullptr, 0)))
       return rc;
   }
   MCK(cudaGetLastError());
@@ -770,7 +770,7 @@ int enqueue_inference(prrtc_proposal* p, const EnvView* d_envs, int U, const int
   for (int l = 1; l < 4; ++l) {
     const int in = p->in_dim[l], out = p->out_dim[l];
     if ((rc = gemm_bf16_ld(p->ih16[l - 1], in, p->w16[l], in, rows, out, in, p->master + p->b_off[l], l < 3,
-                           l < 3 ? nullptr : p->out32, out, l < 3 ? p->ih16[l] : nullptr, out, s, 1, 0, nullptr, 0)))
+                           l < 3 ? nullptr : p->out32, out, l < 3 ? p->ih16[l] : nullptr, out, s, 1, kNextMayStart, nullptr, 0)))
       return rc;
   }
   const int head = kK * (1 + 2 * p->dof);
