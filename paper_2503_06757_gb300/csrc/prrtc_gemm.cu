@@ -1166,11 +1166,11 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
   return PRRTC_OK;
 }
 
-int gemm_gradients(const GradientProduct* p, int n, cudaStream_t stream) {
+int gemm_gradients(const GradientProduct* p, int n, bool ready, cudaStream_t stream) {
   // products of one shape of cluster share a launch while it stays one wave
   ClusterGroup g;
   g.n = 0;
-  g.late = 1;
+  g.late = ready ? 1 : 0;
   g.early = 1;
   int grid = 0, bn = 0, splits = 0;
   const int sms = sm_count();

@@ -471,14 +471,19 @@ int gemm_bf16_ld(const void* a, int lda, const void* b, int ldb, int M, int N, i
                  const void* mask, int ldm);
 // Weight gradients of n layers, dW [out x in] = dZ [rows x out]^T H [rows x
 // in], in as few launches as their sizes allow (all dimensions multiples of 8,
-// all pointers 16-byte aligned).
+// all pointers 16-byte aligned).  ready: the operands are complete and visible
+// before the launch ahead of this call on the stream lets the next one start --
+// it has called wait_before() by then, and writes none of them.  The products
+// then run beside it and each other without a wait of their own; with any other
+// launch ahead (or false) they would read operands that are still being written.
+// The launch after the call has to wait as usual.
 struct GradientProduct {
   const void* dz;
   const void* h;
   float* dw;
   int out, in, rows;
 };
-int gemm_gradients(const GradientProduct* p, int n, cudaStream_t stream);
+int gemm_gradients(const GradientProduct* p, int n, bool ready, cudaStream_t stream);
 int gemm_take_error();
 // Copies the kernels' error word to *out on `stream` (does not clear it).
 cudaError_t gemm_read_error(int* out, cudaStream_t stream);

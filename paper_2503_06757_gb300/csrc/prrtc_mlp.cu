@@ -705,10 +705,12 @@ int backward_rows(prrtc_proposal* p, int rows) {
     cs.first_block[l] = blocks;
     blocks += cs.cols[l] / 32;
   }
+  // Nothing may come between these two launches: the second reads what the first
+  // has waited for, without a wait of its own.
   MCK(launch_overlapped(colsum_kernel, blocks, 256, 0, s, 1, cs));
   // dW = dZ^T H of every layer, both as stored, beside the bias gradients and
   // one another: nothing waits for them but the update
-  return gemm_gradients(dw, 4, s);
+  return gemm_gradients(dw, 4, true, s);
 }
 
 int upload_samples(prrtc_proposal* p, const uint8_t* occ, int n_occ, const float* qs, const float* qg,
