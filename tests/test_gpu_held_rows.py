@@ -34,3 +34,17 @@ def test_lockstep_below_the_limit(workers):
     assert before - torch.cuda.mem_get_info()[0] <= 4 * LIMIT + (1 << 26)
     for k in range(len(items)):
         same(got[k], want[k], (workers, k))
+
+
+def test_serial_gives_large_scratch_back():
+    """70 problems of steps of 0.01: 150 MB of held rows, of which at most 64 MiB stay."""
+    robot = W.dual14()
+    items = problems(robot, shelf(robot, 2), 70)
+    kw = dict(mode=P.MODE_SERIAL, max_iters=3, tree_capacity=4096, path_capacity=4096)
+    span = np.linalg.norm(np.asarray(robot.upper) - np.asarray(robot.lower))
+    assert 1 << 27 < 4 * 16 * 70 * 16 * span / 0.01 < 1 << 28
+    P.prrtc_plan_batch(items, P.params(**kw))  # arenas and the usual scratch
+    before = torch.cuda.mem_get_info()[0]
+    for _ in range(2):
+        P.prrtc_plan_batch(items, P.params(range=0.01, **kw))
+        assert before - torch.cuda.mem_get_info()[0] <= 1 << 26
