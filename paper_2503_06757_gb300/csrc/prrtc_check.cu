@@ -1,9 +1,9 @@
 // prrtc_check.cu -- batched collision verdicts of given configurations
 // (Sec. III-A): sphere-model FK, sphere-vs-primitive and self-collision tests.
-// One lane per configuration; robot tables and the obstacle set are staged in
-// shared memory by TMA bulk copies.  Used for the per-state parity check
-// against the oracle and as the FP32-roofline microbenchmark (collision-free
-// states: every test must run).
+// A lane per configuration, or a warp for calls of few; robot tables and the
+// obstacle set are staged in shared memory by TMA bulk copies.  Used for the
+// per-state parity check against the oracle and as the FP32-roofline
+// microbenchmark.
 #include <algorithm>
 #include <array>
 #include <map>
@@ -18,7 +18,8 @@ namespace prrtc {
 namespace {
 
 constexpr int kMaxCheckWarps = 16;
-// Lanes that make a link pair's tests pay at once instead of through the queue.
+// Lanes that make a link's or a link pair's tests pay at once instead of waiting
+// for a full warp in the queue.
 constexpr int kDirect = 24;
 
 // Robot header, pair tables and the first env_f4 words of the environment into
@@ -194,8 +195,13 @@ __device__ __forceinline__ bool block_hits(const RobotHeader* __restrict__ R, co
 // primitive link by link, 5,900 now), and with 14 joints the latency of the
 // staged reads, because the centres of 32 states take 18 KB: the block takes
 // as many warps as the shared memory holds.  A million states in a shelf scene
-// of 50 obstacles: 481 -> 251 us (both arms 1457 -> 624); without obstacles
-// 144 -> 126 (761 -> 403).
+// of 50 obstacles: 500 -> 213 us (both arms 1711 -> 652); among 600 mixed ones
+// 4220 -> 1520.
+//
+// kTwoStage = false: robots without bounding spheres, with the two-stage check
+// off, distance fields and empty environments.  Spheres meet the obstacles one
+// by one; the queues only cost there (a million states of a point robot between
+// two boxes 43 -> 28 us, of the 7-DoF arm without obstacles 132 -> 93).
 template <bool kTwoStage>
 __global__ void __maxnreg__(128) check_states_kernel(
     const RobotDev* __restrict__ robot, EnvView env, const float* __restrict__ q, int n, uint8_t* __restrict__ valid,
@@ -289,6 +295,7 @@ __global__ void __maxnreg__(128) check_states_kernel(
     if (kTwoStage) {
       int queued = 0, done = 0;
       for (int i = dof - 1; i >= 0; --i) {
+        int enough = 32;
         if (R->sph_begin[i] != R->sph_begin[i + 1]) {
           const float* st = stage + s_bslot[i] * 96 + lane;
           const float r = R->grp[i].w * kReachSlack;
@@ -299,8 +306,12 @@ __global__ void __maxnreg__(128) check_states_kernel(
           const uint32_t m = __ballot_sync(kFull, near);
           if (near) queue[(queued + __popc(m & below)) & 63] = (uint16_t)(i << 5 | lane);
           queued += __popc(m);
+          // In clutter nearly every state has the link and most collide there: mixed
+          // with the next links they would be tested for nothing (both arms among 600
+          // obstacles, 100,000 states with centres 350 us when all wait, 320 so)
+          if (__popc(m) >= kDirect) enough = kDirect;
         }
-        while (queued - done >= 32 || (i == 0 && done < queued)) {
+        while (queued - done >= enough || (i == 0 && done < queued)) {
           __syncwarp();  // the queue and the hits
           const bool mine = done + lane < queued;
           const uint32_t code = queue[(mine ? done + lane : done) & 63];
@@ -437,7 +448,7 @@ __device__ __forceinline__ bool warp_link_stage(const float4* __restrict__ prims
 // The same verdicts for few states: one state per warp.  A lane per joint
 // takes its sine and cosine, every lane runs the chain, a lane per sphere
 // places it, a lane per primitive tests the links and a lane per pair the
-// pairs -- the arithmetic of the kernel below, so the verdicts and centres are
+// pairs -- the arithmetic of the kernel above, so the verdicts and centres are
 // the same.  A few states alone take a warp of the other kernel through every
 // link, primitive and pair in turn, and most of its lanes or warps are idle.
 constexpr int kStateWarps = 4;
