@@ -901,7 +901,7 @@ def run_ours(args):
         extra["ttfs_single_boxes8_ms"] = dict(percentiles(tt), success_rate=ok / 100, keys=100,
                                           launch=dict(blocks=p1.blocks, warps_per_block=p1.warps_per_block),
                                           workload="boxes8: 7-DoF arm, 8 random cuboids, one problem, keys 1..100")
-        # collision-check microbenchmark: collision-free shelf states, every test runs
+        # collision-check microbenchmark: collision-free shelf states, none ends a check early
         pb = probs[0]
         rb, ev = robots[pb.robot.name], envs[0]
         from paper_2503_06757_gb300 import workload as W
@@ -928,15 +928,18 @@ def run_ours(args):
             info = rb.info()
             alg_state = one_stage_ops_per_state(ec, pb.robot.dof, info["n_spheres"], info["n_pairs"])
             alg_gops = len(F) * alg_state / (kms * 1e-3) * 1e-9
+            executed = cc_ops / (kms * 1e-3) * 1e-9
             micro[name] = dict(
-                bound="alu", achieved=alg_gops, peak=peak_gops, unit="Gop/s", frac=alg_gops / peak_gops,
-                executed_gops=cc_ops / (kms * 1e-3) * 1e-9, executed_frac=cc_ops / (kms * 1e-3) * 1e-9 / peak_gops,
+                bound="alu", achieved=executed, peak=peak_gops, unit="Gop/s", frac=executed / peak_gops,
+                one_stage_equivalent_gops=alg_gops, one_stage_equivalent_frac=alg_gops / peak_gops,
                 states=int(len(F)), kernel_ms=kms, states_per_s=len(F) / (kms * 1e-3),
-                executed_ops_per_state=cc_ops / len(F), algorithmic_ops_per_state=alg_state)
+                executed_ops_per_state=cc_ops / len(F), one_stage_ops_per_state=alg_state)
         rb.set_two_stage(True)
         extra["roofline_cc_microbench"] = dict(micro["two_stage"], one_stage=micro["one_stage"],
-                                               workload="1M collision-free 7-DoF states vs one shelf scene "
-                                                        "(every test runs)")
+                                               workload="1M collision-free 7-DoF states vs one shelf scene",
+                                               note="counted as on the main line: bounding spheres and whole links "
+                                                    "skip the tests they rule out, which one_stage_equivalent prices "
+                                                    "all the same")
         # the roofline's denominator checked on the device: an FP32 FMA loop
         fma_rate, fma_ms = P.prrtc_alu_peak(16384)
         extra["alu_peak_microbench"] = dict(

@@ -746,8 +746,8 @@ uint64_t chain_signature(std::initializer_list<uint64_t> vals) {
 
 // Kernel chain of one inference batch on p->stream: occupancy grids of the
 // U distinct environments, the occupancy part of the first layer once per
-// environment, then one fused launch for the rest of the network and the
-// mixture parameters in the planner's rows.
+// environment, then its start / goal part, the three other layers and the
+// mixture parameters in the planner's rows, a launch each.
 int enqueue_inference(prrtc_proposal* p, const EnvView* d_envs, int U, const int* d_row_env, float* const* d_rows,
                       const float* d_qs, const float* d_qg, int B, int rows) {
   const cudaStream_t s = p->stream;
@@ -872,8 +872,7 @@ int prrtc_internal_proposal_stage(prrtc_proposal* p, const EnvView* envs, const 
        (uint64_t)(uintptr_t)p->h1o32, (uint64_t)(uintptr_t)p->wq, (uint64_t)(uintptr_t)p->ih16[0],
        (uint64_t)(uintptr_t)p->ih16[1], (uint64_t)(uintptr_t)p->ih16[2],
        (uint64_t)(uintptr_t)p->d_stage, (uint64_t)(uintptr_t)p->inf_occ,
-       (uint64_t)(uintptr_t)p->x16, (uint64_t)(uintptr_t)p->h16[0], (uint64_t)(uintptr_t)p->h16[1],
-       (uint64_t)(uintptr_t)p->h16[2], (uint64_t)(uintptr_t)p->out32, (uint64_t)(uintptr_t)p->w16[0],
+       (uint64_t)(uintptr_t)p->out32, (uint64_t)(uintptr_t)p->w16[0],
        (uint64_t)(uintptr_t)p->w16[1], (uint64_t)(uintptr_t)p->w16[2], (uint64_t)(uintptr_t)p->w16[3],
        (uint64_t)(uintptr_t)p->master, (uint64_t)(uintptr_t)p->d_lims, gemm_workspace_epoch()});
   p->pend_ok = true;
