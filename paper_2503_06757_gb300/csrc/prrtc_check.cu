@@ -190,9 +190,9 @@ __device__ __forceinline__ bool block_hits(const RobotHeader* __restrict__ R, co
 // fifty, other ones in every lane; in clutter most states collide at their
 // first link, which empties the warp early.
 //
-// What bounds it is instruction issue (75 - 85% of the slots; 10,100
+// What bounds it is instruction issue and its latencies (63% of the slots; 10,100
 // instructions per 32 states of the 7-DoF arm when every lane met every
-// primitive link by link, 5,900 now), and with 14 joints the latency of the
+// primitive link by link, 4,600 now), and with 14 joints the latency of the
 // staged reads, because the centres of 32 states take 18 KB: the block takes
 // as many warps as the shared memory holds.  A million states in a shelf scene
 // of 50 obstacles: 500 -> 213 us (both arms 1711 -> 652); among 600 mixed ones
@@ -656,9 +656,10 @@ static cudaError_t check_wave(const CheckShape& shape, bool two_stage, CheckWave
   return cudaSuccess;
 }
 
-// States up to which a warp each is faster than a lane each: 64 states of the
-// 7-DoF arm 13 / 17 us, of both arms 13 / 29; 4000 14 / 19 and 22 / 31; 8000
-// 21 / 18 and 35 / 31.
+// States up to which a warp each is faster than a lane each.  Either way at the
+// line (us, 6000 states a warp each / 6100 a lane each): 7-DoF arm in a shelf
+// 17.8 / 17.6, among eight boxes 15.6 / 14.9, among 600 obstacles 33 / 70; both
+// arms in a shelf 30.5 / 34.0.  64 states a warp each take 10, 10, 17 and 14.5.
 constexpr int kWarpPerState = 6000;
 
 static cudaError_t state_warps_attribute() {
