@@ -635,7 +635,7 @@ __device__ void worker(const Ctx& c) {
 // the slowest of its iterations (23k cycles on average, 47k the batch of 16),
 // and on hard problems hundreds of rounds in a row add nothing (14,160 iterations
 // for 21 rows in one shelf problem).  200 shelf problems, kernel: serial 76 ->
-// 2.2 ms (one warp a problem before), lockstep with 8 workers 15.5 -> 1.7 ms (one
+// 2.0 ms (one warp a problem before), lockstep with 8 workers 15.4 -> 1.6 ms (one
 // block a problem, one round at a time).
 //
 // Virtual worker v runs on warp v / C of block v % C of the problem's cluster
@@ -772,16 +772,22 @@ __device__ __forceinline__ void flush_counters(ProblemState* S, const WarpCount&
 }
 
 // What the leading block tells its cluster about the next batch; kept in its
-// shared memory and read by every warp after the cluster barrier.
+// shared memory and read by every warp after the barrier.  A batch of a few
+// iterations is the leading block's alone: the others wait for the next one that
+// is not (two cluster barriers and a read of remote memory cost 2 us a batch).
 struct RoundCtl {
   int stop;        // 1: leave the problem
   int it0;         // first iteration of the batch
   int s, n_s, n_o; // tree extended by every iteration, and the trees' rows
   int nb;          // iterations of the batch
-  int committed;   // iterations of the batch before that count
+  int all;         // 1: for every block
+  int committed;   // iterations of the batch before that count: the leading block's ...
+  int committed_all;  // ... and those of the last batch for every block
   int prob;        // problem to run, -1: none left
 };
-static_assert(sizeof(RoundCtl) == 8 * sizeof(int), "one int per lane");
+constexpr int kCtlWords = 10;
+static_assert(sizeof(RoundCtl) == kCtlWords * sizeof(int), "one int per lane");
+constexpr int kAloneIters = 4;  // warps that share an SM without slowing each other
 
 // Barrier over the problem's blocks; global and shared writes before it are
 // visible after it.
@@ -794,10 +800,10 @@ __device__ __forceinline__ void cluster_barrier(int blocks) {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Word `lane` (lane < 8) of the leading block's control record.
+// Word `lane` of the leading block's control record.
 __device__ __forceinline__ int ctl_word(const RoundCtl* ctl, int lane) {
   int v = 0;
-  if (lane < 8) {
+  if (lane < kCtlWords) {
     uint32_t remote;
     asm volatile("mapa.shared::cluster.u32 %0, %1, 0;"
                  : "=r"(remote)
@@ -808,16 +814,16 @@ __device__ __forceinline__ int ctl_word(const RoundCtl* ctl, int lane) {
 }
 
 // How many rounds the next batch runs side by side: twice as many as ran of late
-// between two that changed a tree, less one; twice the rounds since the
-// last change if that is more.  What follows the first change is run again, and
-// every iteration makes its batch slower -- the slowest counts, and the warps
-// share the SM -- so where most rounds change something (open scenes; dynamic
-// domain: every edge moves a radius) few pay, and where hundreds add nothing all
-// do.  Only the schedule depends on it, not the results.  Serial plans, kernel,
-// with every warp of the cluster always at work / so / one warp a problem: one
-// problem among eight boxes 325 / 199 / 185 us, 60 with ten obstacles 26 / 20 /
-// 22 ms, 40 with a dynamic domain among eight boxes 53 / 23 / 22 ms; 200 shelf
-// problems 2.5 / 2.2 / 76 ms.
+// between two that changed a tree, less one, or twice the rounds since the last
+// change if that is more.  What follows the first change is run again, and every
+// iteration makes its batch slower -- the slowest counts, and the warps share the
+// SM -- so where most rounds change something (open scenes; dynamic domain: every
+// edge moves a radius) few pay, and where hundreds add nothing all do.  Only the
+// schedule depends on it, not the results.  Serial plans, kernel, with every warp
+// of the cluster always at work / so / one warp a problem: one problem among eight
+// boxes 325 / 185 / 185 us, 60 with ten obstacles 26 / 20 / 22 ms, 40 with a
+// dynamic domain among eight boxes 53 / 22 / 22 ms; 200 shelf problems 2.5 / 2.0 /
+// 76 ms.
 struct RoundsAhead {
   int len;      // rounds between two changes, x 16, smoothed
   int run;      // rounds since the last change
@@ -847,8 +853,8 @@ __device__ __forceinline__ void rounds_done(RoundsAhead& a, int rounds, bool cha
 // launch's place among the call's.  Nobody else changes the problem, so its
 // state is handed on instead of read back.
 __device__ __forceinline__ void plan_batch(PlanGlobals* g, ProblemState* S, ProblemState* states, int phase,
-                                           const RoundsLimit& lim, int most, const RoundsAhead& a, RoundCtl* ctl,
-                                           int it0, int na, int nb, bool ended) {
+                                           const RoundsLimit& lim, int most, int alone, const RoundsAhead& a,
+                                           RoundCtl* ctl, int it0, int na, int nb, bool ended) {
   const int B = g->workers;
   const int usual = a.len / 8 - 1;  // rounds
   int stop = (ended || slice_over(g)) ? 1 : 0;
@@ -876,7 +882,9 @@ __device__ __forceinline__ void plan_batch(PlanGlobals* g, ProblemState* S, Prob
   ctl->s = (na <= nb) ? 0 : 1;
   ctl->n_s = min(na, nb);
   ctl->n_o = max(na, nb);
-  ctl->nb = min(min(max(max(usual, 2 * a.run), 1), most / B) * B, g->max_iters - it0);
+  const int iters = min(min(max(max(usual, 2 * a.run), 1), most / B) * B, g->max_iters - it0);
+  ctl->nb = iters;
+  ctl->all = stop || iters > alone;
 }
 
 // Batches of one problem by every warp of its cluster (uniform control flow:
@@ -895,35 +903,40 @@ __device__ __forceinline__ void rounds_problem(const Ctx& c, ProblemState* state
   const int B = g->workers, dpad = D->dpad, cap = D->cap, lane = c.lane;
   const int slots = blocks * nwarps;             // warps of the cluster
   const int batch = max(slots / B, 1) * B;       // virtual workers: whole rounds
-  const int me = warp * blocks + rank;
+  const int alone = min(kAloneIters, nwarps);
   const size_t held_stride = (size_t)D->held_rows * dpad;
   unsigned long long* acc = reinterpret_cast<unsigned long long*>(total);
   unsigned long long* one = reinterpret_cast<unsigned long long*>(c.cnt);
   if (rank == 0 && threadIdx.x == 0) {
     s_ahead.len = S->ahead ? S->ahead : max(16 * kAheadStart / (2 * B), 8);
     s_ahead.run = s_ahead.batches = 0;
-    plan_batch(g, S, states, phase, lim, batch, s_ahead, ctl, ld_volatile(&S->iter),
+    plan_batch(g, S, states, phase, lim, batch, alone, s_ahead, ctl, ld_volatile(&S->iter),
                min(ld_volatile(&S->count[0]), cap), min(ld_volatile(&S->count[1]), cap),
                (ld_volatile(&S->done) | ld_volatile(&S->solved)) != 0);
-    ctl->committed = 0;
+    ctl->committed = ctl->committed_all = 0;
   }
-  int ran = 0;  // iterations this warp ran in the batch before
+  int me = INT_MAX;  // this warp's first virtual worker in the batch before
   for (;;) {
-    cluster_barrier(blocks);
+    if (rank == 0) __syncthreads();  // the control record
+    if (rank != 0 || (blocks > 1 && ctl->all)) cluster_barrier(blocks);
     const int word = ctl_word(ctl, lane);
     // the iterations of the batch before count, or are forgotten
-    if (ran && me < __shfl_sync(kFull, word, 6)) {
+    if (me < __shfl_sync(kFull, word, rank == 0 ? 7 : 8)) {
       if (lane < 14) acc[lane] += one[lane];
     }
     warp_count_clear(c.cnt, lane);
     if (__shfl_sync(kFull, word, 0)) break;
     const int it0 = __shfl_sync(kFull, word, 1), s = __shfl_sync(kFull, word, 2), n_s = __shfl_sync(kFull, word, 3);
-    const int n_o = __shfl_sync(kFull, word, 4), nb = __shfl_sync(kFull, word, 5);
-    ran = me < nb ? 1 : 0;
+    const int n_o = __shfl_sync(kFull, word, 4), nb = __shfl_sync(kFull, word, 5), all = __shfl_sync(kFull, word, 6);
+    me = all ? warp * blocks + rank : warp;
     // a warp has several virtual workers only where the batch is one round, all of which count
     for (int v = me; v < nb; v += slots)
       lockstep_iteration<kLean>(c, it0 + v, s, n_s, n_o, meta + v, D->held + (size_t)v * held_stride);
-    cluster_barrier(blocks);
+    if (me >= nb) me = INT_MAX;
+    if (all)
+      cluster_barrier(blocks);
+    else
+      __syncthreads();
     if (rank != 0) continue;
     // The leading block takes the rounds in order.
     if (warp == 0) {
@@ -978,9 +991,10 @@ __device__ __forceinline__ void rounds_problem(const Ctx& c, ProblemState* state
         s_total = sum;
         S->iter = it0 + committed;
         ctl->committed = committed;
+        if (all) ctl->committed_all = committed;
         rounds_done(s_ahead, (committed + B - 1) / B, first != INT_MAX);
         if (first == INT_MAX || sum == 0)
-          plan_batch(g, S, states, phase, lim, batch, s_ahead, ctl, it0 + committed, s ? n_o : n_s, s ? n_s : n_o,
+          plan_batch(g, S, states, phase, lim, batch, alone, s_ahead, ctl, it0 + committed, s ? n_o : n_s, s ? n_s : n_o,
                      false);
       }
     }
@@ -1023,7 +1037,7 @@ __device__ __forceinline__ void rounds_problem(const Ctx& c, ProblemState* state
         if (lane == 0) atomicExch(&S->done, 1);
       }
       if (lane == 0)
-        plan_batch(g, S, states, phase, lim, batch, s_ahead, ctl, it0 + committed, s ? n_o : rows, s ? rows : n_o,
+        plan_batch(g, S, states, phase, lim, batch, alone, s_ahead, ctl, it0 + committed, s ? n_o : rows, s ? rows : n_o,
                    w >= 0);
     }
   }
@@ -1063,7 +1077,7 @@ __global__ void __maxnreg__(128) rounds_kernel(PlanGlobals* __restrict__ g, cons
       ctl.prob = p;
     }
     cluster_barrier(blocks);
-    const int p = __shfl_sync(kFull, ctl_word(&ctl, lane), 7);
+    const int p = __shfl_sync(kFull, ctl_word(&ctl, lane), 9);
     if (p < 0) break;
     const ProblemDesc* D = descs + p;
     const int np_pad = (D->n_pairs + 3) & ~3;
